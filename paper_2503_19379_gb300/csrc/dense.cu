@@ -6,6 +6,7 @@
 
 #include "dfloat.cuh"
 #include "pc_internal.cuh"
+#include "sliced.cuh"
 
 namespace pc {
 
@@ -135,14 +136,31 @@ __global__ void __launch_bounds__(256) gram_tile_partial_kernel(const cplx<T> *_
     }
 }
 
+// Sum of nchunk partial sums, `stride` elements apart, in eight interleaved sums added pairwise: their loads are
+// independent (one chain of loads and adds per chunk was the kernel's time), and the rounding of the sum grows with
+// nchunk / 8.
+__device__ __forceinline__ double2 sum_chunks(const double2 *__restrict__ part, long stride, int nchunk) {
+  double2 s[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) s[u] = cmake<double2>(0.0, 0.0);
+  for (int c = 0; c < nchunk; c += 8) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (c + u < nchunk) s[u] = cadd(s[u], part[(c + u) * stride]);
+  }
+#pragma unroll
+  for (int w = 4; w > 0; w >>= 1)
+#pragma unroll
+    for (int u = 0; u < w; ++u) s[u] = cadd(s[u], s[u + w]);
+  return s[0];
+}
+
 __global__ void gram_reduce_kernel(const double2 *__restrict__ part, int nchunk, int p, int q,
                                    const int *__restrict__ act, double2 *__restrict__ G, long sg) {
   const int bi = blockIdx.x;
   const int b = act ? act[bi] : bi;
   for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < p * q; i += gridDim.y * blockDim.x) {
-    double2 s = cmake<double2>(0.0, 0.0);
-    for (int c = 0; c < nchunk; ++c) s = cadd(s, part[((long)bi * nchunk + c) * p * q + i]);
-    G[(long)b * sg + i] = s;
+    G[(long)b * sg + i] = sum_chunks(part + (long)bi * nchunk * p * q + i, (long)p * q, nchunk);
   }
 }
 
@@ -152,9 +170,11 @@ static int gram_chunks(int nb, long L) {
   return (int)std::min<long>(std::min(want, maxc), 256);
 }
 
-// partial sums per k-point that either Gram path may write: the CUDA-core kernels' chunks, or the tensor-core
-// kernel's (at least tc_min_chunks)
-static int gram_scratch_chunks(int nb, long L) { return std::max(gram_chunks(nb, L), tc_min_chunks(L)); }
+// partial sums per k-point that any Gram path may write: the CUDA-core kernels' chunks, the complex64 tensor-core
+// kernel's (at least tc_min_chunks) and the sliced FP64 kernel's
+static int gram_scratch_chunks(int nb, long L) {
+  return std::max({gram_chunks(nb, L), tc_min_chunks(L), sl_gram_chunks(nb, L)});
+}
 
 size_t gram_scratch_bytes(int nb, long L, int p, int q) {
   return sizeof(double2) * (size_t)nb * gram_scratch_chunks(nb, L) * p * q;
@@ -167,25 +187,28 @@ int launch_gram(int nb, long L, int p, int q, int dtype, const void *A, long sa,
     const int rc = launch_gram_tc(nb, L, p, q, A, sa, B, sb, G, scratch, scratch_bytes, st, act, nb_alloc, sg);
     if (rc != PC_EUNSUPPORTED) return rc;
   }
-  const int nchunk = gram_chunks(nb, L);
   if (gram_scratch_bytes(nb, L, p, q) > scratch_bytes) {
     set_error("gram: scratch too small");
     return PC_EINVAL;
   }
+  if (dtype == PC_C128) {
+    int c = 0;
+    const int rc = launch_gram_sl(nb, L, p, q, PC_C128, A, sa, B, sb, SL_GENERAL, static_cast<double2 *>(scratch),
+                                  gram_scratch_chunks(nb, L), &c, st, act);
+    if (rc) return rc;
+    launch_gram_reduce(nb, c, p, q, static_cast<double2 *>(scratch), act, G, st, sg);
+    PC_CK_LAUNCH();
+    return PC_OK;
+  }
+  const int nchunk = gram_chunks(nb, L);
   long chunk = (L + nchunk - 1) / nchunk;
   chunk = (chunk + GRAM_TL - 1) / GRAM_TL * GRAM_TL;
   double2 *part = static_cast<double2 *>(scratch);
   const int R = std::max(p, q) <= 32 ? 2 : 4;
   const dim3 blk((q + R - 1) / R, (p + R - 1) / R);
-  if (R == 2 && dtype == PC_C128)
-    gram_tile_partial_kernel<double, 2><<<dim3(nchunk, 1, nb), blk, 0, st>>>(
-        static_cast<const double2 *>(A), sa, static_cast<const double2 *>(B), sb, L, p, q, chunk, part, act);
-  else if (R == 2)
+  if (R == 2)
     gram_tile_partial_kernel<float, 2><<<dim3(nchunk, 1, nb), blk, 0, st>>>(
         static_cast<const float2 *>(A), sa, static_cast<const float2 *>(B), sb, L, p, q, chunk, part, act);
-  else if (dtype == PC_C128)
-    gram_partial_kernel<double><<<dim3(nchunk, 1, nb), 256, 0, st>>>(
-        static_cast<const double2 *>(A), sa, static_cast<const double2 *>(B), sb, L, p, q, chunk, part, act);
   else
     gram_partial_kernel<float><<<dim3(nchunk, 1, nb), 256, 0, st>>>(
         static_cast<const float2 *>(A), sa, static_cast<const float2 *>(B), sb, L, p, q, chunk, part, act);
@@ -284,11 +307,8 @@ __global__ void gram_pair_reduce_kernel(const double2 *__restrict__ partG, const
   for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < p * p; e += gridDim.y * blockDim.x) {
     const int i = e / p, j = e - i * p;
     if (i > j) continue;
-    double2 sg = cmake<double2>(0.0, 0.0), sh = sg;
-    for (int c = 0; c < nchunk; ++c) {
-      sg = cadd(sg, partG[((long)bi * nchunk + c) * p * p + e]);
-      sh = cadd(sh, partH[((long)bi * nchunk + c) * p * p + e]);
-    }
+    double2 sg = sum_chunks(partG + (long)bi * nchunk * p * p + e, (long)p * p, nchunk);
+    double2 sh = sum_chunks(partH + (long)bi * nchunk * p * p + e, (long)p * p, nchunk);
     if (i == j) {
       sg.y = 0.0;
       sh.y = 0.0;
@@ -352,12 +372,16 @@ int launch_gram_pair(int nb, long L, int p, int dtype, const void *S, const void
     const int rc = launch_gram_pair_tc(nb, L, p, S, AS, ss, G, H, scratch, scratch_bytes, st, act, nb_alloc, sg);
     if (rc != PC_EUNSUPPORTED) return rc;
   }
-  const int nchunk = gram_chunks(nb, L);
-  long chunk = (L + nchunk - 1) / nchunk;
-  chunk = (chunk + GRAM_TL - 1) / GRAM_TL * GRAM_TL;
   double2 *part = static_cast<double2 *>(scratch);
-  int rc = dtype == PC_C128 ? launch_gram_pair_t<double>(nb, L, p, S, AS, ss, part, nchunk, chunk, st, act)
-                            : launch_gram_pair_t<float>(nb, L, p, S, AS, ss, part, nchunk, chunk, st, act);
+  int nchunk = gram_chunks(nb, L), rc;
+  if (dtype == PC_C128) {
+    rc = launch_gram_sl(nb, L, p, p, PC_C128, S, ss, AS, ss, SL_PAIR, part, gram_scratch_chunks(nb, L), &nchunk, st,
+                        act);
+  } else {
+    long chunk = (L + nchunk - 1) / nchunk;
+    chunk = (chunk + GRAM_TL - 1) / GRAM_TL * GRAM_TL;
+    rc = launch_gram_pair_t<float>(nb, L, p, S, AS, ss, part, nchunk, chunk, st, act);
+  }
   if (rc) return rc;
   gram_pair_reduce_kernel<<<dim3(nb, (p * p + 255) / 256), 256, 0, st>>>(
       part, part + (size_t)nb * nchunk * p * p, nchunk, p, act, static_cast<double2 *>(G), static_cast<double2 *>(H),

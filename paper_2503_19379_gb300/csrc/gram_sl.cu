@@ -1,0 +1,351 @@
+// Gram products of FP64-accurate panels on the tensor cores: complex128 panels (the FP64 solve) and double-float pairs
+// (the mixed solve's block X), sliced exactly into FP16 digits (sliced.cuh).
+//
+// D = A^H B over the L rows, as one real product of the columns' real and imaginary parts: accumulator row 2 i + c is
+// part c of column i of A (M = 128, at most 64 columns), accumulator columns 2 j + c' the parts of a block of up to 32
+// columns of B, once per level. Re = D[re,re] + D[im,im] and Im = D[re,im] - D[im,re] are added as integers.
+//
+// One CTA (17 warps, one CTA per SM) takes a chunk of rows and a block of columns. It works through the chunk in spans
+// of SG_SUPER rows, which share one exponent per column (found by a scan of the span; the second read comes from the
+// L2 cache), in stages of 32 rows: 16 warps turn the stage's elements into digits in the K-major tiles of the tensor
+// core (128-byte swizzle; two stages side by side in the 64-wide tile, so that the digits of one stage are formed while
+// the MMAs of the stage before run), the 17th issues the MMAs, and after every fourth stage (128 rows, the most that
+// FP32 holds exactly) the level sums are drained into 64-bit integer sums in registers. At the end of a span these are
+// scaled and added to FP64 sums in shared memory.
+//
+// Bound: integer instructions of the digit extraction. The pair A^H A, A^H B therefore takes the block's columns of A
+// and of B in one CTA, and the columns of A that the block shares with the left operand are extracted once and stored
+// twice.
+#include <cuda.h>
+#include <cuda_runtime.h>
+
+#include "sliced.cuh"
+
+namespace pc {
+
+namespace {
+
+constexpr int SG_CONV = 512;                  // threads that form digits and drain
+constexpr int SG_THREADS = SG_CONV + 32;      // and the warp that issues the MMAs
+constexpr int SG_ROWS = 32;                   // rows per stage
+constexpr int SG_GROUP = 4;                   // stages per drain
+constexpr int SG_SUPER = 1024;                // rows per common exponent
+constexpr int SG_ND = 7;
+constexpr int SG_TASKS = 3;                   // (64 + 32 columns) x 16 row pairs over 512 threads
+
+__device__ int g_gram_sl_error = 0;
+
+struct SlGramArgs {
+  const void *A, *B;
+  long sa, sb;
+  long L, chunk;
+  int p, q, mode;
+  int nbc, nbp;  // columns per block; accumulator columns per level (2 per operand column, rounded up to 16)
+  double2 *part0, *part1;
+  const int *act;
+};
+
+__device__ __forceinline__ void named_arrive(int id, int count) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+__device__ __forceinline__ void named_sync(int id, int count) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+
+template <typename T>
+__global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs a) {
+  constexpr int ND = SG_ND;
+  extern __shared__ unsigned char smem_raw[];
+  const uint32_t raw = smem_addr(smem_raw);
+  const uint32_t base = (raw + 1023u) & ~1023u;
+  unsigned char *const sm = smem_raw + (base - raw);
+  const uint32_t off_b = ND * 16384u, off_acc = off_b + (uint32_t)(ND * a.nbp) * 128u;
+  const uint32_t off_e = off_acc + 8u * SG_CONV * 8u;  // FP64 sums, then exponents
+  double *const acc = reinterpret_cast<double *>(sm + off_acc);
+  int *const sE = reinterpret_cast<int *>(sm + off_e);
+  const uint32_t off_bar = off_e + 96u * 4u;
+  const uint32_t bars = base + off_bar;
+  uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(sm + off_bar + 16);
+  volatile int *abort = reinterpret_cast<volatile int *>(tmem_holder + 1);
+  volatile int *bad = abort + 1;
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int bi = blockIdx.z, b = a.act ? a.act[bi] : bi;
+  const int j0 = blockIdx.y * a.nbc, nbc = min(a.nbc, a.q - j0);
+  const int pa = a.mode == SL_GENERAL ? a.p : min(a.p, j0 + nbc);  // left columns (upper triangle: i <= j)
+  // the right operand: [columns j0 .. of A (dup), columns j0 .. of B]; the first are extracted with the left operand
+  const int ndup = a.mode == SL_GENERAL ? 0 : nbc, nown = a.mode == SL_SELF ? 0 : nbc;
+  const int ncols = pa + nown;  // columns to extract
+  const T *const Ab = static_cast<const T *>(a.A) + (long)b * a.sa;
+  const T *const Bb = static_cast<const T *>(a.B) + (long)b * a.sb + (long)j0 * a.L;
+  const long L = a.L, r0 = (long)blockIdx.x * a.chunk, r1 = min(L, r0 + a.chunk);
+
+  {
+    float4 *z = reinterpret_cast<float4 *>(sm);
+    const int nz = (int)(off_e / 16u);
+    for (int i = tid; i < nz; i += SG_THREADS) z[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    fence_proxy_async();
+  }
+  if (tid == 0) {
+    bar_init(bars, 1);
+    bar_init(bars + 8u, 1);
+    *abort = 0;
+    *bad = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tmem_holder)),
+                 "r"(512u)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_holder;
+  const bool issuer = warp == SG_CONV / 32;
+
+  // digit tasks: rows 2 rp, 2 rp + 1 of the stage; the two columns of a warp are two apart, so that their digits fall
+  // into different halves of the swizzled 128-byte rows (no bank conflict)
+  const int rp = lane & 15, c0 = (warp >> 1) * 4 + (warp & 1) + 2 * (lane >> 4);
+  // accumulator part of this warp: TMEM lane quarter, 16 columns of each level
+  const int quarter = warp & 3, slot = warp >> 2;
+  const int row = quarter * 32 + lane, ci = row >> 1;
+  const bool odd = row & 1, drains = !issuer && slot * 16 < a.nbp;
+  const uint32_t tdrain = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(slot * 16);
+  // extracted column (index into sE) of operand column jj
+  auto col_of = [&](int jj) { return jj < ndup ? j0 + jj : pa + jj - ndup; };
+
+  int n = 0;  // stages issued
+  for (long t0 = r0; t0 < r1; t0 += SG_SUPER) {
+    const long t1 = min(r1, t0 + SG_SUPER);
+    for (int c = warp; c < ncols; c += SG_THREADS / 32) {
+      const T *x = c < pa ? Ab + (long)c * L : Bb + (long)(c - pa) * L;
+      int mx = 0;
+#pragma unroll 16
+      for (long l = t0 + lane; l < t1; l += 32) mx = max(mx, sl_key(x[l]));
+      mx = sl_exp_of<T>(__reduce_max_sync(0xffffffffu, mx));
+      if (lane == 0) {
+        sE[c] = mx;
+        if (mx >= SL_NONFINITE) *bad = 1;
+      }
+    }
+    __syncthreads();
+    const int ns = (int)((t1 - t0 + SG_ROWS - 1) / SG_ROWS);
+    if (*bad) {
+      // an infinity or a NaN in the span: its products in plain FP64
+      if (drains && ci < pa)
+        for (int k = 0; k < 8; ++k) {
+          const int jj = slot * 8 + k;
+          if (jj >= ndup + nown) break;
+          const T *x = Ab + (long)ci * L, *y = jj < ndup ? Ab + (long)(j0 + jj) * L : Bb + (long)(jj - ndup) * L;
+          double s = 0.0;
+          for (long l = t0; l < t1; ++l) {
+            const double2 u = ld_c128(x + l), v = ld_c128(y + l);
+            s = odd ? fma(u.x, v.y, fma(-u.y, v.x, s)) : fma(u.x, v.x, fma(u.y, v.y, s));
+          }
+          acc[k * SG_CONV + tid] += s;
+        }
+      __syncthreads();
+      if (tid == 0) *bad = 0;
+    } else if (issuer) {
+      for (int s = 0; s < ns; ++s, ++n) {
+        const int buf = n & 1;
+        named_sync(1 + buf, SG_THREADS);
+        if (lane == 0) {
+          tc_fence_after();
+#pragma unroll
+          for (int ks = 0; ks < SG_ROWS / 16; ++ks) {
+            const uint32_t ko = (uint32_t)(buf * 64 + ks * 32);
+            sl_mma_step<ND>(tmem, base, base + off_b, ko, ko, a.nbp, (s & (SG_GROUP - 1)) == 0 && ks == 0);
+          }
+          mma_commit(bars + 8u * buf);
+        }
+        __syncwarp();
+      }
+    } else {
+      long long shi[8], slo[8];  // levels 0 .. 2 and 3 .. 6 of the sums
+#pragma unroll
+      for (int k = 0; k < 8; ++k) shi[k] = slo[k] = 0;
+      T v[SG_TASKS][2];
+      auto load = [&](int k, long s0) {
+        const int c = c0 + 32 * k;
+        const long l = s0 + 2 * rp;
+        v[k][0] = v[k][1] = T{};
+        if (c < ncols) {
+          const T *x = (c < pa ? Ab + (long)c * L : Bb + (long)(c - pa) * L) + l;
+          if (l < t1) v[k][0] = x[0];
+          if (l + 1 < t1) v[k][1] = x[1];
+        }
+      };
+#pragma unroll
+      for (int k = 0; k < SG_TASKS; ++k) load(k, t0);
+      for (int s = 0; s < ns; ++s) {
+        const int buf = n & 1;
+        if (n >= 2) bar_wait(bars + 8u * buf, ((n >> 1) & 1) ^ 1, abort);
+#pragma unroll
+        for (int k = 0; k < SG_TASKS; ++k) {
+          const int c = c0 + 32 * k;
+          if (c < ncols) {
+            const int E = sE[c];
+            unsigned long long m[2][2];
+            sl_split<ND>(v[k][0], E, m[0][0], m[1][0]);
+            sl_split<ND>(v[k][1], E, m[0][1], m[1][1]);
+            load(k, t0 + (long)(s + 1) * SG_ROWS);  // in flight while the digits of the other columns are formed
+            const bool left = c < pa, dup = left && c >= j0 && ndup > 0;
+            const int jr = left ? c - j0 : ndup + c - pa;  // right operand column
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int ra = 2 * c + h, rb = 2 * jr + h;
+              unsigned char *oa = sm + ra * 128 + (((buf * 4 + (rp >> 2)) ^ (ra & 7)) << 4) + (rp & 3) * 4;
+              unsigned char *ob = sm + off_b + rb * 128 + (((buf * 4 + (rp >> 2)) ^ (rb & 7)) << 4) + (rp & 3) * 4;
+#pragma unroll
+              for (int d = 0; d < ND; ++d) {
+                const unsigned x = sl_digits(m[h][0], m[h][1], ND - 1 - d);
+                if (left) *reinterpret_cast<unsigned *>(oa + d * 16384) = x;
+                if (!left || dup) *reinterpret_cast<unsigned *>(ob + d * (a.nbp * 128)) = x;
+              }
+            }
+          }
+        }
+        fence_proxy_async();
+        tc_fence_before();
+        named_arrive(1 + buf, SG_THREADS);
+        ++n;
+        if ((s & (SG_GROUP - 1)) == SG_GROUP - 1 || s == ns - 1) {
+          bar_wait(bars + 8u * buf, ((n - 1) >> 1) & 1, abort);
+          tc_fence_after();
+          if (drains) {
+#pragma unroll
+            for (int lv = 0; lv < ND; ++lv) {
+              uint32_t r[16];
+              tmem_ld16(tdrain + (uint32_t)(lv * a.nbp), r);
+              // the re and im parts of a left column sit in adjacent lanes: even lanes form Re, odd lanes Im
+#pragma unroll
+              for (int k = 0; k < 8; ++k) {
+                const int own = __float2int_rn(__uint_as_float(r[2 * k]));
+                const int o = __shfl_xor_sync(0xffffffffu, __float2int_rn(__uint_as_float(r[2 * k + 1])), 1);
+                const int d = odd ? o - own : own + o;
+                if (lv < 3)
+                  shi[k] += (long long)d * (1 << (8 * (2 - lv)));
+                else
+                  slo[k] += (long long)d * (1 << (8 * (6 - lv)));
+              }
+            }
+          }
+        }
+      }
+      if (drains && ci < pa) {
+        const int EA = sE[ci];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int jj = slot * 8 + k;
+          if (jj < ndup + nown) {
+            const int sc = EA + sE[col_of(jj)] - 2046 - 2 * (sl_bits<ND>() - 1) + 8 * (ND - 1);
+            acc[k * SG_CONV + tid] += sl_to_double(shi[k] + (slo[k] >> 32), (unsigned)slo[k], sc);
+          }
+        }
+      }
+    }
+    __syncthreads();
+  }
+  if (drains && ci < pa) {
+    const long o = ((long)bi * gridDim.x + blockIdx.x) * a.p * a.q;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int jj = slot * 8 + k;
+      if (jj >= ndup + nown) break;
+      const bool dup = jj < ndup;
+      const int j = j0 + (dup ? jj : jj - ndup);
+      double2 *const part = dup || a.mode == SL_GENERAL ? a.part0 : a.part1;
+      if (a.mode == SL_GENERAL || ci <= j)
+        reinterpret_cast<double *>(part + o + (long)ci * a.q + j)[odd] = acc[k * SG_CONV + tid];
+    }
+  }
+  if (issuer && lane == 0 && *abort && n > 0) bar_wait(bars + 8u * ((n - 1) & 1), ((n - 1) >> 1) & 1, abort, false);
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+  }
+  if (tid == 0 && *abort) atomicExch(&g_gram_sl_error, 1);
+}
+
+size_t sg_smem(int nbp) { return 1024 + SG_ND * 16384 + (size_t)SG_ND * nbp * 128 + 8 * SG_CONV * 8 + 96 * 4 + 64; }
+
+}  // namespace
+
+// most chunks per k-point that launch_gram_sl takes (partial-sum scratch sizing)
+int sl_gram_chunks(int nb, long L) {
+  const long want = (4L * sm_count() + nb - 1) / std::max(nb, 1);
+  return (int)std::max<long>(1, std::min<long>({want, L / 128, 256}));
+}
+
+int launch_gram_sl(int nb, long L, int p, int q, int dtype, const void *A, long sa, const void *B, long sb, int mode,
+                   double2 *part, int maxchunk, int *nchunk, cudaStream_t st, const int *act) {
+  SlGramArgs a{};
+  a.A = A;
+  a.B = B;
+  a.sa = sa;
+  a.sb = sb;
+  a.L = L;
+  a.p = p;
+  a.q = q;
+  a.mode = mode;
+  a.act = act;
+  // blocks of up to 32 operand columns (7 levels of 64 accumulator columns in TMEM); a pair's block has two per column
+  const int most_cols = mode == SL_PAIR ? 16 : 32, nblk = (q + most_cols - 1) / most_cols;
+  a.nbc = (q + nblk - 1) / nblk;
+  a.nbp = (2 * a.nbc * (mode == SL_PAIR ? 2 : 1) + 15) / 16 * 16;
+  // the chunk count with the least rows (plus a CTA's fixed cost, about 100 rows) in the longest sequence of CTAs per SM
+  const long per = (long)nb * nblk, nsm = sm_count();
+  const int most = (int)std::max<long>(1, std::min<long>(maxchunk, sl_gram_chunks(nb, L)));
+  double best = 0.0;
+  int c = 1;
+  for (int k = 1; k <= most; ++k) {
+    const long rows = ((L + k - 1) / k + SG_ROWS - 1) / SG_ROWS * SG_ROWS;
+    const double cost = (double)((per * k + nsm - 1) / nsm) * (double)(rows + 100);
+    if (k == 1 || cost < best) {
+      best = cost;
+      c = k;
+    }
+  }
+  a.chunk = std::max<long>(SG_ROWS, ((L + c - 1) / c + SG_ROWS - 1) / SG_ROWS * SG_ROWS);
+  c = (int)std::max<long>(1, (L + a.chunk - 1) / a.chunk);
+  *nchunk = c;
+  a.part0 = part;
+  a.part1 = part + (size_t)nb * c * p * q;
+  const size_t smem = sg_smem(a.nbp);
+  const dim3 grid(c, nblk, nb);
+  // per device: the attribute belongs to the function on the current device
+  static bool configured[64][2] = {};
+  int dev = 0;
+  PC_CK(cudaGetDevice(&dev));
+  const int kind = dtype == PC_DFS ? 1 : 0;
+  if (dev < 0 || dev >= 64 || !configured[dev][kind]) {
+    PC_CK(cudaFuncSetAttribute(kind ? gram_sl_kernel<float4> : gram_sl_kernel<double2>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sg_smem(64)));
+    if (dev >= 0 && dev < 64) configured[dev][kind] = true;
+  }
+  if (kind)
+    gram_sl_kernel<float4><<<grid, SG_THREADS, smem, st>>>(a);
+  else
+    gram_sl_kernel<double2><<<grid, SG_THREADS, smem, st>>>(a);
+  PC_CK_LAUNCH();
+  return PC_OK;
+}
+
+int sliced_check() {
+  int v = 0;
+  PC_CK(cudaMemcpyFromSymbol(&v, g_gram_sl_error, sizeof(int)));
+  if (v) {
+    const int zero = 0;
+    PC_CK(cudaMemcpyToSymbol(g_gram_sl_error, &zero, sizeof(int)));
+    set_error("sliced product kernel: a pipeline wait ran out of time");
+    return PC_ECUDA;
+  }
+  return PC_OK;
+}
+
+}  // namespace pc

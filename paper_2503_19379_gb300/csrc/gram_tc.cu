@@ -40,6 +40,8 @@
 #include <cstdlib>
 
 #include "pc_internal.cuh"
+#include "sliced.cuh"
+#include "tc_ptx.cuh"
 
 namespace pc {
 
@@ -54,73 +56,9 @@ constexpr int TC_NTR = 6;     // transform warps (2..7)
 constexpr int TC_NDR = 12;    // drain warps (8..19), three per TMEM lane quarter
 constexpr int TC_NMAX = 160;  // MMA columns: three accumulators of N columns in the 512 TMEM columns
 constexpr int TC_MAXT = 512;  // K tiles per chunk at most: the drain's FP32 running sums span <= 256 groups
-constexpr unsigned long long TC_WAIT_NS = 1000000000ull;  // 1 s: a kernel call takes milliseconds
 
 __device__ int g_gram_tc_error = 0;
 
-__device__ __forceinline__ uint32_t smem_addr(const void *p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ unsigned long long gtimer() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ void bar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void bar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void bar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool bar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Waits for the completion of the phase of the given parity. Returns false when the abort flag is (or gets) set,
-// or after TC_WAIT_NS, in which case it sets the flag. With honour_abort = false only the time bound ends the wait
-// (used to drain operations in flight).
-__device__ bool bar_wait(uint32_t bar, uint32_t parity, volatile int *abort, bool honour_abort = true) {
-  unsigned long long t0 = 0;
-  for (uint32_t it = 0;; ++it) {
-    if (bar_try_wait(bar, parity)) return true;
-    if ((it & 15) == 15) {
-      if (honour_abort && *abort) return false;
-      const unsigned long long t = gtimer();
-      if (t0 == 0) {
-        t0 = t;
-      } else if (t - t0 > TC_WAIT_NS) {
-        *abort = 1;
-        return false;
-      }
-    }
-  }
-}
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-          dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
-      : "memory");
-}
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// shared-memory matrix descriptor: K-major operand, 128-byte swizzle, 8-row groups 1024 bytes apart
-__device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
-  return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
-         ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
-}
 __device__ __forceinline__ void mma_tf32(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                          uint32_t accumulate) {
   asm volatile(
@@ -130,29 +68,10 @@ __device__ __forceinline__ void mma_tf32(uint32_t dtmem, uint64_t adesc, uint64_
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-               : "memory");
-}
 __device__ __forceinline__ float tf32_rna(float x) {
   uint32_t r;
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
   return __uint_as_float(r);
-}
-// 16 consecutive accumulator columns of this warp's 32 TMEM lanes
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-      "%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
-                 "+r"(r[15])
-               :
-               : "memory");
 }
 // adds 32 accumulator columns (two 16-column loads) into acc
 __device__ __forceinline__ void tmem_add32(uint32_t taddr, float (&acc)[32]) {
@@ -650,7 +569,7 @@ int launch_gram_tc(int nb, long L, int p, int q, const void *A, long sa, const v
   return PC_OK;
 }
 
-// reads and clears the abort flag of the tensor-core Gram kernel (after a synchronisation)
+// reads and clears the abort flags of the tensor-core Gram kernels (after a synchronisation)
 int gram_tc_check() {
   int v = 0;
   PC_CK(cudaMemcpyFromSymbol(&v, g_gram_tc_error, sizeof(int)));
@@ -660,7 +579,7 @@ int gram_tc_check() {
     set_error("tensor-core Gram kernel: a pipeline wait ran out of time");
     return PC_ECUDA;
   }
-  return PC_OK;
+  return sliced_check();
 }
 
 }  // namespace pc

@@ -1,0 +1,218 @@
+// Exact slicing of FP64-accurate values into FP16 integers for the tensor cores (the error-free splitting of
+// Ozaki, Ogita, Oishi and Rump, "Error-free transformations of matrix multiplication by using fast routines of matrix
+// multiplication and its applications", Numer. Algorithms 2012; on tensor cores: Mukunoki, Ozaki, Ogita and Imamura,
+// ISC 2020).
+//
+// A value v is held against a common exponent E (biased as in FP64, at least that of every value it is summed with)
+// as the integer m = round(v 2^(MB - 1 - (E - 1023))), |m| < 2^MB with MB = 8 (ND - 1) + 6, and m is written in ND
+// balanced base-256 digits, m = sum_j d_j 256^(ND-1-j), |d_j| <= 128 (|d_0| <= 64). Digits are exact in FP16, a
+// product of two is an integer of at most 2^14, and the products d_i d'_j of one level k = i + j (at most ND <= 7 pairs)
+// over a sum of 128 terms stay below 2^24: the tensor core's FP32 accumulator holds them exactly, in any order. The
+// level sums L_0 .. L_(ND-1) give sum m m' = 256^(ND-1) sum_k L_k 256^(ND-1-k); the dropped levels k >= ND are
+// below 2^-(8 ND - 2) of the largest product. With ND = 7 that is 2^-54: the product of two FP64 values rounded
+// once, with no rounding at all in the additions of a chunk.
+#pragma once
+#include <cuda_fp16.h>
+
+#include "dfloat.cuh"
+#include "pc_internal.cuh"
+#include "tc_ptx.cuh"
+
+namespace pc {
+
+template <int ND> constexpr int sl_bits() { return 8 * (ND - 1) + 6; }
+constexpr int SL_NONFINITE = 0x7ff;
+constexpr int SL_EMIN = 128;  // common exponents start here: FP64 values too small to reach their last digit become 0
+
+// A key whose maximum over elements gives their common exponent (sl_exp_of): the larger part's magnitude, high bits
+__device__ __forceinline__ int sl_key(double2 v) {
+  return max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff);
+}
+__device__ __forceinline__ int sl_key(float2 v) {
+  return max(__float_as_int(v.x) & 0x7fffffff, __float_as_int(v.y) & 0x7fffffff);
+}
+__device__ __forceinline__ int sl_key(float4 v) {  // a pair's low part is normally far below its high part
+  return max(sl_key(make_float2(v.x, v.z)), sl_key(make_float2(v.y, v.w)));
+}
+// biased FP64 exponent of a key (0x7ff for an infinity or a NaN)
+template <typename T> __device__ __forceinline__ int sl_exp_of(int key) {
+  if constexpr (std::is_same<T, double2>::value) return max(key >> 20, SL_EMIN);
+  const int e = key >> 23;
+  return e == 0xff ? SL_NONFINITE : max(e, 1) + 896;
+}
+
+__device__ __forceinline__ unsigned sl_shr(unsigned x, int s) {  // 0 for s >= 32
+  unsigned r;
+  asm("shr.u32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(s));
+  return r;
+}
+// (mh : ml) >> sh for sh >= 0 with the sign s (0 or -1) applied
+__device__ __forceinline__ long long sl_shift(unsigned mh, unsigned ml, int sh, int s) {
+  const unsigned lo = sl_shr(__funnelshift_rc(ml, mh, sh), max(sh - 32, 0)), hi = sl_shr(mh, sh);
+  return (long long)(((unsigned long long)(hi ^ (unsigned)s) << 32) | (lo ^ (unsigned)s)) - s;
+}
+// 2 m, not yet rounded: v 2^(MB - (E - 1023)); E at least the exponent of v and SL_EMIN
+template <int ND> __device__ __forceinline__ long long sl_raw(double x, int E) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned mh = (__funnelshift_l(lo, hi, 2) & 0x3fffffu) | 0x400000u;  // |v| = (mh : ml) 2^(e - 1077)
+  // zeros and subnormals (e = 0) are shifted out, as E >= SL_EMIN
+  return sl_shift(mh, lo << 2, E + 54 - sl_bits<ND>() - (int)((hi >> 20) & 0x7ff), (int)hi >> 31);
+}
+template <int ND> __device__ __forceinline__ long long sl_raw(float x, int E) {
+  const unsigned u = (unsigned)__float_as_int(x);
+  const int e = (u >> 23) & 0xff;
+  const unsigned m = (u & 0x7fffffu) | (e ? 0x800000u : 0u);
+  return sl_shift(m >> 1, m << 31, E - 896 + 54 - sl_bits<ND>() - max(e, 1), (int)u >> 31);
+}
+// m with every digit moved up by 128, so that digit j is byte ND - 1 - j minus 128; byte 7 holds 0x64 (see sl_digits)
+template <int ND> __device__ __forceinline__ unsigned long long sl_round(long long raw) {
+  unsigned long long b = 0x64ull << 56;
+#pragma unroll
+  for (int k = 0; k < ND; ++k) b |= 0x80ull << (8 * k);
+  return ((unsigned long long)raw + (2 * b + 1)) >> 1;
+}
+// rounded and biased m of the real and imaginary part of an element
+template <int ND>
+__device__ __forceinline__ void sl_split(double2 v, int E, unsigned long long &re, unsigned long long &im) {
+  re = sl_round<ND>(sl_raw<ND>(v.x, E));
+  im = sl_round<ND>(sl_raw<ND>(v.y, E));
+}
+template <int ND>
+__device__ __forceinline__ void sl_split(float2 v, int E, unsigned long long &re, unsigned long long &im) {
+  re = sl_round<ND>(sl_raw<ND>(v.x, E));
+  im = sl_round<ND>(sl_raw<ND>(v.y, E));
+}
+template <int ND>
+__device__ __forceinline__ void sl_split(float4 v, int E, unsigned long long &re, unsigned long long &im) {
+  re = sl_round<ND>(sl_raw<ND>(v.x, E) + sl_raw<ND>(v.y, E));
+  im = sl_round<ND>(sl_raw<ND>(v.z, E) + sl_raw<ND>(v.w, E));
+}
+// byte k of two biased values as FP16 digits (u0 low, u1 high): 0x6400 | byte is 1024 + byte
+__device__ __forceinline__ unsigned sl_digits(unsigned long long u0, unsigned long long u1, int k) {
+  unsigned x;
+  if (k < 4)
+    x = (__byte_perm((unsigned)u0, (unsigned)u1, k | (k << 4) | ((4 + k) << 8) | ((4 + k) << 12)) & 0x00ff00ffu) |
+        0x64006400u;
+  else  // the 0x64 of byte 7 comes along
+    x = __byte_perm((unsigned)(u0 >> 32), (unsigned)(u1 >> 32), (k - 4) | (3 << 4) | (k << 8) | (7 << 12));
+  const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&x), __half2half2(__ushort_as_half(0x6480)));
+  return *reinterpret_cast<const unsigned *>(&h);
+}
+
+// (H 2^32 + Lw) 2^n rounded to FP64; integer arithmetic only (the FP64 pipe retires about 2 operations per clock and SM)
+__device__ __forceinline__ double sl_to_double(long long H, unsigned Lw, int n) {
+  const bool neg = H < 0;
+  if (neg) {
+    Lw = 0u - Lw;
+    H = ~H + (Lw == 0u ? 1 : 0);
+  }
+  unsigned long long top;
+  int ex;  // exponent of the top bit
+  const int z = __clzll(H);
+  if (z < 32) {
+    top = ((unsigned long long)H << z) | (((unsigned long long)Lw << z) >> 32);
+    ex = 95 - z;
+  } else {
+    top = ((unsigned long long)H << 32) | Lw;
+    if (top == 0ull) return 0.0;
+    const int z2 = __clzll((long long)top);
+    top <<= z2;
+    ex = 63 - z2;
+  }
+  const unsigned long long r = top + 1024ull;
+  if (r < top) {
+    top = 1ull << 63;
+    ++ex;
+  } else {
+    top = r;
+  }
+  const int be = ex + n + 1023;
+  if (be >= 1 && be <= 2046)
+    return __longlong_as_double((long long)((top >> 11) & 0xfffffffffffffull) | ((long long)be << 52) |
+                                (neg ? (long long)0x8000000000000000ull : 0ll));
+  const double v = scalbn((double)(top >> 11), ex + n - 52);
+  return neg ? -v : v;
+}
+// the same value as a double-float pair
+__device__ __forceinline__ df sl_to_df(long long H, unsigned Lw, int n) {
+  const bool neg = H < 0;
+  if (neg) {
+    Lw = 0u - Lw;
+    H = ~H + (Lw == 0u ? 1 : 0);
+  }
+  unsigned long long top;
+  int ex;
+  const int z = __clzll(H);
+  if (z < 32) {
+    top = ((unsigned long long)H << z) | (((unsigned long long)Lw << z) >> 32);
+    ex = 95 - z;
+  } else {
+    top = ((unsigned long long)H << 32) | Lw;
+    if (top == 0ull) return df{0.f, 0.f};
+    const int z2 = __clzll((long long)top);
+    top <<= z2;
+    ex = 63 - z2;
+  }
+  // top = h 2^40 + rest, |rest| <= 2^39: the high part's 24 bits, rounded, and the remainder to 31 bits
+  const unsigned h = (unsigned)((top >> 40) + ((top >> 39) & 1ull));
+  const int rest = (int)((long long)(top - ((unsigned long long)h << 40)) >> 9);
+  const int e2 = ex + n;  // value = h 2^(e2 - 23) + rest 2^(e2 - 54)
+  df r;
+  if (e2 >= -60 && e2 <= 126) {
+    r.hi = (float)h * __int_as_float((e2 - 23 + 127) << 23);
+    r.lo = e2 >= -40 ? (float)rest * __int_as_float((e2 - 54 + 127) << 23) : ldexpf((float)rest, e2 - 54);
+  } else {
+    r.hi = ldexpf((float)h, e2 - 23);
+    r.lo = isinf(r.hi) ? 0.f : ldexpf((float)rest, e2 - 54);
+  }
+  if (neg) {
+    r.hi = -r.hi;
+    r.lo = -r.lo;
+  }
+  return r;
+}
+
+// D (+)= A B^T, FP16 operands, FP32 accumulator
+__device__ __forceinline__ void mma_f16(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                        uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// instruction descriptor: D FP32 (bits 4-5 = 1), A and B FP16 (0), both K-major, N >> 3 at bits 17-22, M >> 4 at 24-28
+__device__ __forceinline__ uint32_t idesc_f16(int M, int N) {
+  return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+// The MMAs of one K step (16 values) for all digit pairs of levels below ND. A: ND slices of 128 rows of 128 bytes;
+// B: ND slices of nbp rows each, one after the other, so that one instruction multiplies slice i of A with several
+// slices of B: slice j lands in the accumulator columns of level i + j (level k at column k nbp).
+template <int ND>
+__device__ __forceinline__ void sl_mma_step(uint32_t tmem, uint32_t a, uint32_t b, uint32_t ko_a, uint32_t ko_b, int nbp,
+                                            bool first) {
+  const int most = 256 / nbp;  // slices per instruction (N <= 256)
+#pragma unroll
+  for (int i = 0; i < ND; ++i) {
+    const uint64_t ad = sdesc(a + (uint32_t)i * 16384u + ko_a);
+    for (int j = 0; j < ND - i; j += most) {
+      const int cnt = min(ND - i - j, most);
+      mma_f16(tmem + (uint32_t)((i + j) * nbp), ad, sdesc(b + (uint32_t)(j * nbp) * 128u + ko_b), idesc_f16(128, cnt * nbp),
+              (first && i == 0) ? 0u : 1u);
+    }
+  }
+}
+
+// products per launch that a time-out voided (sliced kernels), read and cleared after a synchronisation
+int sliced_check();
+// Gram products of FP64-accurate panels (gram_sl.cu), dtype PC_C128 or PC_DFS, one array part[bi][chunk][p][q] per
+// product: SL_GENERAL A^H B; SL_PAIR A^H A, then A^H B, both upper triangles (q = p); SL_SELF the upper triangle of
+// A^H A
+constexpr int SL_GENERAL = 0, SL_PAIR = 1, SL_SELF = 2;
+int sl_gram_chunks(int nb, long L);
+int launch_gram_sl(int nb, long L, int p, int q, int dtype, const void *A, long sa, const void *B, long sb, int mode,
+                   double2 *part, int maxchunk, int *nchunk, cudaStream_t st, const int *act);
+
+}  // namespace pc

@@ -1,0 +1,102 @@
+"""Products of FP64-accurate panels on the tensor cores (exact FP16 digit slices) through the C ABI.
+
+Tolerance of the Gram products. A value is rounded to 2^-54 of the largest part M of its column, and the digit pairs
+below level 6 are dropped: 6 pairs of random digits (uniform on [-128, 127], rms 74) at level 7, 2^(40 + 12.4 + 1.3)
+against M_a M_b >= 2^106 in the same units, so 2^-52.3 M_a M_b (rms) for each of the 2 L real products of an entry.
+Six standard deviations of their sum, 6 sqrt(2 L) 2^-52.2 M_a M_b, bound it; the FP64 sums over spans and chunks add
+a few 2^-53 of the entry.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pcmod():
+    from paper_2503_19379_gb300 import build as b
+    b.build()
+    import paper_2503_19379_gb300 as p
+    return p
+
+
+def rand(seed, shape):
+    g = np.random.default_rng(seed)
+    x = g.standard_normal(shape) + 1j * g.standard_normal(shape)
+    return x * np.exp(2.0 * g.standard_normal(shape[:-1]))[..., None]  # columns of different sizes
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def top(A):
+    return np.maximum(np.abs(A.real), np.abs(A.imag)).max(axis=2)
+
+
+def check(got, A, B, upper=False):
+    L = A.shape[2]
+    # the reference sums in extended precision, so that its own rounding stays below the tolerance
+    ref = np.einsum("bil,bjl->bij", A.conj().astype(np.clongdouble), B.astype(np.clongdouble))
+    tol = 6.0 * np.sqrt(2.0 * L) * 2.0 ** -52.2 * top(A)[:, :, None] * top(B)[:, None, :] + 2.0 ** -50 * np.abs(ref)
+    ratio = np.abs(got - ref) / np.maximum(tol, np.finfo(np.float64).tiny)
+    if upper:
+        ratio = np.triu(ratio)
+    assert np.all(ratio <= 1.0), float(np.max(ratio))
+
+
+@pytest.mark.parametrize("nb,p,L", [(1, 1, 1), (2, 16, 31), (1, 17, 33), (3, 32, 128), (1, 33, 129), (2, 48, 1025),
+                                    (1, 64, 2100), (4, 21, 1536), (1, 39, 12288)])
+def test_gram_pair_sliced(pcmod, nb, p, L):
+    S = rand(p + L, (nb, p, L))
+    w = np.random.default_rng(L).uniform(0.5, 40.0, L)
+    AS = S * w
+    G, H = (x.cpu().numpy() for x in pcmod.gram_pair(dev(S), dev(AS)))
+    for got, B in ((G, S), (H, AS)):
+        check(got, S, B, upper=True)  # the lower triangle is its mirror
+        assert np.array_equal(got, got.conj().transpose(0, 2, 1))
+
+
+@pytest.mark.parametrize("nb,p,q,L", [(1, 1, 1, 7), (2, 5, 33, 640), (1, 64, 64, 1500), (3, 40, 32, 96),
+                                      (1, 12, 24, 999)])
+def test_gram_sliced(pcmod, nb, p, q, L):
+    A, B = rand(p, (nb, p, L)), rand(100 + q, (nb, q, L))
+    check(pcmod.gram(dev(A), dev(B)).cpu().numpy(), A, B)
+
+
+@pytest.mark.parametrize("bits", [0x3FFFFFFFFFFFFFFF, 0x3FF7F7F7F7F7F7F7, 0x3FF8080808080808])
+def test_gram_extreme_digits(pcmod, bits):
+    """Constant columns whose digits are all at an end of their range: the level sums are the largest possible, and a
+    rounding of the accumulator would show. All products are equal, so only the dropped levels' part remains:
+    at most 6 2^54 of 2^106 per product."""
+    v = np.array([bits], dtype=np.uint64).view(np.float64)[0]
+    L = 4096
+    S = np.full((1, 64, L), v * (1 - 1j))
+    G, _ = (x.cpu().numpy() for x in pcmod.gram_pair(dev(S), dev(S)))
+    ref = float(2 * np.longdouble(v) ** 2 * L)
+    assert np.max(np.abs(G - ref)) <= 7 * 2.0 ** -52 * ref
+
+
+def test_gram_nonfinite(pcmod):
+    """An infinity or a NaN reaches exactly the entries of its columns, as in plain FP64 sums."""
+    S = rand(3, (1, 10, 2500))
+    S[0, 3, 1500] = np.inf
+    S[0, 7, 10] = np.nan
+    G, H = (x.cpu().numpy()[0] for x in pcmod.gram_pair(dev(S), dev(S)))
+    touched = np.zeros((10, 10), dtype=bool)
+    touched[[3, 7], :] = touched[:, [3, 7]] = True
+    assert np.array_equal(~np.isfinite(G.real), touched) and np.array_equal(~np.isfinite(H.real), touched)
+    ok = [i for i in range(10) if i not in (3, 7)]
+    check(G[None][:, ok][:, :, ok], S[:, ok], S[:, ok])
+
+
+def test_gram_zero_and_tiny_columns(pcmod):
+    """Zero columns give exact zeros; a column of a scale far from the others' keeps its relative accuracy."""
+    S = rand(4, (1, 6, 700))
+    S[0, 2] = 0.0
+    S[0, 4] *= 2.0 ** -300
+    S[0, 5] *= 2.0 ** 300
+    G, _ = (x.cpu().numpy() for x in pcmod.gram_pair(dev(S), dev(S)))
+    assert np.all(G[0, 2] == 0.0) and np.all(G[0, :, 2] == 0.0)
+    check(G, S, S)
