@@ -414,7 +414,7 @@ int launch_gram_pair_coupled(int nb, long L, int p, int q2, int dtype, const voi
 // per thread, QB outputs. Products and sums run in the precision T of S and Y; Z is a complex64 addend (the
 // complex64 correction added to the FP64 block in the mixed-precision update). Each column group re-reads S, so
 // the launcher takes the width that covers q in the fewest groups with the fewest idle columns (complex64: one
-// group of up to 24 columns, 48 accumulator registers; complex128: 16).
+// group of up to 24 columns, 48 accumulator registers).
 constexpr int UPD_PMAX = 64;
 
 template <typename T, int QB>
@@ -493,11 +493,11 @@ int launch_block_update(int nb, long L, int p, int q, int dtype, const void *S, 
     set_error("block_update: at most 64 input columns");
     return PC_EINVAL;
   }
+  // complex128: on the tensor cores (faster at every size measured, see update_sl.cu); not the
+  // addend and the sum of no columns, which no solve asks for
+  if (dtype == PC_C128 && p > 0 && !Z) return launch_update_sl(nb, L, p, q, S, ss, C, sc, Y, sy, st, act);
   if (dtype == PC_C128) {
-    if (update_width(q, {8, 16}) == 8)
-      block_update_t<double, 8>(nb, L, p, q, S, ss, C, sc, Y, sy, st, act, Z, sz);
-    else
-      block_update_t<double, 16>(nb, L, p, q, S, ss, C, sc, Y, sy, st, act, Z, sz);
+    block_update_t<double, 8>(nb, L, p, q, S, ss, C, sc, Y, sy, st, act, Z, sz);
   } else {
     switch (update_width(q, {8, 10, 12, 16, 20, 24})) {
       case 8: block_update_t<float, 8>(nb, L, p, q, S, ss, C, sc, Y, sy, st, act, Z, sz); break;

@@ -13,7 +13,12 @@
 // FP32 holds exactly) the level sums are drained into 64-bit integer sums in registers. At the end of a span these are
 // scaled and added to FP64 sums in shared memory.
 //
-// Bound: integer instructions of the digit extraction. The pair A^H A, A^H B therefore takes the block's columns of A
+// Eight levels of seven digits leave less error than the FP64 sums they replace, in every entry of G and H (against
+// extended precision, N = 8 to 32, smooth and random panels); seven levels left up to 1.8 times more off the diagonal.
+//
+// Bound: integer instructions of the digit extraction (8 k-points x 48 columns at N = 32: 2.19 ms, of which a variant
+// without the scan saves 0.3 ms, without the MMAs 0.4 ms, and the extraction alone takes 1.0 ms; the tensor pipe is 24%
+// busy). The CUDA cores' FP64 pipe took 23.6 ms, and 1.77 ms against 64 us for one k-point of 24 columns at N = 16. The pair A^H A, A^H B therefore takes the block's columns of A
 // and of B in one CTA, and the columns of A that the block shares with the left operand are extracted once and stored
 // twice.
 #include <cuda.h>
@@ -30,7 +35,8 @@ constexpr int SG_THREADS = SG_CONV + 32;      // and the warp that issues the MM
 constexpr int SG_ROWS = 32;                   // rows per stage
 constexpr int SG_GROUP = 4;                   // stages per drain
 constexpr int SG_SUPER = 1024;                // rows per common exponent
-constexpr int SG_ND = 7;
+constexpr int SG_ND = 7;                      // digits
+constexpr int SG_NL = 8;                      // levels of digit products
 constexpr int SG_TASKS = 3;                   // (64 + 32 columns) x 16 row pairs over 512 threads
 
 __device__ int g_gram_sl_error = 0;
@@ -45,21 +51,14 @@ struct SlGramArgs {
   const int *act;
 };
 
-__device__ __forceinline__ void named_arrive(int id, int count) {
-  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
-}
-__device__ __forceinline__ void named_sync(int id, int count) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
-}
-
 template <typename T>
 __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs a) {
-  constexpr int ND = SG_ND;
+  constexpr int ND = SG_ND, NL = SG_NL;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_addr(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   unsigned char *const sm = smem_raw + (base - raw);
-  const uint32_t off_b = ND * 16384u, off_acc = off_b + (uint32_t)(ND * a.nbp) * 128u;
+  const uint32_t off_b = ND * 16384u, off_acc = off_b + (uint32_t)(NL * a.nbp) * 128u;
   const uint32_t off_e = off_acc + 8u * SG_CONV * 8u;  // FP64 sums, then exponents
   double *const acc = reinterpret_cast<double *>(sm + off_acc);
   int *const sE = reinterpret_cast<int *>(sm + off_e);
@@ -157,14 +156,14 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
 #pragma unroll
           for (int ks = 0; ks < SG_ROWS / 16; ++ks) {
             const uint32_t ko = (uint32_t)(buf * 64 + ks * 32);
-            sl_mma_step<ND>(tmem, base, base + off_b, ko, ko, a.nbp, (s & (SG_GROUP - 1)) == 0 && ks == 0);
+            sl_mma_step<ND, NL>(tmem, base, base + off_b, ko, ko, a.nbp, (s & (SG_GROUP - 1)) == 0 && ks == 0);
           }
           mma_commit(bars + 8u * buf);
         }
         __syncwarp();
       }
     } else {
-      long long shi[8], slo[8];  // levels 0 .. 2 and 3 .. 6 of the sums
+      long long shi[8], slo[8];  // the levels before the last four, and the last four
 #pragma unroll
       for (int k = 0; k < 8; ++k) shi[k] = slo[k] = 0;
       T v[SG_TASKS][2];
@@ -201,7 +200,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
               unsigned char *ob = sm + off_b + rb * 128 + (((buf * 4 + (rp >> 2)) ^ (rb & 7)) << 4) + (rp & 3) * 4;
 #pragma unroll
               for (int d = 0; d < ND; ++d) {
-                const unsigned x = sl_digits(m[h][0], m[h][1], ND - 1 - d);
+                const unsigned x = sl_digits<ND>(m[h][0], m[h][1], ND - 1 - d);
                 if (left) *reinterpret_cast<unsigned *>(oa + d * 16384) = x;
                 if (!left || dup) *reinterpret_cast<unsigned *>(ob + d * (a.nbp * 128)) = x;
               }
@@ -217,7 +216,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
           tc_fence_after();
           if (drains) {
 #pragma unroll
-            for (int lv = 0; lv < ND; ++lv) {
+            for (int lv = 0; lv < NL; ++lv) {
               uint32_t r[16];
               tmem_ld16(tdrain + (uint32_t)(lv * a.nbp), r);
               // the re and im parts of a left column sit in adjacent lanes: even lanes form Re, odd lanes Im
@@ -226,10 +225,10 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
                 const int own = __float2int_rn(__uint_as_float(r[2 * k]));
                 const int o = __shfl_xor_sync(0xffffffffu, __float2int_rn(__uint_as_float(r[2 * k + 1])), 1);
                 const int d = odd ? o - own : own + o;
-                if (lv < 3)
-                  shi[k] += (long long)d * (1 << (8 * (2 - lv)));
+                if (lv < NL - 4)
+                  shi[k] += (long long)d * (1 << (8 * (NL - 5 - lv)));
                 else
-                  slo[k] += (long long)d * (1 << (8 * (6 - lv)));
+                  slo[k] += (long long)d * (1 << (8 * (NL - 1 - lv)));
               }
             }
           }
@@ -241,7 +240,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
         for (int k = 0; k < 8; ++k) {
           const int jj = slot * 8 + k;
           if (jj < ndup + nown) {
-            const int sc = EA + sE[col_of(jj)] - 2046 - 2 * (sl_bits<ND>() - 1) + 8 * (ND - 1);
+            const int sc = EA + sE[col_of(jj)] - 2046 - 2 * (sl_bits<ND>() - 1) + 8 * (2 * ND - 1 - NL);
             acc[k * SG_CONV + tid] += sl_to_double(shi[k] + (slo[k] >> 32), (unsigned)slo[k], sc);
           }
         }
@@ -272,7 +271,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
   if (tid == 0 && *abort) atomicExch(&g_gram_sl_error, 1);
 }
 
-size_t sg_smem(int nbp) { return 1024 + SG_ND * 16384 + (size_t)SG_ND * nbp * 128 + 8 * SG_CONV * 8 + 96 * 4 + 64; }
+size_t sg_smem(int nbp) { return 1024 + SG_ND * 16384 + (size_t)SG_NL * nbp * 128 + 8 * SG_CONV * 8 + 96 * 4 + 64; }
 
 }  // namespace
 
@@ -294,7 +293,7 @@ int launch_gram_sl(int nb, long L, int p, int q, int dtype, const void *A, long 
   a.q = q;
   a.mode = mode;
   a.act = act;
-  // blocks of up to 32 operand columns (7 levels of 64 accumulator columns in TMEM); a pair's block has two per column
+  // blocks of up to 32 operand columns (8 levels of 64 accumulator columns fill TMEM); a pair's block has two per column
   const int most_cols = mode == SL_PAIR ? 16 : 32, nblk = (q + most_cols - 1) / most_cols;
   a.nbc = (q + nblk - 1) / nblk;
   a.nbp = (2 * a.nbc * (mode == SL_PAIR ? 2 : 1) + 15) / 16 * 16;
@@ -342,10 +341,10 @@ int sliced_check() {
   if (v) {
     const int zero = 0;
     PC_CK(cudaMemcpyToSymbol(g_gram_sl_error, &zero, sizeof(int)));
-    set_error("sliced product kernel: a pipeline wait ran out of time");
+    set_error("sliced Gram kernel: a pipeline wait ran out of time");
     return PC_ECUDA;
   }
-  return PC_OK;
+  return update_sl_check();
 }
 
 }  // namespace pc

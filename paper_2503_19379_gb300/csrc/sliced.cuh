@@ -6,11 +6,11 @@
 // A value v is held against a common exponent E (biased as in FP64, at least that of every value it is summed with)
 // as the integer m = round(v 2^(MB - 1 - (E - 1023))), |m| < 2^MB with MB = 8 (ND - 1) + 6, and m is written in ND
 // balanced base-256 digits, m = sum_j d_j 256^(ND-1-j), |d_j| <= 128 (|d_0| <= 64). Digits are exact in FP16, a
-// product of two is an integer of at most 2^14, and the products d_i d'_j of one level k = i + j (at most ND <= 7 pairs)
-// over a sum of 128 terms stay below 2^24: the tensor core's FP32 accumulator holds them exactly, in any order. The
-// level sums L_0 .. L_(ND-1) give sum m m' = 256^(ND-1) sum_k L_k 256^(ND-1-k); the dropped levels k >= ND are
-// below 2^-(8 ND - 2) of the largest product. With ND = 7 that is 2^-54: the product of two FP64 values rounded
-// once, with no rounding at all in the additions of a chunk.
+// product of two is an integer of at most 2^14, and the products d_i d'_j of one level k = i + j (at most 8 pairs)
+// over a sum of 128 terms stay within 2^24: the tensor core's FP32 accumulator holds them exactly, in any order. The
+// level sums L_0 .. L_(NL-1) give sum m m' = 256^(2 ND - 1 - NL) sum_k L_k 256^(NL-1-k). A product is off by the
+// dropped levels k >= NL (random digits have rms 74; a pair at level 8 is 2^-60 of the largest product) and by the
+// rounding of its factors, 2^-(8 ND - 1.2) of the largest (rms); the additions do not round at all.
 #pragma once
 #include <cuda_fp16.h>
 
@@ -53,10 +53,12 @@ __device__ __forceinline__ long long sl_shift(unsigned mh, unsigned ml, int sh, 
 }
 // 2 m, not yet rounded: v 2^(MB - (E - 1023)); E at least the exponent of v and SL_EMIN
 template <int ND> __device__ __forceinline__ long long sl_raw(double x, int E) {
+  constexpr int PS = sl_bits<ND>() - 52;  // the 53-bit significand's place in 2 m
+  static_assert(PS > 0 && PS <= 10, "FP64 values take seven or eight digits");
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned mh = (__funnelshift_l(lo, hi, 2) & 0x3fffffu) | 0x400000u;  // |v| = (mh : ml) 2^(e - 1077)
+  const unsigned mh = (__funnelshift_l(lo, hi, PS) & ((1u << (20 + PS)) - 1u)) | (1u << (20 + PS));
   // zeros and subnormals (e = 0) are shifted out, as E >= SL_EMIN
-  return sl_shift(mh, lo << 2, E + 54 - sl_bits<ND>() - (int)((hi >> 20) & 0x7ff), (int)hi >> 31);
+  return sl_shift(mh, lo << PS, E - (int)((hi >> 20) & 0x7ff), (int)hi >> 31);
 }
 template <int ND> __device__ __forceinline__ long long sl_raw(float x, int E) {
   const unsigned u = (unsigned)__float_as_int(x);
@@ -64,21 +66,18 @@ template <int ND> __device__ __forceinline__ long long sl_raw(float x, int E) {
   const unsigned m = (u & 0x7fffffu) | (e ? 0x800000u : 0u);
   return sl_shift(m >> 1, m << 31, E - 896 + 54 - sl_bits<ND>() - max(e, 1), (int)u >> 31);
 }
-// m with every digit moved up by 128, so that digit j is byte ND - 1 - j minus 128; byte 7 holds 0x64 (see sl_digits)
+// m with every digit moved up by 128, so that digit j is byte ND - 1 - j minus 128; with seven digits byte 7 holds 0x64
+// (see sl_digits)
 template <int ND> __device__ __forceinline__ unsigned long long sl_round(long long raw) {
-  unsigned long long b = 0x64ull << 56;
+  unsigned long long b = ND < 8 ? 0x64ull << 56 : 0ull;
 #pragma unroll
   for (int k = 0; k < ND; ++k) b |= 0x80ull << (8 * k);
-  return ((unsigned long long)raw + (2 * b + 1)) >> 1;
+  if constexpr (ND < 8) return ((unsigned long long)raw + (2 * b + 1)) >> 1;
+  return (unsigned long long)((raw + 1) >> 1) + b;
 }
 // rounded and biased m of the real and imaginary part of an element
 template <int ND>
 __device__ __forceinline__ void sl_split(double2 v, int E, unsigned long long &re, unsigned long long &im) {
-  re = sl_round<ND>(sl_raw<ND>(v.x, E));
-  im = sl_round<ND>(sl_raw<ND>(v.y, E));
-}
-template <int ND>
-__device__ __forceinline__ void sl_split(float2 v, int E, unsigned long long &re, unsigned long long &im) {
   re = sl_round<ND>(sl_raw<ND>(v.x, E));
   im = sl_round<ND>(sl_raw<ND>(v.y, E));
 }
@@ -88,12 +87,13 @@ __device__ __forceinline__ void sl_split(float4 v, int E, unsigned long long &re
   im = sl_round<ND>(sl_raw<ND>(v.z, E) + sl_raw<ND>(v.w, E));
 }
 // byte k of two biased values as FP16 digits (u0 low, u1 high): 0x6400 | byte is 1024 + byte
-__device__ __forceinline__ unsigned sl_digits(unsigned long long u0, unsigned long long u1, int k) {
+template <int ND> __device__ __forceinline__ unsigned sl_digits(unsigned long long u0, unsigned long long u1, int k) {
   unsigned x;
-  if (k < 4)
-    x = (__byte_perm((unsigned)u0, (unsigned)u1, k | (k << 4) | ((4 + k) << 8) | ((4 + k) << 12)) & 0x00ff00ffu) |
-        0x64006400u;
-  else  // the 0x64 of byte 7 comes along
+  if (ND == 8 || k < 4) {
+    const int kk = k & 3;
+    x = (__byte_perm(k < 4 ? (unsigned)u0 : (unsigned)(u0 >> 32), k < 4 ? (unsigned)u1 : (unsigned)(u1 >> 32),
+                     kk | (kk << 4) | ((4 + kk) << 8) | ((4 + kk) << 12)) & 0x00ff00ffu) | 0x64006400u;
+  } else  // the 0x64 of byte 7 comes along
     x = __byte_perm((unsigned)(u0 >> 32), (unsigned)(u1 >> 32), (k - 4) | (3 << 4) | (k << 8) | (7 << 12));
   const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&x), __half2half2(__ushort_as_half(0x6480)));
   return *reinterpret_cast<const unsigned *>(&h);
@@ -133,45 +133,6 @@ __device__ __forceinline__ double sl_to_double(long long H, unsigned Lw, int n) 
   const double v = scalbn((double)(top >> 11), ex + n - 52);
   return neg ? -v : v;
 }
-// the same value as a double-float pair
-__device__ __forceinline__ df sl_to_df(long long H, unsigned Lw, int n) {
-  const bool neg = H < 0;
-  if (neg) {
-    Lw = 0u - Lw;
-    H = ~H + (Lw == 0u ? 1 : 0);
-  }
-  unsigned long long top;
-  int ex;
-  const int z = __clzll(H);
-  if (z < 32) {
-    top = ((unsigned long long)H << z) | (((unsigned long long)Lw << z) >> 32);
-    ex = 95 - z;
-  } else {
-    top = ((unsigned long long)H << 32) | Lw;
-    if (top == 0ull) return df{0.f, 0.f};
-    const int z2 = __clzll((long long)top);
-    top <<= z2;
-    ex = 63 - z2;
-  }
-  // top = h 2^40 + rest, |rest| <= 2^39: the high part's 24 bits, rounded, and the remainder to 31 bits
-  const unsigned h = (unsigned)((top >> 40) + ((top >> 39) & 1ull));
-  const int rest = (int)((long long)(top - ((unsigned long long)h << 40)) >> 9);
-  const int e2 = ex + n;  // value = h 2^(e2 - 23) + rest 2^(e2 - 54)
-  df r;
-  if (e2 >= -60 && e2 <= 126) {
-    r.hi = (float)h * __int_as_float((e2 - 23 + 127) << 23);
-    r.lo = e2 >= -40 ? (float)rest * __int_as_float((e2 - 54 + 127) << 23) : ldexpf((float)rest, e2 - 54);
-  } else {
-    r.hi = ldexpf((float)h, e2 - 23);
-    r.lo = isinf(r.hi) ? 0.f : ldexpf((float)rest, e2 - 54);
-  }
-  if (neg) {
-    r.hi = -r.hi;
-    r.lo = -r.lo;
-  }
-  return r;
-}
-
 // D (+)= A B^T, FP16 operands, FP32 accumulator
 __device__ __forceinline__ void mma_f16(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                         uint32_t accumulate) {
@@ -187,26 +148,40 @@ __device__ __forceinline__ uint32_t idesc_f16(int M, int N) {
   return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// The MMAs of one K step (16 values) for all digit pairs of levels below ND. A: ND slices of 128 rows of 128 bytes;
-// B: ND slices of nbp rows each, one after the other, so that one instruction multiplies slice i of A with several
-// slices of B: slice j lands in the accumulator columns of level i + j (level k at column k nbp).
-template <int ND>
+// The MMAs of one K step (16 values) for all digit pairs of levels below NL. A: ND slices of 128 rows of 128 bytes;
+// B: NL slices of nbp rows each, one after the other, so that one instruction multiplies slice i of A with several
+// slices of B: slice j lands in the accumulator columns of level i + j (level k at column k nbp). The slices of B past ND
+// are zero: the first instructions of a sum (i = 0) start the accumulators of all NL levels. An instruction's N is a
+// multiple of 16; where nbp is 8 mod 16 (allowed for ND = NL even), odd counts take one slice more, into an unused
+// level NL.
+template <int ND, int NL>
 __device__ __forceinline__ void sl_mma_step(uint32_t tmem, uint32_t a, uint32_t b, uint32_t ko_a, uint32_t ko_b, int nbp,
                                             bool first) {
-  const int most = 256 / nbp;  // slices per instruction (N <= 256)
+  const int odd = (nbp >> 3) & 1;
+  const int most = (256 / nbp) & ~odd;  // slices per instruction (N <= 256)
 #pragma unroll
   for (int i = 0; i < ND; ++i) {
     const uint64_t ad = sdesc(a + (uint32_t)i * 16384u + ko_a);
-    for (int j = 0; j < ND - i; j += most) {
-      const int cnt = min(ND - i - j, most);
+    const int count = NL - i;
+    for (int j = 0; j < count; j += most) {
+      int cnt = min(count - j, most);
+      cnt += cnt & odd;
       mma_f16(tmem + (uint32_t)((i + j) * nbp), ad, sdesc(b + (uint32_t)(j * nbp) * 128u + ko_b), idesc_f16(128, cnt * nbp),
               (first && i == 0) ? 0u : 1u);
     }
   }
 }
 
-// products per launch that a time-out voided (sliced kernels), read and cleared after a synchronisation
+__device__ __forceinline__ void named_arrive(int id, int count) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+__device__ __forceinline__ void named_sync(int id, int count) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+
+// time-out flags of the sliced kernels, read and cleared after a synchronisation
 int sliced_check();
+int update_sl_check();
 // Gram products of FP64-accurate panels (gram_sl.cu), dtype PC_C128 or PC_DFS, one array part[bi][chunk][p][q] per
 // product: SL_GENERAL A^H B; SL_PAIR A^H A, then A^H B, both upper triangles (q = p); SL_SELF the upper triangle of
 // A^H A
@@ -214,5 +189,9 @@ constexpr int SL_GENERAL = 0, SL_PAIR = 1, SL_SELF = 2;
 int sl_gram_chunks(int nb, long L);
 int launch_gram_sl(int nb, long L, int p, int q, int dtype, const void *A, long sa, const void *B, long sb, int mode,
                    double2 *part, int maxchunk, int *nchunk, cudaStream_t st, const int *act);
+
+// Y = S C (+ Z) for complex128 blocks (update_sl.cu), 1 <= p <= 64
+int launch_update_sl(int nb, long L, int p, int q, const void *S, long ss, const void *C, long sc, void *Y,
+                     long sy, cudaStream_t st, const int *act);
 
 }  // namespace pc

@@ -1,10 +1,14 @@
 """Products of FP64-accurate panels on the tensor cores (exact FP16 digit slices) through the C ABI.
 
-Tolerance of the Gram products. A value is rounded to 2^-54 of the largest part M of its column, and the digit pairs
-below level 6 are dropped: 6 pairs of random digits (uniform on [-128, 127], rms 74) at level 7, 2^(40 + 12.4 + 1.3)
-against M_a M_b >= 2^106 in the same units, so 2^-52.3 M_a M_b (rms) for each of the 2 L real products of an entry.
-Six standard deviations of their sum, 6 sqrt(2 L) 2^-52.2 M_a M_b, bound it; the FP64 sums over spans and chunks add
-a few 2^-53 of the entry.
+Tolerance of the Gram products. A value is rounded to an integer m whose largest in the column is at least 2^53 (M): a
+uniform error of +-1/2, rms 2^-54.8 M, and 2^-54.3 M_a M_b for each of the 2 L real products of an entry; the digit
+pairs of levels 8 and above are far smaller. Six standard deviations of their sum, 6 sqrt(2 L) 2^-54.2 M_a M_b, bound it;
+the FP64 sums over spans and chunks add a few 2^-53 of the entry.
+
+Block updates: one exponent per row and per column of the coefficients (scaled by the largest entry of their row), eight
+digits (m up to 2^61 and more): T = max_i(|s_li| c_i) max_i(|c_ij| / c_i) takes the place of M_a M_b. The seven digit
+pairs of level 8 are dropped, 2^(48 + 12.4 + 1.4) of 2^122 (random digits, rms 74 each): 2^-60.2 T (rms) for each of
+the 2 p real products, and the total is rounded once.
 """
 import numpy as np
 import pytest
@@ -39,7 +43,7 @@ def check(got, A, B, upper=False):
     L = A.shape[2]
     # the reference sums in extended precision, so that its own rounding stays below the tolerance
     ref = np.einsum("bil,bjl->bij", A.conj().astype(np.clongdouble), B.astype(np.clongdouble))
-    tol = 6.0 * np.sqrt(2.0 * L) * 2.0 ** -52.2 * top(A)[:, :, None] * top(B)[:, None, :] + 2.0 ** -50 * np.abs(ref)
+    tol = 6.0 * np.sqrt(2.0 * L) * 2.0 ** -54.2 * top(A)[:, :, None] * top(B)[:, None, :] + 2.0 ** -50 * np.abs(ref)
     ratio = np.abs(got - ref) / np.maximum(tol, np.finfo(np.float64).tiny)
     if upper:
         ratio = np.triu(ratio)
@@ -69,13 +73,13 @@ def test_gram_sliced(pcmod, nb, p, q, L):
 def test_gram_extreme_digits(pcmod, bits):
     """Constant columns whose digits are all at an end of their range: the level sums are the largest possible, and a
     rounding of the accumulator would show. All products are equal, so only the dropped levels' part remains:
-    at most 6 2^54 of 2^106 per product."""
+    at most 5 2^46 of 2^106 per product, below the rounding of the FP64 sums over spans."""
     v = np.array([bits], dtype=np.uint64).view(np.float64)[0]
     L = 4096
     S = np.full((1, 64, L), v * (1 - 1j))
     G, _ = (x.cpu().numpy() for x in pcmod.gram_pair(dev(S), dev(S)))
     ref = float(2 * np.longdouble(v) ** 2 * L)
-    assert np.max(np.abs(G - ref)) <= 7 * 2.0 ** -52 * ref
+    assert np.max(np.abs(G - ref)) <= 8 * 2.0 ** -53 * ref
 
 
 def test_gram_nonfinite(pcmod):
@@ -100,3 +104,43 @@ def test_gram_zero_and_tiny_columns(pcmod):
     G, _ = (x.cpu().numpy() for x in pcmod.gram_pair(dev(S), dev(S)))
     assert np.all(G[0, 2] == 0.0) and np.all(G[0, :, 2] == 0.0)
     check(G, S, S)
+
+
+def check_update(Y, S, C):
+    p = S.shape[1]
+    ref = np.einsum("bpl,bpq->bql", S.astype(np.clongdouble), C.astype(np.clongdouble))
+    part = lambda A: np.maximum(np.abs(A.real), np.abs(A.imag))
+    ci = part(C).max(axis=2)
+    T = (part(S) * ci[:, :, None]).max(axis=1)[:, None, :] * (part(C) / ci[:, :, None]).max(axis=1)[:, :, None]
+    tol = 6.0 * np.sqrt(2.0 * p) * 2.0 ** -59.5 * T + 2.0 ** -52 * np.abs(ref)
+    ratio = np.abs(Y - ref) / tol
+    assert np.all(ratio <= 1.0), float(np.max(ratio))
+
+
+@pytest.mark.parametrize("nb,p,q,L", [(1, 1, 1, 1), (2, 16, 3, 127), (1, 17, 8, 129), (3, 32, 33, 640), (1, 33, 24, 1000),
+                                      (2, 48, 25, 2500), (1, 49, 16, 128), (1, 64, 64, 5000), (200, 9, 4, 300)])
+def test_block_update_sliced(pcmod, nb, p, q, L):
+    S = rand(p + L, (nb, p, L))
+    g = np.random.default_rng(q)
+    C = g.standard_normal((nb, p, q)) + 1j * g.standard_normal((nb, p, q))
+    C /= np.abs(S).max(axis=2)[:, :, None]  # small columns with large coefficients, as preconditioned residuals have
+    check_update(pcmod.block_update(dev(S), dev(C)).cpu().numpy(), S, C)
+
+
+def test_block_update_nonfinite_and_zero(pcmod):
+    """An infinity stays in its row, a NaN coefficient in its column; zero rows give zeros."""
+    S = rand(8, (1, 20, 400))
+    g = np.random.default_rng(9)
+    C = g.standard_normal((1, 20, 12)) + 1j * g.standard_normal((1, 20, 12))
+    S[0, 4, 77] = np.inf
+    S[0, :, 200] = 0.0
+    Y = pcmod.block_update(dev(S), dev(C)).cpu().numpy()
+    bad = ~np.isfinite(Y[0])
+    assert bad[:, 77].all() and bad.sum() == 12 and np.all(Y[0, :, 200] == 0.0)
+    S[0, 4, 77] = 1.0
+    C[0, 3, 5] = np.nan
+    Y = pcmod.block_update(dev(S), dev(C)).cpu().numpy()
+    assert np.isnan(Y[0, 5]).all() and np.isfinite(np.delete(Y[0], 5, axis=0)).all()
+    ok = [j for j in range(12) if j != 5]
+    ref = np.einsum("pl,pq->ql", S[0], C[0][:, ok])
+    assert np.max(np.abs(Y[0][ok] - ref)) <= 1e-12 * np.max(np.abs(ref))
