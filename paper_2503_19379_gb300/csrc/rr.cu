@@ -1,6 +1,6 @@
 // Batched Rayleigh-Ritz step of LOBPCG (Section 5.1): for every k-point the pencil (H, G) = (S^H Op S, S^H S) of
-// its search space S = [X | W | P] (n <= 64 columns) is reduced to its m lowest Ritz pairs, one thread block per
-// k-point, everything in shared memory, FP64.
+// its search space S = [X | W | P] (n <= 64 columns) is reduced to its m lowest Ritz pairs by a cluster of 4, 2 or 1
+// thread blocks per k-point, everything in shared memory, FP64.
 //
 //   1. unit-diagonal scaling D of G (a zero column gets D = 0 and is dropped below);
 //   2. Cholesky of D G D with diagonal pivoting, stopped when the largest remaining pivot is below `drop`: the
@@ -16,7 +16,8 @@
 //
 // A GB300 SM retires about 2 FP64 FMA per clock, so one warp-wide FP64 instruction holds the FP64 unit of its SM
 // sub-partition for tens of cycles and the kernel is bound by its count of FP64 warp instructions on the longest
-// chain. Every phase is therefore spread over the block and over the four sub-partitions: substitutions
+// chain (measured: 64 to 76 cycles per FP64 warp instruction, the same for 1 active lane and for 32, dependent or not).
+// Every phase is therefore spread over the block and over the four sub-partitions: substitutions
 // column-oriented (one rank-1 row update per step for all threads), matrix-vector products split by rows and column
 // quarters, the back-transformation for all wanted vectors at once (short shuffle trees per vector), shared
 // matrices with an odd leading dimension (row-wise access by consecutive threads hits distinct banks), reciprocals
@@ -25,9 +26,19 @@
 // make the FP32 bracket exact for a matrix within a few eps32 |T|; the bracket is widened by 16 eps32 |T| and
 // verified by two FP64 counts, with the Gershgorin interval as fallback), then in FP64 to the absolute width
 // eps64 |T| (LAPACK's default for bisection, below which the FP64 Sturm count itself is not accurate).
+//
+// Where SMs are free the blocks of a cluster divide what divides without a change in any entry's arithmetic (the result
+// is the same bit for bit whatever the cluster size): the columns of the substitutions, the eigenvalues, and their
+// vectors. The factorisation and the tridiagonalisation are repeated in every block: an exchange costs about 1000
+// cycles, a step of the reduction has two, and its scalar chain (4000 cycles) stays. 15 pencils, n = 57, m = 19, in
+// thousands of cycles with 1 and with 4 blocks: Cholesky 280, 288; substitutions 465, 182; tridiagonalisation 622, 623;
+// bisection 740, 633 (13 Sturm counts one after the other); inverse iteration 232, 220; back-transformation 323, 207.
+// The launch takes 1.34 ms with one block per pencil, 1.07 ms with four.
 #include <cfloat>
 #include <climits>
 #include <cmath>
+
+#include <cooperative_groups.h>
 
 #include "pc_internal.cuh"
 
@@ -43,10 +54,14 @@ constexpr double RR_EPS = 2.220446049250313e-16;
 __device__ __forceinline__ double2 shfl_xor_d2(double2 v, int mask) {
   return make_double2(__shfl_xor_sync(0xffffffffu, v.x, mask), __shfl_xor_sync(0xffffffffu, v.y, mask));
 }
+// sum over the warp, in every lane: the lower half-warp sums x and the upper half y, one FP64 instruction a level
 __device__ __forceinline__ double2 warp_sum_d2(double2 v) {
+  const bool up = threadIdx.x & 16;
+  double t = (up ? v.y : v.x) + __shfl_xor_sync(0xffffffffu, up ? v.x : v.y, 16);
 #pragma unroll
-  for (int o = 16; o; o >>= 1) v = cadd(v, shfl_xor_d2(v, o));
-  return v;
+  for (int o = 8; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  const double w = __shfl_xor_sync(0xffffffffu, t, 16);
+  return up ? make_double2(w, t) : make_double2(t, w);
 }
 __device__ __forceinline__ double warp_sum_d(double v) {
 #pragma unroll
@@ -60,28 +75,21 @@ __device__ void tri_factor(const double *d, const double *e, int r, double lam, 
   double *u0i = f, *u1 = f + r, *u2 = f + 2 * r, *l = f + 3 * r, *piv = f + 4 * r;
   double ca = d[0] - lam, cb = r > 1 ? e[0] : 0.0;
   for (int i = 0; i < r - 1; ++i) {
+    // both pivot choices through selects: lanes with different choices share every FP64 instruction
     const double sub = e[i];
     const double ai1 = d[i + 1] - lam, bi1 = (i + 1 < r - 1) ? e[i + 1] : 0.0;
-    if (fabs(ca) >= fabs(sub)) {
-      if (ca == 0.0) ca = tiny;
-      const double ic = 1.0 / ca;
-      l[i] = sub * ic;
-      piv[i] = 0.0;
-      u0i[i] = ic;
-      u1[i] = cb;
-      u2[i] = 0.0;
-      ca = ai1 - l[i] * cb;
-      cb = bi1;
-    } else {
-      const double is = 1.0 / sub;
-      l[i] = ca * is;
-      piv[i] = 1.0;
-      u0i[i] = is;
-      u1[i] = ai1;
-      u2[i] = bi1;
-      ca = cb - l[i] * ai1;
-      cb = -l[i] * bi1;
-    }
+    const bool keep = fabs(ca) >= fabs(sub);
+    double pv = keep ? ca : sub;
+    if (pv == 0.0) pv = tiny;
+    const double ip = __drcp_rn(pv), li = (keep ? sub : ca) * ip;
+    const double nb = keep ? cb : ai1;
+    l[i] = li;
+    piv[i] = keep ? 0.0 : 1.0;
+    u0i[i] = ip;
+    u1[i] = nb;
+    u2[i] = keep ? 0.0 : bi1;
+    ca = fma(-li, nb, keep ? ai1 : cb);
+    cb = keep ? bi1 : -li * bi1;
   }
   if (ca == 0.0) ca = tiny;
   u0i[r - 1] = 1.0 / ca;
@@ -89,20 +97,23 @@ __device__ void tri_factor(const double *d, const double *e, int r, double lam, 
 
 __device__ void tri_solve(const double *f, int r, double *y) {
   const double *u0i = f, *u1 = f + r, *u2 = f + 2 * r, *l = f + 3 * r, *piv = f + 4 * r;
+  double c = y[0];
   for (int i = 0; i < r - 1; ++i) {
-    if (piv[i] != 0.0) {
-      const double yi = y[i];
-      y[i] = y[i + 1];
-      y[i + 1] = yi - l[i] * y[i + 1];
-    } else {
-      y[i + 1] -= l[i] * y[i];
-    }
+    const bool swap = piv[i] != 0.0;
+    const double nx = y[i + 1], top = swap ? nx : c;
+    y[i] = top;
+    c = fma(-l[i], top, swap ? c : nx);
   }
+  y[r - 1] = c;
+  double y1 = 0.0, y2 = 0.0;
   for (int i = r - 1; i >= 0; --i) {
     double s = y[i];
-    if (i + 1 < r) s -= u1[i] * y[i + 1];
-    if (i + 2 < r) s -= u2[i] * y[i + 2];
-    y[i] = s * u0i[i];
+    if (i + 1 < r) s = fma(-u1[i], y1, s);
+    if (i + 2 < r) s = fma(-u2[i], y2, s);
+    s *= u0i[i];
+    y[i] = s;
+    y2 = y1;
+    y1 = s;
   }
 }
 
@@ -173,6 +184,8 @@ size_t rr_smem(int n, int m) {
          sizeof(float) * 2 * (size_t)n + sizeof(int) * (2 * (size_t)n + m) + 64;
 }
 
+// CS: thread blocks per pencil (a cluster)
+template <int CS>
 __global__ void __launch_bounds__(RR_THREADS) rr_kernel(const double2 *__restrict__ Gg, const double2 *__restrict__ Hg,
                                                         int n, int m, double drop, double *__restrict__ thetag,
                                                         double2 *__restrict__ coefg, int *__restrict__ rankg,
@@ -198,7 +211,15 @@ __global__ void __launch_bounds__(RR_THREADS) rr_kernel(const double2 *__restric
   __shared__ double s_il, s_lkk, s_tau2[2], s_gl, s_gu, s_tn, s_pivmin;
   __shared__ double2 s_alpha2[2], s_Kp[2];
   const int tid = threadIdx.x, nt = blockDim.x, warp = tid >> 5, lane = tid & 31, nwarp = nt >> 5;
-  const int b = act ? act[blockIdx.x] : (int)blockIdx.x;
+  const int rank = CS > 1 ? (int)(blockIdx.x % CS) : 0;
+  const int b = act ? act[blockIdx.x / CS] : (int)(blockIdx.x / CS);
+  const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  auto csync = [&] {  // the pencil's blocks
+    if constexpr (CS > 1)
+      cluster.sync();
+    else
+      __syncthreads();
+  };
   const double2 *G = Gg + (long)b * sg;
   const double2 *H = Hg + (long)b * sg;
   double *Z = reinterpret_cast<double *>(B);
@@ -312,12 +333,15 @@ __global__ void __launch_bounds__(RR_THREADS) rr_kernel(const double2 *__restric
   __syncthreads();
 
   // 3. H3 = L^{-1} H_r L^{-H}: two column-oriented forward substitutions with U (row i, once final, updates all rows
-  // below it: four FP64 FMA per entry; the rows are scaled by 1/L_ii at the end), a conjugate transpose in between
+  // below it: four FP64 FMA per entry; the rows are scaled by 1/L_ii at the end), a conjugate transpose in between. The
+  // columns are independent: each block of the cluster takes its share, and the blocks exchange them through
+  // distributed shared memory for the transpose and at the end.
+  const int wc = (r + CS - 1) / CS, jc0 = min(r, rank * wc), nc = min(r, jc0 + wc) - jc0;
   for (int pass = 0; pass < 2; ++pass) {
     for (int i = 0; i + 1 < r; ++i) {
       const int below = r - i - 1;
-      for (int e = tid; e < below * r; e += nt) {
-        const int q = e / r, kk = i + 1 + q, j = e - q * r;
+      for (int e = tid; e < below * nc; e += nt) {
+        const int q = e / nc, kk = i + 1 + q, j = jc0 + e - q * nc;
         const double2 c = Vh[kk * LD + i], y = B[i * LD + j];
         double2 v = B[kk * LD + j];
         v.x = fma(-c.x, y.x, fma(c.y, y.y, v.x));
@@ -326,24 +350,41 @@ __global__ void __launch_bounds__(RR_THREADS) rr_kernel(const double2 *__restric
       }
       __syncthreads();
     }
-    for (int e = tid; e < r * r; e += nt) {
-      const int i = e / r, j = e % r;
+    for (int e = tid; e < r * nc; e += nt) {
+      const int i = e / nc, j = jc0 + e - i * nc;
       B[i * LD + j] = cscale(B[i * LD + j], dinv[i]);
     }
-    __syncthreads();
     if (pass == 0) {
-      for (int e = tid; e < r * r; e += nt) {
-        const int i = e / r, j = e % r;
-        if (i < j) {
-          const double2 x = B[i * LD + j], y = B[j * LD + i];
-          B[i * LD + j] = cmake<double2>(y.x, -y.y);
-          B[j * LD + i] = cmake<double2>(x.x, -x.y);
-        } else if (i == j) {
-          B[i * LD + i].y = -B[i * LD + i].y;
+      // own columns of the conjugate transpose: B'[i][j] = conj(B[j][i]), column i from its block
+      constexpr int NR = (RR_MAXN * ((RR_MAXN + CS - 1) / CS) + RR_THREADS - 1) / RR_THREADS;
+      double2 t[NR];
+      csync();
+#pragma unroll
+      for (int u = 0; u < NR; ++u) {
+        const int e = tid + u * RR_THREADS;
+        if (e < r * nc) {
+          const int j = jc0 + e / r, i = e % r;
+          const double2 *src = B;
+          if constexpr (CS > 1) src = cluster.map_shared_rank(B, i / wc);
+          t[u] = src[j * LD + i];
         }
+      }
+      csync();
+#pragma unroll
+      for (int u = 0; u < NR; ++u) {
+        const int e = tid + u * RR_THREADS;
+        if (e < r * nc) B[(e % r) * LD + jc0 + e / r] = cmake<double2>(t[u].x, -t[u].y);
       }
       __syncthreads();
     }
+  }
+  csync();
+  if constexpr (CS > 1) {
+    for (int e = tid; e < r * r; e += nt) {
+      const int i = e / r, j = e - i * r, o = j / wc;
+      if (o != rank) B[i * LD + j] = cluster.map_shared_rank(B, o)[i * LD + j];
+    }
+    cluster.sync();
   }
   for (int e = tid; e < r * r; e += nt) {
     const int i = e / r, j = e % r;
@@ -376,23 +417,21 @@ __global__ void __launch_bounds__(RR_THREADS) rr_kernel(const double2 *__restric
       sig = fma(x.x, x.x, fma(x.y, x.y, sig));
     }
     sig = warp_sum_d(sig);
+    __syncwarp();
+    // the reciprocal roots of |x|^2 (even lanes) and |x0|^2 (odd lanes) in one go
+    const double2 x0 = vb[0];
+    const double a0 = fma(x0.x, x0.x, x0.y * x0.y), arg = lane & 1 ? a0 : sig;
+    const double rs = arg > 0.0 ? rsqrt(arg) : 0.0, ra = __shfl_sync(0xffffffffu, rs, 1);
+    __syncwarp();
     if (lane == 0) {
-      const double2 x0 = vb[0];
       if (sig == 0.0) {
         s_tau2[slot] = 0.0;
       } else {
-        const double a0 = fma(x0.x, x0.x, x0.y * x0.y);
-        const double nrm = sig * rsqrt(sig);
-        double2 ph = cmake<double2>(1.0, 0.0);
-        double ax0 = 0.0;
-        if (a0 > 0.0) {
-          const double ra = rsqrt(a0);
-          ax0 = a0 * ra;
-          ph = cmake<double2>(x0.x * ra, x0.y * ra);
-        }
+        const double nrm = sig * rs, ax0 = a0 * ra;
+        const double2 ph = a0 > 0.0 ? cmake<double2>(x0.x * ra, x0.y * ra) : cmake<double2>(1.0, 0.0);
         s_alpha2[slot] = cmake<double2>(-ph.x * nrm, -ph.y * nrm);
         vb[0] = cmake<double2>(fma(ph.x, nrm, x0.x), fma(ph.y, nrm, x0.y));
-        s_tau2[slot] = 1.0 / fma(nrm, ax0, sig);
+        s_tau2[slot] = __drcp_rn(fma(nrm, ax0, sig));
       }
     }
   };
@@ -536,11 +575,12 @@ __global__ void __launch_bounds__(RR_THREADS) rr_kernel(const double2 *__restric
 
   // 5. bisection: eigenvalue j (ascending) of T on a group of G lanes (G = 8 up to 32 wanted eigenvalues)
   const int mm = m < r ? m : r;
+  const int wm = (mm + CS - 1) / CS, ja = min(mm, rank * wm), jb = min(mm, ja + wm);  // this block's eigenpairs
   {
     const int G = mm <= nt / 8 ? 8 : (mm <= nt / 4 ? 4 : (mm <= nt / 2 ? 2 : 1));
-    if (tid < ((mm * G + 31) & ~31)) {
-      const int j = tid / G, s = tid % G, base = (tid & 31) & ~(G - 1);
-      const bool active = j < mm;
+    if (tid < (((jb - ja) * G + 31) & ~31)) {
+      const int j = ja + tid / G, s = tid % G, base = (tid & 31) & ~(G - 1);
+      const bool active = j < jb;
       const int jj = active ? j : 0;
       const double tn = s_tn, pivmin = s_pivmin;
       // FP32 bracket
@@ -561,10 +601,14 @@ __global__ void __launch_bounds__(RR_THREADS) rr_kernel(const double2 *__restric
         hi = s_gu;
       }
       multisect<double>(dd, e2, r, pivmin, jj, s, G, active, lo, hi, RR_EPS * tn, 2.0 * RR_EPS, 200);
-      if (active && s == 0) w[j] = 0.5 * (lo + hi);
+      if (active && s == 0) {
+        w[j] = 0.5 * (lo + hi);
+        if constexpr (CS > 1)
+          for (int o = 1; o < CS; ++o) cluster.map_shared_rank(w, (rank + o) % CS)[j] = 0.5 * (lo + hi);
+      }
     }
   }
-  __syncthreads();
+  csync();
   if (tid == 0) {
     int mp = 0;
     for (int j = 0; j < mm; ++j) {
@@ -577,9 +621,11 @@ __global__ void __launch_bounds__(RR_THREADS) rr_kernel(const double2 *__restric
 
   // 6. inverse iteration, cluster position by cluster position; Z (r x mm, column-major by j) lives in B
   const int maxpos = s_maxpos;
-  // eigenvector j on warp j % 4, lane j / 4: the sequential solves run on all four SM sub-partitions
+  // the eigenvectors of this block, and the earlier members of the first one's cluster; one vector per warp % 4 and
+  // lane: the sequential solves run on all four SM sub-partitions
+  const int jfirst = ja < jb ? ja - pos[ja] : ja;
   for (int round = 0; round <= maxpos; ++round) {
-    for (int j = warp + 4 * lane; warp < 4 && j < mm; j += 128) {
+    for (int j = jfirst + warp + 4 * lane; warp < 4 && j < jb; j += 128) {
       if (pos[j] != round) continue;
       double work[5 * RR_MAXN];
       double *z = Z + (long)j * r;
@@ -617,9 +663,10 @@ __global__ void __launch_bounds__(RR_THREADS) rr_kernel(const double2 *__restric
   while (2 * C <= 32 && 2 * C * mm <= nt) C *= 2;
   if (mm > 0 && zsz + (long)r * YLD + mm <= (long)n * LD) {
     double2 *Y = B + zsz, *sj = Y + (long)r * YLD;
-    for (int e = tid; e < r * mm; e += nt) {
-      const int i = e / mm, j = e - i * mm;
-      Y[(long)i * YLD + j] = cscale(phi[i], Z[(long)j * r + i]);
+    const int ml = jb - ja;  // own vectors, columns 0 .. ml - 1 of Y
+    for (int e = tid; e < r * ml; e += nt) {
+      const int i = e / ml, j = e - i * ml;
+      Y[(long)i * YLD + j] = cscale(phi[i], Z[(long)(ja + j) * r + i]);
     }
     __syncthreads();
     for (int k = r - 3; k >= 0; --k) {
@@ -627,21 +674,21 @@ __global__ void __launch_bounds__(RR_THREADS) rr_kernel(const double2 *__restric
       if (tk == 0.0) continue;  // uniform over the block
       const int t = r - k - 1;
       // s_j = tau v_k^H Y[k+1:, j]
-      if (tid < ((C * mm + 31) & ~31)) {  // whole warps (the shuffles)
+      if (tid < ((C * ml + 31) & ~31)) {  // whole warps (the shuffles)
         const int j = tid / C, c = tid - j * C;
         double2 acc = cmake<double2>(0.0, 0.0);
-        if (j < mm)
+        if (j < ml)
           for (int i = c; i < t; i += C) {
             const double2 v = Vh[k * LD + i], y = Y[(long)(k + 1 + i) * YLD + j];  // acc += conj(v) y
             acc.x = fma(v.x, y.x, fma(v.y, y.y, acc.x));
             acc.y = fma(v.x, y.y, fma(-v.y, y.x, acc.y));
           }
         for (int o = C >> 1; o; o >>= 1) acc = cadd(acc, shfl_xor_d2(acc, o));
-        if (j < mm && c == 0) sj[j] = cscale(acc, tk);
+        if (j < ml && c == 0) sj[j] = cscale(acc, tk);
       }
       __syncthreads();
-      for (int e = tid; e < t * mm; e += nt) {
-        const int i = e / mm, j = e - i * mm;
+      for (int e = tid; e < t * ml; e += nt) {
+        const int i = e / ml, j = e - i * ml;
         const double2 v = Vh[k * LD + i], sv = sj[j];  // Y -= v s
         double2 y = Y[(long)(k + 1 + i) * YLD + j];
         y.x = fma(-v.x, sv.x, fma(v.y, sv.y, y.x));
@@ -659,8 +706,8 @@ __global__ void __launch_bounds__(RR_THREADS) rr_kernel(const double2 *__restric
     }
     __syncthreads();
     for (int i = r - 1; i > 0; --i) {
-      for (int e = tid; e < i * mm; e += nt) {
-        const int l = e / mm, j = e - l * mm;
+      for (int e = tid; e < i * ml; e += nt) {
+        const int l = e / ml, j = e - l * ml;
         const double2 c = Vh[i * LD + l], y = Y[(long)i * YLD + j];  // Y[l] -= conj(c) Y[i]
         double2 v = Y[(long)l * YLD + j];
         v.x = fma(-c.x, y.x, fma(-c.y, y.y, v.x));
@@ -669,18 +716,25 @@ __global__ void __launch_bounds__(RR_THREADS) rr_kernel(const double2 *__restric
       }
       __syncthreads();
     }
-    for (int e = tid; e < n * m; e += nt) out[e] = cmake<double2>(0.0, 0.0);
-    __syncthreads();
-    for (int e = tid; e < r * mm; e += nt) {
-      const int i = e / mm, j = e - i * mm;
-      out[perm[i] * m + j] = cscale(Y[(long)i * YLD + j], dinv[i] * dsc[perm[i]]);
+    // rows of dropped directions and columns past the rank are zero
+    const int ncol = ml + (rank == 0 ? m - mm : 0);
+    for (int e = tid; e < n * ncol; e += nt) {
+      const int i = e / ncol, q = e - i * ncol;
+      out[i * m + (q < ml ? ja + q : mm + q - ml)] = cmake<double2>(0.0, 0.0);
     }
-    for (int j = tid; j < m; j += nt) thetag[(long)b * m + j] = j < mm ? w[j] : 0.0;
-    if (rankg && tid == 0) rankg[b] = r;
+    __syncthreads();
+    for (int e = tid; e < r * ml; e += nt) {
+      const int i = e / ml, j = e - i * ml;
+      out[perm[i] * m + ja + j] = cscale(Y[(long)i * YLD + j], dinv[i] * dsc[perm[i]]);
+    }
+    for (int j = tid; j < m && rank == 0; j += nt) thetag[(long)b * m + j] = j < mm ? w[j] : 0.0;
+    if (rankg && tid == 0 && rank == 0) rankg[b] = r;
     return;
   }
   // Otherwise one warp per Ritz vector held in registers (lane l owns rows l and l + 32).
-  for (int j = warp; j < m; j += nwarp) {
+  const int own = jb - ja, todo = own + (rank == 0 ? m - mm : 0);  // block 0 also takes the columns past the rank
+  for (int u = warp; u < todo; u += nwarp) {
+    const int j = u < own ? ja + u : mm + u - own;
     double2 y0 = cmake<double2>(0.0, 0.0), y1 = y0;
     const int i0 = lane, i1 = lane + 32;
     if (j < mm) {
@@ -716,7 +770,7 @@ __global__ void __launch_bounds__(RR_THREADS) rr_kernel(const double2 *__restric
     }
     if (lane == 0) thetag[(long)b * m + j] = j < mm ? w[j] : 0.0;
   }
-  if (rankg && tid == 0) rankg[b] = r;
+  if (rankg && tid == 0 && rank == 0) rankg[b] = r;
 }
 
 }  // namespace
@@ -735,15 +789,30 @@ int launch_rr(int nb, int n, int m, const void *G, const void *H, double drop, d
     set_error("rayleigh_ritz: need m <= n <= %d", RR_MAXN);
     return PC_EINVAL;
   }
-  static bool configured = false;
-  if (!configured) {
-    PC_CK(cudaFuncSetAttribute(rr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)rr_smem(RR_MAXN, RR_MAXN)));
-    configured = true;
+  // blocks per pencil: as many as leave every block an SM of its own (they take most of its shared memory)
+  const int nsm = sm_count(), cs = 4 * nb <= nsm ? 4 : (2 * nb <= nsm ? 2 : 1);
+  const auto kernel = cs == 4 ? rr_kernel<4> : (cs == 2 ? rr_kernel<2> : rr_kernel<1>);
+  static bool configured[64][3] = {};  // per device and block count
+  int dev = 0;
+  PC_CK(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64 || !configured[dev][cs >> 1]) {
+    PC_CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rr_smem(RR_MAXN, RR_MAXN)));
+    if (dev >= 0 && dev < 64) configured[dev][cs >> 1] = true;
   }
-  rr_kernel<<<nb, RR_THREADS, rr_smem(n, m), st>>>(static_cast<const double2 *>(G), static_cast<const double2 *>(H),
-                                                    n, m, drop, theta, static_cast<double2 *>(coef), rank, act,
-                                                    sg > 0 ? sg : (long)n * n, sc > 0 ? sc : (long)n * m);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(nb * cs));
+  cfg.blockDim = dim3(RR_THREADS);
+  cfg.dynamicSmemBytes = rr_smem(n, m);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cs;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cs > 1 ? 1 : 0;
+  PC_CK(cudaLaunchKernelEx(&cfg, kernel, static_cast<const double2 *>(G), static_cast<const double2 *>(H), n, m, drop,
+                           theta, static_cast<double2 *>(coef), rank, act, sg > 0 ? sg : (long)n * n,
+                           sc > 0 ? sc : (long)n * m));
   PC_CK_LAUNCH();
   return PC_OK;
 }
