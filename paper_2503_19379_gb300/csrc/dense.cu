@@ -136,32 +136,40 @@ __global__ void __launch_bounds__(256) gram_tile_partial_kernel(const cplx<T> *_
     }
 }
 
-// Sum of nchunk partial sums, `stride` elements apart, in eight interleaved sums added pairwise: their loads are
-// independent (one chain of loads and adds per chunk was the kernel's time), and the rounding of the sum grows with
-// nchunk / 8.
-__device__ __forceinline__ double2 sum_chunks(const double2 *__restrict__ part, long stride, int nchunk) {
-  double2 s[8];
-#pragma unroll
-  for (int u = 0; u < 8; ++u) s[u] = cmake<double2>(0.0, 0.0);
-  for (int c = 0; c < nchunk; c += 8) {
-#pragma unroll
-    for (int u = 0; u < 8; ++u)
-      if (c + u < nchunk) s[u] = cadd(s[u], part[(c + u) * stride]);
+// Chunk sums in FP64. Eight threads per entry (threadIdx.y) each add every eighth chunk, then the eight sums are added
+// pairwise: one thread per entry, walking 100 chunks and more for few entries, took 120 us per pencil of 57 columns
+// (latency), and the rounding of the sum grows with nchunk / 8. Entry i of the block: threadIdx.x, 32 per block.
+constexpr int RED_X = 32, RED_Y = 8;
+
+__device__ __forceinline__ double2 sum_chunks(const double2 *__restrict__ part, long stride, int nchunk, bool on,
+                                              double2 (*red)[RED_X]) {
+  double2 s = cmake<double2>(0.0, 0.0);
+  if (on) {
+#pragma unroll 4
+    for (int c = threadIdx.y; c < nchunk; c += RED_Y) s = cadd(s, part[c * stride]);
   }
+  red[threadIdx.y][threadIdx.x] = s;
+  __syncthreads();
 #pragma unroll
-  for (int w = 4; w > 0; w >>= 1)
-#pragma unroll
-    for (int u = 0; u < w; ++u) s[u] = cadd(s[u], s[u + w]);
-  return s[0];
+  for (int w = RED_Y / 2; w > 0; w >>= 1) {
+    if ((int)threadIdx.y < w) red[threadIdx.y][threadIdx.x] = cadd(red[threadIdx.y][threadIdx.x], red[threadIdx.y + w][threadIdx.x]);
+    __syncthreads();
+  }
+  s = red[0][threadIdx.x];
+  __syncthreads();
+  return s;
 }
 
-__global__ void gram_reduce_kernel(const double2 *__restrict__ part, int nchunk, int p, int q,
-                                   const int *__restrict__ act, double2 *__restrict__ G, long sg) {
+__global__ void __launch_bounds__(RED_X *RED_Y) gram_reduce_kernel(const double2 *__restrict__ part, int nchunk, int p,
+                                                                   int q, const int *__restrict__ act,
+                                                                   double2 *__restrict__ G, long sg) {
+  __shared__ double2 red[RED_Y][RED_X];
   const int bi = blockIdx.x;
   const int b = act ? act[bi] : bi;
-  for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < p * q; i += gridDim.y * blockDim.x) {
-    G[(long)b * sg + i] = sum_chunks(part + (long)bi * nchunk * p * q + i, (long)p * q, nchunk);
-  }
+  const int i = blockIdx.y * RED_X + threadIdx.x;
+  const bool on = i < p * q;
+  const double2 s = sum_chunks(part + (long)bi * nchunk * p * q + i, (long)p * q, nchunk, on, red);
+  if (on && threadIdx.y == 0) G[(long)b * sg + i] = s;
 }
 
 static int gram_chunks(int nb, long L) {
@@ -213,8 +221,7 @@ int launch_gram(int nb, long L, int p, int q, int dtype, const void *A, long sa,
     gram_partial_kernel<float><<<dim3(nchunk, 1, nb), 256, 0, st>>>(
         static_cast<const float2 *>(A), sa, static_cast<const float2 *>(B), sb, L, p, q, chunk, part, act);
   PC_CK_LAUNCH();
-  gram_reduce_kernel<<<dim3(nb, (p * q + 255) / 256), 256, 0, st>>>(part, nchunk, p, q, act, static_cast<double2 *>(G),
-                                                                    sg > 0 ? sg : (long)p * q);
+  launch_gram_reduce(nb, nchunk, p, q, part, act, G, st, sg);
   PC_CK_LAUNCH();
   return PC_OK;
 }
@@ -298,26 +305,23 @@ __global__ void __launch_bounds__(256) gram_pair_partial_kernel(const cplx<T> *_
     }
 }
 
-// sums the chunks of the upper triangle and mirrors it: G[j][i] = conj(G[i][j])
-__global__ void gram_pair_reduce_kernel(const double2 *__restrict__ partG, const double2 *__restrict__ partH,
-                                        int nchunk, int p, const int *__restrict__ act, double2 *__restrict__ G,
-                                        double2 *__restrict__ H, long sgb) {
+// sums the chunks of the upper triangle and mirrors it: G[j][i] = conj(G[i][j]); blockIdx.z 0: G, 1: H
+__global__ void __launch_bounds__(RED_X *RED_Y) gram_pair_reduce_kernel(const double2 *__restrict__ part, int nchunk,
+                                                                        int p, const int *__restrict__ act,
+                                                                        double2 *__restrict__ G, double2 *__restrict__ H,
+                                                                        long sgb) {
+  __shared__ double2 red[RED_Y][RED_X];
   const int bi = blockIdx.x;
   const int b = act ? act[bi] : bi;
-  for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < p * p; e += gridDim.y * blockDim.x) {
-    const int i = e / p, j = e - i * p;
-    if (i > j) continue;
-    double2 sg = sum_chunks(partG + (long)bi * nchunk * p * p + e, (long)p * p, nchunk);
-    double2 sh = sum_chunks(partH + (long)bi * nchunk * p * p + e, (long)p * p, nchunk);
-    if (i == j) {
-      sg.y = 0.0;
-      sh.y = 0.0;
-    }
-    G[(long)b * sgb + i * p + j] = sg;
-    H[(long)b * sgb + i * p + j] = sh;
-    G[(long)b * sgb + j * p + i] = cmake<double2>(sg.x, -sg.y);
-    H[(long)b * sgb + j * p + i] = cmake<double2>(sh.x, -sh.y);
-  }
+  const int e = blockIdx.y * RED_X + threadIdx.x, i = e / p, j = e - i * p;
+  const bool on = e < p * p && i <= j;
+  const double2 *src = part + (blockIdx.z ? (size_t)gridDim.x * nchunk * p * p : 0) + (long)bi * nchunk * p * p + e;
+  double2 s = sum_chunks(src, (long)p * p, nchunk, on, red);
+  if (!on || threadIdx.y != 0) return;
+  if (i == j) s.y = 0.0;
+  double2 *out = (blockIdx.z ? H : G) + (long)b * sgb;
+  out[i * p + j] = s;
+  out[j * p + i] = cmake<double2>(s.x, -s.y);
 }
 
 size_t gram_pair_scratch_bytes(int nb, long L, int p) {
@@ -326,15 +330,19 @@ size_t gram_pair_scratch_bytes(int nb, long L, int p) {
 
 void launch_gram_pair_reduce(int nb, int nchunk, int p, const double2 *part, const int *act, void *G, void *H,
                              cudaStream_t st, long sg) {
-  gram_pair_reduce_kernel<<<dim3(nb, (p * p + 255) / 256), 256, 0, st>>>(
-      part, part + (size_t)nb * nchunk * p * p, nchunk, p, act, static_cast<double2 *>(G), static_cast<double2 *>(H),
-      sg > 0 ? sg : (long)p * p);
+  gram_pair_reduce_kernel<<<dim3(nb, (p * p + RED_X - 1) / RED_X, 2), dim3(RED_X, RED_Y), 0, st>>>(
+      part, nchunk, p, act, static_cast<double2 *>(G), static_cast<double2 *>(H), sg > 0 ? sg : (long)p * p);
 }
 
 void launch_gram_reduce(int nb, int nchunk, int p, int q, const double2 *part, const int *act, void *G,
                         cudaStream_t st, long sg) {
-  gram_reduce_kernel<<<dim3(nb, (p * q + 255) / 256), 256, 0, st>>>(part, nchunk, p, q, act, static_cast<double2 *>(G),
-                                                                    sg > 0 ? sg : (long)p * q);
+  gram_reduce_kernel<<<dim3(nb, (p * q + RED_X - 1) / RED_X), dim3(RED_X, RED_Y), 0, st>>>(
+      part, nchunk, p, q, act, static_cast<double2 *>(G), sg > 0 ? sg : (long)p * q);
+}
+
+void launch_gram_self_reduce(int nb, int nchunk, int p, const double2 *part, const int *act, void *G, cudaStream_t st) {
+  gram_pair_reduce_kernel<<<dim3(nb, (p * p + RED_X - 1) / RED_X, 1), dim3(RED_X, RED_Y), 0, st>>>(
+      part, nchunk, p, act, static_cast<double2 *>(G), nullptr, (long)p * p);
 }
 
 template <typename T>
@@ -383,9 +391,7 @@ int launch_gram_pair(int nb, long L, int p, int dtype, const void *S, const void
     rc = launch_gram_pair_t<float>(nb, L, p, S, AS, ss, part, nchunk, chunk, st, act);
   }
   if (rc) return rc;
-  gram_pair_reduce_kernel<<<dim3(nb, (p * p + 255) / 256), 256, 0, st>>>(
-      part, part + (size_t)nb * nchunk * p * p, nchunk, p, act, static_cast<double2 *>(G), static_cast<double2 *>(H),
-      sg > 0 ? sg : (long)p * p);
+  launch_gram_pair_reduce(nb, nchunk, p, part, act, G, H, st, sg);
   PC_CK_LAUNCH();
   return PC_OK;
 }
@@ -1122,9 +1128,7 @@ extern "C" int pc_gram_pair_noalloc(int nb, long L, int p, int dtype, const void
   rc = dtype == PC_C128 ? launch_gram_pair_t<double>(nb, L, p, S, AS, ss, part, nchunk, chunk, st, nullptr)
                         : launch_gram_pair_t<float>(nb, L, p, S, AS, ss, part, nchunk, chunk, st, nullptr);
   if (rc) return rc;
-  gram_pair_reduce_kernel<<<dim3(nb, (p * p + 255) / 256), 256, 0, st>>>(
-      part, part + (size_t)nb * nchunk * p * p, nchunk, p, nullptr, static_cast<double2 *>(G),
-      static_cast<double2 *>(H), (long)p * p);
+  launch_gram_pair_reduce(nb, nchunk, p, part, nullptr, G, H, st);
   PC_CK_LAUNCH();
   return PC_OK;
 }

@@ -670,22 +670,6 @@ __global__ void __launch_bounds__(528) gram_df_kernel(const float4 *__restrict__
   part[((long)bi * gridDim.x + blockIdx.x) * p * p + i * p + j] = make_double2(df_to(re), df_to(im));
 }
 
-// chunk sums of the upper triangle in FP64, mirrored
-__global__ void gram_df_reduce_kernel(const double2 *__restrict__ part, int nchunk, int p, const int *__restrict__ act,
-                                      double2 *__restrict__ G) {
-  const int bi = blockIdx.x;
-  const int b = act ? act[bi] : bi;
-  for (int e = threadIdx.x; e < p * p; e += blockDim.x) {
-    const int i = e / p, j = e - i * p;
-    if (i > j) continue;
-    double2 sg = make_double2(0.0, 0.0);
-    for (int c = 0; c < nchunk; ++c) sg = cadd(sg, part[((long)bi * nchunk + c) * p * p + e]);
-    if (i == j) sg.y = 0.0;
-    G[(long)b * p * p + i * p + j] = sg;
-    G[(long)b * p * p + j * p + i] = make_double2(sg.x, -sg.y);
-  }
-}
-
 static int df_chunks(int nb, long L) {
   long want = std::max<long>(1, (8L * sm_count() + nb - 1) / std::max(nb, 1));
   return (int)std::min<long>(std::min<long>(want, std::max<long>(1, L / 512)), 128);
@@ -709,7 +693,7 @@ int launch_gram_df(int nb, long L, int p, const void *X, long sx, void *G, void 
   gram_df_kernel<<<dim3(nchunk, 1, nb), p * (p + 1) / 2, 0, st>>>(static_cast<const float4 *>(X), sx, L, p, chunk,
                                                                    part, act);
   PC_CK_LAUNCH();
-  gram_df_reduce_kernel<<<nb, 256, 0, st>>>(part, nchunk, p, act, static_cast<double2 *>(G));
+  launch_gram_self_reduce(nb, nchunk, p, part, act, G, st);
   PC_CK_LAUNCH();
   return PC_OK;
 }

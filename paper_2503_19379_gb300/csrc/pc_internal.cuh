@@ -229,6 +229,7 @@ size_t gram_pair_scratch_bytes(int nb, long L, int p);
 // reductions of per-chunk partial sums ([nb][nchunk][p][q] double2; the pair: G block then H block, upper triangles)
 void launch_gram_pair_reduce(int nb, int nchunk, int p, const double2 *part, const int *act, void *G, void *H,
                              cudaStream_t st, long sg = 0);
+void launch_gram_self_reduce(int nb, int nchunk, int p, const double2 *part, const int *act, void *G, cudaStream_t st);
 void launch_gram_reduce(int nb, int nchunk, int p, int q, const double2 *part, const int *act, void *G,
                         cudaStream_t st, long sg = 0);
 // complex64 Gram products on the tensor cores (gram_tc.cu); PC_EUNSUPPORTED when the shape does not fit
