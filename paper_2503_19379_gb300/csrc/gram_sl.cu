@@ -9,18 +9,21 @@
 // of SG_SUPER rows, which share one exponent per column (found by a scan of the span; the second read comes from the
 // L2 cache), in stages of 32 rows: 16 warps turn the stage's elements into digits in the K-major tiles of the tensor
 // core (128-byte swizzle; two stages side by side in the 64-wide tile, so that the digits of one stage are formed while
-// the MMAs of the stage before run), the 17th issues the MMAs, and after every fourth stage (128 rows, the most that
-// FP32 holds exactly) the level sums are drained into 64-bit integer sums in registers. At the end of a span these are
+// the MMAs of the stage before run), the 17th issues the MMAs, and after every group of rows that FP32 holds
+// exactly (SlForm::KMAX) the level sums are drained into 64-bit integer sums in registers. At the end of a span these are
 // scaled and added to FP64 sums in shared memory.
 //
-// Eight levels of seven digits leave less error than the FP64 sums they replace, in every entry of G and H (against
-// extended precision, N = 8 to 32, smooth and random panels); seven levels left up to 1.8 times more off the diagonal.
+// Complex128 panels take seven digits in eight levels, which leaves less error than the FP64 sums they replace, in every
+// entry of G and H (against extended precision, N = 8 to 32, smooth and random panels; seven levels left up to 1.8 times
+// more off the diagonal). Pairs take seven digits of base 128: 1e-15 of the diagonal, the double-float sums 3e-14.
 //
-// Bound: integer instructions of the digit extraction (8 k-points x 48 columns at N = 32: 2.19 ms, of which a variant
-// without the scan saves 0.3 ms, without the MMAs 0.4 ms, and the extraction alone takes 1.0 ms; the tensor pipe is 24%
-// busy). The CUDA cores' FP64 pipe took 23.6 ms, and 1.77 ms against 64 us for one k-point of 24 columns at N = 16. The pair A^H A, A^H B therefore takes the block's columns of A
-// and of B in one CTA, and the columns of A that the block shares with the left operand are extracted once and stored
-// twice.
+// Bound: the latency of a stage (load, digits, hand-off to the tensor core, drain), then integer instructions of the digit
+// extraction. 8 k-points x 48 complex128 columns at N = 32: 23.6 ms on the FP64 pipe, 1.92 ms here (without the scan
+// 0.3 ms less, without the MMAs 0.4 ms, without the drains 0.2 ms); one k-point of 24 columns at N = 16: 1.77 ms and
+// 64 us. X^H X of 4 k-points x 19 pair columns at N = 64: 1.61 ms in double-float arithmetic, 1.11 ms here; of one
+// k-point x 13 at N = 16: 60 and 24 us. The pair A^H A, A^H B takes the block's columns of A and of B in one CTA, and the
+// columns of A that the block shares with the left operand are extracted once and stored twice.
+
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -33,11 +36,7 @@ namespace {
 constexpr int SG_CONV = 512;                  // threads that form digits and drain
 constexpr int SG_THREADS = SG_CONV + 32;      // and the warp that issues the MMAs
 constexpr int SG_ROWS = 32;                   // rows per stage
-constexpr int SG_GROUP = 4;                   // stages per drain
 constexpr int SG_SUPER = 1024;                // rows per common exponent
-constexpr int SG_ND = 7;                      // digits
-constexpr int SG_NL = 8;                      // levels of digit products
-constexpr int SG_TASKS = 3;                   // (64 + 32 columns) x 16 row pairs over 512 threads
 
 __device__ int g_gram_sl_error = 0;
 
@@ -51,9 +50,11 @@ struct SlGramArgs {
   const int *act;
 };
 
-template <typename T>
+// TASKS: at most 32 TASKS columns to extract (each thread two rows of every 32nd column); DEPTH: stages loaded ahead
+template <typename T, int TASKS, int DEPTH>
 __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs a) {
-  constexpr int ND = SG_ND, NL = SG_NL;
+  using F = SlForm<T>;
+  constexpr int ND = F::ND, NL = F::NL, GROUP = F::KMAX / SG_ROWS;  // stages per drain
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_addr(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -116,13 +117,13 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
   auto col_of = [&](int jj) { return jj < ndup ? j0 + jj : pa + jj - ndup; };
 
   int n = 0;  // stages issued
-  for (long t0 = r0; t0 < r1; t0 += SG_SUPER) {
-    const long t1 = min(r1, t0 + SG_SUPER);
+  for (long span0 = r0; span0 < r1; span0 += SG_SUPER) {
+    const long span1 = min(r1, span0 + SG_SUPER);
     for (int c = warp; c < ncols; c += SG_THREADS / 32) {
       const T *x = c < pa ? Ab + (long)c * L : Bb + (long)(c - pa) * L;
       int mx = 0;
 #pragma unroll 16
-      for (long l = t0 + lane; l < t1; l += 32) mx = max(mx, sl_key(x[l]));
+      for (long l = span0 + lane; l < span1; l += 32) mx = max(mx, sl_key(x[l]));
       mx = sl_exp_of<T>(__reduce_max_sync(0xffffffffu, mx));
       if (lane == 0) {
         sE[c] = mx;
@@ -130,7 +131,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
       }
     }
     __syncthreads();
-    const int ns = (int)((t1 - t0 + SG_ROWS - 1) / SG_ROWS);
+    const int ns = (int)((span1 - span0 + SG_ROWS - 1) / SG_ROWS);
     if (*bad) {
       // an infinity or a NaN in the span: its products in plain FP64
       if (drains && ci < pa)
@@ -139,7 +140,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
           if (jj >= ndup + nown) break;
           const T *x = Ab + (long)ci * L, *y = jj < ndup ? Ab + (long)(j0 + jj) * L : Bb + (long)(jj - ndup) * L;
           double s = 0.0;
-          for (long l = t0; l < t1; ++l) {
+          for (long l = span0; l < span1; ++l) {
             const double2 u = ld_c128(x + l), v = ld_c128(y + l);
             s = odd ? fma(u.x, v.y, fma(-u.y, v.x, s)) : fma(u.x, v.x, fma(u.y, v.y, s));
           }
@@ -151,12 +152,12 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
       for (int s = 0; s < ns; ++s, ++n) {
         const int buf = n & 1;
         named_sync(1 + buf, SG_THREADS);
-        if (lane == 0) {
+        if (elect_one()) {
           tc_fence_after();
 #pragma unroll
           for (int ks = 0; ks < SG_ROWS / 16; ++ks) {
             const uint32_t ko = (uint32_t)(buf * 64 + ks * 32);
-            sl_mma_step<ND, NL>(tmem, base, base + off_b, ko, ko, a.nbp, (s & (SG_GROUP - 1)) == 0 && ks == 0);
+            sl_mma_step<ND, NL>(tmem, base, base + off_b, ko, ko, a.nbp, (s & (GROUP - 1)) == 0 && ks == 0);
           }
           mma_commit(bars + 8u * buf);
         }
@@ -166,31 +167,56 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
       long long shi[8], slo[8];  // the levels before the last four, and the last four
 #pragma unroll
       for (int k = 0; k < 8; ++k) shi[k] = slo[k] = 0;
-      T v[SG_TASKS][2];
-      auto load = [&](int k, long s0) {
+      T ring[DEPTH][TASKS][2];
+      auto load = [&](T(&v)[2], int k, int s) {
         const int c = c0 + 32 * k;
-        const long l = s0 + 2 * rp;
-        v[k][0] = v[k][1] = T{};
+        const long l = span0 + (long)s * SG_ROWS + 2 * rp;
+        v[0] = v[1] = T{};
         if (c < ncols) {
           const T *x = (c < pa ? Ab + (long)c * L : Bb + (long)(c - pa) * L) + l;
-          if (l < t1) v[k][0] = x[0];
-          if (l + 1 < t1) v[k][1] = x[1];
+          if (l < span1) v[0] = x[0];
+          if (l + 1 < span1) v[1] = x[1];
         }
       };
 #pragma unroll
-      for (int k = 0; k < SG_TASKS; ++k) load(k, t0);
-      for (int s = 0; s < ns; ++s) {
+      for (int d = 0; d < DEPTH; ++d)
+#pragma unroll
+        for (int k = 0; k < TASKS; ++k) load(ring[d][k], k, d);
+      for (int s0 = 0; s0 < ns; s0 += DEPTH)
+#pragma unroll
+      for (int dd = 0; dd < DEPTH; ++dd) {
+        const int s = s0 + dd;
+        if (s >= ns) break;
         const int buf = n & 1;
         if (n >= 2) bar_wait(bars + 8u * buf, ((n >> 1) & 1) ^ 1, abort);
 #pragma unroll
-        for (int k = 0; k < SG_TASKS; ++k) {
+        for (int k = 0; k < TASKS; ++k) {
           const int c = c0 + 32 * k;
           if (c < ncols) {
             const int E = sE[c];
-            unsigned long long m[2][2];
-            sl_split<ND>(v[k][0], E, m[0][0], m[1][0]);
-            sl_split<ND>(v[k][1], E, m[0][1], m[1][1]);
-            load(k, t0 + (long)(s + 1) * SG_ROWS);  // in flight while the digits of the other columns are formed
+            unsigned x[2][ND];  // the digits of rows 2 rp and 2 rp + 1, real and imaginary parts
+            if constexpr (std::is_same<T, double2>::value) {
+              unsigned long long m[2][2];
+              sl_split<ND>(ring[dd][k][0], E, m[0][0], m[1][0]);
+              sl_split<ND>(ring[dd][k][1], E, m[0][1], m[1][1]);
+#pragma unroll
+              for (int d = 0; d < ND; ++d) {
+                x[0][d] = sl_digits<ND>(m[0][0], m[0][1], ND - 1 - d);
+                x[1][d] = sl_digits<ND>(m[1][0], m[1][1], ND - 1 - d);
+              }
+            } else {
+              const float f = sl7_scale(E);
+              unsigned t0[ND], t1[ND];
+              sl7_digits(ring[dd][k][0].x, ring[dd][k][0].y, f, t0);
+              sl7_digits(ring[dd][k][1].x, ring[dd][k][1].y, f, t1);
+#pragma unroll
+              for (int d = 0; d < ND; ++d) x[0][d] = sl7_pack(t0[d], t1[d]);
+              sl7_digits(ring[dd][k][0].z, ring[dd][k][0].w, f, t0);
+              sl7_digits(ring[dd][k][1].z, ring[dd][k][1].w, f, t1);
+#pragma unroll
+              for (int d = 0; d < ND; ++d) x[1][d] = sl7_pack(t0[d], t1[d]);
+            }
+            load(ring[dd][k], k, s + DEPTH);  // in flight while the digits of the other columns are stored
             const bool left = c < pa, dup = left && c >= j0 && ndup > 0;
             const int jr = left ? c - j0 : ndup + c - pa;  // right operand column
 #pragma unroll
@@ -200,9 +226,8 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
               unsigned char *ob = sm + off_b + rb * 128 + (((buf * 4 + (rp >> 2)) ^ (rb & 7)) << 4) + (rp & 3) * 4;
 #pragma unroll
               for (int d = 0; d < ND; ++d) {
-                const unsigned x = sl_digits<ND>(m[h][0], m[h][1], ND - 1 - d);
-                if (left) *reinterpret_cast<unsigned *>(oa + d * 16384) = x;
-                if (!left || dup) *reinterpret_cast<unsigned *>(ob + d * (a.nbp * 128)) = x;
+                if (left) *reinterpret_cast<unsigned *>(oa + d * 16384) = x[h][d];
+                if (!left || dup) *reinterpret_cast<unsigned *>(ob + d * (a.nbp * 128)) = x[h][d];
               }
             }
           }
@@ -211,7 +236,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
         tc_fence_before();
         named_arrive(1 + buf, SG_THREADS);
         ++n;
-        if ((s & (SG_GROUP - 1)) == SG_GROUP - 1 || s == ns - 1) {
+        if ((s & (GROUP - 1)) == GROUP - 1 || s == ns - 1) {
           bar_wait(bars + 8u * buf, ((n - 1) >> 1) & 1, abort);
           tc_fence_after();
           if (drains) {
@@ -225,10 +250,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
                 const int own = __float2int_rn(__uint_as_float(r[2 * k]));
                 const int o = __shfl_xor_sync(0xffffffffu, __float2int_rn(__uint_as_float(r[2 * k + 1])), 1);
                 const int d = odd ? o - own : own + o;
-                if (lv < NL - 4)
-                  shi[k] += (long long)d * (1 << (8 * (NL - 5 - lv)));
-                else
-                  slo[k] += (long long)d * (1 << (8 * (NL - 1 - lv)));
+                sl_level_add<F>(shi[k], slo[k], lv, d);
               }
             }
           }
@@ -240,8 +262,10 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
         for (int k = 0; k < 8; ++k) {
           const int jj = slot * 8 + k;
           if (jj < ndup + nown) {
-            const int sc = EA + sE[col_of(jj)] - 2046 - 2 * (sl_bits<ND>() - 1) + 8 * (2 * ND - 1 - NL);
-            acc[k * SG_CONV + tid] += sl_to_double(shi[k] + (slo[k] >> 32), (unsigned)slo[k], sc);
+            long long H;
+            unsigned Lw;
+            sl_join<F>(shi[k], slo[k], H, Lw);
+            acc[k * SG_CONV + tid] += sl_to_double(H, Lw, sl_weight<F>(EA, sE[col_of(jj)]));
           }
         }
       }
@@ -271,7 +295,9 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
   if (tid == 0 && *abort) atomicExch(&g_gram_sl_error, 1);
 }
 
-size_t sg_smem(int nbp) { return 1024 + SG_ND * 16384 + (size_t)SG_NL * nbp * 128 + 8 * SG_CONV * 8 + 96 * 4 + 64; }
+template <typename F> size_t sg_smem(int nbp) {
+  return 1024 + F::ND * 16384 + (size_t)F::NL * nbp * 128 + 8 * SG_CONV * 8 + 96 * 4 + 64;
+}
 
 }  // namespace
 
@@ -315,22 +341,30 @@ int launch_gram_sl(int nb, long L, int p, int q, int dtype, const void *A, long 
   *nchunk = c;
   a.part0 = part;
   a.part1 = part + (size_t)nb * c * p * q;
-  const size_t smem = sg_smem(a.nbp);
+  using F64 = SlForm<double2>;
+  using FDF = SlForm<float4>;
+  const size_t smem = dtype == PC_DFS ? sg_smem<FDF>(a.nbp) : sg_smem<F64>(a.nbp);
   const dim3 grid(c, nblk, nb);
-  // per device: the attribute belongs to the function on the current device
-  static bool configured[64][2] = {};
+  // columns that a block extracts: its left columns, up to all p, and its own of B
+  const int ncols = p + (mode == SL_SELF ? 0 : a.nbc);
+  const int kind = dtype == PC_DFS ? 0 : (ncols <= 32 ? 1 : (ncols <= 64 ? 2 : 3));
+  if (kind == 0 && ncols > 32) {
+    set_error("gram_sl: at most 32 columns of double-float pairs");
+    return PC_EINVAL;
+  }
+  const auto kernel = kind == 0   ? gram_sl_kernel<float4, 1, 3>
+                      : kind == 1 ? gram_sl_kernel<double2, 1, 3>
+                      : kind == 2 ? gram_sl_kernel<double2, 2, 1>
+                                  : gram_sl_kernel<double2, 3, 1>;
+  static bool configured[64][4] = {};  // per device
   int dev = 0;
   PC_CK(cudaGetDevice(&dev));
-  const int kind = dtype == PC_DFS ? 1 : 0;
   if (dev < 0 || dev >= 64 || !configured[dev][kind]) {
-    PC_CK(cudaFuncSetAttribute(kind ? gram_sl_kernel<float4> : gram_sl_kernel<double2>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sg_smem(64)));
+    PC_CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)(kind ? sg_smem<F64>(64) : sg_smem<FDF>(64))));
     if (dev >= 0 && dev < 64) configured[dev][kind] = true;
   }
-  if (kind)
-    gram_sl_kernel<float4><<<grid, SG_THREADS, smem, st>>>(a);
-  else
-    gram_sl_kernel<double2><<<grid, SG_THREADS, smem, st>>>(a);
+  kernel<<<grid, SG_THREADS, smem, st>>>(a);
   PC_CK_LAUNCH();
   return PC_OK;
 }

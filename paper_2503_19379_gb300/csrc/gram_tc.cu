@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) gram_tc_kernel(const TcArgs a, 
     const int yA = (int)(b * a.cppA), yB = (int)(b * a.cppB), yR = (int)(b * a.cppR);
     const int nstage = (ntile + TC_SPT - 1) / TC_SPT;
     int issued = 0;
-    if (lane == 0) {
+    if (elect_one()) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
       if (a.RB > 0) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmR)) : "memory");
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) gram_tc_kernel(const TcArgs a, 
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       bool ok = true;
       for (int g = 0; g < ngroup && ok; ++g) {
         const int v = g & 1;

@@ -5,13 +5,14 @@
 //   op_df_kernel / opz_df_kernel  AX = Op X (the stencil of stencil.cu; differences, shifts, M0, gamma in
 //                     double-float), or, in the solver, the residual epilogue: R = AX - X Theta and complex64 copies
 //                     of R, X and AX, plus column norms (AX itself is not stored)
-//   update_df_kernel  X' = X C + Z  (Z: the complex64 correction [W P] coef_{W,P})
-//   gram_df_kernel    G = X^H X  (upper triangle, Hermitian mirror)
+//   launch_update_df  X' = X C + Z  (Z: the complex64 correction [W P] coef_{W,P}; on the tensor cores, update_sl.cu)
+//   launch_gram_df    G = X^H X  (on the tensor cores, gram_sl.cu)
 #include <cmath>
 #include <type_traits>
 
 #include "dfloat.cuh"
 #include "pc_internal.cuh"
+#include "sliced.cuh"
 
 namespace pc {
 
@@ -542,141 +543,22 @@ int launch_op_df_resid(pc_ctx *ctx, int nb, int m, const void *X, long sx, const
 }
 
 // ---------------------------------------------------------------- block update Y = X C + Z
-// One row per thread, QB output columns per block row of the grid (QB from the column count so that few columns
-// are computed for nothing: 19 columns take two blocks of 10, not three of 8). Coefficients in shared memory as
-// double-float (re, im, -im); each term is a dfsum multiply-add (12 FP32 operations per real term).
-template <int QB>
-__global__ void __launch_bounds__(256) update_df_kernel(const float4 *__restrict__ X, long sx,
-                                                       const double2 *__restrict__ Cm, long sc,
-                                                       float4 *__restrict__ Y, long sy,
-                                                       const float2 *__restrict__ Z, long sz, long L, int p, int q,
-                                                       const int *__restrict__ act) {
-  __shared__ df Cs[64][QB][3];  // (re, im, -im) of C[i][j0 + c]
-  const int b = act ? act[blockIdx.z] : (int)blockIdx.z;
-  const int j0 = blockIdx.y * QB;
-  const double2 *Cb = Cm + (long)b * sc;
-  for (int i = threadIdx.x; i < p * QB; i += blockDim.x) {
-    const int r = i / QB, c = i - r * QB;
-    const double2 v = (j0 + c < q) ? Cb[r * q + j0 + c] : make_double2(0.0, 0.0);
-    Cs[r][c][0] = df_from(v.x);
-    Cs[r][c][1] = df_from(v.y);
-    Cs[r][c][2] = df_from(-v.y);
-  }
-  __syncthreads();
-  const long l = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (l >= L) return;
-  const float4 *Xb = X + (long)b * sx;
-  dfsum re[QB], im[QB];
-#pragma unroll
-  for (int c = 0; c < QB; ++c) re[c] = im[c] = dfsum{0.f, 0.f};
-  for (int i = 0; i < p; ++i) {
-    const cdf xv = ld_cdf(Xb + (long)i * L + l);
-#pragma unroll
-    for (int c = 0; c < QB; ++c) {
-      // (xr + i xi)(cr + i ci) = (xr cr - xi ci) + i (xr ci + xi cr)
-      dfsum_mac(re[c], xv.re, Cs[i][c][0]);
-      dfsum_mac(re[c], xv.im, Cs[i][c][2]);
-      dfsum_mac(im[c], xv.re, Cs[i][c][1]);
-      dfsum_mac(im[c], xv.im, Cs[i][c][0]);
-    }
-  }
-  float4 *Yb = Y + (long)b * sy;
-  const float2 *Zb = Z ? Z + (long)b * sz : nullptr;
-#pragma unroll
-  for (int c = 0; c < QB; ++c)
-    if (j0 + c < q) {
-      if (Zb) {
-        const float2 z = Zb[(long)(j0 + c) * L + l];
-        dfsum_addf(re[c], z.x);
-        dfsum_addf(im[c], z.y);
-      }
-      st_cdf(Yb + (long)(j0 + c) * L + l, cdf{dfsum_value(re[c]), dfsum_value(im[c])});
-    }
-}
-
+// On the tensor cores (update_sl.cu).
 int launch_update_df(int nb, long L, int p, int q, const void *X, long sx, const void *C, long sc, void *Y, long sy,
                      const void *Z, long sz, cudaStream_t st, const int *act) {
   if (nb == 0 || q == 0) return PC_OK;
-  if (p > 64) {
-    set_error("update_df: at most 64 input columns");
+  if (p < 1 || p > 32) {
+    set_error("update_df: 1 to 32 input columns");
     return PC_EINVAL;
   }
-  // blocks of columns: 8 wide unless 10 wastes fewer (q = 19: 2 x 10 instead of 3 x 8)
-  const int nb8 = (q + 7) / 8, nb10 = (q + 9) / 10;
-  const bool wide = nb10 * 10 < nb8 * 8;
-  const unsigned gx = (unsigned)((L + 255) / 256);
-  if (wide)
-    update_df_kernel<10><<<dim3(gx, nb10, nb), 256, 0, st>>>(static_cast<const float4 *>(X), sx,
-                                                             static_cast<const double2 *>(C), sc, static_cast<float4 *>(Y),
-                                                             sy, static_cast<const float2 *>(Z), sz, L, p, q, act);
-  else
-    update_df_kernel<8><<<dim3(gx, nb8, nb), 256, 0, st>>>(static_cast<const float4 *>(X), sx,
-                                                           static_cast<const double2 *>(C), sc, static_cast<float4 *>(Y),
-                                                           sy, static_cast<const float2 *>(Z), sz, L, p, q, act);
-  PC_CK_LAUNCH();
-  return PC_OK;
+  return launch_update_sl(nb, L, p, q, PC_DFS, X, sx, C, sc, Y, sy, Z, sz, st, act);
 }
 
 // ---------------------------------------------------------------- Gram G = X^H X of the FP64 block
 // (X^H AX is not formed here: the mixed solve takes it as Theta X^H X + R^H X, R = AX - X Theta.)
-constexpr int DF_TL = 32;
-
-// One thread per upper-triangle entry (i <= j): p(p+1)/2 threads; grid (nchunk, 1, nb).
-__global__ void __launch_bounds__(528) gram_df_kernel(const float4 *__restrict__ X, long sx, long L, int p,
-                                                     long chunk, double2 *__restrict__ part,
-                                                     const int *__restrict__ act) {
-  __shared__ cdf Xs[32][DF_TL + 1];
-  __shared__ unsigned char pi[528], pj[528];
-  const int bi = blockIdx.z;
-  const int b = act ? act[bi] : bi;
-  const float4 *Xb = X + (long)b * sx;
-  const int tid = threadIdx.x, nthr = blockDim.x;
-  if (tid == 0) {
-    int t = 0;
-    for (int i = 0; i < p; ++i)
-      for (int j = i; j < p; ++j, ++t) {
-        pi[t] = (unsigned char)i;
-        pj[t] = (unsigned char)j;
-      }
-  }
-  __syncthreads();
-  const int i = pi[tid], j = pj[tid];
-  // two independent sums (even and odd rows of each tile): twice the instruction-level parallelism of one chain
-  dfsum re0{0.f, 0.f}, im0{0.f, 0.f}, re1{0.f, 0.f}, im1{0.f, 0.f};
-  const long beg = (long)blockIdx.x * chunk, end = min(L, beg + chunk);
-  for (long l0 = beg; l0 < end; l0 += DF_TL) {
-    for (int e = tid; e < p * DF_TL; e += nthr) {
-      const int col = e / DF_TL, t = e - col * DF_TL;
-      const long l = l0 + t;
-      Xs[col][t] = l < end ? ld_cdf(Xb + (long)col * L + l) : cdf{df{0.f, 0.f}, df{0.f, 0.f}};
-    }
-    __syncthreads();
-#pragma unroll 2
-    for (int t = 0; t < DF_TL; t += 2) {
-      const cdf a = Xs[i][t], c = Xs[j][t], a1 = Xs[i][t + 1], c1 = Xs[j][t + 1];
-      // conj(a) c = (ar cr + ai ci) + i (ar ci - ai cr)
-      dfsum_mac(re0, a.re, c.re);
-      dfsum_mac(re1, a1.re, c1.re);
-      dfsum_mac(im0, a.re, c.im);
-      dfsum_mac(im1, a1.re, c1.im);
-      dfsum_mac(re0, a.im, c.im);
-      dfsum_mac(re1, a1.im, c1.im);
-      dfsum_mac(im0, df_neg(a.im), c.re);
-      dfsum_mac(im1, df_neg(a1.im), c1.re);
-    }
-    __syncthreads();
-  }
-  const df re = df_add(dfsum_value(re0), dfsum_value(re1)), im = df_add(dfsum_value(im0), dfsum_value(im1));
-  part[((long)bi * gridDim.x + blockIdx.x) * p * p + i * p + j] = make_double2(df_to(re), df_to(im));
-}
-
-static int df_chunks(int nb, long L) {
-  long want = std::max<long>(1, (8L * sm_count() + nb - 1) / std::max(nb, 1));
-  return (int)std::min<long>(std::min<long>(want, std::max<long>(1, L / 512)), 128);
-}
-
+// On the tensor cores (gram_sl.cu).
 size_t gram_df_scratch_bytes(int nb, long L, int p) {
-  return sizeof(double2) * (size_t)nb * df_chunks(nb, L) * p * p;
+  return sizeof(double2) * (size_t)nb * sl_gram_chunks(nb, L) * p * p;
 }
 
 int launch_gram_df(int nb, long L, int p, const void *X, long sx, void *G, void *scratch, size_t scratch_bytes,
@@ -686,13 +568,10 @@ int launch_gram_df(int nb, long L, int p, const void *X, long sx, void *G, void 
     set_error("gram_df: at most 32 columns and enough scratch");
     return PC_EINVAL;
   }
-  const int nchunk = df_chunks(nb, L);
-  long chunk = (L + nchunk - 1) / nchunk;
-  chunk = (chunk + DF_TL - 1) / DF_TL * DF_TL;
   double2 *part = static_cast<double2 *>(scratch);
-  gram_df_kernel<<<dim3(nchunk, 1, nb), p * (p + 1) / 2, 0, st>>>(static_cast<const float4 *>(X), sx, L, p, chunk,
-                                                                   part, act);
-  PC_CK_LAUNCH();
+  int nchunk = 0;
+  const int rc = launch_gram_sl(nb, L, p, p, PC_DFS, X, sx, X, sx, SL_SELF, part, sl_gram_chunks(nb, L), &nchunk, st, act);
+  if (rc) return rc;
   launch_gram_self_reduce(nb, nchunk, p, part, act, G, st);
   PC_CK_LAUNCH();
   return PC_OK;

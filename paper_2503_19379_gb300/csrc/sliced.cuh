@@ -28,17 +28,15 @@ constexpr int SL_EMIN = 128;  // common exponents start here: FP64 values too sm
 __device__ __forceinline__ int sl_key(double2 v) {
   return max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff);
 }
-__device__ __forceinline__ int sl_key(float2 v) {
-  return max(__float_as_int(v.x) & 0x7fffffff, __float_as_int(v.y) & 0x7fffffff);
-}
 __device__ __forceinline__ int sl_key(float4 v) {  // a pair's low part is normally far below its high part
-  return max(sl_key(make_float2(v.x, v.z)), sl_key(make_float2(v.y, v.w)));
+  return max(max(__float_as_int(v.x) & 0x7fffffff, __float_as_int(v.z) & 0x7fffffff),
+             max(__float_as_int(v.y) & 0x7fffffff, __float_as_int(v.w) & 0x7fffffff));
 }
 // biased FP64 exponent of a key (0x7ff for an infinity or a NaN)
 template <typename T> __device__ __forceinline__ int sl_exp_of(int key) {
   if constexpr (std::is_same<T, double2>::value) return max(key >> 20, SL_EMIN);
   const int e = key >> 23;
-  return e == 0xff ? SL_NONFINITE : max(e, 1) + 896;
+  return e == 0xff ? SL_NONFINITE : max(e, 6) + 896;  // (not below 902: sl_scale stays an FP32 number)
 }
 
 __device__ __forceinline__ unsigned sl_shr(unsigned x, int s) {  // 0 for s >= 32
@@ -60,12 +58,6 @@ template <int ND> __device__ __forceinline__ long long sl_raw(double x, int E) {
   // zeros and subnormals (e = 0) are shifted out, as E >= SL_EMIN
   return sl_shift(mh, lo << PS, E - (int)((hi >> 20) & 0x7ff), (int)hi >> 31);
 }
-template <int ND> __device__ __forceinline__ long long sl_raw(float x, int E) {
-  const unsigned u = (unsigned)__float_as_int(x);
-  const int e = (u >> 23) & 0xff;
-  const unsigned m = (u & 0x7fffffu) | (e ? 0x800000u : 0u);
-  return sl_shift(m >> 1, m << 31, E - 896 + 54 - sl_bits<ND>() - max(e, 1), (int)u >> 31);
-}
 // m with every digit moved up by 128, so that digit j is byte ND - 1 - j minus 128; with seven digits byte 7 holds 0x64
 // (see sl_digits)
 template <int ND> __device__ __forceinline__ unsigned long long sl_round(long long raw) {
@@ -81,11 +73,6 @@ __device__ __forceinline__ void sl_split(double2 v, int E, unsigned long long &r
   re = sl_round<ND>(sl_raw<ND>(v.x, E));
   im = sl_round<ND>(sl_raw<ND>(v.y, E));
 }
-template <int ND>
-__device__ __forceinline__ void sl_split(float4 v, int E, unsigned long long &re, unsigned long long &im) {
-  re = sl_round<ND>(sl_raw<ND>(v.x, E) + sl_raw<ND>(v.y, E));
-  im = sl_round<ND>(sl_raw<ND>(v.z, E) + sl_raw<ND>(v.w, E));
-}
 // byte k of two biased values as FP16 digits (u0 low, u1 high): 0x6400 | byte is 1024 + byte
 template <int ND> __device__ __forceinline__ unsigned sl_digits(unsigned long long u0, unsigned long long u1, int k) {
   unsigned x;
@@ -97,6 +84,72 @@ template <int ND> __device__ __forceinline__ unsigned sl_digits(unsigned long lo
     x = __byte_perm((unsigned)(u0 >> 32), (unsigned)(u1 >> 32), (k - 4) | (3 << 4) | (k << 8) | (7 << 12));
   const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&x), __half2half2(__ushort_as_half(0x6480)));
   return *reinterpret_cast<const unsigned *>(&h);
+}
+
+// Double-float pairs take digits in base 128 (seven: 48 bits, their precision), formed on the FP32 pipe: adding
+// M_k = (1.5 2^23 + 0x6480) 2^-7k to the rest y rounds it to a multiple of 2^-7k and leaves the digit, |d_k| <= 64, plus
+// 0x6480 in the low 16 bits of the sum: the FP16 number 1024 + 128 + d_k. (The integer route of the FP64 values costs
+// twice the instructions for a pair, on the pipe of half the rate. Base 128, because a rest of exactly 1/2 would
+// overflow a digit of base 256 here.)
+// y = v f has |y| < 64 for |v| < 2^(E - 1022)
+__device__ __forceinline__ float sl7_scale(int E) { return __int_as_float(max(1155 - E, 0) << 23); }
+template <int ND> __device__ __forceinline__ void sl7_digits(float hi, float lo, float f, unsigned (&t)[ND]) {
+  static_assert(ND <= 8, "at most eight digits");
+  constexpr float M = 12582912.0f + 25728.0f;
+  constexpr float Mk[8] = {M,           M * 0x1p-7f,  M * 0x1p-14f, M * 0x1p-21f,
+                           M * 0x1p-28f, M * 0x1p-35f, M * 0x1p-42f, M * 0x1p-49f};
+  float y = hi * f;
+  // lo in two parts, each added where the sum with the rest of hi is exact
+  const float l = lo * f, l1 = (l + Mk[4]) - Mk[4], l2 = l - l1;
+#pragma unroll
+  for (int k = 0; k < ND; ++k) {
+    if (k == 3) y += l1;
+    if (k == 5) y += l2;
+    const float s = y + Mk[k];
+    t[k] = (unsigned)__float_as_int(s);
+    y -= s - Mk[k];
+  }
+}
+// the FP16 digits of two values (a low, b high)
+__device__ __forceinline__ unsigned sl7_pack(unsigned a, unsigned b) {
+  const unsigned x = __byte_perm(a, b, 0x5410);
+  const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&x), __half2half2(__ushort_as_half(0x6480)));
+  return *reinterpret_cast<const unsigned *>(&h);
+}
+
+// Per element type: bits per digit, digits, levels of digit products, rows of K whose level sums FP32 holds exactly
+template <typename T> struct SlForm;
+template <> struct SlForm<double2> {  // sums over many rows
+  static constexpr int RB = 8, ND = 7, NL = 8, KMAX = 128;
+};
+template <> struct SlForm<float4> {
+  // (digits 3 and 5 take the low part's share: up to 72 and 128)
+  static constexpr int RB = 7, ND = 7, NL = 7, KMAX = 256;
+};
+template <typename T> struct SlFormShort;  // sums over the columns of a block
+template <> struct SlFormShort<double2> {
+  static constexpr int RB = 8, ND = 8, NL = 8, KMAX = 128;
+};
+template <> struct SlFormShort<float4> {
+  static constexpr int RB = 7, ND = 8, NL = 8, KMAX = 256;
+};
+// sum_k L_k 2^(RB (NL-1-k)) times this power of two is the sum of products of values held at exponents Ea and Eb
+template <typename F> __device__ __forceinline__ int sl_weight(int Ea, int Eb) {
+  return Ea + Eb - 2056 - F::RB * (F::NL - 1);
+}
+// The weighted level sum from the sum hi of the levels before the last four and the sum lo of the last four (each in
+// units of its last level), as H 2^32 + low word
+template <typename F> __device__ __forceinline__ void sl_join(long long hi, long long lo, long long &H, unsigned &Lw) {
+  constexpr int S = 32 - 4 * F::RB;
+  lo += (hi & ((1ll << S) - 1)) << (4 * F::RB);
+  H = (hi >> S) + (lo >> 32);
+  Lw = (unsigned)lo;
+}
+template <typename F> __device__ __forceinline__ void sl_level_add(long long &hi, long long &lo, int lv, int x) {
+  if (lv < F::NL - 4)
+    hi += (long long)x * (1 << (F::RB * (F::NL - 5 - lv)));
+  else
+    lo += (long long)x * (1 << (F::RB * (F::NL - 1 - lv)));
 }
 
 // (H 2^32 + Lw) 2^n rounded to FP64; integer arithmetic only (the FP64 pipe retires about 2 operations per clock and SM)
@@ -133,6 +186,26 @@ __device__ __forceinline__ double sl_to_double(long long H, unsigned Lw, int n) 
   const double v = scalbn((double)(top >> 11), ex + n - 52);
   return neg ? -v : v;
 }
+// the pair sum_k L_k 2^-7k 2^n from level sums (integers of FP32), plus an FP32 addend
+__device__ __forceinline__ df sl7_value(const float (&L)[8], int n, float z) {
+  df s = two_sum(L[0], L[1] * 0x1p-7f);
+  float e = s.lo;
+  s = two_sum(s.hi, L[2] * 0x1p-14f);
+  e += s.lo;
+  s = two_sum(s.hi, L[3] * 0x1p-21f);
+  e += s.lo;
+  e += fmaf(fmaf(fmaf(L[7], 0x1p-7f, L[6]), 0x1p-7f, L[5]), 0x1p-7f, L[4]) * 0x1p-28f;
+  if (n >= -60 && n <= 100) {  // both parts stay normal
+    const float f = __int_as_float((n + 127) << 23);
+    s.hi *= f;
+    e *= f;
+  } else {
+    s.hi = ldexpf(s.hi, n);
+    e = ldexpf(e, n);
+  }
+  return df_addf(quick_two_sum(s.hi, e), z);
+}
+
 // D (+)= A B^T, FP16 operands, FP32 accumulator
 __device__ __forceinline__ void mma_f16(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                         uint32_t accumulate) {
@@ -190,8 +263,8 @@ int sl_gram_chunks(int nb, long L);
 int launch_gram_sl(int nb, long L, int p, int q, int dtype, const void *A, long sa, const void *B, long sb, int mode,
                    double2 *part, int maxchunk, int *nchunk, cudaStream_t st, const int *act);
 
-// Y = S C (+ Z) for complex128 blocks (update_sl.cu), 1 <= p <= 64
-int launch_update_sl(int nb, long L, int p, int q, const void *S, long ss, const void *C, long sc, void *Y,
-                     long sy, cudaStream_t st, const int *act);
+// Y = S C (+ Z, a complex64 addend, for pairs) for PC_C128 (1 <= p <= 64) or PC_DFS (1 <= p <= 32) blocks (update_sl.cu)
+int launch_update_sl(int nb, long L, int p, int q, int dtype, const void *S, long ss, const void *C, long sc, void *Y,
+                     long sy, const void *Z, long sz, cudaStream_t st, const int *act);
 
 }  // namespace pc

@@ -64,6 +64,15 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
       : "memory");
 }
+// True in one lane of a converged warp. tcgen05.mma and its companions belong into a branch on this: their descriptors
+// are warp-uniform registers, and only here does the compiler know that a single lane is active. In a branch on the
+// lane or thread index it serialises over the lanes instead, 174 cycles per MMA whatever its size; in this branch an
+// MMA of 128 x N x 16 (FP16) takes its N / 2 cycles, 40 at least (measured, N = 16 to 256).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(e));
+  return e != 0;
+}
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }

@@ -1,5 +1,5 @@
-// Block updates Y = S C of complex128 blocks on the tensor cores (S: L x p, C: p x q complex), sliced exactly into
-// FP16 digits (sliced.cuh).
+// Block updates Y = S C on the tensor cores (S: L x p, C: p x q complex), sliced exactly into FP16 digits (sliced.cuh):
+// complex128 blocks, and blocks of double-float pairs with a complex64 addend, Y = S C + Z (the mixed solve's block X).
 //
 // One real product per tile of 128 rows: accumulator row = row of S, K = the 2 p real and imaginary parts of a row,
 // accumulator columns 2 j + c = parts of up to 32 columns of Y, once per level. Row l is held against one exponent
@@ -15,11 +15,19 @@
 // as a stage's are used. The epilogue adds the levels as 64-bit integers and rounds once, in integer arithmetic (the
 // FP64 pipe retires about 2 operations per clock and SM).
 //
-// Bound: integer instructions of the digit extraction and the epilogue. 8 k-points, 48 -> 16 columns at N = 32:
-// 4.00 ms on the FP64 pipe (1.21 TFLOP/s, all of it), 0.53 ms here; 4 k-points, 57 -> 19 at N = 64: 27.5 and 2.67 ms;
-// one k-point, 24 -> 8 at N = 16: 54.8 and 17.0 us; the smallest size tried (8 -> 4 columns of 1536 rows): 21.9 and
-// 17.9 us. (For complex64 the same scheme with four digits was slower than the FP32 pipe: 1.29 against 0.97 ms for
-// 57 -> 19 columns at N = 64.)
+// A tile's first two stages are converted before the epilogue of the tile before it, so that the MMAs run meanwhile.
+//
+// Complex128 takes eight digits (the error against extended precision is 4.7e-17 of the result, that of FP64 sums 1.3e-16
+// to 3.4e-16; seven digits left 1.1e-15). Pairs take eight digits of base 128 (2.5e-15, the double-float sums 2.0e-14;
+// seven left 5.4e-14 where C is near the identity).
+//
+// Bound: instructions of the digit extraction and the epilogue. Complex128, 8 k-points, 48 -> 16 columns at N = 32:
+// 4.00 ms on the FP64 pipe (1.21 TFLOP/s, all of it), 0.48 ms here; 4 k-points, 57 -> 19 at N = 64: 27.5 and 2.7 ms; one
+// k-point, 24 -> 8 at N = 16: 54.8 and 17.0 us; the smallest size tried (8 -> 4 columns of 1536 rows): 21.9 and 17.9 us.
+// Pairs, 4 k-points, 19 -> 19 columns at N = 64: 2.03 ms in double-float arithmetic, 1.16 ms here (without the MMAs
+// 0.25 ms less, without the digits 0.3 ms, without the epilogue 0.44 ms); 2 k-points, 12 -> 12 at N = 8: 16.9 and 12.9 us.
+// (For complex64 the same scheme with four digits was slower than the FP32 pipe: 1.29 against 0.97 ms for 57 -> 19
+// columns at N = 64.)
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -32,7 +40,6 @@ namespace {
 constexpr int SU_THREADS = 512;
 constexpr int SU_COLS = 16;  // columns per stage
 constexpr int SU_BAD = 1 << 20;
-constexpr int SU_ND = 8;
 
 __device__ int g_update_sl_error = 0;
 
@@ -43,6 +50,8 @@ struct SlUpdateArgs {
   long sc;
   void *Y;
   long sy;
+  const float2 *Z;
+  long sz;
   long L;
   int p, q, nbc, nbp, ntile;
   uint32_t tmem_cols;
@@ -59,11 +68,12 @@ __device__ __forceinline__ void tmem_wait4(uint32_t (&r)[4]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3])::"memory");
 }
 
-// NS: stages (p <= 16 NS)
-template <int NS>
+// T: element type of S and Y; NS: stages (p <= 16 NS)
+template <typename T, int NS>
 __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdateArgs a) {
-  using T = double2;
-  constexpr int ND = SU_ND;
+  using F = SlFormShort<T>;
+  constexpr int ND = F::ND, NL = F::NL;
+  constexpr bool F64 = std::is_same<T, double2>::value;
   constexpr int NC = 4 * NS;          // columns per thread
   constexpr int NATOM = (NS + 1) / 2;  // 64-wide operand tiles of C
   extern __shared__ unsigned char smem_raw[];
@@ -71,9 +81,9 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
   const uint32_t base = (raw + 1023u) & ~1023u;
   unsigned char *const sm = smem_raw + (base - raw);
   const uint32_t off_b = ND * 16384u, atom = (uint32_t)(ND * a.nbp) * 128u, off_e = off_b + NATOM * atom;
-  int *const sE = reinterpret_cast<int *>(sm + off_e);  // [2][4][128] row exponents (per tile parity and column quarter)
-  int *const sCA = sE + 1024, *const sCB = sCA + 64;    // exponents of the rows and columns of C
-  const uint32_t off_bar = off_e + (1024u + 128u) * 4u;
+  int *const sE = reinterpret_cast<int *>(sm + off_e);  // [3][4][128] row exponents (three tiles in turn, by column quarter)
+  int *const sCA = sE + 1536, *const sCB = sCA + 64;    // exponents of the rows and columns of C
+  const uint32_t off_bar = off_e + (1536u + 128u) * 4u;
   const uint32_t bars = base + off_bar;
   uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(sm + off_bar + 16);
   volatile int *abort = reinterpret_cast<volatile int *>(tmem_holder + 1);
@@ -146,15 +156,36 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
     const int i = t / nbc, j = t - i * nbc;
     const double2 c = Cb[(long)i * a.q + j];
     const int E = sCB[j] + sCA[i], ii = i & 31, kc = ii >> 2;  // four columns (8 values) per 16-byte chunk
-    const unsigned long long cr = sl_round<ND>(sl_raw<ND>(c.x, E)), ci = sl_round<ND>(sl_raw<ND>(c.y, E)),
-                             cn = sl_round<ND>(sl_raw<ND>(-c.y, E));
+    unsigned x0[ND], x1[ND];  // digits of (cr, -ci) and (ci, cr)
+    if constexpr (F64) {
+      const unsigned long long cr = sl_round<ND>(sl_raw<ND>(c.x, E)), ci = sl_round<ND>(sl_raw<ND>(c.y, E)),
+                               cn = sl_round<ND>(sl_raw<ND>(-c.y, E));
+#pragma unroll
+      for (int d = 0; d < ND; ++d) {
+        x0[d] = sl_digits<ND>(cr, cn, ND - 1 - d);
+        x1[d] = sl_digits<ND>(ci, cr, ND - 1 - d);
+      }
+    } else {
+      // scaled in FP64 (|c| 2^(5 - (E - 1023)) < 64), then as pairs
+      const double f = __longlong_as_double((long long)min(max(2051 - E, 1), 2046) << 52);
+      const df re = df_from(c.x * f), im = df_from(c.y * f);
+      unsigned tr[ND], ti[ND], tn[ND];
+      sl7_digits(re.hi, re.lo, 1.0f, tr);
+      sl7_digits(im.hi, im.lo, 1.0f, ti);
+      sl7_digits(-im.hi, -im.lo, 1.0f, tn);
+#pragma unroll
+      for (int d = 0; d < ND; ++d) {
+        x0[d] = sl7_pack(tr[d], tn[d]);
+        x1[d] = sl7_pack(ti[d], tr[d]);
+      }
+    }
     // (x + i y)(cr + i ci): row 2 j holds (cr, -ci), row 2 j + 1 holds (ci, cr)
 #pragma unroll
     for (int d = 0; d < ND; ++d) {
       const int rr = d * a.nbp + 2 * j;
       unsigned char *o = sm + off_b + (i >> 5) * atom + (ii & 3) * 4;
-      *reinterpret_cast<unsigned *>(o + rr * 128 + ((kc ^ (rr & 7)) << 4)) = sl_digits<ND>(cr, cn, ND - 1 - d);
-      *reinterpret_cast<unsigned *>(o + (rr + 1) * 128 + ((kc ^ ((rr + 1) & 7)) << 4)) = sl_digits<ND>(ci, cr, ND - 1 - d);
+      *reinterpret_cast<unsigned *>(o + rr * 128 + ((kc ^ (rr & 7)) << 4)) = x0[d];
+      *reinterpret_cast<unsigned *>(o + (rr + 1) * 128 + ((kc ^ ((rr + 1) & 7)) << 4)) = x1[d];
     }
   }
   fence_proxy_async();
@@ -162,8 +193,159 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
   const int quarter = warp & 3, slot = warp >> 2;
   const uint32_t tdrain = tmem + ((uint32_t)(quarter * 32) << 16);
   T *const Yb = static_cast<T *>(a.Y) + (long)b * a.sy + (long)j0 * L;
-  int n = 0, par = 0;
-  for (long tile = blockIdx.x; tile < a.ntile; tile += gridDim.x, par ^= 1) {
+  const float2 *const Zb = a.Z ? a.Z + (long)b * a.sz + (long)j0 * L : nullptr;
+  // Z of the epilogue's outputs, loaded before the digits of the next tile are formed
+  constexpr int NZ = F64 ? 1 : 8;
+  float2 z[NZ];
+  auto load_z = [&](long tile) {
+    if constexpr (!F64) {
+      const long l = tile * 128 + quarter * 32 + lane;
+#pragma unroll
+      for (int u = 0; u < NZ; ++u) {
+        const int j = 2 * slot + 8 * (u >> 1) + (u & 1);
+        z[u] = Zb && j < nbc && l < L ? Zb[(long)j * L + l] : make_float2(0.f, 0.f);
+      }
+    }
+  };
+  auto convert = [&](int s, int n, long tile, int ex) {
+    const int buf = n & 1;
+    if (n >= 2) bar_wait(bars + 8u * buf, ((n >> 1) & 1) ^ 1, abort);
+    unsigned char *o = sm + r * 128 + (((buf * 4 + g) ^ (r & 7)) << 4);
+    if constexpr (F64) {
+      unsigned long long m[8];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int i = min(s * SU_COLS + 4 * g + c, a.p - 1);  // (columns past p are zero)
+        sl_split<ND>(v[4 * s + c], ex - sCA[i], m[2 * c], m[2 * c + 1]);
+      }
+      load(s, tile + gridDim.x);
+#pragma unroll
+      for (int d = 0; d < ND; ++d) {
+        uint4 x;
+        x.x = sl_digits<ND>(m[0], m[1], ND - 1 - d);
+        x.y = sl_digits<ND>(m[2], m[3], ND - 1 - d);
+        x.z = sl_digits<ND>(m[4], m[5], ND - 1 - d);
+        x.w = sl_digits<ND>(m[6], m[7], ND - 1 - d);
+        *reinterpret_cast<uint4 *>(o + d * 16384) = x;
+      }
+    } else if (s * SU_COLS + 4 * g < a.p) {
+      // (with at most two stages a quarter without columns keeps the zeros of the start)
+      unsigned x[4][ND];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int i = min(s * SU_COLS + 4 * g + c, a.p - 1);
+        const float f = sl7_scale(ex - sCA[i]);
+        const float4 e = v[4 * s + c];
+        unsigned tr[ND], ti[ND];
+        sl7_digits(e.x, e.y, f, tr);
+        sl7_digits(e.z, e.w, f, ti);
+#pragma unroll
+        for (int d = 0; d < ND; ++d) x[c][d] = sl7_pack(tr[d], ti[d]);
+      }
+      load(s, tile + gridDim.x);
+#pragma unroll
+      for (int d = 0; d < ND; ++d)
+        *reinterpret_cast<uint4 *>(o + d * 16384) = make_uint4(x[0][d], x[1][d], x[2][d], x[3][d]);
+    }
+    fence_proxy_async();
+  };
+  // the MMAs of stages s0 .. s1 - 1 (converted by all threads), the first of them the n-th
+  auto issue = [&](int s0, int s1, int n) {
+    tc_fence_before();
+    if (warp == 0) {
+      named_sync(1 + (n & 1), SU_THREADS);
+      if (elect_one()) {
+        tc_fence_after();
+        for (int s = s0; s < s1; ++s) {
+          const int buf = (n + s - s0) & 1, nks = a.p - s * SU_COLS > SU_COLS / 2 ? 2 : 1;  // K steps of 8 columns
+          for (int ks = 0; ks < nks; ++ks)
+            sl_mma_step<ND, NL>(tmem, base, base + off_b + (s >> 1) * atom, (uint32_t)(buf * 64 + ks * 32),
+                                (uint32_t)((s & 1) * 64 + ks * 32), a.nbp, s == 0 && ks == 0);
+          mma_commit(bars + 8u * buf);
+        }
+      }
+      __syncwarp();
+    } else {
+      named_arrive(1 + (n & 1), SU_THREADS);
+    }
+  };
+  // the tile whose n-th stage was its last
+  auto epilogue = [&](long tile, int n, int par) {
+    bar_wait(bars + 8u * (n & 1), (n >> 1) & 1, abort);
+    tc_fence_after();
+    // epilogue: lane = row, four accumulator columns (two columns of Y) at a time
+    const int row = quarter * 32 + lane;
+    const long l = tile * 128 + row;
+    int E = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) E = max(E, sE[par * 512 + k * 128 + row]);
+#pragma unroll
+    for (int it = 0; it < 4; ++it) {
+      const int c0 = 4 * slot + 16 * it;
+      if (c0 >= 2 * nbc) break;
+      __syncwarp();
+      uint32_t w[NL][4];
+#pragma unroll
+      for (int lv = 0; lv < NL; ++lv) tmem_ld4(tdrain + (uint32_t)(lv * a.nbp + c0), w[lv]);
+#pragma unroll
+      for (int lv = 0; lv < NL; ++lv) tmem_wait4(w[lv]);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int j = (c0 >> 1) + h;
+        if (j >= nbc || l >= L) continue;
+        T out;
+        if (bad || E >= SU_BAD) {
+          // an infinity or a NaN in the row or in C: plain FP64
+          double re = 0.0, im = 0.0;
+          for (int i = 0; i < a.p; ++i) {
+            const double2 x = ld_c128(Sb + (long)i * L + l), c = Cb[(long)i * a.q + j];
+            re = fma(x.x, c.x, fma(-x.y, c.y, re));
+            im = fma(x.x, c.y, fma(x.y, c.x, im));
+          }
+          if constexpr (F64) {
+            out = make_double2(re, im);
+          } else {
+            if (Zb) {
+              re += (double)Zb[(long)j * L + l].x;
+              im += (double)Zb[(long)j * L + l].y;
+            }
+            const cdf d = cdf_from(make_double2(re, im));
+            out = make_float4(d.re.hi, d.re.lo, d.im.hi, d.im.lo);
+          }
+        } else if constexpr (F64) {
+          const int sc = sl_weight<F>(E, sCB[j]);
+          long long H[2];
+          unsigned lo[2];
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            long long hi = 0, s = 0;
+#pragma unroll
+            for (int lv = 0; lv < NL; ++lv) sl_level_add<F>(hi, s, lv, __float2int_rn(__uint_as_float(w[lv][2 * h + u])));
+            sl_join<F>(hi, s, H[u], lo[u]);
+          }
+          out = make_double2(sl_to_double(H[0], lo[0], sc), sl_to_double(H[1], lo[1], sc));
+        } else {
+          const int sc = sl_weight<F>(E, sCB[j]) + F::RB * (NL - 1);
+          float lr[NL], li[NL];
+#pragma unroll
+          for (int lv = 0; lv < NL; ++lv) {
+            lr[lv] = __uint_as_float(w[lv][2 * h]);
+            li[lv] = __uint_as_float(w[lv][2 * h + 1]);
+          }
+          const float2 zz = z[2 * it + h];
+          const df re = sl7_value(lr, sc, zz.x), im = sl7_value(li, sc, zz.y);
+          out = make_float4(re.hi, re.lo, im.hi, im.lo);
+        }
+        Yb[(long)j * L + l] = out;
+      }
+    }
+  };
+  // A tile's first two stages are converted before the epilogue of the tile before, whose MMAs run meanwhile
+  constexpr int AHEAD = NS < 2 ? NS : 2;
+  int n = 0, par = 0, ppar = 0;  // stages converted; exponent buffers of this tile and the one before
+  long prev = -1;
+  for (long tile = blockIdx.x; tile < a.ntile; tile += gridDim.x) {
+    if (prev >= 0) load_z(prev);
     // exponent of the row
     int ex = 0;
 #pragma unroll
@@ -179,96 +361,23 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
 #pragma unroll
     for (int k = 0; k < 4; ++k) ex = max(ex, sE[par * 512 + k * 128 + r]);
 #pragma unroll
-    for (int s = 0; s < NS; ++s) {
-      const int buf = n & 1;
-      if (n >= 2) bar_wait(bars + 8u * buf, ((n >> 1) & 1) ^ 1, abort);
-      unsigned long long m[8];
+    for (int s = 0; s < AHEAD; ++s) convert(s, n + s, tile, ex);
+    if (prev >= 0) epilogue(prev, n - 1, ppar);
+    issue(0, AHEAD, n);
+    n += AHEAD;
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int i = min(s * SU_COLS + 4 * g + c, a.p - 1);  // (columns past p are zero)
-        sl_split<ND>(v[4 * s + c], ex - sCA[i], m[2 * c], m[2 * c + 1]);
-      }
-      load(s, tile + gridDim.x);
-      unsigned char *o = sm + r * 128 + (((buf * 4 + g) ^ (r & 7)) << 4);
-#pragma unroll
-      for (int d = 0; d < ND; ++d) {
-        uint4 x;
-        x.x = sl_digits<ND>(m[0], m[1], ND - 1 - d);
-        x.y = sl_digits<ND>(m[2], m[3], ND - 1 - d);
-        x.z = sl_digits<ND>(m[4], m[5], ND - 1 - d);
-        x.w = sl_digits<ND>(m[6], m[7], ND - 1 - d);
-        *reinterpret_cast<uint4 *>(o + d * 16384) = x;
-      }
-      fence_proxy_async();
-      tc_fence_before();
-      if (warp == 0) {
-        named_sync(1 + buf, SU_THREADS);
-        if (lane == 0) {
-          tc_fence_after();
-          const int nks = a.p - s * SU_COLS > SU_COLS / 2 ? 2 : 1;  // K steps of 8 columns
-          for (int ks = 0; ks < nks; ++ks)
-            sl_mma_step<ND, ND>(tmem, base, base + off_b + (s >> 1) * atom, (uint32_t)(buf * 64 + ks * 32),
-                            (uint32_t)((s & 1) * 64 + ks * 32), a.nbp, s == 0 && ks == 0);
-          mma_commit(bars + 8u * buf);
-        }
-        __syncwarp();
-      } else {
-        named_arrive(1 + buf, SU_THREADS);
-      }
+    for (int s = AHEAD; s < NS; ++s) {
+      convert(s, n, tile, ex);
+      issue(s, s + 1, n);
       ++n;
     }
-    bar_wait(bars + 8u * ((n - 1) & 1), ((n - 1) >> 1) & 1, abort);
-    tc_fence_after();
-    // epilogue: lane = row, four accumulator columns (two columns of Y) at a time
-    const int row = quarter * 32 + lane;
-    const long l = tile * 128 + row;
-    int E = 0;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) E = max(E, sE[par * 512 + k * 128 + row]);
-    for (int c0 = 4 * slot; c0 < 2 * nbc; c0 += 16) {
-      __syncwarp();
-      uint32_t w[ND][4];
-#pragma unroll
-      for (int lv = 0; lv < ND; ++lv) tmem_ld4(tdrain + (uint32_t)(lv * a.nbp + c0), w[lv]);
-#pragma unroll
-      for (int lv = 0; lv < ND; ++lv) tmem_wait4(w[lv]);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int j = (c0 >> 1) + h;
-        if (j >= nbc || l >= L) continue;
-        T out;
-        if (bad || E >= SU_BAD) {
-          // an infinity or a NaN in the row or in C: plain FP64
-          double re = 0.0, im = 0.0;
-          for (int i = 0; i < a.p; ++i) {
-            const double2 x = ld_c128(Sb + (long)i * L + l), c = Cb[(long)i * a.q + j];
-            re = fma(x.x, c.x, fma(-x.y, c.y, re));
-            im = fma(x.x, c.y, fma(x.y, c.x, im));
-          }
-          out = make_double2(re, im);
-        } else {
-          const int sc = E + sCB[j] - 2046 - 2 * (sl_bits<ND>() - 1) + 8 * (ND - 1);
-          long long H[2];
-          unsigned lo[2];
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            long long hi = 0, s = 0;
-#pragma unroll
-            for (int lv = 0; lv < ND; ++lv) {
-              const int x = __float2int_rn(__uint_as_float(w[lv][2 * h + u]));
-              if (lv < ND - 4)
-                hi += (long long)x * (1 << (8 * (ND - 5 - lv)));
-              else
-                s += (long long)x * (1 << (8 * (ND - 1 - lv)));
-            }
-            H[u] = hi + (s >> 32);
-            lo[u] = (unsigned)s;
-          }
-          out = make_double2(sl_to_double(H[0], lo[0], sc), sl_to_double(H[1], lo[1], sc));
-        }
-        Yb[(long)j * L + l] = out;
-      }
-    }
+    prev = tile;
+    ppar = par;
+    par = par == 2 ? 0 : par + 1;
+  }
+  if (prev >= 0) {
+    load_z(prev);
+    epilogue(prev, n - 1, ppar);
   }
   __syncwarp();
   if (tid == 0 && *abort && n > 0) bar_wait(bars + 8u * ((n - 1) & 1), ((n - 1) >> 1) & 1, abort, false);
@@ -281,18 +390,20 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
   if (tid == 0 && *abort) atomicExch(&g_update_sl_error, 1);
 }
 
-template <int NS>
+template <typename T, int NS>
 int launch_su(SlUpdateArgs a, int nb, cudaStream_t st) {
   // columns of Y per block: all levels of 2 nbc columns in TMEM, the digits of C and of one tile in shared memory
-  constexpr int ND = SU_ND, most_cols = NS > 2 ? 20 : 32;
+  using F = SlFormShort<T>;
+  constexpr int ND = F::ND, most_cols = NS > 2 ? 20 : 32;
+  constexpr int NPAD = F::NL % 2 == 0 ? 8 : 16;  // (see sl_mma_step)
   const int nqb = (a.q + most_cols - 1) / most_cols;
   a.nbc = (a.q + nqb - 1) / nqb;
-  a.nbp = (2 * a.nbc + 7) / 8 * 8;
+  a.nbp = (2 * a.nbc + NPAD - 1) / NPAD * NPAD;
   a.ntile = (int)((a.L + 127) / 128);
   a.tmem_cols = 32;
   while (a.tmem_cols < (uint32_t)((ND + ((a.nbp >> 3) & 1)) * a.nbp)) a.tmem_cols *= 2;
   auto smem_of = [](int nbp) {
-    return (size_t)1024 + ND * 16384 + (size_t)((NS + 1) / 2) * ND * nbp * 128 + (1024 + 128) * 4 + 64;
+    return (size_t)1024 + ND * 16384 + (size_t)((NS + 1) / 2) * ND * nbp * 128 + (1536 + 128) * 4 + 64;
   };
   // CTAs per k-point and column block: the least tiles (plus about one for the setup) in the longest sequence per SM
   const long per = (long)nb * nqb, nsm = sm_count();
@@ -309,20 +420,20 @@ int launch_su(SlUpdateArgs a, int nb, cudaStream_t st) {
   int dev = 0;
   PC_CK(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64 || !configured[dev]) {
-    PC_CK(cudaFuncSetAttribute(update_sl_kernel<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    PC_CK(cudaFuncSetAttribute(update_sl_kernel<T, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)smem_of(2 * most_cols)));
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
   // a CTA's 512 threads of 128 registers take the SM: no second CTA waits for its TMEM columns there
-  update_sl_kernel<NS><<<dim3(gx, nqb, nb), SU_THREADS, smem_of(a.nbp), st>>>(a);
+  update_sl_kernel<T, NS><<<dim3(gx, nqb, nb), SU_THREADS, smem_of(a.nbp), st>>>(a);
   PC_CK_LAUNCH();
   return PC_OK;
 }
 
 }  // namespace
 
-int launch_update_sl(int nb, long L, int p, int q, const void *S, long ss, const void *C, long sc, void *Y,
-                     long sy, cudaStream_t st, const int *act) {
+int launch_update_sl(int nb, long L, int p, int q, int dtype, const void *S, long ss, const void *C, long sc, void *Y,
+                     long sy, const void *Z, long sz, cudaStream_t st, const int *act) {
   SlUpdateArgs a{};
   a.S = S;
   a.ss = ss;
@@ -330,15 +441,18 @@ int launch_update_sl(int nb, long L, int p, int q, const void *S, long ss, const
   a.sc = sc;
   a.Y = Y;
   a.sy = sy;
+  a.Z = static_cast<const float2 *>(Z);
+  a.sz = sz;
   a.L = L;
   a.p = p;
   a.q = q;
   a.act = act;
+  if (dtype == PC_DFS) return p <= SU_COLS ? launch_su<float4, 1>(a, nb, st) : launch_su<float4, 2>(a, nb, st);
   switch ((p + SU_COLS - 1) / SU_COLS) {
-    case 1: return launch_su<1>(a, nb, st);
-    case 2: return launch_su<2>(a, nb, st);
-    case 3: return launch_su<3>(a, nb, st);
-    default: return launch_su<4>(a, nb, st);
+    case 1: return launch_su<double2, 1>(a, nb, st);
+    case 2: return launch_su<double2, 2>(a, nb, st);
+    case 3: return launch_su<double2, 3>(a, nb, st);
+    default: return launch_su<double2, 4>(a, nb, st);
   }
 }
 

@@ -25,7 +25,7 @@ def test_same_bits_for_every_cluster_size(pcmod, n, m, rank):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     out = []
     for nb in (1, sms // 4 + 1, sms // 2 + 1):  # 4, 2 and 1 blocks per pencil
-        Gt, Ht = (torch.from_numpy(np.ascontiguousarray(np.broadcast_to(x, (nb, n, n)))).cuda() for x in (G, H))
+        Gt, Ht = (torch.from_numpy(np.tile(x, (nb, 1, 1))).cuda() for x in (G, H))
         theta, coef, rk = pcmod.rayleigh_ritz(Gt, Ht, m, 1e-12)
         assert torch.equal(theta, theta[:1].expand_as(theta)) and torch.equal(coef, coef[:1].expand_as(coef))
         out.append((theta[0], coef[0], int(rk[0])))

@@ -144,3 +144,15 @@ def test_block_update_nonfinite_and_zero(pcmod):
     ok = [j for j in range(12) if j != 5]
     ref = np.einsum("pl,pq->ql", S[0], C[0][:, ok])
     assert np.max(np.abs(Y[0][ok] - ref)) <= 1e-12 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("nbands,guard", [(1, 0), (3, 1), (10, 6), (11, 6), (12, 9)])
+def test_mixed_solve_block_widths(pcmod, nbands, guard):
+    """The mixed solve's block X (double-float pairs: Gram and update) at 1, 4, 16, 17 and 21 columns. Residuals of
+    1e-6 leave eigenvalue errors of about 1e-12 over the relative gap (at least 1e-4 here)."""
+    N, k = 8, [[0.9, 0.4, -0.3], [1.7, -0.2, 0.8], [0.3, 2.1, 1.0]]
+    eps = pcmod.eps_spheres(N, [[0.5, 0.5, 0.5, 0.3, 13.0]], 1.0)
+    a = pcmod.Solver(N, eps, precision=1, guard=guard).solve(k, nbands, 1e-6)
+    b = pcmod.Solver(N, eps, precision=0, guard=guard).solve(k, nbands, 1e-8)
+    assert a["status"] == 0 and b["status"] == 0
+    assert np.max(np.abs(a["evals"] - b["evals"]) / b["evals"]) <= 1e-8
