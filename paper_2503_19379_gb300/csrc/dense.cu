@@ -172,6 +172,69 @@ __global__ void __launch_bounds__(RED_X *RED_Y) gram_reduce_kernel(const double2
   if (on && threadIdx.y == 0) G[(long)b * sg + i] = s;
 }
 
+// Narrow complex64 products (p, q <= 16): 8 x 8 tiles of outputs, a thread holding 8 x 4 of them for its rows (threads
+// 0-127 the first four columns of B, 128-255 the others). The sums of a thread (about 20 rows) are FP32, added over the
+// lanes in FP32 and over the warps and chunks in FP64. Bound: HBM. The tensor-core kernel's hand-offs per K tile cost
+// the same for narrow panels as for wide ones: 16 samples x 8 columns at N = 32, 317 us there.
+// grid (nchunk, tiles of p x tiles of q, nb)
+constexpr int GN_T = 8;
+
+__global__ void __launch_bounds__(256, 2) gram_narrow_kernel(const float2 *__restrict__ A, long sa,
+                                                             const float2 *__restrict__ B, long sb, long L, int p, int q,
+                                                             long chunk, double2 *__restrict__ part,
+                                                             const int *__restrict__ act) {
+  __shared__ float red[8][64];
+  const int bi = blockIdx.z, b = act ? act[bi] : bi;
+  const int tq = (q + GN_T - 1) / GN_T, i0 = (int)blockIdx.y / tq * GN_T, jt = (int)blockIdx.y % tq * GN_T;
+  const int half = threadIdx.x >> 7, j0 = jt + 4 * half, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const float2 *Ab = A + (long)b * sa + (long)i0 * L, *Bb = B + (long)b * sb;
+  const int np = min(GN_T, p - i0), nq = min(4, q - j0);  // (nq <= 0: nothing of this half is wanted)
+  float acc[64];  // (i, j, part): 8 i + 2 j + part
+#pragma unroll
+  for (int u = 0; u < 64; ++u) acc[u] = 0.f;
+  const long beg = (long)blockIdx.x * chunk, end = min(L, beg + chunk);
+  for (long l = beg + (threadIdx.x & 127); l < end; l += 128) {
+    float2 a[GN_T], v[4];
+#pragma unroll
+    for (int i = 0; i < GN_T; ++i) a[i] = i < np ? Ab[(long)i * L + l] : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = j < nq ? Bb[(long)(j0 + j) * L + l] : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < GN_T; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        float &x = acc[8 * i + 2 * j], &y = acc[8 * i + 2 * j + 1];
+        x = fmaf(a[i].x, v[j].x, fmaf(a[i].y, v[j].y, x));
+        y = fmaf(a[i].x, v[j].y, fmaf(-a[i].y, v[j].x, y));
+      }
+  }
+  // lane l of the warp ends with the warp's sums 2 l and 2 l + 1: each step halves the entries a lane holds
+#pragma unroll
+  for (int w = 16, cnt = 32; w > 0; w >>= 1, cnt >>= 1) {
+    const bool up = lane & w;
+#pragma unroll
+    for (int u = 0; u < cnt; ++u) {
+      const float give = up ? acc[u] : acc[u + cnt], keep = up ? acc[u + cnt] : acc[u];
+      acc[u] = keep + __shfl_xor_sync(0xffffffffu, give, w);
+    }
+  }
+  red[warp][2 * lane] = acc[0];
+  red[warp][2 * lane + 1] = acc[1];
+  __syncthreads();
+  if ((threadIdx.x & 127) < 32) {
+    const int e = threadIdx.x & 31, i = e >> 2, j = e & 3;  // complex output (i, j) of this half
+    if (i < np && j < nq) {
+      double x = 0.0, y = 0.0;
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        x += (double)red[4 * half + w][2 * e];
+        y += (double)red[4 * half + w][2 * e + 1];
+      }
+      part[((long)bi * gridDim.x + blockIdx.x) * p * q + (i0 + i) * q + j0 + j] = make_double2(x, y);
+    }
+  }
+}
+
 static int gram_chunks(int nb, long L) {
   long want = std::max<long>(1, (4L * sm_count() + nb - 1) / std::max(nb, 1));
   long maxc = std::max<long>(1, L / 512);
@@ -191,7 +254,7 @@ size_t gram_scratch_bytes(int nb, long L, int p, int q) {
 int launch_gram(int nb, long L, int p, int q, int dtype, const void *A, long sa, const void *B, long sb, void *G,
                 void *scratch, size_t scratch_bytes, cudaStream_t st, const int *act, int nb_alloc, long sg) {
   if (nb == 0 || p == 0 || q == 0) return PC_OK;
-  if (dtype == PC_C64) {
+  if (dtype == PC_C64 && (p > 16 || q > 16)) {
     const int rc = launch_gram_tc(nb, L, p, q, A, sa, B, sb, G, scratch, scratch_bytes, st, act, nb_alloc, sg);
     if (rc != PC_EUNSUPPORTED) return rc;
   }
@@ -214,7 +277,10 @@ int launch_gram(int nb, long L, int p, int q, int dtype, const void *A, long sa,
   double2 *part = static_cast<double2 *>(scratch);
   const int R = std::max(p, q) <= 32 ? 2 : 4;
   const dim3 blk((q + R - 1) / R, (p + R - 1) / R);
-  if (R == 2)
+  if (p <= 16 && q <= 16)
+    gram_narrow_kernel<<<dim3(nchunk, ((p + GN_T - 1) / GN_T) * ((q + GN_T - 1) / GN_T), nb), 256, 0, st>>>(
+        static_cast<const float2 *>(A), sa, static_cast<const float2 *>(B), sb, L, p, q, chunk, part, act);
+  else if (R == 2)
     gram_tile_partial_kernel<float, 2><<<dim3(nchunk, 1, nb), blk, 0, st>>>(
         static_cast<const float2 *>(A), sa, static_cast<const float2 *>(B), sb, L, p, q, chunk, part, act);
   else
@@ -469,9 +535,85 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
     }
 }
 
+// complex64, two adjacent rows per thread (even L, 16-byte aligned panels): a coefficient read from shared memory feeds
+// two rows and comes in pairs, 10 shared-memory loads for 160 FMA at QB = 20 where one row a thread has 20 for 80. The
+// sums are those of block_update_kernel, in the same order. Bound: FP32 pipe. 4 k-points, 57 -> 19 columns at N = 64:
+// 0.94 ms with one row a thread, 0.76 ms here. A second product S2 C2 of the same widths can follow (S2 null: none).
+template <int QB>
+__global__ void __launch_bounds__(256, 2)
+    block_update2_kernel(const float2 *__restrict__ S, long ss, const double2 *__restrict__ Cm, long sc,
+                         float2 *__restrict__ Y, long sy, const float2 *__restrict__ Z, long sz, long L, int p, int q,
+                         const int *__restrict__ act, const float2 *__restrict__ S2, const double2 *__restrict__ Cm2) {
+  static_assert(QB % 2 == 0, "coefficients are read in pairs");
+  __shared__ float4 Cs[UPD_PMAX][QB / 2];
+  const int b = act ? act[blockIdx.z] : (int)blockIdx.z;
+  const int j0 = blockIdx.y * QB;
+  const long l = 2 * ((long)blockIdx.x * blockDim.x + threadIdx.x);
+  float2 a0[QB], a1[QB];
+#pragma unroll
+  for (int c = 0; c < QB; ++c) a0[c] = a1[c] = make_float2(0.f, 0.f);
+  for (int pass = 0; pass < (S2 ? 2 : 1); ++pass) {
+    const double2 *Cb = (pass ? Cm2 : Cm) + (long)b * sc;
+    if (pass) __syncthreads();
+    for (int i = threadIdx.x; i < p * QB; i += blockDim.x) {
+      const int r = i / QB, c = i - r * QB;
+      const double2 v = (j0 + c < q) ? Cb[r * q + j0 + c] : cmake<double2>(0.0, 0.0);
+      reinterpret_cast<float2 *>(Cs[r])[c] = make_float2((float)v.x, (float)v.y);
+    }
+    __syncthreads();
+    if (l >= L) continue;
+    const float2 *Sb = (pass ? S2 : S) + (long)b * ss + l;
+    float4 nx = p > 0 ? *reinterpret_cast<const float4 *>(Sb) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = 0; i < p; ++i) {
+      const float4 s = nx;
+      if (i + 1 < p) nx = *reinterpret_cast<const float4 *>(Sb + (long)(i + 1) * L);
+#pragma unroll
+      for (int c = 0; c < QB; c += 2) {
+        const float4 w = Cs[i][c / 2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float cx = h ? w.z : w.x, cy = h ? w.w : w.y;
+          a0[c + h].x = fmaf(s.x, cx, fmaf(-s.y, cy, a0[c + h].x));
+          a0[c + h].y = fmaf(s.x, cy, fmaf(s.y, cx, a0[c + h].y));
+          a1[c + h].x = fmaf(s.z, cx, fmaf(-s.w, cy, a1[c + h].x));
+          a1[c + h].y = fmaf(s.z, cy, fmaf(s.w, cx, a1[c + h].y));
+        }
+      }
+    }
+  }
+  if (l >= L) return;
+  float2 *Yb = Y + (long)b * sy + l;
+  const float2 *Zb = Z ? Z + (long)b * sz + l : nullptr;
+#pragma unroll
+  for (int c = 0; c < QB; ++c)
+    if (j0 + c < q) {
+      float4 v = make_float4(a0[c].x, a0[c].y, a1[c].x, a1[c].y);
+      if (Zb) {
+        const float4 z = *reinterpret_cast<const float4 *>(Zb + (long)(j0 + c) * L);
+        v.x += z.x;
+        v.y += z.y;
+        v.z += z.z;
+        v.w += z.w;
+      }
+      *reinterpret_cast<float4 *>(Yb + (long)(j0 + c) * L) = v;
+    }
+}
+
 template <typename T, int QB>
 static void block_update_t(int nb, long L, int p, int q, const void *S, long ss, const void *C, long sc, void *Y,
                            long sy, cudaStream_t st, const int *act, const void *Z, long sz) {
+  if constexpr (std::is_same<T, float>::value) {
+    // two rows a thread once that leaves two blocks per SM (8 k-points x 1536 rows, 39 -> 12: 18 us with one row, 23 with
+    // two)
+    const uintptr_t at = (uintptr_t)S | (uintptr_t)Y | (uintptr_t)Z;
+    const dim3 g((unsigned)((L / 2 + 255) / 256), (unsigned)((q + QB - 1) / QB), nb);
+    if (((L | ss | sy | sz) & 1) == 0 && (at & 15) == 0 && (long)g.x * g.y * g.z >= 2L * sm_count()) {
+      block_update2_kernel<QB><<<g, 256, 0, st>>>(static_cast<const float2 *>(S), ss, static_cast<const double2 *>(C), sc,
+                                                  static_cast<float2 *>(Y), sy, static_cast<const float2 *>(Z), sz, L, p,
+                                                  q, act, nullptr, nullptr);
+      return;
+    }
+  }
   const dim3 grid((unsigned)((L + 255) / 256), (unsigned)((q + QB - 1) / QB), nb);
   block_update_kernel<T, QB><<<grid, 256, 0, st>>>(static_cast<const cplx<T> *>(S), ss,
                                                    static_cast<const double2 *>(C), sc, static_cast<cplx<T> *>(Y), sy,
@@ -515,6 +657,31 @@ int launch_block_update(int nb, long L, int p, int q, int dtype, const void *S, 
       default: block_update_t<float, 24>(nb, L, p, q, S, ss, C, sc, Y, sy, st, act, Z, sz); break;
     }
   }
+  PC_CK_LAUNCH();
+  return PC_OK;
+}
+
+// Y = S C + S2 C2, complex64, p <= 64 columns each (q <= 16: one pass over S and S2; the general shapes in two)
+int launch_block_update_sum(int nb, long L, int p, int q, const void *S, const void *C, const void *S2, const void *C2,
+                            long ss, long sc, void *Y, long sy, cudaStream_t st) {
+  if (nb == 0 || q == 0) return PC_OK;
+  const uintptr_t at = (uintptr_t)S | (uintptr_t)S2 | (uintptr_t)Y;
+  if (p > UPD_PMAX || q > 16 || ((L | ss | sy) & 1) || (at & 15)) {
+    const int rc = launch_block_update(nb, L, p, q, PC_C64, S, ss, C, sc, Y, sy, st, nullptr);
+    return rc ? rc : launch_block_update(nb, L, p, q, PC_C64, S2, ss, C2, sc, Y, sy, st, nullptr, Y, sy);
+  }
+  const dim3 g((unsigned)((L / 2 + 255) / 256), 1, nb);
+  auto run = [&](auto kernel) {
+    kernel<<<g, 256, 0, st>>>(static_cast<const float2 *>(S), ss, static_cast<const double2 *>(C), sc,
+                              static_cast<float2 *>(Y), sy, nullptr, 0, L, p, q, nullptr,
+                              static_cast<const float2 *>(S2), static_cast<const double2 *>(C2));
+  };
+  if (q <= 8)
+    run(block_update2_kernel<8>);
+  else if (q <= 12)
+    run(block_update2_kernel<12>);
+  else
+    run(block_update2_kernel<16>);
   PC_CK_LAUNCH();
   return PC_OK;
 }

@@ -27,6 +27,7 @@ namespace pc {
 namespace ws {
 
 constexpr int C1 = PC_WS_C1, C2 = PC_WS_C2, NBMAX = 16, TPB = 256;
+constexpr int MAXSPLIT = 64;  // ranges of a gradient sum (head_grad_kernel, conv_wgrad_kernel)
 
 struct Offs {
   long W1, b1, W2, b2, Fa, fa, Fc, fc, Wh, bh, Wv, bv, total;
@@ -53,7 +54,7 @@ Offs offsets(int nb) {
 
 // device workspace of one forward + backward pass over S samples (offsets in bytes, 256-aligned)
 struct Work {
-  size_t phi, a1, a2, z, pool, dy, coarse, G, B, Cx, Cv, dX, dcoarse, dz, da2, da1, dsa, dsc, loss, gram, total;
+  size_t phi, a1, a2, z, pool, dy, coarse, G, B, Cx, Cv, dX, dcoarse, dz, da2, da1, dsa, dsc, loss, gram, part, total;
 };
 
 Work work_layout(int N, int nb, int S) {
@@ -86,6 +87,7 @@ Work work_layout(int N, int nb, int S) {
   w.dsc = take(sizeof(float) * (size_t)S * C2);
   w.loss = take(sizeof(double) * (size_t)S);
   w.gram = take(std::max<size_t>(16, gram_scratch_bytes(S, L, nb, nb)));
+  w.part = take(sizeof(float) * MAXSPLIT * std::max<size_t>(C1 * C2 * 28, 6 * NBMAX * (C2 + 1)));
   w.total = p;
   return w;
 }
@@ -183,21 +185,16 @@ __global__ void __launch_bounds__(TPB) film_head_kernel(const float *__restrict_
 __global__ void __launch_bounds__(TPB) pool_value_kernel(const float *__restrict__ z, const float *__restrict__ P,
                                                          const Offs of, const float *__restrict__ phi, int nb, long m3,
                                                          float *__restrict__ pool, float *__restrict__ y) {
-  __shared__ float red[TPB];
   __shared__ float sp[C2];
-  const int s = blockIdx.x;
-  for (int c = 0; c < C2; ++c) {
+  const int s = blockIdx.x, lane = threadIdx.x & 31;
+  for (int c = threadIdx.x >> 5; c < C2; c += TPB / 32) {  // one warp per channel
     float acc = 0.0f;
-    for (long q = threadIdx.x; q < m3; q += blockDim.x) acc += z[((long)s * C2 + c) * m3 + q];
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-      if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) sp[c] = red[0] / (float)m3;
-    __syncthreads();
+    for (long q = lane; q < m3; q += 32) acc += z[((long)s * C2 + c) * m3 + q];
+#pragma unroll
+    for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) sp[c] = acc / (float)m3;
   }
+  __syncthreads();
   if ((int)threadIdx.x < C2) pool[(long)s * C2 + threadIdx.x] = sp[threadIdx.x];
   if ((int)threadIdx.x < nb) {
     const int b = threadIdx.x;
@@ -209,36 +206,40 @@ __global__ void __launch_bounds__(TPB) pool_value_kernel(const float *__restrict
 }
 
 // X[s][b][comp][i] = periodic linear interpolation of the coarse block: along each axis fine point i = 4 j + r takes
-// (1 - r/4) c_j + (r/4) c_{j+1}. grid (ceil(N^3 / 256), 3 nb, S)
+// (1 - r/4) c_j + (r/4) c_{j+1}. A thread forms the four fine points of one coarse x: eight coarse values for four
+// points, two 16-byte stores. Bound: HBM writes (62 us with one point a thread at 16 samples x 8 bands, N = 32).
+// grid (ceil(N^3 / 1024), 3 nb, S)
 __global__ void __launch_bounds__(TPB) upsample_kernel(const float2 *__restrict__ coarse, float2 *__restrict__ X,
                                                        int logN) {
   const int N = 1 << logN, M = N >> 2, logM = logN - 2;
   const long n = 1L << (3 * logN), m3 = 1L << (3 * logM);
-  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long i = 4 * ((long)blockIdx.x * blockDim.x + threadIdx.x);
   if (i >= n) return;
   const long col = (long)blockIdx.z * gridDim.y + blockIdx.y;  // (s, band, component)
   const float2 *c = coarse + col * m3;
-  const int ix = (int)(i & (N - 1)), iy = (int)((i >> logN) & (N - 1)), iz = (int)(i >> (2 * logN));
-  int j0[3], j1[3];
-  float w1[3];
-  const int id[3] = {ix, iy, iz};
+  const int jx0 = (int)(i & (N - 1)) >> 2, iy = (int)((i >> logN) & (N - 1)), iz = (int)(i >> (2 * logN));
+  const int jx1 = (jx0 + 1) & (M - 1), jy0 = iy >> 2, jy1 = (jy0 + 1) & (M - 1), jz0 = iz >> 2, jz1 = (jz0 + 1) & (M - 1);
+  const float wy = 0.25f * (float)(iy & 3), wz = 0.25f * (float)(iz & 3);
+  float2 v[8];
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    j0[a] = id[a] >> 2;
-    j1[a] = (j0[a] + 1) & (M - 1);
-    w1[a] = 0.25f * (float)(id[a] & 3);
-  }
-  float2 acc = make_float2(0.0f, 0.0f);
+  for (int t = 0; t < 8; ++t)
+    v[t] = c[((long)((t & 4) ? jz1 : jz0) << (2 * logM)) + ((long)((t & 2) ? jy1 : jy0) << logM) + ((t & 1) ? jx1 : jx0)];
+  float2 out[4];
 #pragma unroll
-  for (int t = 0; t < 8; ++t) {
-    const int jx = (t & 1) ? j1[0] : j0[0], jy = (t & 2) ? j1[1] : j0[1], jz = (t & 4) ? j1[2] : j0[2];
-    const float w = ((t & 1) ? w1[0] : 1.0f - w1[0]) * ((t & 2) ? w1[1] : 1.0f - w1[1]) *
-                    ((t & 4) ? w1[2] : 1.0f - w1[2]);
-    const float2 v = c[((long)jz << (2 * logM)) + ((long)jy << logM) + jx];
-    acc.x = fmaf(w, v.x, acc.x);
-    acc.y = fmaf(w, v.y, acc.y);
+  for (int r = 0; r < 4; ++r) {
+    const float wx = 0.25f * (float)r;
+    float2 acc = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      const float w = ((t & 1) ? wx : 1.0f - wx) * ((t & 2) ? wy : 1.0f - wy) * ((t & 4) ? wz : 1.0f - wz);
+      acc.x = fmaf(w, v[t].x, acc.x);
+      acc.y = fmaf(w, v[t].y, acc.y);
+    }
+    out[r] = acc;
   }
-  X[col * n + i] = acc;
+  float4 *o = reinterpret_cast<float4 *>(X + col * n + i);
+  o[0] = make_float4(out[0].x, out[0].y, out[1].x, out[1].y);
+  o[1] = make_float4(out[2].x, out[2].y, out[3].x, out[3].y);
 }
 
 // ------------------------------------------------------------------------------------------------------ loss
@@ -358,12 +359,16 @@ __global__ void __launch_bounds__(TPB) upsample_bwd_kernel(const float2 *__restr
     for (int ty = -3; ty <= 3; ++ty) {
       const float wzy = wz * (1.0f - 0.25f * (float)abs(ty));
       const long yo = zo + ((long)((4 * jy + ty) & mask) << logN);
+      // x = 4 jx - 4 .. 4 jx + 3 as four 16-byte loads (4 jx - 4 itself is not used)
+      const float4 *lo = reinterpret_cast<const float4 *>(d + yo + ((4 * jx - 4) & mask));
+      const float4 *hi = reinterpret_cast<const float4 *>(d + yo + 4 * jx);
+      const float4 v0 = lo[0], v1 = lo[1], v2 = hi[0], v3 = hi[1];
+      const float2 v[7] = {{v0.z, v0.w}, {v1.x, v1.y}, {v1.z, v1.w}, {v2.x, v2.y}, {v2.z, v2.w}, {v3.x, v3.y}, {v3.z, v3.w}};
 #pragma unroll
       for (int tx = -3; tx <= 3; ++tx) {
         const float w = wzy * (1.0f - 0.25f * (float)abs(tx));
-        const float2 v = d[yo + ((4 * jx + tx) & mask)];
-        acc.x = fmaf(w, v.x, acc.x);
-        acc.y = fmaf(w, v.y, acc.y);
+        acc.x = fmaf(w, v[tx + 3].x, acc.x);
+        acc.y = fmaf(w, v[tx + 3].y, acc.y);
       }
     }
   }
@@ -417,30 +422,57 @@ template <int K> __device__ __forceinline__ void block_sum(float (*red)[TPB], co
   }
 }
 
-// dWh[o][c] = sum_{s,q} dh[s][o][q] z[s][c][q], dbh[o] = sum dh (dh: channel o = 2 bc + ri of the coarse gradient).
-// grid (6 nb), TPB threads
+// Sums over samples and points are cut into `split` ranges, one block each, whose partial sums reduce_part_kernel adds in
+// order: one block per output (48 and 24 blocks for the head and the first convolution at 8 bands) left most SMs idle.
+// out[e] for e < count: part[0][e] + part[1][e] + ...; entries e with e % row == row - 1 go to bias, the others to out.
+__global__ void __launch_bounds__(TPB) reduce_part_kernel(const float *__restrict__ part, int split, int count, int row,
+                                                          int per_bias, float *__restrict__ out, float *__restrict__ bias) {
+  const int e = blockIdx.x * TPB + threadIdx.x;
+  if (e >= count) return;
+  float s = 0.0f;
+  for (int k = 0; k < split; ++k) s += part[(long)k * count + e];
+  const int r = e / row, c = e - r * row;
+  if (c < row - 1)
+    out[(long)r * (row - 1) + c] = s;
+  else if (r % per_bias == 0)
+    bias[r / per_bias] = s;
+}
+
+// ranges for `blocks` outputs of `tot` terms: enough for four blocks per SM, at least 512 terms each
+int split_for(long blocks, long tot) {
+  const long want = (4L * sm_count() + blocks - 1) / blocks;
+  return (int)std::max<long>(1, std::min<long>({want, tot / 512, (long)MAXSPLIT}));
+}
+
+// dWh[o][c] = sum_{s,q} dh[s][o][q] z[s][c][q], dbh[o] = sum dh (dh: channel o = 2 bc + ri of the coarse gradient), as
+// partial sums part[range][o][C2 + 1]. grid (3 nb, split), TPB threads
 __global__ void __launch_bounds__(TPB) head_grad_kernel(const float2 *__restrict__ dc, const float *__restrict__ z,
-                                                        int nb, int S, long m3, float *__restrict__ gWh,
-                                                        float *__restrict__ gbh) {
+                                                        int nb, int S, long m3, float *__restrict__ part) {
   __shared__ float red[C2 + 1][TPB];
-  const int o = blockIdx.x, bc = o >> 1, ri = o & 1;
-  float acc[C2 + 1];
+  const int bc = blockIdx.x;
+  float acc[2][C2 + 1];
 #pragma unroll
-  for (int c = 0; c <= C2; ++c) acc[c] = 0.0f;
-  const long tot = (long)S * m3;
-  for (long t = threadIdx.x; t < tot; t += blockDim.x) {
+  for (int c = 0; c <= C2; ++c) acc[0][c] = acc[1][c] = 0.0f;
+  const long tot = (long)S * m3, len = (tot + gridDim.y - 1) / gridDim.y, t0 = blockIdx.y * len;
+  for (long t = t0 + threadIdx.x; t < min(tot, t0 + len); t += blockDim.x) {
     const int s = (int)(t / m3);
     const long q = t - (long)s * m3;
-    const float2 d2 = dc[((long)s * 3 * nb + bc) * m3 + q];
-    const float d = ri ? d2.y : d2.x;
+    const float2 d = dc[((long)s * 3 * nb + bc) * m3 + q];
 #pragma unroll
-    for (int c = 0; c < C2; ++c) acc[c] = fmaf(d, z[((long)s * C2 + c) * m3 + q], acc[c]);
-    acc[C2] += d;
+    for (int c = 0; c < C2; ++c) {
+      const float zc = z[((long)s * C2 + c) * m3 + q];
+      acc[0][c] = fmaf(d.x, zc, acc[0][c]);
+      acc[1][c] = fmaf(d.y, zc, acc[1][c]);
+    }
+    acc[0][C2] += d.x;
+    acc[1][C2] += d.y;
   }
-  block_sum<C2 + 1>(red, acc);
-  if (threadIdx.x == 0) {
-    for (int c = 0; c < C2; ++c) gWh[o * C2 + c] = red[c][0];
-    gbh[o] = red[C2][0];
+#pragma unroll
+  for (int ri = 0; ri < 2; ++ri) {
+    block_sum<C2 + 1>(red, acc[ri]);
+    if ((int)threadIdx.x <= C2)
+      part[((long)blockIdx.y * 6 * nb + 2 * bc + ri) * (C2 + 1) + threadIdx.x] = red[threadIdx.x][0];
+    __syncthreads();
   }
 }
 
@@ -495,12 +527,12 @@ __global__ void small_grads_kernel(const float *__restrict__ dsa, const float *_
   }
 }
 
-// dW[o][c][t] = sum_{s,q} dout[s][o][q] in[s][c][2q + d - 1], db[o] = sum dout (written by the c = 0 block).
-// grid (COUT, CIN), TPB threads
+// dW[o][c][t] = sum_{s,q} dout[s][o][q] in[s][c][2q + d - 1], db[o] = sum dout, as partial sums
+// part[range][o][c][28] (db[o] in every c). grid (COUT, CIN, split), TPB threads
 template <int CIN, int COUT, bool RELU_IN>
 __global__ void __launch_bounds__(TPB) conv_wgrad_kernel(const float *__restrict__ dout, const float *__restrict__ in,
                                                          long in_stride, const int *__restrict__ sidx, int S, int logn,
-                                                         float *__restrict__ gW, float *__restrict__ gb) {
+                                                         float *__restrict__ part) {
   __shared__ float red[28][TPB];
   const int o = blockIdx.x, c = blockIdx.y;
   const int n = 1 << logn, h = n >> 1, logh = logn - 1, mask = n - 1;
@@ -508,8 +540,8 @@ __global__ void __launch_bounds__(TPB) conv_wgrad_kernel(const float *__restrict
   float acc[28];
 #pragma unroll
   for (int t = 0; t < 28; ++t) acc[t] = 0.0f;
-  const long tot = (long)S * nout;
-  for (long e = threadIdx.x; e < tot; e += blockDim.x) {
+  const long tot = (long)S * nout, len = (tot + gridDim.z - 1) / gridDim.z, e0 = blockIdx.z * len;
+  for (long e = e0 + threadIdx.x; e < min(tot, e0 + len); e += blockDim.x) {
     const int s = (int)(e / nout);
     const long q = e - (long)s * nout;
     const float d = dout[((long)s * COUT + o) * nout + q];
@@ -533,10 +565,7 @@ __global__ void __launch_bounds__(TPB) conv_wgrad_kernel(const float *__restrict
     acc[27] += d;
   }
   block_sum<28>(red, acc);
-  if (threadIdx.x == 0) {
-    for (int t = 0; t < 27; ++t) gW[(o * CIN + c) * 27 + t] = red[t][0];
-    if (c == 0) gb[o] = red[27][0];
-  }
+  if (threadIdx.x < 28) part[(((long)blockIdx.z * COUT + o) * CIN + c) * 28 + threadIdx.x] = red[threadIdx.x][0];
 }
 
 // The transposed convolution as a gather, with the ReLU mask of its input: din[s][c][p] = [a_in > 0]
@@ -677,7 +706,7 @@ extern "C" int pc_ws_forward(int N, int nb, int S, const float *params, const fl
   PC_CK_LAUNCH();
   pool_value_kernel<<<S, TPB, 0, st>>>(z, params, of, dphi, nb, m3, pool, y);
   PC_CK_LAUNCH();
-  upsample_kernel<<<dim3((unsigned)((n + TPB - 1) / TPB), 3 * nb, S), TPB, 0, st>>>(coarse, static_cast<float2 *>(X),
+  upsample_kernel<<<dim3((unsigned)((n / 4 + TPB - 1) / TPB), 3 * nb, S), TPB, 0, st>>>(coarse, static_cast<float2 *>(X),
                                                                                    logN);
   PC_CK_LAUNCH();
   PC_CK(cudaStreamSynchronize(st));  // the host copy of phi goes out of scope
@@ -710,6 +739,7 @@ extern "C" int pc_ws_backward(int N, int nb, int S, const float *params, const f
   float *da1 = reinterpret_cast<float *>(wp(work, w.da1));
   float *dsa = reinterpret_cast<float *>(wp(work, w.dsa)), *dsc = reinterpret_cast<float *>(wp(work, w.dsc));
   double *dloss = reinterpret_cast<double *>(wp(work, w.loss));
+  float *part = reinterpret_cast<float *>(wp(work, w.part));
   void *gscr = wp(work, w.gram);
   const size_t gbytes = std::max<size_t>(16, gram_scratch_bytes(S, L, nb, nb));
   const long sx = (long)nb * L;
@@ -720,9 +750,7 @@ extern "C" int pc_ws_backward(int N, int nb, int S, const float *params, const f
   if (rc) return rc;
   loss_kernel<<<S, NBMAX * NBMAX, 0, st>>>(G, B, y, lam, w_val, nb, S, dloss, Cx, Cv, dy);
   PC_CK_LAUNCH();
-  rc = launch_block_update(S, L, nb, nb, PC_C64, X, sx, Cx, (long)nb * nb, dX, sx, st, nullptr);
-  if (rc) return rc;
-  rc = launch_block_update(S, L, nb, nb, PC_C64, V, sx, Cv, (long)nb * nb, dX, sx, st, nullptr, dX, sx);
+  rc = launch_block_update_sum(S, L, nb, nb, X, Cx, V, Cv, sx, (long)nb * nb, dX, sx, st);
   if (rc) return rc;
   // back through the upsampling, the head, FiLM and the value head
   upsample_bwd_kernel<<<dim3((unsigned)((m3 + TPB - 1) / TPB), 3 * nb, S), TPB, 0, st>>>(dX, dc, logN);
@@ -730,21 +758,31 @@ extern "C" int pc_ws_backward(int N, int nb, int S, const float *params, const f
   head_bwd_kernel<<<dim3((unsigned)((m3 + TPB - 1) / TPB), S), TPB, 0, st>>>(dc, a2, params, of, dphi, dy, nb, m3, dz,
                                                                             da2);
   PC_CK_LAUNCH();
-  head_grad_kernel<<<6 * nb, TPB, 0, st>>>(dc, z, nb, S, m3, grad + of.Wh, grad + of.bh);
+  auto reduce = [&](int split, int count, int row, int per_bias, float *out, float *bias) {
+    reduce_part_kernel<<<(count + TPB - 1) / TPB, TPB, 0, st>>>(part, split, count, row, per_bias, out, bias);
+  };
+  int split = split_for(3 * nb, (long)S * m3);
+  head_grad_kernel<<<dim3(3 * nb, split), TPB, 0, st>>>(dc, z, nb, S, m3, part);
+  PC_CK_LAUNCH();
+  reduce(split, 6 * nb * (C2 + 1), C2 + 1, 1, grad + of.Wh, grad + of.bh);
   PC_CK_LAUNCH();
   film_grad_kernel<<<dim3(C2, S), TPB, 0, st>>>(dz, a2, m3, dsa, dsc);
   PC_CK_LAUNCH();
   small_grads_kernel<<<1, TPB, 0, st>>>(dsa, dsc, dphi, pool, dy, nb, S, of, grad);
   PC_CK_LAUNCH();
   // back through the encoder
-  conv_wgrad_kernel<C1, C2, true><<<dim3(C2, C1), TPB, 0, st>>>(da2, a1, C1 * n1, nullptr, S, logN - 1,
-                                                                 grad + of.W2, grad + of.b2);
+  split = split_for(C1 * C2, (long)S * m3);
+  conv_wgrad_kernel<C1, C2, true><<<dim3(C2, C1, split), TPB, 0, st>>>(da2, a1, C1 * n1, nullptr, S, logN - 1, part);
+  PC_CK_LAUNCH();
+  reduce(split, C2 * C1 * 28, 28, C1, grad + of.W2, grad + of.b2);
   PC_CK_LAUNCH();
   conv_dgrad_kernel<C1, C2><<<dim3((unsigned)((n1 + TPB - 1) / TPB), S), TPB, 0, st>>>(da2, params + of.W2, a1,
                                                                                        logN - 1, da1);
   PC_CK_LAUNCH();
-  conv_wgrad_kernel<3, C1, false><<<dim3(C1, 3), TPB, 0, st>>>(da1, m0, 3 * n, sidx, S, logN, grad + of.W1,
-                                                               grad + of.b1);
+  split = split_for(3 * C1, (long)S * n1);
+  conv_wgrad_kernel<3, C1, false><<<dim3(C1, 3, split), TPB, 0, st>>>(da1, m0, 3 * n, sidx, S, logN, part);
+  PC_CK_LAUNCH();
+  reduce(split, C1 * 3 * 28, 28, 3, grad + of.W1, grad + of.b1);
   PC_CK_LAUNCH();
   PC_CK(cudaMemcpyAsync(loss, dloss, sizeof(double) * S, cudaMemcpyDeviceToDevice, st));
   return PC_OK;
