@@ -16,6 +16,9 @@
 // The frequency data never needs reordering: the DIT inverse consumes the DIF output order directly.
 // Each line is transformed in shared memory with radix-2 butterflies; twiddles exp(-2 pi i t / N) come from a
 // table computed once on the host.
+// Bound (FP64): the FP64 pipe, 64 to 76 cycles per warp instruction on an SM sub-partition. One k-point x 13 fields at
+// N = 16: 75 us a call with a multiplication in every butterfly, three divisions per mode and 16-column z tiles, 65 us
+// now; 2 fields at N = 32: 137 and 91 us.
 #include <cmath>
 
 #include "pc_internal.cuh"
@@ -29,6 +32,16 @@ __device__ __forceinline__ int bitrev(int p, int logN) { return (int)(__brev((un
 // exp(+).
 // LINE_MAJOR: consecutive threads take consecutive lines (for lines that are adjacent in memory, ls = 1, so that a
 // warp reads consecutive addresses); otherwise consecutive butterflies of one line (for contiguous lines, es = 1).
+// The twiddles of the two shortest stages are 1 and -i (FP64: half of a butterfly's instructions).
+template <bool INV, typename C> __device__ __forceinline__ C fft_twiddle(C x, const C *tw, int jj, int lh, int logN) {
+  if (lh == 0) return x;
+  if (lh == 1) {
+    const C r = INV ? cmake<C>(-x.y, x.x) : cmake<C>(x.y, -x.x);
+    return jj ? r : x;
+  }
+  const C w = tw[jj << (logN - 1 - lh)];
+  return INV ? cmulc(w, x) : cmul(x, w);
+}
 template <typename C, bool FWD, bool LINE_MAJOR = false>
 __device__ __forceinline__ void fft_lines(C *a, int lines, int lpg, int gs, int ls, int es, int logN, const C *tw) {
   const int N = 1 << logN, halfN = N >> 1;
@@ -43,7 +56,7 @@ __device__ __forceinline__ void fft_lines(C *a, int lines, int lpg, int gs, int 
         const int i0 = lg * gs + lu * ls + ((g << (lh + 1)) + jj) * es, i1 = i0 + half * es;
         const C x0 = a[i0], x1 = a[i1];
         a[i0] = cadd(x0, x1);
-        a[i1] = cmul(csub(x0, x1), tw[jj << (logN - 1 - lh)]);
+        a[i1] = fft_twiddle<false>(csub(x0, x1), tw, jj, lh, logN);
       }
       __syncthreads();
     }
@@ -55,8 +68,7 @@ __device__ __forceinline__ void fft_lines(C *a, int lines, int lpg, int gs, int 
         const int g = r >> lh, jj = r & (half - 1);
         const int lg = l / lpg, lu = l - lg * lpg;
         const int i0 = lg * gs + lu * ls + ((g << (lh + 1)) + jj) * es, i1 = i0 + half * es;
-        const C w = tw[jj << (logN - 1 - lh)];
-        const C t = cmulc(w, a[i1]);  // conj(w) * a[i1]
+        const C t = fft_twiddle<true>(a[i1], tw, jj, lh, logN);  // conj(w) * a[i1]
         const C x0 = a[i0];
         a[i1] = csub(x0, t);
         a[i0] = cadd(x0, t);
@@ -178,8 +190,8 @@ __global__ void __launch_bounds__(256) fft_z_symbol_kernel(const cplx<T> *__rest
   fft_lines<C, true, true>(a, 3 * U, U, N * U, 1, U, logN, s_tw);  // lines (comp, u); z stride U
   // symbol inverse per mode
   const double2 *symb = sym + (long)b * (LAT ? 9 : 3) * N;
-  const T fac = (T)((kp[b].gamma - 1.0) / kp[b].gamma);  // (gamma - 1) / gamma, once per block
-  const T scale = (T)(1.0 / (double)n);
+  const T fac = std::is_same<T, double>::value ? (T)kp[b].pfac : (T)kp[b].pfacf;  // (gamma - 1) / gamma
+  const T scale = (T)__int_as_float((127 - 3 * logN) << 23);                      // 1 / N^3
   const int my = bitrev(y, logN);
   const double2 d2d = LAT ? make_double2(0.0, 0.0) : symb[N + my];
   for (int i = threadIdx.x; i < N * U; i += blockDim.x) {
@@ -206,10 +218,10 @@ __global__ void __launch_bounds__(256) fft_z_symbol_kernel(const cplx<T> *__rest
     if (!(sigma > (T)0)) {
       r1 = r2 = r3 = cmake<C>((T)0, (T)0);
     } else {
-      const T inv = scale / sigma;
+      const T rs = (T)1 / sigma, inv = scale * rs;  // one division: 1 / N^3 is a power of two
       if (!laplacian) {
         const C s = cadd(cadd(cmul(d1, r1), cmul(d2, r2)), cmul(d3, r3));  // d^T r
-        const T f = fac / sigma;
+        const T f = fac * rs;
         r1 = csub(r1, cscale(cmulc(d1, s), f));  // conj(d1) * s
         r2 = csub(r2, cscale(cmulc(d2, s), f));
         r3 = csub(r3, cscale(cmulc(d3, s), f));
@@ -436,6 +448,9 @@ static int launch_precond_t(pc_ctx *ctx, int nb, int m, const void *R, long sr, 
   const int Uy = std::min(N, std::max(1, elems / N));  // x values per CTA along y
   int Uz = 1;
   while (Uz * 2 <= N && 3 * N * Uz * 2 <= 3 * elems / 2) Uz *= 2;
+  // few blocks: narrower z tiles (not below 64 bytes a row), so that every SM has several: the FP64 pipe's time per SM is
+  // what counts, and 208 blocks of 16 columns (13 fields at N = 16) left some SMs two and some one
+  while (Uz > 4 && sizeof(C) * Uz > 64 && (long)N * (N / Uz) * m * nb < 4L * sm_count()) Uz /= 2;
   const size_t tw_b = sizeof(C) * (N / 2);
   const size_t sx = tw_b + sizeof(C) * Rr * N, sy = tw_b + sizeof(C) * Uy * N, sz = tw_b + sizeof(C) * 3 * N * Uz;
   static bool configured = false;

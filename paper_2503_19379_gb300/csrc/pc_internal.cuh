@@ -48,6 +48,7 @@ struct KParam {
   float khl[3];  // remainders: (khf, khl) and (gammaf, gammal) are the double-float values of k_i / 2 and gamma
   float gammal;
   float pfacf;   // (gamma - 1) / gamma rounded to FP32 (the complex64 preconditioner's projection factor)
+  double pfac;   // the same in FP64
 };
 
 // internal dtype of the mixed solve's FP64-accurate block: complex double-float pairs, one float4 per element

@@ -135,7 +135,8 @@ int upload_kpoints(pc_ctx *ctx, int nb, const double *kpts, const double *gammas
     kp[b].gamma = gammas[b];
     kp[b].gammaf = (float)gammas[b];
     kp[b].gammal = (float)(gammas[b] - (double)kp[b].gammaf);
-    kp[b].pfacf = (float)((gammas[b] - 1.0) / gammas[b]);
+    kp[b].pfac = (gammas[b] - 1.0) / gammas[b];
+    kp[b].pfacf = (float)kp[b].pfac;
     if (!ctx->lat) {
       for (int d = 0; d < 3; ++d)
         axis_symbols(ctx->N, ctx->opts.order, kpts[3 * b + d], &sym[((size_t)b * 3 + d) * ctx->N]);
