@@ -16,17 +16,90 @@
 
 namespace pc {
 
+// ---------------------------------------------------------------- packed complex double-float
+// A complex double-float as two packed FP32 pairs, hi = (re.hi, im.hi) and lo = (re.lo, im.lo): every operation runs on
+// both parts with one instruction (add, mul, fma .f32x2). Their rate in results is that of the scalar ones (measured: 124
+// and 119 per clock and SM), in half the issue slots, and the stencils below are bound by issue (71% of the cycles
+// with the FMA pipe 60% busy; complex128 blocks of 15 k-points x 16 fields at N = 32: 1.10 ms with scalar operations,
+// 1.01 ms with these). The operations and their order are those of dfloat.cuh: the same bits.
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, 0xbf800000bf800000ull, a); }  // b (-1, -1) + a
+__device__ __forceinline__ f32x2 swap2(f32x2 v) {
+  const float2 t = unpack2(v);
+  return pack2(t.y, t.x);
+}
+
+struct zdf {
+  f32x2 hi, lo;
+};
+__device__ __forceinline__ zdf zdf_quick(f32x2 a, f32x2 b) {  // quick_two_sum
+  zdf r;
+  r.hi = add2(a, b);
+  r.lo = sub2(b, sub2(r.hi, a));
+  return r;
+}
+__device__ __forceinline__ zdf cdf_add(zdf x, zdf y) {
+  const f32x2 s = add2(x.hi, y.hi), bb = sub2(s, x.hi);
+  const f32x2 e = add2(sub2(x.hi, sub2(s, bb)), sub2(y.hi, bb));
+  return zdf_quick(s, add2(e, add2(x.lo, y.lo)));
+}
+__device__ __forceinline__ zdf cdf_sub(zdf x, zdf y) {
+  const f32x2 s = sub2(x.hi, y.hi), bb = sub2(s, x.hi);
+  const f32x2 e = sub2(sub2(x.hi, sub2(s, bb)), add2(y.hi, bb));
+  return zdf_quick(s, add2(e, sub2(x.lo, y.lo)));
+}
+// a s for a real double-float s (df_mul(a, s) for both parts)
+__device__ __forceinline__ zdf cdf_scale(zdf a, df s) {
+  const f32x2 sh = pack2(s.hi, s.hi), sl = pack2(s.lo, s.lo);
+  const f32x2 p = mul2(a.hi, sh);
+  f32x2 e = fma2(a.hi, sh, mul2(p, 0xbf800000bf800000ull));
+  e = fma2(a.hi, sl, e);
+  e = fma2(a.lo, sh, e);
+  return zdf_quick(p, e);
+}
+// i k s for a real double-float k as the pairs (-k, k) in kp and (k, -k) in km: df_mul(k, .) of the exchanged parts
+struct kdf {
+  f32x2 hp, lp, hm, lm;
+};
+__device__ __forceinline__ kdf kdf_of(float hi, float lo) {
+  return kdf{pack2(-hi, hi), pack2(-lo, lo), pack2(hi, -hi), pack2(lo, -lo)};
+}
+__device__ __forceinline__ zdf imul(zdf s, f32x2 kh, f32x2 kl, f32x2 nkh, f32x2 nkl) {
+  const f32x2 sh = swap2(s.hi), sl = swap2(s.lo);
+  const f32x2 p = mul2(kh, sh);
+  f32x2 e = fma2(nkh, sh, p);  // minus the rounding error of p
+  e = fma2(nkh, sl, e);
+  e = fma2(nkl, sh, e);
+  zdf r;
+  r.hi = sub2(p, e);
+  r.lo = sub2(sub2(p, r.hi), e);
+  return r;
+}
+
+__device__ __forceinline__ zdf ld_zdf(const double2 *p) {
+  const double2 v = *p;
+  const df re = df_from(v.x), im = df_from(v.y);
+  return zdf{pack2(re.hi, im.hi), pack2(re.lo, im.lo)};
+}
+__device__ __forceinline__ zdf ld_zdf(const float4 *p) {
+  const float4 v = *p;
+  return zdf{pack2(v.x, v.z), pack2(v.y, v.w)};
+}
+__device__ __forceinline__ cdf to_cdf(zdf z) {
+  const float2 h = unpack2(z.hi), l = unpack2(z.lo);
+  return cdf{df{h.x, l.x}, df{h.y, l.y}};
+}
+__device__ __forceinline__ void st_cdf(double2 *p, zdf z) { st_cdf(p, to_cdf(z)); }
+__device__ __forceinline__ void st_cdf(float4 *p, zdf z) { st_cdf(p, to_cdf(z)); }
+
 // ---------------------------------------------------------------- stencil
 // (D f)_r = ih (f_{r+1} - f_r) + i kh (f_r + f_{r+1});  (D' g)_r = ih (g_{r-1} - g_r) - i kh (g_{r-1} + g_r)
-__device__ __forceinline__ cdf dfwd_df(cdf f0, cdf f1, float ih, df kh) {
-  const cdf a = cdf_sub(f1, f0), s = cdf_add(f0, f1);
-  // ih a + i kh s = (ih a.re - kh s.im) + i (ih a.im + kh s.re)
-  return cdf{df_sub(df_scale2(a.re, ih), df_mul(kh, s.im)), df_add(df_scale2(a.im, ih), df_mul(kh, s.re))};
+__device__ __forceinline__ zdf dfwd_df(zdf f0, zdf f1, f32x2 ih, const kdf &k) {
+  const zdf a = cdf_sub(f1, f0), s = cdf_add(f0, f1);
+  return cdf_add(zdf{mul2(a.hi, ih), mul2(a.lo, ih)}, imul(s, k.hp, k.lp, k.hm, k.lm));
 }
-__device__ __forceinline__ cdf dbwd_df(cdf gm, cdf g0, float ih, df kh) {
-  const cdf a = cdf_sub(gm, g0), s = cdf_add(gm, g0);
-  // ih a - i kh s = (ih a.re + kh s.im) + i (ih a.im - kh s.re)
-  return cdf{df_add(df_scale2(a.re, ih), df_mul(kh, s.im)), df_sub(df_scale2(a.im, ih), df_mul(kh, s.re))};
+__device__ __forceinline__ zdf dbwd_df(zdf gm, zdf g0, f32x2 ih, const kdf &k) {
+  const zdf a = cdf_sub(gm, g0), s = cdf_add(gm, g0);
+  return cdf_add(zdf{mul2(a.hi, ih), mul2(a.lo, ih)}, imul(s, k.hm, k.lm, k.hp, k.lp));
 }
 
 // Residual epilogue of the stencil (the mixed solve's phase 2): instead of AX the kernel writes, per point,
@@ -41,6 +114,9 @@ struct ResidArgs {
   double *part;  // [nb][m][blocks per field][2]
 };
 
+__device__ __forceinline__ float2 cdf_round(zdf a) { return unpack2(add2(a.hi, a.lo)); }
+__device__ __forceinline__ float2 cdf_high(zdf a) { return unpack2(a.hi); }
+__device__ __forceinline__ float2 cdf_high(cdf a) { return make_float2(a.re.hi, a.im.hi); }
 __device__ __forceinline__ float2 cdf_round(cdf a) { return make_float2(a.re.hi + a.re.lo, a.im.hi + a.im.lo); }
 __device__ __forceinline__ df ld_m0(const float2 *p) {
   const float2 v = *p;
@@ -48,15 +124,16 @@ __device__ __forceinline__ df ld_m0(const float2 *p) {
 }
 
 // writes the three components of one point; returns |r|^2 and |x|^2 contributions
-__device__ __forceinline__ void resid_point(const ResidArgs &ra, int b, int j, long n, long gi, df th, const cdf (&y)[3],
-                                            const cdf (&x)[3], float &sr, float &sxx) {
+template <typename Z>
+__device__ __forceinline__ void resid_point(const ResidArgs &ra, int b, int j, long n, long gi, df th, const Z (&y)[3],
+                                            const Z (&x)[3], float &sr, float &sxx) {
   const long L = 3 * n;
   float2 *r1 = ra.R1 + (long)b * ra.sr1 + (long)j * L, *r2 = ra.R2 + (long)b * ra.sr2 + (long)j * L;
   float2 *x32 = ra.X32 + (long)b * ra.sx32 + (long)j * L, *ax32 = ra.AX32 + (long)b * ra.sax32 + (long)j * L;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    const cdf r = cdf_sub(y[c], cdf_scale(x[c], th));
-    const float2 rf = cdf_round(r), xf = make_float2(x[c].re.hi, x[c].im.hi);
+    const Z r = cdf_sub(y[c], cdf_scale(x[c], th));
+    const float2 rf = cdf_round(r), xf = cdf_high(x[c]);
     const long o = c * n + gi;
     r1[o] = rf;
     r2[o] = rf;
@@ -95,7 +172,7 @@ __device__ __forceinline__ void resid_block_sum(const ResidArgs &ra, float sr, f
 }
 
 template <int TX, int TY, int TZ> constexpr size_t op_df_smem_bytes() {
-  return sizeof(cdf) * (size_t)(3 * (TZ + 2) * (TY + 2) * (TX + 2) + 3 * (TZ + 1) * (TY + 1) * (TX + 1) +
+  return sizeof(zdf) * (size_t)(3 * (TZ + 2) * (TY + 2) * (TX + 2) + 3 * (TZ + 1) * (TY + 1) * (TX + 1) +
                                 (TZ + 1) * (TY + 1) * (TX + 1));
 }
 
@@ -117,9 +194,9 @@ __global__ void __launch_bounds__(256) op_df_kernel(const df_store_t<RES> *__res
   constexpr int VX = TX + 2, VY = TY + 2, VZ = TZ + 2;
   constexpr int EX = TX + 1, EY = TY + 1, EZ = TZ + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cdf *v = reinterpret_cast<cdf *>(smem_raw);
-  cdf *e = v + 3 * VZ * VY * VX;
-  cdf *c = e + 3 * EZ * EY * EX;
+  zdf *v = reinterpret_cast<zdf *>(smem_raw);
+  zdf *e = v + 3 * VZ * VY * VX;
+  zdf *c = e + 3 * EZ * EY * EX;
   const int N = 1 << logN, mask = N - 1;
   const long n = 1L << (3 * logN);
   const int b = act ? act[blockIdx.z] : (int)blockIdx.z;
@@ -133,9 +210,9 @@ __global__ void __launch_bounds__(256) op_df_kernel(const df_store_t<RES> *__res
   const XS *Xb = X + (long)b * sx + (long)j * 3 * n;
   XS *Yb = Y + (long)b * sy + (long)j * 3 * n;
   const KParam p = kp[b];
-  const df kh0 = kp_df(p.khf[0], p.khl[0]), kh1 = kp_df(p.khf[1], p.khl[1]), kh2 = kp_df(p.khf[2], p.khl[2]);
+  const kdf kh0 = kdf_of(p.khf[0], p.khl[0]), kh1 = kdf_of(p.khf[1], p.khl[1]), kh2 = kdf_of(p.khf[2], p.khl[2]);
   const df gam = kp_df(p.gammaf, p.gammal);
-  const float ih = (float)N;
+  const f32x2 ih = pack2((float)N, (float)N);
 
   for (int i = threadIdx.x; i < 3 * VZ * VY * VX; i += blockDim.x) {
     int lx = i % VX, r = i / VX;
@@ -143,19 +220,19 @@ __global__ void __launch_bounds__(256) op_df_kernel(const df_store_t<RES> *__res
     r /= VY;
     int lz = r % VZ, comp = r / VZ;
     int gx = (x0 + lx - 1) & mask, gy = (y0 + ly - 1) & mask, gz = (z0 + lz - 1) & mask;
-    v[i] = ld_cdf(Xb + comp * n + ((long)gz << (2 * logN)) + ((long)gy << logN) + gx);
+    v[i] = ld_zdf(Xb + comp * n + ((long)gz << (2 * logN)) + ((long)gy << logN) + gx);
   }
   __syncthreads();
   for (int i = threadIdx.x; i < EZ * EY * EX; i += blockDim.x) {
     const int ex = i % EX, ey = (i / EX) % EY, ez = i / (EX * EY);
 #define VV(comp, dz, dy, dx) v[(((comp) * VZ + ez + 1 + (dz)) * VY + ey + 1 + (dy)) * VX + ex + 1 + (dx)]
-    const cdf v1 = VV(0, 0, 0, 0), v2 = VV(1, 0, 0, 0), v3 = VV(2, 0, 0, 0);
-    const cdf d3v2 = dbwd_df(VV(1, -1, 0, 0), v2, ih, kh2);
-    const cdf d2v3 = dbwd_df(VV(2, 0, -1, 0), v3, ih, kh1);
-    const cdf d3v1 = dbwd_df(VV(0, -1, 0, 0), v1, ih, kh2);
-    const cdf d1v3 = dbwd_df(VV(2, 0, 0, -1), v3, ih, kh0);
-    const cdf d2v1 = dbwd_df(VV(0, 0, -1, 0), v1, ih, kh1);
-    const cdf d1v2 = dbwd_df(VV(1, 0, 0, -1), v2, ih, kh0);
+    const zdf v1 = VV(0, 0, 0, 0), v2 = VV(1, 0, 0, 0), v3 = VV(2, 0, 0, 0);
+    const zdf d3v2 = dbwd_df(VV(1, -1, 0, 0), v2, ih, kh2);
+    const zdf d2v3 = dbwd_df(VV(2, 0, -1, 0), v3, ih, kh1);
+    const zdf d3v1 = dbwd_df(VV(0, -1, 0, 0), v1, ih, kh2);
+    const zdf d1v3 = dbwd_df(VV(2, 0, 0, -1), v3, ih, kh0);
+    const zdf d2v1 = dbwd_df(VV(0, 0, -1, 0), v1, ih, kh1);
+    const zdf d1v2 = dbwd_df(VV(1, 0, 0, -1), v2, ih, kh0);
 #undef VV
     const int gx = (x0 + ex) & mask, gy = (y0 + ey) & mask, gz = (z0 + ez) & mask;
     const long gi = ((long)gz << (2 * logN)) + ((long)gy << logN) + gx;
@@ -164,7 +241,7 @@ __global__ void __launch_bounds__(256) op_df_kernel(const df_store_t<RES> *__res
     e[EZ * EY * EX + eo] = cdf_scale(cdf_sub(d1v3, d3v1), ld_m0(m0 + n + gi));
     e[2 * EZ * EY * EX + eo] = cdf_scale(cdf_sub(d2v1, d1v2), ld_m0(m0 + 2 * n + gi));
 #define WW(comp, dz, dy, dx) v[(((comp) * VZ + ez + (dz)) * VY + ey + (dy)) * VX + ex + (dx)]
-    cdf cc = dfwd_df(WW(0, 0, 0, 0), WW(0, 0, 0, 1), ih, kh0);
+    zdf cc = dfwd_df(WW(0, 0, 0, 0), WW(0, 0, 0, 1), ih, kh0);
     cc = cdf_add(cc, dfwd_df(WW(1, 0, 0, 0), WW(1, 0, 1, 0), ih, kh1));
     cc = cdf_add(cc, dfwd_df(WW(2, 0, 0, 0), WW(2, 1, 0, 0), ih, kh2));
 #undef WW
@@ -176,20 +253,20 @@ __global__ void __launch_bounds__(256) op_df_kernel(const df_store_t<RES> *__res
     const int lx = i % TX, ly = (i / TX) % TY, lz = i / (TX * TY);
 #define EE(comp, dz, dy, dx) e[(((comp) * EZ + lz + (dz)) * EY + ly + (dy)) * EX + lx + (dx)]
 #define CC(dz, dy, dx) c[((lz + 1 + (dz)) * EY + ly + 1 + (dy)) * EX + lx + 1 + (dx)]
-    const cdf c0 = CC(0, 0, 0);
-    const cdf e1 = EE(0, 0, 0, 0), e2 = EE(1, 0, 0, 0), e3 = EE(2, 0, 0, 0);
-    cdf y1 = cdf_sub(dfwd_df(e3, EE(2, 0, 1, 0), ih, kh1), dfwd_df(e2, EE(1, 1, 0, 0), ih, kh2));
+    const zdf c0 = CC(0, 0, 0);
+    const zdf e1 = EE(0, 0, 0, 0), e2 = EE(1, 0, 0, 0), e3 = EE(2, 0, 0, 0);
+    zdf y1 = cdf_sub(dfwd_df(e3, EE(2, 0, 1, 0), ih, kh1), dfwd_df(e2, EE(1, 1, 0, 0), ih, kh2));
     y1 = cdf_add(y1, cdf_scale(dbwd_df(CC(0, 0, -1), c0, ih, kh0), gam));
-    cdf y2 = cdf_sub(dfwd_df(e1, EE(0, 1, 0, 0), ih, kh2), dfwd_df(e3, EE(2, 0, 0, 1), ih, kh0));
+    zdf y2 = cdf_sub(dfwd_df(e1, EE(0, 1, 0, 0), ih, kh2), dfwd_df(e3, EE(2, 0, 0, 1), ih, kh0));
     y2 = cdf_add(y2, cdf_scale(dbwd_df(CC(0, -1, 0), c0, ih, kh1), gam));
-    cdf y3 = cdf_sub(dfwd_df(e2, EE(1, 0, 0, 1), ih, kh0), dfwd_df(e1, EE(0, 0, 1, 0), ih, kh1));
+    zdf y3 = cdf_sub(dfwd_df(e2, EE(1, 0, 0, 1), ih, kh0), dfwd_df(e1, EE(0, 0, 1, 0), ih, kh1));
     y3 = cdf_add(y3, cdf_scale(dbwd_df(CC(-1, 0, 0), c0, ih, kh2), gam));
 #undef EE
 #undef CC
     const long gi = ((long)(z0 + lz) << (2 * logN)) + ((long)(y0 + ly) << logN) + x0 + lx;
     if constexpr (RES) {
 #define XV(comp) v[(((comp) * VZ + lz + 1) * VY + ly + 1) * VX + lx + 1]
-      const cdf yv[3] = {y1, y2, y3}, xv[3] = {XV(0), XV(1), XV(2)};
+      const zdf yv[3] = {y1, y2, y3}, xv[3] = {XV(0), XV(1), XV(2)};
 #undef XV
       resid_point(ra, b, j, n, gi, df_from(ra.theta[(long)b * ra.m + j]), yv, xv, sr, sxx);
     } else {
@@ -225,7 +302,7 @@ static int launch_op_df_t(pc_ctx *ctx, int nb, int m, const void *X, long sx, vo
 // z-marching version (the blocking of opz_kernel in stencil.cu): a TX x TY column tile walks ZC planes with ring
 // buffers of v (2 planes), e = M0 A' v (2 planes) and c = B v (2 planes).
 template <int TX, int TY> constexpr size_t opz_df_smem_bytes() {
-  return sizeof(cdf) * (size_t)(2 * 3 * (TY + 2) * (TX + 2) + 2 * 3 * (TY + 1) * (TX + 1) + 2 * (TY + 1) * (TX + 1));
+  return sizeof(zdf) * (size_t)(2 * 3 * (TY + 2) * (TX + 2) + 2 * 3 * (TY + 1) * (TX + 1) + 2 * (TY + 1) * (TX + 1));
 }
 
 template <int TX, int TY, bool RES>
@@ -239,9 +316,9 @@ __global__ void __launch_bounds__(TX * TY) opz_df_kernel(const df_store_t<RES> *
   constexpr int EX = TX + 1, EY = TY + 1, EP = EX * EY;
   constexpr int NT = TX * TY;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cdf *vbuf = reinterpret_cast<cdf *>(smem_raw);
-  cdf *ebuf = vbuf + 2 * 3 * VP;
-  cdf *cbuf = ebuf + 2 * 3 * EP;
+  zdf *vbuf = reinterpret_cast<zdf *>(smem_raw);
+  zdf *ebuf = vbuf + 2 * 3 * VP;
+  zdf *cbuf = ebuf + 2 * 3 * EP;
   const int N = 1 << logN, mask = N - 1;
   const long n = 1L << (3 * logN), plane = 1L << (2 * logN);
   const int b = act ? act[blockIdx.z] : (int)blockIdx.z;
@@ -255,33 +332,33 @@ __global__ void __launch_bounds__(TX * TY) opz_df_kernel(const df_store_t<RES> *
   const XS *Xb = X + (long)b * sx + (long)j * 3 * n;
   XS *Yb = Y + (long)b * sy + (long)j * 3 * n;
   const KParam &p = kp[b];
-  const df kh0 = kp_df(p.khf[0], p.khl[0]), kh1 = kp_df(p.khf[1], p.khl[1]), kh2 = kp_df(p.khf[2], p.khl[2]);
+  const kdf kh0 = kdf_of(p.khf[0], p.khl[0]), kh1 = kdf_of(p.khf[1], p.khl[1]), kh2 = kdf_of(p.khf[2], p.khl[2]);
   const df gam = kp_df(p.gammaf, p.gammal);
-  const float ih = (float)N;
+  const f32x2 ih = pack2((float)N, (float)N);
   const int tid = threadIdx.x;
   auto load_v = [&](int slot, int z) {
     const int gz = z & mask;
-    cdf *vs = vbuf + slot * 3 * VP;
+    zdf *vs = vbuf + slot * 3 * VP;
     for (int i = tid; i < 3 * VP; i += NT) {
       const int comp = i / VP, r = i - comp * VP, ly = r / VX, lx = r - ly * VX;
       const int gx = (x0 + lx - 1) & mask, gy = (y0 + ly - 1) & mask;
-      vs[i] = ld_cdf(Xb + comp * n + gz * plane + ((long)gy << logN) + gx);
+      vs[i] = ld_zdf(Xb + comp * n + gz * plane + ((long)gy << logN) + gx);
     }
   };
   auto make_e = [&](int eslot, int z, int sz, int szm) {
-    const cdf *v0 = vbuf + sz * 3 * VP, *vm = vbuf + szm * 3 * VP;
-    cdf *es = ebuf + eslot * 3 * EP;
+    const zdf *v0 = vbuf + sz * 3 * VP, *vm = vbuf + szm * 3 * VP;
+    zdf *es = ebuf + eslot * 3 * EP;
     const int gz = z & mask;
     for (int i = tid; i < EP; i += NT) {
       const int ey = i / EX, ex = i - ey * EX;
       const int o = (ey + 1) * VX + ex + 1;
-      const cdf v1 = v0[o], v2 = v0[VP + o], v3 = v0[2 * VP + o];
-      const cdf d3v2 = dbwd_df(vm[VP + o], v2, ih, kh2);
-      const cdf d2v3 = dbwd_df(v0[2 * VP + o - VX], v3, ih, kh1);
-      const cdf d3v1 = dbwd_df(vm[o], v1, ih, kh2);
-      const cdf d1v3 = dbwd_df(v0[2 * VP + o - 1], v3, ih, kh0);
-      const cdf d2v1 = dbwd_df(v0[o - VX], v1, ih, kh1);
-      const cdf d1v2 = dbwd_df(v0[VP + o - 1], v2, ih, kh0);
+      const zdf v1 = v0[o], v2 = v0[VP + o], v3 = v0[2 * VP + o];
+      const zdf d3v2 = dbwd_df(vm[VP + o], v2, ih, kh2);
+      const zdf d2v3 = dbwd_df(v0[2 * VP + o - VX], v3, ih, kh1);
+      const zdf d3v1 = dbwd_df(vm[o], v1, ih, kh2);
+      const zdf d1v3 = dbwd_df(v0[2 * VP + o - 1], v3, ih, kh0);
+      const zdf d2v1 = dbwd_df(v0[o - VX], v1, ih, kh1);
+      const zdf d1v2 = dbwd_df(v0[VP + o - 1], v2, ih, kh0);
       const long gi = gz * plane + ((long)((y0 + ey) & mask) << logN) + ((x0 + ex) & mask);
       es[i] = cdf_scale(cdf_sub(d3v2, d2v3), ld_m0(m0 + gi));
       es[EP + i] = cdf_scale(cdf_sub(d1v3, d3v1), ld_m0(m0 + n + gi));
@@ -289,12 +366,12 @@ __global__ void __launch_bounds__(TX * TY) opz_df_kernel(const df_store_t<RES> *
     }
   };
   auto make_c = [&](int cslot, int sz, int szp) {
-    const cdf *v0 = vbuf + sz * 3 * VP, *vp = vbuf + szp * 3 * VP;
-    cdf *cs = cbuf + cslot * EP;
+    const zdf *v0 = vbuf + sz * 3 * VP, *vp = vbuf + szp * 3 * VP;
+    zdf *cs = cbuf + cslot * EP;
     for (int i = tid; i < EP; i += NT) {
       const int cy = i / EX, cx = i - cy * EX;
       const int o = cy * VX + cx;
-      cdf cc = dfwd_df(v0[o], v0[o + 1], ih, kh0);
+      zdf cc = dfwd_df(v0[o], v0[o + 1], ih, kh0);
       cc = cdf_add(cc, dfwd_df(v0[VP + o], v0[VP + o + VX], ih, kh1));
       cc = cdf_add(cc, dfwd_df(v0[2 * VP + o], vp[2 * VP + o], ih, kh2));
       cs[i] = cc;
@@ -316,24 +393,24 @@ __global__ void __launch_bounds__(TX * TY) opz_df_kernel(const df_store_t<RES> *
     make_c(1 - sc, sv, 1 - sv);
     __syncthreads();
     {
-      const cdf *e0 = ebuf + se * 3 * EP, *e1p = ebuf + (1 - se) * 3 * EP;
-      const cdf *cm = cbuf + sc * EP, *c0p = cbuf + (1 - sc) * EP;
+      const zdf *e0 = ebuf + se * 3 * EP, *e1p = ebuf + (1 - se) * 3 * EP;
+      const zdf *cm = cbuf + sc * EP, *c0p = cbuf + (1 - sc) * EP;
       const int ly = tid / TX, lx = tid - ly * TX;
       const int eo = ly * EX + lx;
       const int co = (ly + 1) * EX + lx + 1;
-      const cdf c0 = c0p[co];
-      const cdf e1 = e0[eo], e2 = e0[EP + eo], e3 = e0[2 * EP + eo];
-      cdf y1 = cdf_sub(dfwd_df(e3, e0[2 * EP + eo + EX], ih, kh1), dfwd_df(e2, e1p[EP + eo], ih, kh2));
+      const zdf c0 = c0p[co];
+      const zdf e1 = e0[eo], e2 = e0[EP + eo], e3 = e0[2 * EP + eo];
+      zdf y1 = cdf_sub(dfwd_df(e3, e0[2 * EP + eo + EX], ih, kh1), dfwd_df(e2, e1p[EP + eo], ih, kh2));
       y1 = cdf_add(y1, cdf_scale(dbwd_df(c0p[co - 1], c0, ih, kh0), gam));
-      cdf y2 = cdf_sub(dfwd_df(e1, e1p[eo], ih, kh2), dfwd_df(e3, e0[2 * EP + eo + 1], ih, kh0));
+      zdf y2 = cdf_sub(dfwd_df(e1, e1p[eo], ih, kh2), dfwd_df(e3, e0[2 * EP + eo + 1], ih, kh0));
       y2 = cdf_add(y2, cdf_scale(dbwd_df(c0p[co - EX], c0, ih, kh1), gam));
-      cdf y3 = cdf_sub(dfwd_df(e2, e0[EP + eo + 1], ih, kh0), dfwd_df(e1, e0[eo + EX], ih, kh1));
+      zdf y3 = cdf_sub(dfwd_df(e2, e0[EP + eo + 1], ih, kh0), dfwd_df(e1, e0[eo + EX], ih, kh1));
       y3 = cdf_add(y3, cdf_scale(dbwd_df(cm[co], c0, ih, kh2), gam));
       const long gi = (long)z * plane + ((long)(y0 + ly) << logN) + x0 + lx;
       if constexpr (RES) {
-        const cdf *v0 = vbuf + sv * 3 * VP;  // plane z
+        const zdf *v0 = vbuf + sv * 3 * VP;  // plane z
         const int o = (ly + 1) * VX + lx + 1;
-        const cdf yv[3] = {y1, y2, y3}, xv[3] = {v0[o], v0[VP + o], v0[2 * VP + o]};
+        const zdf yv[3] = {y1, y2, y3}, xv[3] = {v0[o], v0[VP + o], v0[2 * VP + o]};
         resid_point(ra, b, j, n, gi, th, yv, xv, sr, sxx);
       } else {
         st_cdf(Yb + gi, y1);
