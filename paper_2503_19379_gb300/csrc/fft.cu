@@ -534,7 +534,7 @@ extern "C" int pc_apply_precond(pc_ctx *ctx, int nb, const double *kpts, const d
   PC_REQUIRE(ctx && kpts && gammas && R && W, "pc_apply_precond: null argument");
   PC_REQUIRE(nb >= 0 && m >= 0, "pc_apply_precond: negative size");
   PC_REQUIRE(dtype == PC_C128 || dtype == PC_C64, "pc_apply_precond: bad dtype %d", dtype);
-  int rc = upload_kpoints(ctx, nb, kpts, gammas);
+  int rc = upload_kpoints(ctx, nb, kpts, gammas, false);
   if (rc) return rc;
   const long blk = (long)m * 3 * ctx->n;
   return launch_precond(ctx, nb, m, dtype, R, blk, W, blk, nullptr);

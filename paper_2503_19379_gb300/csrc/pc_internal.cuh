@@ -155,6 +155,15 @@ struct pc_ctx {
   pc::DevBuf symd;          // per-k axis symbols d_i(m) complex128 [nb][3][N]; general lattice: [nb][3][3][N]
   pc::DevBuf scratch;       // general scratch (partial sums)
   int kcap = 0;             // capacity (k-points) of kparam / symd
+  // host tables of the axis symbols (see axis_symbols), and pinned staging of upload_kpoints
+  std::vector<double> symS, symZ, symE;
+  struct Stage {
+    void *p = nullptr;
+    size_t bytes = 0;
+    cudaEvent_t done = nullptr;  // the last copies from p have completed
+  };
+  Stage stage[2];
+  int stage_next = 0;
   // solver buffers
   pc::DevBuf S[2], AS[2], Gm, Hm, coef, theta, norms, rnorm, rank, flag;
   // mixed-precision solve: FP64 block X, complex64 residual copy, coupling R^H S, FP64 X^H X, phases, masks
@@ -184,6 +193,13 @@ struct pc_ctx {
     for (cudaStream_t s : rrstream)
       if (s) cudaStreamDestroy(s);
     if (pinned) cudaFreeHost(pinned);
+    for (Stage &s : stage) {
+      if (s.done) {
+        cudaEventSynchronize(s.done);
+        cudaEventDestroy(s.done);
+      }
+      if (s.p) cudaFreeHost(s.p);
+    }
     for (auto &p : pending) {
       cudaEventDestroy(p.a);
       cudaEventDestroy(p.b);
@@ -208,8 +224,9 @@ int harvest_timing(pc_ctx *ctx);
 // A (row-major) and b = A^{-1} (row-major) from the lattice vectors a_1, a_2, a_3 stored one after the other
 // (lattice[3 n + c] = component c of a_{n+1}); nonzero when the vectors are numerically dependent
 int invert_lattice(const double *lattice, double *amat, double *binv);
-// uploads kparams (and symbol tables) for nb k-points into the context; returns 0 or an error code
-int upload_kpoints(pc_ctx *ctx, int nb, const double *kpts, const double *gammas);
+// uploads kparams (and symbol tables) for nb k-points into the context; returns 0 or an error code. The copies are on
+// ctx->stream; with `wait` they have completed on return (for callers that go on to other streams)
+int upload_kpoints(pc_ctx *ctx, int nb, const double *kpts, const double *gammas, bool wait = true);
 // kernels launched by the solver (all on ctx->stream)
 int launch_apply_op(pc_ctx *ctx, int nb, int m, int dtype, const void *X, long sx, void *Y, long sy,
                     const int *act);

@@ -35,6 +35,7 @@ void set_error(const char *fmt, ...) {
 
 int cuda_fail(cudaError_t e, const char *what, const char *file, int line) {
   set_error("CUDA error %d (%s) in %s at %s:%d", (int)e, cudaGetErrorString(e), what, file, line);
+  (void)cudaGetLastError();  // reported: the next call's launch check starts clean
   return e == cudaErrorMemoryAllocation ? PC_ENOMEM : PC_ECUDA;
 }
 
@@ -42,10 +43,14 @@ int cuda_fail(cudaError_t e, const char *what, const char *file, int line) {
 // matrices by the FFT): d_i(m) = i e^{i th/2} (S_i(m) + k_i Z_i(m)), th = 2 pi m / N, with
 // S_i(m) = (2/h) sum_s c_s sin((s - 1/2) th) and Z_i(m) = 2 sum_s d_s cos((s - 1/2) th); for k = 1 (c_1 = 1,
 // d_1 = 1/2) this is i e^{i th/2} ((2/h) sin(th/2) + k_i cos(th/2))
-static void axis_symbols(int N, int order, double k_i, double2 *out) {
-  const double h = 1.0 / N;
+// The parts that do not depend on k are formed once per context (symbol_tables): S, Z and (-sin(th/2), cos(th/2)).
+static void symbol_tables(pc_ctx *ctx) {
+  const int N = ctx->N, order = ctx->opts.order;
   double c[4], d[4];
   stencil_coefficients(order, c, d);
+  ctx->symS.resize(N);
+  ctx->symZ.resize(N);
+  ctx->symE.resize(2 * N);
   for (int mm = 0; mm < N; ++mm) {
     const double th = 2.0 * M_PI * mm / N;
     double S = 0.0, Z = 0.0;
@@ -53,30 +58,33 @@ static void axis_symbols(int N, int order, double k_i, double2 *out) {
       S += c[q - 1] * std::sin((q - 0.5) * th);
       Z += d[q - 1] * std::cos((q - 0.5) * th);
     }
-    const double mag = (2.0 / h) * S + k_i * (2.0 * Z);
-    // i e^{i th/2} = -sin(th/2) + i cos(th/2)
-    out[mm].x = -std::sin(0.5 * th) * mag;
-    out[mm].y = std::cos(0.5 * th) * mag;
+    ctx->symS[mm] = S;
+    ctx->symZ[mm] = Z;
+    ctx->symE[2 * mm] = -std::sin(0.5 * th);  // i e^{i th/2} = -sin(th/2) + i cos(th/2)
+    ctx->symE[2 * mm + 1] = std::cos(0.5 * th);
+  }
+}
+
+static void axis_symbols(const pc_ctx *ctx, double k_i, double2 *out) {
+  const int N = ctx->N;
+  const double h = 1.0 / N;
+  for (int mm = 0; mm < N; ++mm) {
+    const double mag = (2.0 / h) * ctx->symS[mm] + k_i * (2.0 * ctx->symZ[mm]);
+    out[mm].x = ctx->symE[2 * mm] * mag;
+    out[mm].y = ctx->symE[2 * mm + 1] * mag;
   }
 }
 
 // General lattice (Section 4.2.2): D_hat_i = sum_j b_ji K_j + i L_i has the symbol
 // d_i = sum_j i e^{i th_j/2} (b_ji S(m_j) + [j = i] k_i Z(m_j)), a sum of one table per axis j. This writes the table
 // of axis j for component i: weights wS = b_ji and wZ = k_i (j = i) or 0.
-static void lattice_part_symbols(int N, int order, double wS, double wZ, double2 *out) {
+static void lattice_part_symbols(const pc_ctx *ctx, double wS, double wZ, double2 *out) {
+  const int N = ctx->N;
   const double h = 1.0 / N;
-  double c[4], d[4];
-  stencil_coefficients(order, c, d);
   for (int mm = 0; mm < N; ++mm) {
-    const double th = 2.0 * M_PI * mm / N;
-    double S = 0.0, Z = 0.0;
-    for (int q = 1; q <= order; ++q) {
-      S += c[q - 1] * std::sin((q - 0.5) * th);
-      Z += d[q - 1] * std::cos((q - 0.5) * th);
-    }
-    const double mag = wS * ((2.0 / h) * S) + wZ * (2.0 * Z);
-    out[mm].x = -std::sin(0.5 * th) * mag;
-    out[mm].y = std::cos(0.5 * th) * mag;
+    const double mag = wS * ((2.0 / h) * ctx->symS[mm]) + wZ * (2.0 * ctx->symZ[mm]);
+    out[mm].x = ctx->symE[2 * mm] * mag;
+    out[mm].y = ctx->symE[2 * mm + 1] * mag;
   }
 }
 
@@ -116,7 +124,7 @@ void spurious_mask(const std::vector<int> &redo, int m, int nbands, double tol, 
     }
 }
 
-int upload_kpoints(pc_ctx *ctx, int nb, const double *kpts, const double *gammas) {
+int upload_kpoints(pc_ctx *ctx, int nb, const double *kpts, const double *gammas, bool wait) {
   if (nb <= 0) return PC_OK;
   const int tabs = ctx->lat ? 9 : 3;  // symbol tables per k-point: d_i by axis, or the parts (i, j) of d_i
   if (nb > ctx->kcap) {
@@ -124,8 +132,27 @@ int upload_kpoints(pc_ctx *ctx, int nb, const double *kpts, const double *gammas
     PC_CK(ctx->symd.reserve(sizeof(double2) * tabs * (size_t)ctx->N * nb));
     ctx->kcap = nb;
   }
-  std::vector<KParam> kp(nb);
-  std::vector<double2> sym((size_t)tabs * ctx->N * nb);
+  // Staged in one of two pinned buffers: without `wait` the call returns while the copies are still queued, and the buffer
+  // is filled again once its event says that they are done. (From pageable memory each call waited for the stream: 10
+  // to 20 us between two passes of a step.)
+  pc_ctx::Stage &sg = ctx->stage[ctx->stage_next];
+  ctx->stage_next ^= 1;
+  const size_t symc = (size_t)tabs * ctx->N * nb, need = sizeof(double2) * symc + sizeof(KParam) * nb;
+  // not under stream capture (a replay would copy whatever the staging buffer holds by then): the wait's error, as before
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  PC_CK(cudaStreamIsCapturing(ctx->stream, &cap));
+  if (cap != cudaStreamCaptureStatusNone) PC_CK(cudaStreamSynchronize(ctx->stream));
+  if (!sg.done) PC_CK(cudaEventCreateWithFlags(&sg.done, cudaEventDisableTiming));
+  PC_CK(cudaEventSynchronize(sg.done));
+  if (need > sg.bytes) {
+    if (sg.p) cudaFreeHost(sg.p);
+    sg.p = nullptr;
+    sg.bytes = 0;
+    PC_CK(cudaMallocHost(&sg.p, need));
+    sg.bytes = need;
+  }
+  double2 *const sym = static_cast<double2 *>(sg.p);
+  KParam *const kp = reinterpret_cast<KParam *>(sym + symc);
   for (int b = 0; b < nb; ++b) {
     for (int d = 0; d < 3; ++d) {
       kp[b].k[d] = kpts[3 * b + d];
@@ -139,17 +166,18 @@ int upload_kpoints(pc_ctx *ctx, int nb, const double *kpts, const double *gammas
     kp[b].pfacf = (float)kp[b].pfac;
     if (!ctx->lat) {
       for (int d = 0; d < 3; ++d)
-        axis_symbols(ctx->N, ctx->opts.order, kpts[3 * b + d], &sym[((size_t)b * 3 + d) * ctx->N]);
+        axis_symbols(ctx, kpts[3 * b + d], &sym[((size_t)b * 3 + d) * ctx->N]);
     } else {
       for (int i = 0; i < 3; ++i)
         for (int j = 0; j < 3; ++j)
-          lattice_part_symbols(ctx->N, ctx->opts.order, ctx->binv[3 * j + i], j == i ? kpts[3 * b + i] : 0.0,
+          lattice_part_symbols(ctx, ctx->binv[3 * j + i], j == i ? kpts[3 * b + i] : 0.0,
                                &sym[(((size_t)b * 3 + i) * 3 + j) * ctx->N]);
     }
   }
-  PC_CK(cudaMemcpyAsync(ctx->kparam.p, kp.data(), sizeof(KParam) * nb, cudaMemcpyHostToDevice, ctx->stream));
-  PC_CK(cudaMemcpyAsync(ctx->symd.p, sym.data(), sizeof(double2) * sym.size(), cudaMemcpyHostToDevice, ctx->stream));
-  PC_CK(cudaStreamSynchronize(ctx->stream));  // host staging vectors go out of scope
+  PC_CK(cudaMemcpyAsync(ctx->kparam.p, kp, sizeof(KParam) * nb, cudaMemcpyHostToDevice, ctx->stream));
+  PC_CK(cudaMemcpyAsync(ctx->symd.p, sym, sizeof(double2) * symc, cudaMemcpyHostToDevice, ctx->stream));
+  PC_CK(cudaEventRecord(sg.done, ctx->stream));
+  if (wait) PC_CK(cudaStreamSynchronize(ctx->stream));
   return PC_OK;
 }
 
@@ -273,6 +301,7 @@ extern "C" int pc_setup(pc_ctx **out, int N, const double *eps_edges, const doub
   ctx->lat = general;
   std::memcpy(ctx->amat, amat, sizeof(amat));
   std::memcpy(ctx->binv, binv, sizeof(binv));
+  symbol_tables(ctx);
   std::vector<double> m0(3 * n);
   std::vector<float> m0f(3 * n);
   std::vector<float2> m0p(3 * n);  // double-float pairs of m0

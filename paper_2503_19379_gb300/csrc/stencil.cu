@@ -750,7 +750,7 @@ extern "C" int pc_apply_op(pc_ctx *ctx, int nb, const double *kpts, const double
   PC_REQUIRE(ctx && kpts && gammas && X && Y, "pc_apply_op: null argument");
   PC_REQUIRE(nb >= 0 && m >= 0, "pc_apply_op: negative size");
   PC_REQUIRE(dtype == PC_C128 || dtype == PC_C64 || dtype == PC_C128_DF, "pc_apply_op: bad dtype %d", dtype);
-  int rc = upload_kpoints(ctx, nb, kpts, gammas);
+  int rc = upload_kpoints(ctx, nb, kpts, gammas, false);
   if (rc) return rc;
   const long blk = (long)m * 3 * ctx->n;
   if (dtype == PC_C128_DF) return launch_apply_op_df(ctx, nb, m, X, blk, Y, blk, nullptr);
@@ -762,7 +762,7 @@ extern "C" int pc_apply_half(pc_ctx *ctx, int nb, const double *kpts, int m, con
   PC_REQUIRE(nb >= 0 && m >= 0, "pc_apply_half: negative size");
   if (nb == 0 || m == 0) return PC_OK;
   std::vector<double> g(nb, 1.0);
-  int rc = upload_kpoints(ctx, nb, kpts, g.data());
+  int rc = upload_kpoints(ctx, nb, kpts, g.data(), false);
   if (rc) return rc;
   if (ctx->opts.order > 1 || ctx->lat) return launch_half_k(ctx, nb, m, X, E, C);
   dim3 grid((unsigned)((ctx->n + 255) / 256), m, nb);
@@ -777,7 +777,7 @@ extern "C" int pc_recompute_norms(pc_ctx *ctx, int nb, const double *kpts, int m
   PC_REQUIRE(ctx && kpts && X && out, "pc_recompute_norms: null argument");
   PC_REQUIRE(nb >= 0 && m >= 0 && m <= 64, "pc_recompute_norms: bad size");
   std::vector<double> g(nb, 1.0);
-  int rc = upload_kpoints(ctx, nb, kpts, g.data());
+  int rc = upload_kpoints(ctx, nb, kpts, g.data(), false);
   if (rc) return rc;
   PC_CK(ctx->scratch.reserve(recompute_scratch_bytes(ctx->n, nb, m)));
   return launch_recompute(ctx, nb, m, X, (long)m * 3 * ctx->n, out, nullptr, ctx->scratch.p, ctx->scratch.bytes);
