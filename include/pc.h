@@ -111,9 +111,9 @@ int pc_setup(pc_ctx **out, int N, const double *eps_edges, const double *lattice
  *   evecs:  device [nk][nbands][3][N][N][N] complex128, unit 2-norm, or NULL.
  *   iters:  host [nk] LOBPCG iterations (summed over gamma doublings), or NULL.
  *   resid:  host [nk][nbands] final relative residuals, or NULL.
- * All k-points are solved together (batched kernels). Returns PC_NOT_CONVERGED if some k-point hit maxiter and
- * PC_SPURIOUS if Algorithm 4.1 still saw a spurious eigenvalue after max_doublings (results are filled in both
- * cases). With PC_PREC_MIXED, a k-point whose FP64-accurate phase stops converging or reaches maxiter is solved
+ * All k-points are solved together (batched kernels). Returns PC_NOT_CONVERGED if some k-point had not converged after
+ * maxiter iterations and PC_SPURIOUS if Algorithm 4.1 still saw a spurious eigenvalue after max_doublings (results
+ * are filled in both cases). With PC_PREC_MIXED, a k-point whose FP64-accurate phase stops converging or reaches maxiter is solved
  * again by the FP64 solve, started from its current block (pc_get_fp64_finish tells which; its iteration count is
  * the sum of both). Synchronises the context stream before returning. */
 int pc_solve(pc_ctx *ctx, int nk, const double *kpts, int nbands, double tol, double *evals, void *evecs,

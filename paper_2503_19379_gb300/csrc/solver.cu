@@ -638,12 +638,14 @@ extern "C" int pc_solve(pc_ctx *ctx, int nk, const double *kpts, int nbands, dou
       }
     }
     std::vector<int> conv;
+    std::vector<char> missed(nb, 0);  // out of iterations before the tolerance (converging in the last one counts)
     for (int b : act) {
       bool ok = true;
       for (int j = 0; j < nbands; ++j) {
         const double r = h_norms[((size_t)b * m + j) * 2], x = h_norms[((size_t)b * m + j) * 2 + 1];
         if (!(r <= tol * std::fabs(h_theta[(size_t)b * m + j]) * x)) ok = false;
       }
+      missed[b] = !ok;
       if (ok || it - round_start[b] >= maxiter) conv.push_back(b);
     }
     // Algorithm 4.1 on the k-points that just converged
@@ -667,7 +669,7 @@ extern "C" int pc_solve(pc_ctx *ctx, int nk, const double *kpts, int nbands, dou
           redo.push_back(b);
         } else {
           if (spurious) status = std::max(status, PC_SPURIOUS);
-          if (capped) status = std::max(status, PC_NOT_CONVERGED);
+          if (missed[b]) status = std::max(status, PC_NOT_CONVERGED);
           fin.push_back(b);
         }
       }

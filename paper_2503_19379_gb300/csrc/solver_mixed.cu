@@ -308,7 +308,6 @@ class MixedSolve {
           redo.push_back(b);
         } else {
           if (spurious) S.status = std::max(S.status, (int)PC_SPURIOUS);
-          if (capped) S.status = std::max(S.status, (int)PC_NOT_CONVERGED);
           fin.push_back(b);
         }
       }
