@@ -4,18 +4,24 @@
 //   2. along z, all three components of U consecutive (x, y) columns: forward transform, the exact inverse of the
 //      mode's 3x3 symbol sigma I + (gamma - 1) conj(d) d^T times 1/N^3, inverse transform;
 //   3. inverse transforms along y and x of each plane.
-// Every line transform of length N = N1 N2 (N1 <= N2 <= 16, both powers of two) is split in two (Cooley-Tukey with
-// n = n1 + N1 n2, k = k2 + N2 k1): N1 threads each take one DFT of length N2 over the stride-N1 elements of the
-// line in registers, multiply by the twiddles W_N^(n1 k2), exchange through shared memory, and take N2/N1 DFTs of
-// length N1. Inputs and outputs are in natural order, so the symbol is applied at the natural mode indices. The
-// small DFTs are radix-2 decimation in time on registers with the constant roots of unity of order 16.
+// A line transform of length N = N1 N2 (N2 = N up to 16, 8 at N = 32, 16 above) is a DFT of length N2 and one of length N1 (Cooley-Tukey) with
+// the twiddles W_N between them; a thread holds N2 elements in registers. The small DFTs are radix-2 decimation in time on
+// registers with the constant roots of unity of order 16. Inputs and outputs are in natural order, so the symbol is
+// applied at the natural mode indices.
 //
-// Shared-memory layouts are chosen so that every warp access touches each bank pair at most twice (two wavefronts
-// for 32 eight-byte accesses, the minimum): the x pass of the plane kernel runs with consecutive threads on the
-// N1 pieces of a line (coalesced global loads of N1 consecutive elements per row), its exchange rows padded to
-// N + N1 entries with the pieces at stride N2 + 1; the y pass runs with consecutive threads on consecutive columns
-// (conflict-free row segments in shared memory and coalesced 256-byte stores to global memory); the z pass has
-// consecutive threads on consecutive columns as well.
+// What bounds the passes besides HBM is the trips through shared memory and the barriers around them, so the steps are
+// ordered for few of both. Plane pass: the first axis' length-N2 DFTs; the length-N1 DFTs of both axes on an N1 x N1 block
+// of a thread (N = 128: one axis after the other); the second axis' length-N2 DFTs, two exchanges in all. z pass: the
+// length-N2 DFTs; then a thread takes the N1 modes of one residue and all three components through the length-N1 DFTs,
+// the symbol and the inverse DFTs back; the inverse length-N2 DFTs. The middle steps write where they read, so
+// one buffer serves and a step needs one barrier. 76 fields of N = 64: 0.71 ms with the axes one after the other, an
+// exchange and a transposition each, N1 <= N2 split nearly even and the modes gathered once more for the symbol; 0.54 ms
+// so (5.2 TB/s over the three passes). 256 fields of N = 32: 315 and 250 us; 20 of N = 128: 1.72 and 1.54 ms. Passes over
+// blocks of fields that would stay in L2 were slower at every block size (0.61 to 0.95 ms): the launches get too small.
+//
+// Shared-memory layouts: every half warp touches each bank pair once. In a plane, the N1 pieces of a row are N2 + 1 apart,
+// which makes the row stride N1 (mod N2); loads and stores of rows are N1 consecutive elements per thread group (32 bytes
+// at N = 64), those of columns are consecutive threads on consecutive columns, as in the z pass.
 #include <cmath>
 
 #include "pc_internal.cuh"
@@ -88,25 +94,22 @@ template <bool INV> __device__ __forceinline__ float2 twmul(float2 x, float2 w) 
              : make_float2(x.x * w.x - x.y * w.y, x.x * w.y + x.y * w.x);
 }
 
-// Split of a length-N transform: N1 <= N2 <= 16.
+// Split of a length-N transform.
 template <int N> struct Split {
-  static constexpr int N1 = N <= 8 ? 2 : (N <= 32 ? 4 : (N <= 128 ? 8 : 16));
-  static constexpr int N2 = N / N1;
-  static_assert(N1 * N2 == N && N1 <= N2 && N2 <= 16, "unsupported length");
+  static constexpr int N2 = N < 16 ? N : (N == 32 ? 8 : 16);  // (32 = 2 x 16: 262 us for 256 fields; 4 x 8: 250)
+  static constexpr int N1 = N / N2;
+  static_assert(N1 * N2 == N && N1 <= 8, "unsupported length");
 };
 
-// planes per CTA (about 512 threads; P divides the 3N planes of a field) and whether the plane kernel's exchange
-// shares the plane buffer (for N = 128 two N x (N + N1) buffers would not fit in shared memory)
+// planes per CTA (at least 128 threads where the planes of a component allow it; P divides the 3 N planes of a field)
 template <int N> struct PlaneCfg {
-  static constexpr int N1 = Split<N>::N1;
-  static constexpr int P0 = (N * N1 >= 512) ? 1 : 512 / (N * N1);
+  static constexpr int N1 = Split<N>::N1, N2 = Split<N>::N2;
+  static constexpr int P0 = (N * N1 >= 128) ? 1 : 128 / (N * N1);
   static constexpr int P = P0 < N ? P0 : N;
-  static constexpr int LD = N + N1;  // row stride (elements) of the plane and exchange buffers
-  static constexpr bool SINGLE = N >= 128;
+  static constexpr int PN = N2 + 1;   // stride of the N1 pieces of a row
+  static constexpr int LD = N1 * PN;  // row stride of the plane
   static constexpr int THREADS = P * N * N1;
-  static constexpr size_t smem() {
-    return sizeof(float2) * ((size_t)(SINGLE ? 1 : 2) * P * N * LD + N);
-  }
+  static constexpr size_t smem() { return sizeof(float2) * ((size_t)P * N * LD + N); }
 };
 
 // twiddle table W_N^t = exp(-2 pi i t / N), t < N, from the context's table of the first N / 2
@@ -125,134 +128,128 @@ __global__ void __launch_bounds__(PlaneCfg<N>::THREADS) fft_plane_kernel(const f
                                                                          const float2 *__restrict__ tw,
                                                                          const int *__restrict__ act) {
   using CF = PlaneCfg<N>;
-  constexpr int N1 = Split<N>::N1, N2 = Split<N>::N2, P = CF::P, LD = CF::LD, Q = N2 / N1;
+  constexpr int N1 = CF::N1, N2 = CF::N2, P = CF::P, LD = CF::LD, PN = CF::PN, T = CF::THREADS;
   constexpr bool INV = !FWD;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2 *s_tw = reinterpret_cast<float2 *>(smem_raw);
-  float2 *A = s_tw + N;                                  // planes [P N rows][LD]
-  float2 *E = CF::SINGLE ? A : A + (size_t)P * N * LD;   // exchange [P N rows][LD]
+  float2 *A = s_tw + N;  // planes [P N rows][N1 pieces, PN apart][N2]
   const long n = (long)N * N * N;
   const int b = act ? act[blockIdx.z] : (int)blockIdx.z;
   const long off = (long)blockIdx.y * 3 * n + (long)blockIdx.x * P * N * N;
   const float2 *src = in + (long)b * si + off;
   float2 *dst = out + (long)b * so + off;
   load_twiddles(s_tw, tw, N);
+  const int tid = threadIdx.x;
+  // a thread's share of the outer steps: of a row (plane, y) the elements n1 + N1 j, or of a column the rows m1 + N1 j
+  const int n1 = tid % N1, row = tid / N1;
+  const int x = tid % N, m1 = tid / N % N1, pl = tid / (N * N1);
+  const int xs = x / N2 * PN + x % N2;  // the column's place in a row
   float2 v[N2];
 
-  // ---- first pass: along x (forward) or y (inverse) on lines owned by N1 consecutive threads
-  // forward: line = row (plane, y), loads of the row's elements x = n1 + N1 n2 straight from global memory
-  // inverse: line = column (plane, x): consecutive threads on consecutive columns
-  const int tid = threadIdx.x;
-  if (FWD) {
-    const int n1 = tid % N1, row = tid / N1;
+  // ---- the first axis' DFTs of length N2 over its elements n1 + N1 j; result k2 of piece n1 to n1 N2 + k2
 #pragma unroll
-    for (int j = 0; j < N2; ++j) v[j] = src[(long)row * N + n1 + N1 * j];
-    __syncthreads();  // twiddle table
-    dft<N2, INV>(v);
+  for (int j = 0; j < N2; ++j) v[j] = FWD ? src[row * N + n1 + N1 * j] : src[(pl * N + m1 + N1 * j) * N + x];
+  __syncthreads();  // twiddle table
+  dft<N2, INV>(v);
 #pragma unroll
-    for (int j = 1; j < N2; ++j) v[j] = twmul<INV>(v[j], s_tw[n1 * j]);
+  for (int j = 1; j < N2; ++j)
+    if (N1 > 1) v[j] = twmul<INV>(v[j], s_tw[(FWD ? n1 : m1) * j]);
 #pragma unroll
-    for (int j = 0; j < N2; ++j) E[row * LD + n1 * (N2 + 1) + j] = v[j];
-    __syncthreads();
-    const int t = n1;
-    float2 u[N2];
-#pragma unroll
-    for (int q = 0; q < Q; ++q)
-#pragma unroll
-      for (int a = 0; a < N1; ++a) u[q * N1 + a] = E[row * LD + a * (N2 + 1) + t + N1 * q];
-#pragma unroll
-    for (int q = 0; q < Q; ++q) dft<N1, INV>(u + q * N1);
-    if (CF::SINGLE) __syncthreads();  // E is A: every exchange read done before the plane is written
-#pragma unroll
-    for (int q = 0; q < Q; ++q)
-#pragma unroll
-      for (int a = 0; a < N1; ++a) A[row * LD + t + N1 * q + N2 * a] = u[q * N1 + a];
-  } else {
-    const int x = tid % N, r = tid / N, p = r % P, m1 = r / P;
-#pragma unroll
-    for (int j = 0; j < N2; ++j) v[j] = src[(long)p * N * N + (long)(m1 + N1 * j) * N + x];
-    __syncthreads();
-    dft<N2, INV>(v);
-#pragma unroll
-    for (int j = 1; j < N2; ++j) v[j] = twmul<INV>(v[j], s_tw[m1 * j]);
-#pragma unroll
-    for (int j = 0; j < N2; ++j) E[(p * N + m1 * N2 + j) * LD + x] = v[j];
-    __syncthreads();
-    float2 u[N2];
-#pragma unroll
-    for (int q = 0; q < Q; ++q)
-#pragma unroll
-      for (int a = 0; a < N1; ++a) u[q * N1 + a] = E[(p * N + a * N2 + m1 + N1 * q) * LD + x];
-#pragma unroll
-    for (int q = 0; q < Q; ++q) dft<N1, INV>(u + q * N1);
-    if (CF::SINGLE) __syncthreads();
-#pragma unroll
-    for (int q = 0; q < Q; ++q)
-#pragma unroll
-      for (int a = 0; a < N1; ++a) A[(p * N + m1 + N1 * q + N2 * a) * LD + x] = u[q * N1 + a];
-  }
+  for (int j = 0; j < N2; ++j) A[FWD ? row * LD + n1 * PN + j : (pl * N + m1 * N2 + j) * LD + xs] = v[j];
   __syncthreads();
 
-  // ---- second pass: along y (forward) or x (inverse)
-  if (FWD) {
-    // line = column (plane, x), consecutive threads on consecutive columns; results stored straight to global memory
-    const int x = tid % N, r = tid / N, p = r % P, m1 = r / P;
+  // ---- DFTs of length N1 of both axes, in place. Stride N2 on both: the second axis' elements r + N2 i, result k1 of
+  // residue r times W_N^(r k1)
+  if constexpr (N1 > 1 && N1 <= 4) {
+    for (int i = tid; i < P * N2 * N2; i += T) {
+      const int ix = i % N2, iy = i / N2 % N2, rr = FWD ? iy : ix;
+      float2 *B = A + (i / (N2 * N2) * N + iy) * LD + ix;
+      float2 w[N1][N1];  // [y][x]
 #pragma unroll
-    for (int j = 0; j < N2; ++j) v[j] = A[(p * N + m1 + N1 * j) * LD + x];
-    dft<N2, INV>(v);
+      for (int e = 0; e < N1; ++e)
 #pragma unroll
-    for (int j = 1; j < N2; ++j) v[j] = twmul<INV>(v[j], s_tw[m1 * j]);
-    if (CF::SINGLE) __syncthreads();
+        for (int c = 0; c < N1; ++c) w[e][c] = B[e * N2 * LD + c * PN];
 #pragma unroll
-    for (int j = 0; j < N2; ++j) E[(p * N + m1 * N2 + j) * LD + x] = v[j];
+      for (int axis = 0; axis < 2; ++axis) {  // the first axis, then the second
+        if ((axis == 0) == FWD) {
+#pragma unroll
+          for (int e = 0; e < N1; ++e) dft<N1, INV>(w[e]);
+        } else {
+#pragma unroll
+          for (int c = 0; c < N1; ++c) {
+            float2 q[N1];
+#pragma unroll
+            for (int e = 0; e < N1; ++e) q[e] = w[e][c];
+            dft<N1, INV>(q);
+#pragma unroll
+            for (int e = 0; e < N1; ++e) w[e][c] = q[e];
+          }
+        }
+      }
+#pragma unroll
+      for (int k = 1; k < N1; ++k) {
+        const float2 t = s_tw[rr * k];
+#pragma unroll
+        for (int c = 0; c < N1; ++c) {
+          float2 &z = FWD ? w[k][c] : w[c][k];
+          z = twmul<INV>(z, t);
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < N1; ++e)
+#pragma unroll
+        for (int c = 0; c < N1; ++c) B[e * N2 * LD + c * PN] = w[e][c];
+    }
     __syncthreads();
-    float2 u[N2];
+  } else if constexpr (N1 > 4) {
+    // one axis after the other: rows then columns (forward), columns then rows (inverse)
 #pragma unroll
-    for (int q = 0; q < Q; ++q)
+    for (int s = 0; s < 2; ++s) {
+      const bool rows = FWD == (s == 0);
+      for (int i = tid; i < P * N * N2; i += T) {
+        // rows: (row, ix) of the row's pieces; columns: (plane, iy, x)
+        const int r = rows ? i % N2 : i / N % N2;
+        float2 *B = rows ? A + i / N2 * LD + r
+                         : A + (i / (N * N2) * N + r) * LD + i % N / N2 * PN + i % N % N2;
+        const int st = rows ? PN : N2 * LD;
+        float2 w[N1];
 #pragma unroll
-      for (int a = 0; a < N1; ++a) u[q * N1 + a] = E[(p * N + a * N2 + m1 + N1 * q) * LD + x];
+        for (int e = 0; e < N1; ++e) w[e] = B[e * st];
+        dft<N1, INV>(w);
+        if (s == 1) {
 #pragma unroll
-    for (int q = 0; q < Q; ++q) dft<N1, INV>(u + q * N1);
+          for (int k = 1; k < N1; ++k) w[k] = twmul<INV>(w[k], s_tw[r * k]);
+        }
 #pragma unroll
-    for (int q = 0; q < Q; ++q)
+        for (int e = 0; e < N1; ++e) B[e * st] = w[e];
+      }
+      __syncthreads();
+    }
+  }
+
+  // ---- the second axis' DFTs of length N2 over the residues of k1 = n1 (m1): outputs k1 + N1 k2
 #pragma unroll
-      for (int a = 0; a < N1; ++a) dst[(long)p * N * N + (long)(m1 + N1 * q + N2 * a) * N + x] = u[q * N1 + a];
-  } else {
-    // line = row (plane, y), the N1 pieces on consecutive threads; stores of N1 consecutive elements per row
-    const int n1 = tid % N1, row = tid / N1;
+  for (int j = 0; j < N2; ++j) v[j] = A[FWD ? (pl * N + m1 * N2 + j) * LD + xs : row * LD + n1 * PN + j];
+  dft<N2, INV>(v);
 #pragma unroll
-    for (int j = 0; j < N2; ++j) v[j] = A[row * LD + n1 + N1 * j];
-    dft<N2, INV>(v);
-#pragma unroll
-    for (int j = 1; j < N2; ++j) v[j] = twmul<INV>(v[j], s_tw[n1 * j]);
-    if (CF::SINGLE) __syncthreads();
-#pragma unroll
-    for (int j = 0; j < N2; ++j) E[row * LD + n1 * (N2 + 1) + j] = v[j];
-    __syncthreads();
-    const int t = n1;
-    float2 u[N2];
-#pragma unroll
-    for (int q = 0; q < Q; ++q)
-#pragma unroll
-      for (int a = 0; a < N1; ++a) u[q * N1 + a] = E[row * LD + a * (N2 + 1) + t + N1 * q];
-#pragma unroll
-    for (int q = 0; q < Q; ++q) dft<N1, INV>(u + q * N1);
-#pragma unroll
-    for (int q = 0; q < Q; ++q)
-#pragma unroll
-      for (int a = 0; a < N1; ++a) dst[(long)row * N + t + N1 * q + N2 * a] = u[q * N1 + a];
+  for (int j = 0; j < N2; ++j) {
+    if (FWD)
+      dst[(pl * N + m1 + N1 * j) * N + x] = v[j];
+    else
+      dst[row * N + n1 + N1 * j] = v[j];
   }
 }
 
-// columns per CTA of the z pass: about 384 threads (3 U N1), U <= N^2
+// columns per CTA of the z pass, and threads: one per task of the outer steps (3 N1 U), or a third of that where the
+// middle step's N2 U tasks would leave more of them idle (N = 32, 128). The other choice: 271 against 250 us for 256
+// fields of N = 32, 585 against 545 us for 76 of N = 64, 1.60 against 1.53 ms for 20 of N = 128
 template <int N> struct ZCfg {
   static constexpr int N1 = Split<N>::N1;
-  static constexpr int U0 = 512 / (3 * N1) >= 64 ? 64 : (512 / (3 * N1) >= 32 ? 32 : 16);
-  static constexpr int U = U0 <= N * N ? U0 : N * N;
-  static constexpr int THREADS = 3 * U * N1;
+  static constexpr int U = N == 64 ? 16 : 32;
+  static constexpr int THREADS = U * N1 * (3 * N1 <= Split<N>::N2 ? 3 : 1);
   static constexpr size_t smem() {
-    // exchange [3][N][U], modes [3][N][U], twiddles N, symbols: x/y parts [U][3][2] and z part [3][N]
-    return sizeof(float2) * (2 * (size_t)3 * N * U + N + 6 * (size_t)U + 3 * (size_t)N);
+    // elements [3][N][U], twiddles N, symbols: x/y parts [3][U] and z part [3][N]
+    return sizeof(float2) * ((size_t)3 * N * U + N + 3 * (size_t)U + 3 * (size_t)N);
   }
 };
 
@@ -267,12 +264,11 @@ __global__ void __launch_bounds__(ZCfg<N>::THREADS) fft_zsym_kernel(const float2
                                                                     const KParam *__restrict__ kp,
                                                                     const int *__restrict__ act, int laplacian) {
   using CF = ZCfg<N>;
-  constexpr int N1 = Split<N>::N1, N2 = Split<N>::N2, U = CF::U, Q = N2 / N1;
+  constexpr int N1 = Split<N>::N1, N2 = Split<N>::N2, U = CF::U, T = CF::THREADS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2 *E = reinterpret_cast<float2 *>(smem_raw);  // [3][N][U]
-  float2 *S = E + 3 * N * U;                         // [3][N][U]
-  float2 *s_tw = S + 3 * N * U;                      // [N]
-  float2 *dxy = s_tw + N;                            // [U][3]: x and y parts of d_i at each column
+  float2 *s_tw = E + 3 * N * U;                      // [N]
+  float2 *dxy = s_tw + N;                            // [3][U]: x and y parts of d_i at each column
   float2 *dz = dxy + 3 * U;                          // [3][N]: z part of d_i (on the cube: d_3 itself)
   const long n = (long)N * N * N;
   const int b = act ? act[blockIdx.z] : (int)blockIdx.z;
@@ -296,7 +292,7 @@ __global__ void __launch_bounds__(ZCfg<N>::THREADS) fft_zsym_kernel(const float2
         re = d.x;
         im = d.y;
       }
-      dxy[u * 3 + c] = make_float2((float)re, (float)im);
+      dxy[c * U + u] = make_float2((float)re, (float)im);
     }
     for (int i = threadIdx.x; i < 3 * N; i += blockDim.x) {
       const int c = i / N, zz = i % N;
@@ -304,88 +300,84 @@ __global__ void __launch_bounds__(ZCfg<N>::THREADS) fft_zsym_kernel(const float2
       dz[i] = make_float2((float)d.x, (float)d.y);
     }
   }
-  const int tid = threadIdx.x;
-  const int u = tid % U, r = tid / U, n1 = r % N1, c = r / N1;
-  float2 v[N2];
+  const int tid = threadIdx.x, u = tid % U;  // (U divides T: a thread stays on its column)
+  // forward along z, the DFTs of length N2 over z = n1 + N1 j: result k2 to n1 N2 + k2
+  constexpr int R1 = 3 * N1 * U / T;
 #pragma unroll
-  for (int j = 0; j < N2; ++j) v[j] = in[base_i + (long)c * n + (long)(n1 + N1 * j) * N * N + u];
-  __syncthreads();  // twiddles and symbols
-  // forward along z
-  dft<N2, false>(v);
+  for (int it = 0; it < R1; ++it) {
+    const int r = (tid + it * T) / U, n1 = r % N1, c = r / N1;
+    float2 v[N2];
 #pragma unroll
-  for (int j = 1; j < N2; ++j) v[j] = twmul<false>(v[j], s_tw[n1 * j]);
+    for (int j = 0; j < N2; ++j) v[j] = in[base_i + (long)c * n + (n1 + N1 * j) * N * N + u];
+    if (it == 0) __syncthreads();  // twiddles and symbols
+    dft<N2, false>(v);
 #pragma unroll
-  for (int j = 0; j < N2; ++j) E[(c * N + n1 * N2 + j) * U + u] = v[j];
+    for (int j = 1; j < N2; ++j)
+      if (N1 > 1) v[j] = twmul<false>(v[j], s_tw[n1 * j]);
+#pragma unroll
+    for (int j = 0; j < N2; ++j) E[(c * N + n1 * N2 + j) * U + u] = v[j];
+  }
   __syncthreads();
-  const int t = n1;
-  float2 w[N2];
-#pragma unroll
-  for (int q = 0; q < Q; ++q)
-#pragma unroll
-    for (int a = 0; a < N1; ++a) w[q * N1 + a] = E[(c * N + a * N2 + t + N1 * q) * U + u];
-#pragma unroll
-  for (int q = 0; q < Q; ++q) dft<N1, false>(w + q * N1);
-  // mode kz = k2 + N2 k1 with k2 = t + N1 q: all three components into S
-#pragma unroll
-  for (int q = 0; q < Q; ++q)
-#pragma unroll
-    for (int a = 0; a < N1; ++a) S[(c * N + t + N1 * q + N2 * a) * U + u] = w[q * N1 + a];
-  __syncthreads();
-  // the symbol's inverse, one mode (all three components) per thread and step: consecutive threads on consecutive
-  // columns, each mode's sigma, reciprocal and d^T r formed once
+  // the modes kz = k2 + N2 k1 of residue k2: DFTs of length N1, the symbol's inverse on all three components, the DFTs back
+  // and their twiddles
   {
     const float fac = kp[b].pfacf;  // (gamma - 1) / gamma
     const float scale = 1.0f / (float)n;
-    for (int i = tid; i < U * N; i += CF::THREADS) {
-      const int uu = i % U, kz = i / U;
-      const float2 d1 = cadd(dxy[uu * 3 + 0], dz[kz]), d2 = cadd(dxy[uu * 3 + 1], dz[N + kz]);
-      const float2 d3 = cadd(dxy[uu * 3 + 2], dz[2 * N + kz]);
-      const float sigma = d1.x * d1.x + d1.y * d1.y + d2.x * d2.x + d2.y * d2.y + d3.x * d3.x + d3.y * d3.y;
-      float2 *m = S + kz * U + uu;
-      float2 r1 = m[0], r2 = m[N * U], r3 = m[2 * N * U];
-      if (!(sigma > 0.f)) {
-        r1 = r2 = r3 = make_float2(0.f, 0.f);
-      } else {
-        const float rs = __frcp_rn(sigma);
-        if (!laplacian) {
-          // r_c - (gamma - 1) / (gamma sigma) conj(d_c) (d^T r)
-          const float2 sd = cscale(cadd(cadd(cmul(d1, r1), cmul(d2, r2)), cmul(d3, r3)), fac * rs);
-          r1 = csub(r1, cmulc(d1, sd));
-          r2 = csub(r2, cmulc(d2, sd));
-          r3 = csub(r3, cmulc(d3, sd));
-        }
-        const float f = scale * rs;
-        r1 = cscale(r1, f);
-        r2 = cscale(r2, f);
-        r3 = cscale(r3, f);
+    const float2 e1 = dxy[u], e2 = dxy[U + u], e3 = dxy[2 * U + u];
+    for (int k2 = tid / U; k2 < N2; k2 += T / U) {
+      float2 *B = E + k2 * U + u;
+      float2 w[3][N1];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+#pragma unroll
+        for (int a = 0; a < N1; ++a) w[c][a] = B[(c * N + a * N2) * U];
+        dft<N1, false>(w[c]);
       }
-      m[0] = r1;
-      m[N * U] = r2;
-      m[2 * N * U] = r3;
+#pragma unroll
+      for (int a = 0; a < N1; ++a) {
+        const int kz = k2 + N2 * a;
+        const float2 d1 = LAT ? cadd(e1, dz[kz]) : e1, d2 = LAT ? cadd(e2, dz[N + kz]) : e2;
+        const float2 d3 = LAT ? cadd(e3, dz[2 * N + kz]) : dz[2 * N + kz];
+        const float sigma = d1.x * d1.x + d1.y * d1.y + d2.x * d2.x + d2.y * d2.y + d3.x * d3.x + d3.y * d3.y;
+        float2 &r1 = w[0][a], &r2 = w[1][a], &r3 = w[2][a];
+        if (!(sigma > 0.f)) {
+          r1 = r2 = r3 = make_float2(0.f, 0.f);
+        } else {
+          const float rs = __frcp_rn(sigma);
+          if (!laplacian) {
+            // r_c - (gamma - 1) / (gamma sigma) conj(d_c) (d^T r)
+            const float2 sd = cscale(cadd(cadd(cmul(d1, r1), cmul(d2, r2)), cmul(d3, r3)), fac * rs);
+            r1 = csub(r1, cmulc(d1, sd));
+            r2 = csub(r2, cmulc(d2, sd));
+            r3 = csub(r3, cmulc(d3, sd));
+          }
+          const float f = scale * rs;
+          r1 = cscale(r1, f);
+          r2 = cscale(r2, f);
+          r3 = cscale(r3, f);
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        dft<N1, true>(w[c]);
+#pragma unroll
+        for (int a = 0; a < N1; ++a)
+          B[(c * N + a * N2) * U] = a == 0 ? w[c][a] : twmul<true>(w[c][a], s_tw[a * k2]);
+      }
     }
   }
   __syncthreads();
+  // inverse along z: the DFTs of length N2 over k2, outputs z = n1 + N1 j
 #pragma unroll
-  for (int q = 0; q < Q; ++q)
+  for (int it = 0; it < R1; ++it) {
+    const int r = (tid + it * T) / U, n1 = r % N1, c = r / N1;
+    float2 v[N2];
 #pragma unroll
-    for (int a = 0; a < N1; ++a) w[q * N1 + a] = S[(c * N + t + N1 * q + N2 * a) * U + u];
-  // inverse along z: the length-N1 DFTs first (over k1), twiddles, exchange, the length-N2 DFTs (over k2)
+    for (int j = 0; j < N2; ++j) v[j] = E[(c * N + n1 * N2 + j) * U + u];
+    dft<N2, true>(v);
 #pragma unroll
-  for (int q = 0; q < Q; ++q) dft<N1, true>(w + q * N1);
-#pragma unroll
-  for (int q = 0; q < Q; ++q)
-#pragma unroll
-    for (int a = 0; a < N1; ++a) {
-      const int k2 = t + N1 * q;  // w[q N1 + a] now holds Z[n1 = a][k2]
-      const float2 z = k2 == 0 || a == 0 ? w[q * N1 + a] : twmul<true>(w[q * N1 + a], s_tw[a * k2]);
-      E[(c * N + a * N2 + k2) * U + u] = z;  // E was last read before the previous barrier
-    }
-  __syncthreads();
-#pragma unroll
-  for (int j = 0; j < N2; ++j) v[j] = E[(c * N + n1 * N2 + j) * U + u];
-  dft<N2, true>(v);
-#pragma unroll
-  for (int j = 0; j < N2; ++j) out[base_o + (long)c * n + (long)(n1 + N1 * j) * N * N + u] = v[j];
+    for (int j = 0; j < N2; ++j) out[base_o + (long)c * n + (n1 + N1 * j) * N * N + u] = v[j];
+  }
 }
 
 template <int N>
