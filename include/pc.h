@@ -144,7 +144,7 @@ const char *pc_last_error(void);
 #define PC_STAGE_STENCIL 0   /* a1: Op X (fused stencil) */
 #define PC_STAGE_PRECOND 1   /* a2: FFT preconditioner (5 kernels per call) */
 #define PC_STAGE_GRAM 2      /* a3: Gram products S^H S, S^H AS */
-#define PC_STAGE_RR 3        /* a4: Rayleigh-Ritz (small dense, one block per k-point) */
+#define PC_STAGE_RR 3        /* a4: Rayleigh-Ritz (small dense, a cluster of up to 4 blocks per k-point) */
 #define PC_STAGE_UPDATE 4    /* a5: block updates S C */
 #define PC_STAGE_RESIDUAL 5  /* a5: residual and column norms */
 #define PC_STAGE_RECOMPUTE 6 /* a6: Algorithm 4.1 norms */
@@ -233,16 +233,18 @@ int pc_apply_precond(pc_ctx *ctx, int nb, const double *kpts, const double *gamm
                      const void *R, void *W);
 
 /* a3: G_b = A_b^H B_b for tall-skinny blocks (L rows; p and q columns, column stride L; batch strides sa, sb in
- * elements). G: device complex128 [nb][p][q] row-major. p, q <= 64. dtype applies to A and B. PC_C128: FP64
- * products and sums. PC_C64: FP32 products and partial sums over chunks of the rows, chunks added in FP64; where L
- * is a multiple of 16 and the panels are 16-byte aligned this runs on the tensor cores (TF32 operands split into
- * hi + lo, accumulators drained every 64 rows), otherwise on the CUDA cores. */
+ * elements). G: device complex128 [nb][p][q] row-major. p, q <= 64. dtype applies to A and B. PC_C128: exact products
+ * of the values rounded to 54 bits below the largest of a column's 1024 rows, on the tensor cores (FP16 digits, integer
+ * sums), with FP64 sums over the spans of rows: at most the error of FP64 products and sums. Columns with an infinity
+ * or a NaN take plain FP64. PC_C64: FP32 products and partial sums over chunks of the rows, chunks added in FP64; where
+ * p or q is above 16, L is a multiple of 16 and the panels are 16-byte aligned this runs on the tensor cores (TF32
+ * operands split into hi + lo, accumulators drained every 64 rows), otherwise on the CUDA cores. */
 int pc_gram(int nb, long L, int p, int q, int dtype, const void *A, long sa, const void *B, long sb, void *G,
             void *stream);
 
 /* a3: the Rayleigh-Ritz pencil of one panel: G_b = S_b^H S_b and H_b = S_b^H AS_b, with S_b and AS_b of p columns
  * (length L, column stride L, the same batch stride ss for both). Op is Hermitian, so both outputs are Hermitian:
- * only the upper triangle is accumulated (FP64) and the lower triangle is its conjugate mirror. G, H: device
+ * only the upper triangle is accumulated and the lower triangle is its conjugate mirror. G, H: device
  * complex128 [nb][p][p]. p <= 64; dtype applies to S and AS, with the accumulation of pc_gram for that dtype. */
 int pc_gram_pair(int nb, long L, int p, int dtype, const void *S, long ss, const void *AS, void *G, void *H,
                  void *stream);
@@ -263,9 +265,9 @@ int pc_gram_pair_coupled(int nb, long L, int p, int q, const void *S, long ss, c
  * This entry point has no counterpart in the paper; it is an interface convenience.
  *   Limit: 2 * 16 * nb * p * p <= 4 MiB, i.e. nb * p * p <= 131072 (for example 32 k-points of 64 columns);
  *   larger requests return PC_EINVAL with a message. Arguments and layout are those of pc_gram_pair. Results agree
- *   with pc_gram_pair within rounding, but not bit for bit: complex64 panels are always summed on the CUDA cores
- *   (FP32 products and partial sums over row chunks, chunks added in FP64), never on the tensor-core path that
- *   pc_gram_pair takes for them. The call is asynchronous: it returns once the work is enqueued on `stream`
+ *   with pc_gram_pair within rounding, but not bit for bit: panels are always summed on the CUDA cores (complex64:
+ *   FP32 products and partial sums over row chunks, chunks added in FP64; complex128: FP64), never on the tensor-core
+ *   paths that pc_gram_pair takes for them. The call is asynchronous: it returns once the work is enqueued on `stream`
  *   (pc_gram_pair waits for its stream), so G and H are valid only after the caller synchronises with `stream`.
  *   The first call on each device looks up the array's device address (cudaGetSymbolAddress) with that device
  *   current; make that first call before any stream capture. Every call reuses the same array and only reads
@@ -275,7 +277,9 @@ int pc_gram_pair_noalloc(int nb, long L, int p, int dtype, const void *S, long s
                          void *stream);
 
 /* a5: Y_b = S_b C_b: S_b has p columns of length L (batch stride ss), C_b device complex128 [p][q] row-major
- * (batch stride p*q), Y_b has q columns (batch stride sy). p <= 64, q <= 64. dtype applies to S and Y. */
+ * (batch stride p*q), Y_b has q columns (batch stride sy). p <= 64, q <= 64. dtype applies to S and Y. PC_C128: exact
+ * products on the tensor cores (FP16 digits against one exponent per row of S and column of C, integer sums, one
+ * rounding); rows with an infinity or a NaN take plain FP64. PC_C64: FP32. */
 int pc_block_update(int nb, long L, int p, int q, int dtype, const void *S, long ss, const void *C, void *Y,
                     long sy, void *stream);
 

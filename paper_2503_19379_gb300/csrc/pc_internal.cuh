@@ -161,6 +161,16 @@ struct pc_ctx {
     void *p = nullptr;
     size_t bytes = 0;
     cudaEvent_t done = nullptr;  // the last copies from p have completed
+    // room for `need` bytes, all copies from p done
+    cudaError_t reserve(size_t need) {
+      cudaError_t e = done ? cudaEventSynchronize(done) : cudaEventCreateWithFlags(&done, cudaEventDisableTiming);
+      if (e != cudaSuccess || need <= bytes) return e;
+      if (p) cudaFreeHost(p);
+      p = nullptr;
+      bytes = 0;
+      if ((e = cudaMallocHost(&p, need)) == cudaSuccess) bytes = need;
+      return e;
+    }
   };
   Stage stage[2];
   int stage_next = 0;

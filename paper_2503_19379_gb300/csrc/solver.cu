@@ -142,15 +142,7 @@ int upload_kpoints(pc_ctx *ctx, int nb, const double *kpts, const double *gammas
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   PC_CK(cudaStreamIsCapturing(ctx->stream, &cap));
   if (cap != cudaStreamCaptureStatusNone) PC_CK(cudaStreamSynchronize(ctx->stream));
-  if (!sg.done) PC_CK(cudaEventCreateWithFlags(&sg.done, cudaEventDisableTiming));
-  PC_CK(cudaEventSynchronize(sg.done));
-  if (need > sg.bytes) {
-    if (sg.p) cudaFreeHost(sg.p);
-    sg.p = nullptr;
-    sg.bytes = 0;
-    PC_CK(cudaMallocHost(&sg.p, need));
-    sg.bytes = need;
-  }
+  PC_CK(sg.reserve(need));
   double2 *const sym = static_cast<double2 *>(sg.p);
   KParam *const kp = reinterpret_cast<KParam *>(sym + symc);
   for (int b = 0; b < nb; ++b) {
@@ -335,6 +327,10 @@ extern "C" int pc_setup(pc_ctx **out, int N, const double *eps_edges, const doub
       (e = cudaMemcpy(ctx->twd.p, tw.data(), sizeof(double2) * (N / 2), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = cudaMemcpy(ctx->twf.p, twf.data(), sizeof(float2) * (N / 2), cudaMemcpyHostToDevice)) != cudaSuccess)
     return fail(cuda_fail(e, "upload", __FILE__, __LINE__));
+  // the staging of upload_kpoints, for up to 8 k-points (30 us of a first call's 130 otherwise)
+  for (pc_ctx::Stage &s : ctx->stage)
+    if ((e = s.reserve((sizeof(double2) * (general ? 9 : 3) * N + sizeof(KParam)) * 8)) != cudaSuccess)
+      return fail(cuda_fail(e, "staging", __FILE__, __LINE__));
   *out = ctx;
   return PC_OK;
 }
