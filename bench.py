@@ -71,15 +71,16 @@ def stage_roofline(stage, d, precision, peaks, src):
     """Roofline entry for one stage: algorithmic work per launch / average event time of a launch."""
     calls = max(d["calls"], 1)
     t = d["ms"] / calls / 1e3
-    if precision == "fp64" or stage in ("rr", "recompute"):
+    # (the FP64 Gram products and updates are digit-sliced tensor-core products, not FP64-pipe work: their bytes below)
+    if (precision == "fp64" and stage not in ("gram", "update")) or stage in ("rr", "recompute"):
         achieved = d["flops"] / calls / t / 1e12
         line = {"bound": "alu", "kernel": stage, "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                 "frac": achieved / FP64_PEAK_TFLOPS, "traffic": None,
                 "peak_source": "derived: 152 SMs x 2 FP64 FMA/clk x 2 x 2.07 GHz (FP64 CUDA cores)"}
         if stage == "rr":
-            line["note"] = ("one CTA per pencil: a launch for a k-point group occupies one SM per active k-point of "
-                            "the group, so the fraction of the occupied SMs' FP64 peak is 152 / (active k-points) x "
-                            "frac; the stage time is the interval on the group's stream while the other groups "
+            line["note"] = ("a cluster of at most four CTAs per pencil: a launch for a k-point group occupies that many "
+                            "SMs per active k-point of the group, so the fraction of the occupied SMs' FP64 peak is "
+                            "higher than frac by 152 / (occupied SMs); the stage time is the interval on the group's stream while the other groups "
                             "share the GPU")
         return line
     if stage == "dfloat":
@@ -88,7 +89,9 @@ def stage_roofline(stage, d, precision, peaks, src):
         return {"bound": "alu", "kernel": stage, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": None,
                 "peak_source": "derived: FP32 peak (152 SMs x 128 lanes x 2 x 2.07 GHz) / 9 FP32 ops per "
-                               "double-float flop"}
+                               "double-float flop",
+                "note": "the stage's update and Gram block run as digit-sliced products on the tensor cores, its "
+                        "stencil on the FP32 pipe; the fraction is of double-float arithmetic on the FP32 pipe"}
     achieved = d["bytes"] / calls / t / 1e9
     peak = float(peaks["hbm_gbs"])
     line = {"bound": "hbm", "kernel": stage, "achieved": achieved, "peak": peak, "unit": "GB/s",

@@ -643,7 +643,7 @@ int launch_block_update(int nb, long L, int p, int q, int dtype, const void *S, 
   }
   // complex128: on the tensor cores (faster at every size measured, see update_sl.cu); not the
   // addend and the sum of no columns, which no solve asks for
-  if (dtype == PC_C128 && p > 0 && !Z) 
+  if (dtype == PC_C128 && p > 0 && !Z)
     return launch_update_sl(nb, L, p, q, PC_C128, S, ss, C, sc, Y, sy, nullptr, 0, st, act);
   if (dtype == PC_C128) {
     block_update_t<double, 8>(nb, L, p, q, S, ss, C, sc, Y, sy, st, act, Z, sz);

@@ -13,7 +13,8 @@
 // Phase 1 (every k-point starts here): X and AX in complex64 as well, until the complex64 residual stops falling.
 // Phase 2: X stored as double-float pairs (hi + lo FP32, ~48 bits); X' = X C_X + P' (complex64 correction),
 // AX' = Op X' by the stencil fused with the residual R = AX' - X' Theta (AX' itself is never stored), and the X-X
-// Gram block X^H X, all three in double-float arithmetic (mixed_df.cu) on the FP32 pipe. The X-X block of the
+// Gram block X^H X, all three in double-float accuracy (the stencil in FP32 pairs, mixed_df.cu; the update and the Gram
+// block as exact digit products on the tensor cores, update_sl.cu and gram_sl.cu). The X-X block of the
 // projected operator is Theta X^H X + R^H X (AX = X Theta + R), with R^H X from the complex64 product R^H [X | Q]:
 // its rounding is eps32 |R| |X|, small because R is.
 // Convergence and Algorithm 4.1 are decided in phase 2 only, on FP64 residuals and FP64 norms. A k-point whose
@@ -29,7 +30,7 @@
 // iteration of a group ends with its residual norms copied to the host and an event; the host then serves the
 // groups in turn -- waits for a group's event, takes its convergence decisions, enqueues its next iteration -- so
 // that while it waits for one group the other groups' kernels occupy the GPU. This hides the latency-bound steps (the Rayleigh-Ritz
-// kernel runs one block per k-point, the host decisions leave the GPU idle) behind bandwidth-bound kernels.
+// kernel runs at most four blocks per k-point, the host decisions leave the GPU idle) behind bandwidth-bound kernels.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
