@@ -635,16 +635,17 @@ static int update_width(int q, std::initializer_list<int> widths) {
 }
 
 int launch_block_update(int nb, long L, int p, int q, int dtype, const void *S, long ss, const void *C, long sc,
-                        void *Y, long sy, cudaStream_t st, const int *act, const void *Z, long sz) {
+                        void *Y, long sy, cudaStream_t st, const int *act, const void *Z, long sz, bool each) {
   if (nb == 0 || q == 0) return PC_OK;
   if (p > UPD_PMAX) {
     set_error("block_update: at most 64 input columns");
     return PC_EINVAL;
   }
-  // complex128: on the tensor cores (faster at every size measured, see update_sl.cu); not the
-  // addend and the sum of no columns, which no solve asks for
+  // complex128: on the tensor cores (update_sl.cu: faster than the FP64 pipe at every size measured, 8 -> 4 columns of 1536
+  // rows and up; `each` also where C picks single columns, 1.6 against 4.0 ms for 48 -> 16 of 8 k-points at N = 32); not
+  // the addend and the sum of no columns, which no solve asks for
   if (dtype == PC_C128 && p > 0 && !Z)
-    return launch_update_sl(nb, L, p, q, PC_C128, S, ss, C, sc, Y, sy, nullptr, 0, st, act);
+    return launch_update_sl(nb, L, p, q, PC_C128, S, ss, C, sc, Y, sy, nullptr, 0, st, act, each);
   if (dtype == PC_C128) {
     block_update_t<double, 8>(nb, L, p, q, S, ss, C, sc, Y, sy, st, act, Z, sz);
   } else {
@@ -1215,7 +1216,8 @@ extern "C" int pc_block_update(int nb, long L, int p, int q, int dtype, const vo
   PC_REQUIRE(S && C && Y, "pc_block_update: null argument");
   PC_REQUIRE(nb >= 0 && L >= 0 && p >= 0 && q >= 0 && p <= 64 && q <= 64, "pc_block_update: bad sizes");
   PC_REQUIRE(dtype == PC_C128 || dtype == PC_C64, "pc_block_update: bad dtype");
-  return launch_block_update(nb, L, p, q, dtype, S, ss, C, (long)p * q, Y, sy, (cudaStream_t)stream, nullptr);
+  return launch_block_update(nb, L, p, q, dtype, S, ss, C, (long)p * q, Y, sy, (cudaStream_t)stream, nullptr, nullptr, 0,
+                             true);
 }
 
 extern "C" int pc_residual(int nb, long L, int m, const void *X, const void *AX, const double *theta, void *R,

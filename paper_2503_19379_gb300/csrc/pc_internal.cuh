@@ -280,7 +280,8 @@ int tc_min_chunks(long L);
 int gram_tc_check();
 // Y = S C (+ Z, a complex64 addend, if Z is not null); arithmetic in the precision of dtype
 int launch_block_update(int nb, long L, int p, int q, int dtype, const void *S, long ss, const void *C, long sc,
-                        void *Y, long sy, cudaStream_t st, const int *act, const void *Z = nullptr, long sz = 0);
+                        void *Y, long sy, cudaStream_t st, const int *act, const void *Z = nullptr, long sz = 0,
+                        bool each = false);
 int launch_block_update_sum(int nb, long L, int p, int q, const void *S, const void *C, const void *S2, const void *C2,
                             long ss, long sc, void *Y, long sy, cudaStream_t st);
 // sg, sc: batch strides of G/H and of coef in elements; <= 0 means packed (n n, n m)

@@ -263,8 +263,9 @@ int sl_gram_chunks(int nb, long L);
 int launch_gram_sl(int nb, long L, int p, int q, int dtype, const void *A, long sa, const void *B, long sb, int mode,
                    double2 *part, int maxchunk, int *nchunk, cudaStream_t st, const int *act);
 
-// Y = S C (+ Z, a complex64 addend, for pairs) for PC_C128 (1 <= p <= 64) or PC_DFS (1 <= p <= 32) blocks (update_sl.cu)
+// Y = S C (+ Z, a complex64 addend, for pairs) for PC_C128 (1 <= p <= 64) or PC_DFS (1 <= p <= 32) blocks (update_sl.cu);
+// each (PC_C128): every output to the accuracy of its own terms, otherwise to that of its row's largest
 int launch_update_sl(int nb, long L, int p, int q, int dtype, const void *S, long ss, const void *C, long sc, void *Y,
-                     long sy, const void *Z, long sz, cudaStream_t st, const int *act);
+                     long sy, const void *Z, long sz, cudaStream_t st, const int *act, bool each = false);
 
 }  // namespace pc

@@ -6,7 +6,10 @@
 // E_l = max_i (e(S_li) + a_i), where a_i is the exponent of the largest entry of row i of C; row i of C is scaled by
 // 2^-a_i, and its columns have exponents of their own. So a small column of S with large coefficients (a preconditioned
 // residual) is held as accurately as a large one with small coefficients: every term S_li C_ij is rounded relative to
-// the largest term of its row.
+// the largest term that its row and its column of C could form. That leaves an output few digits if all its own terms are
+// far smaller (a small column of S that C picks out). The solves take it, since their errors count against the norm of a
+// row; for other callers (EACH) the kernel finds such outputs and forms them in plain FP64: per output a bit is set where
+// some term comes within a few bits of that largest one, from the exponents that the digits need anyway.
 //
 // One CTA (512 threads, one per SM) keeps the digits of C in shared memory and walks over row tiles of one k-point. A
 // thread owns one row and a quarter of the columns (16-byte digit stores, no bank conflicts); it holds its elements in
@@ -22,7 +25,8 @@
 // seven left 5.4e-14 where C is near the identity).
 //
 // Bound: instructions of the digit extraction and the epilogue. Complex128, 8 k-points, 48 -> 16 columns at N = 32:
-// 4.00 ms on the FP64 pipe (1.21 TFLOP/s, all of it), 0.48 ms here; 4 k-points, 57 -> 19 at N = 64: 27.5 and 2.7 ms; one
+// 4.00 ms on the FP64 pipe (1.21 TFLOP/s, all of it), 0.48 ms here (EACH: 0.51 ms for smooth fields and dense C; 2.1 ms
+// for C near the identity, where a fifth of the outputs takes FP64); 4 k-points, 57 -> 19 at N = 64: 27.5 and 2.7 ms; one
 // k-point, 24 -> 8 at N = 16: 54.8 and 17.0 us; the smallest size tried (8 -> 4 columns of 1536 rows): 21.9 and 17.9 us.
 // Pairs, 4 k-points, 19 -> 19 columns at N = 64: 2.03 ms in double-float arithmetic, 1.16 ms here (without the MMAs
 // 0.25 ms less, without the digits 0.3 ms, without the epilogue 0.44 ms); 2 k-points, 12 -> 12 at N = 8: 16.9 and 12.9 us.
@@ -30,6 +34,8 @@
 // columns at N = 64.)
 #include <cuda.h>
 #include <cuda_runtime.h>
+
+#include <cmath>
 
 #include "sliced.cuh"
 
@@ -40,6 +46,7 @@ namespace {
 constexpr int SU_THREADS = 512;
 constexpr int SU_COLS = 16;  // columns per stage
 constexpr int SU_BAD = 1 << 20;
+constexpr int SU_SLACK = 5;  // most bits between an output's largest term and its row's (launch_update_sl)
 
 __device__ int g_update_sl_error = 0;
 
@@ -54,6 +61,7 @@ struct SlUpdateArgs {
   long sz;
   long L;
   int p, q, nbc, nbp, ntile;
+  int slack;
   uint32_t tmem_cols;
   const int *act;
 };
@@ -68,8 +76,11 @@ __device__ __forceinline__ void tmem_wait4(uint32_t (&r)[4]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3])::"memory");
 }
 
-// T: element type of S and Y; NS: stages (p <= 16 NS)
-template <typename T, int NS>
+// words of shared memory past the exponents of C with EACH: sM and sNear of update_sl_kernel
+constexpr int su_each_words(bool each) { return each ? 1536 + 2 * 65 * (SU_SLACK + 3) : 0; }
+
+// T: element type of S and Y; NS: stages (p <= 16 NS); EACH: every output as accurate as its own terms, not as its row's
+template <typename T, int NS, bool EACH>
 __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdateArgs a) {
   using F = SlFormShort<T>;
   constexpr int ND = F::ND, NL = F::NL;
@@ -83,7 +94,12 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
   const uint32_t off_b = ND * 16384u, atom = (uint32_t)(ND * a.nbp) * 128u, off_e = off_b + NATOM * atom;
   int *const sE = reinterpret_cast<int *>(sm + off_e);  // [3][4][128] row exponents (three tiles in turn, by column quarter)
   int *const sCA = sE + 1536, *const sCB = sCA + 64;    // exponents of the rows and columns of C
-  const uint32_t off_bar = off_e + (1536u + 128u) * 4u;
+  // with EACH, bit j of a word for output j: sM [3][4][128] outputs of a row that the digits serve (laid out as sE), and
+  // sNear [slack + 3][65], at k and i: outputs whose coefficient in row i of C is at most k - 2 (.x) and k - 1 (.y) bits
+  // below the largest that its column allows
+  unsigned *const sM = reinterpret_cast<unsigned *>(sCB + 64);
+  uint2 *const sNear = reinterpret_cast<uint2 *>(sM + 1536);
+  const uint32_t off_bar = off_e + (uint32_t)(1536 + 128 + su_each_words(EACH)) * 4u;
   const uint32_t bars = base + off_bar;
   uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(sm + off_bar + 16);
   volatile int *abort = reinterpret_cast<volatile int *>(tmem_holder + 1);
@@ -152,6 +168,17 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
   }
   __syncthreads();
   const bool bad = *badC != 0;
+  if constexpr (EACH) {
+    for (int i = warp; i < a.p; i += SU_THREADS / 32) {
+      const int d = lane < nbc ? sCB[lane] + sCA[i] - (sl_key(Cb[(long)i * a.q + lane]) >> 20) : SU_BAD;
+      unsigned m = 0u;
+      for (int k = 0; k < a.slack + 3; ++k) {
+        const unsigned up = k ? __ballot_sync(0xffffffffu, d <= k - 1) : 0u;
+        if (lane == 0) sNear[k * 65 + i] = make_uint2(m, up);
+        m = up;
+      }
+    }
+  }
   for (int t = tid; t < a.p * nbc && !bad; t += SU_THREADS) {
     const int i = t / nbc, j = t - i * nbc;
     const double2 c = Cb[(long)i * a.q + j];
@@ -269,6 +296,67 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
       named_arrive(1 + (n & 1), SU_THREADS);
     }
   };
+  // This warp's columns of Y: 2 slot + 8 it, and the next
+  const unsigned own = (nbc < 32 ? (1u << nbc) - 1u : ~0u) & (0x03030303u << (2 * slot));
+  // Output j of the rows row0 + r in plain FP64, for the lanes r of `todo`: a row with an infinity or a NaN (or C with
+  // one), or an output that the digits do not serve. Up to half of the rows are taken eight at a time, the terms of a row
+  // shared over four lanes; otherwise a lane takes its own row, past the terms of zero coefficients where the row is
+  // finite. (An FP64 instruction takes the warp 64 cycles whatever the number of active lanes: p + 4 of them for eight rows
+  // of the first form, 4 p for the second.)
+  auto plain_fp64 = [&](unsigned todo, long row0, int j, bool finite) {
+    double2 out = make_double2(0.0, 0.0);
+    if (__popc(todo) <= 16) {
+      const int at = __popc(todo & ((1u << lane) - 1u));  // this lane's place among the rows
+      unsigned rest = todo;
+      for (int first = 0; rest; first += 8) {
+        unsigned t = rest;
+        for (int k = 0; k < 8; ++k) {
+          if (k < (lane >> 2)) t &= t - 1;
+          rest &= rest - 1;
+        }
+        double2 v = make_double2(0.0, 0.0);
+        if (t) {
+          const double2 *x = Cb + j;
+          const T *y = Sb + row0 + __ffs(t) - 1;
+#pragma unroll 4
+          for (int i = lane & 3; i < a.p; i += 4) {
+            const double2 u = ld_c128(y + (long)i * L), c = x[(long)i * a.q];
+            v.x = fma(u.x, c.x, fma(-u.y, c.y, v.x));
+            v.y = fma(u.x, c.y, fma(u.y, c.x, v.y));
+          }
+        }
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+          v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+          v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+        }
+        const int from = 4 * ((at - first) & 7);
+        const double2 w = make_double2(__shfl_sync(0xffffffffu, v.x, from), __shfl_sync(0xffffffffu, v.y, from));
+        if (at >= first && at < first + 8) out = w;
+      }
+    } else if ((todo >> lane) & 1u) {
+      for (int i = 0; i < a.p; ++i) {
+        const double2 c = Cb[(long)i * a.q + j];
+        if (finite && c.x == 0.0 && c.y == 0.0) continue;
+        const double2 u = ld_c128(Sb + (long)i * L + row0 + lane);
+        out.x = fma(u.x, c.x, fma(-u.y, c.y, out.x));
+        out.y = fma(u.x, c.y, fma(u.y, c.x, out.y));
+      }
+    }
+    if ((todo >> lane) & 1u) {
+      const long o = (long)j * L + row0 + lane;
+      if constexpr (F64) {
+        Yb[o] = out;
+      } else {
+        if (Zb) {
+          out.x += (double)Zb[o].x;
+          out.y += (double)Zb[o].y;
+        }
+        const cdf d = cdf_from(out);
+        Yb[o] = make_float4(d.re.hi, d.re.lo, d.im.hi, d.im.lo);
+      }
+    }
+  };
   // the tile whose n-th stage was its last
   auto epilogue = [&](long tile, int n, int par) {
     bar_wait(bars + 8u * (n & 1), (n >> 1) & 1, abort);
@@ -277,8 +365,12 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
     const int row = quarter * 32 + lane;
     const long l = tile * 128 + row;
     int E = 0;
+    unsigned served = EACH ? 0u : ~0u;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) E = max(E, sE[par * 512 + k * 128 + row]);
+    for (int k = 0; k < 4; ++k) {
+      E = max(E, sE[par * 512 + k * 128 + row]);
+      if constexpr (EACH) served |= sM[par * 512 + k * 128 + row];
+    }
 #pragma unroll
     for (int it = 0; it < 4; ++it) {
       const int c0 = 4 * slot + 16 * it;
@@ -294,25 +386,7 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
         const int j = (c0 >> 1) + h;
         if (j >= nbc || l >= L) continue;
         T out;
-        if (bad || E >= SU_BAD) {
-          // an infinity or a NaN in the row or in C: plain FP64
-          double re = 0.0, im = 0.0;
-          for (int i = 0; i < a.p; ++i) {
-            const double2 x = ld_c128(Sb + (long)i * L + l), c = Cb[(long)i * a.q + j];
-            re = fma(x.x, c.x, fma(-x.y, c.y, re));
-            im = fma(x.x, c.y, fma(x.y, c.x, im));
-          }
-          if constexpr (F64) {
-            out = make_double2(re, im);
-          } else {
-            if (Zb) {
-              re += (double)Zb[(long)j * L + l].x;
-              im += (double)Zb[(long)j * L + l].y;
-            }
-            const cdf d = cdf_from(make_double2(re, im));
-            out = make_float4(d.re.hi, d.re.lo, d.im.hi, d.im.lo);
-          }
-        } else if constexpr (F64) {
+        if constexpr (F64) {
           const int sc = sl_weight<F>(E, sCB[j]);
           long long H[2];
           unsigned lo[2];
@@ -339,6 +413,16 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
         Yb[(long)j * L + l] = out;
       }
     }
+    // the outputs that the digits do not serve, over what was stored
+    const unsigned plain = l >= L ? 0u : (bad || E >= SU_BAD ? ~0u : ~served);
+    if (__any_sync(0xffffffffu, plain & own)) {
+#pragma unroll 1
+      for (unsigned js = own; js; js &= js - 1) {
+        const int j = __ffs(js) - 1;
+        const unsigned todo = __ballot_sync(0xffffffffu, (plain >> j) & 1u);
+        if (todo) plain_fp64(todo, tile * 128 + quarter * 32, j, E < SU_BAD);
+      }
+    }
   };
   // A tile's first two stages are converted before the epilogue of the tile before, whose MMAs run meanwhile
   constexpr int AHEAD = NS < 2 ? NS : 2;
@@ -360,6 +444,21 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < 4; ++k) ex = max(ex, sE[par * 512 + k * 128 + r]);
+    if constexpr (EACH) {
+      // an output is served if one of its terms is within `slack` bits of the largest that its row and column allow, or
+      // two of this thread's terms within slack + 1
+      unsigned served = 0, seen = 0;
+#pragma unroll
+      for (int k = 0; k < NC; ++k) {
+        const int i = (k >> 2) * SU_COLS + 4 * g + (k & 3);
+        if (i < a.p) {
+          const uint2 m = sNear[max(a.slack + 2 - (ex - sCA[i] - (sl_key(v[k]) >> 20)), 0) * 65 + i];
+          served |= m.x | (seen & m.y);
+          seen |= m.y;
+        }
+      }
+      sM[par * 512 + g * 128 + r] = served;
+    }
 #pragma unroll
     for (int s = 0; s < AHEAD; ++s) convert(s, n + s, tile, ex);
     if (prev >= 0) epilogue(prev, n - 1, ppar);
@@ -375,6 +474,7 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
     ppar = par;
     par = par == 2 ? 0 : par + 1;
   }
+  if (EACH) __syncthreads();  // (sM of the last tile)
   if (prev >= 0) {
     load_z(prev);
     epilogue(prev, n - 1, ppar);
@@ -390,7 +490,7 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
   if (tid == 0 && *abort) atomicExch(&g_update_sl_error, 1);
 }
 
-template <typename T, int NS>
+template <typename T, int NS, bool EACH = false>
 int launch_su(SlUpdateArgs a, int nb, cudaStream_t st) {
   // columns of Y per block: all levels of 2 nbc columns in TMEM, the digits of C and of one tile in shared memory
   using F = SlFormShort<T>;
@@ -403,7 +503,7 @@ int launch_su(SlUpdateArgs a, int nb, cudaStream_t st) {
   a.tmem_cols = 32;
   while (a.tmem_cols < (uint32_t)((ND + ((a.nbp >> 3) & 1)) * a.nbp)) a.tmem_cols *= 2;
   auto smem_of = [](int nbp) {
-    return (size_t)1024 + ND * 16384 + (size_t)((NS + 1) / 2) * ND * nbp * 128 + (1536 + 128) * 4 + 64;
+    return (size_t)1024 + ND * 16384 + (size_t)((NS + 1) / 2) * ND * nbp * 128 + (1536 + 128 + su_each_words(EACH)) * 4 + 64;
   };
   // CTAs per k-point and column block: the least tiles (plus about one for the setup) in the longest sequence per SM
   const long per = (long)nb * nqb, nsm = sm_count();
@@ -420,12 +520,12 @@ int launch_su(SlUpdateArgs a, int nb, cudaStream_t st) {
   int dev = 0;
   PC_CK(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64 || !configured[dev]) {
-    PC_CK(cudaFuncSetAttribute(update_sl_kernel<T, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    PC_CK(cudaFuncSetAttribute(update_sl_kernel<T, NS, EACH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)smem_of(2 * most_cols)));
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
   // a CTA's 512 threads of 128 registers take the SM: no second CTA waits for its TMEM columns there
-  update_sl_kernel<T, NS><<<dim3(gx, nqb, nb), SU_THREADS, smem_of(a.nbp), st>>>(a);
+  update_sl_kernel<T, NS, EACH><<<dim3(gx, nqb, nb), SU_THREADS, smem_of(a.nbp), st>>>(a);
   PC_CK_LAUNCH();
   return PC_OK;
 }
@@ -433,7 +533,7 @@ int launch_su(SlUpdateArgs a, int nb, cudaStream_t st) {
 }  // namespace
 
 int launch_update_sl(int nb, long L, int p, int q, int dtype, const void *S, long ss, const void *C, long sc, void *Y,
-                     long sy, const void *Z, long sz, cudaStream_t st, const int *act) {
+                     long sy, const void *Z, long sz, cudaStream_t st, const int *act, bool each) {
   SlUpdateArgs a{};
   a.S = S;
   a.ss = ss;
@@ -448,11 +548,16 @@ int launch_update_sl(int nb, long L, int p, int q, int dtype, const void *S, lon
   a.q = q;
   a.act = act;
   if (dtype == PC_DFS) return p <= SU_COLS ? launch_su<float4, 1>(a, nb, st) : launch_su<float4, 2>(a, nb, st);
+  // EACH: the error of a digit product is 2^-60.2 sqrt(2 p) (rms) of the largest term that a row of S and a column of C
+  // could form. An output with a term within 2^slack of that is off by 2^-54 of its own terms, no more than FP64 sums. The
+  // others take FP64; where S and C are dense they are few (48 -> 16 columns: none of 10^5 outputs of random panels, 2 in
+  // 10^4 of smooth fields).
+  a.slack = std::min(SU_SLACK, (int)std::floor(6.2 - 0.5 * std::log2(2.0 * p)));
   switch ((p + SU_COLS - 1) / SU_COLS) {
-    case 1: return launch_su<double2, 1>(a, nb, st);
-    case 2: return launch_su<double2, 2>(a, nb, st);
-    case 3: return launch_su<double2, 3>(a, nb, st);
-    default: return launch_su<double2, 4>(a, nb, st);
+    case 1: return each ? launch_su<double2, 1, true>(a, nb, st) : launch_su<double2, 1>(a, nb, st);
+    case 2: return each ? launch_su<double2, 2, true>(a, nb, st) : launch_su<double2, 2>(a, nb, st);
+    case 3: return each ? launch_su<double2, 3, true>(a, nb, st) : launch_su<double2, 3>(a, nb, st);
+    default: return each ? launch_su<double2, 4, true>(a, nb, st) : launch_su<double2, 4>(a, nb, st);
   }
 }
 
