@@ -234,9 +234,10 @@ int pc_apply_precond(pc_ctx *ctx, int nb, const double *kpts, const double *gamm
 
 /* a3: G_b = A_b^H B_b for tall-skinny blocks (L rows; p and q columns, column stride L; batch strides sa, sb in
  * elements). G: device complex128 [nb][p][q] row-major. p, q <= 64. dtype applies to A and B. PC_C128: exact products
- * of the values rounded to 54 bits below the largest of a column's 1024 rows, on the tensor cores (FP16 digits, integer
- * sums), with FP64 sums over the spans of rows: at most the error of FP64 products and sums. Columns with an infinity
- * or a NaN take plain FP64. PC_C64: FP32 products and partial sums over chunks of the rows, chunks added in FP64; where
+ * of the values rounded to 54 bits below the largest of a column's 1024 rows at most, on the tensor cores (FP16 digits,
+ * integer sums), with FP64 sums over the spans of rows; entries whose columns share too few rows of normal size, and
+ * those of columns with an infinity or a NaN, in plain FP64. Every entry is within 2 L 2^-52 sum |a||b|, twice the
+ * a-priori bound of FP64 products and sums. PC_C64: FP32 products and partial sums over chunks of the rows, chunks added in FP64; where
  * p or q is above 16, L is a multiple of 16 and the panels are 16-byte aligned this runs on the tensor cores (TF32
  * operands split into hi + lo, accumulators drained every 64 rows), otherwise on the CUDA cores. */
 int pc_gram(int nb, long L, int p, int q, int dtype, const void *A, long sa, const void *B, long sb, void *G,

@@ -13,13 +13,18 @@
 // exactly (SlForm::KMAX) the level sums are drained into 64-bit integer sums in registers. At the end of a span these are
 // scaled and added to FP64 sums in shared memory.
 //
+// Digits are exact relative to the largest values of the two columns in the span, which need not meet: columns that are
+// large in different rows have a product far below that of their largest values. So the rows of a complex128 span in which
+// a column is within two bits of its largest are marked while the digits are formed, and an entry whose columns share too
+// few of them is formed in plain FP64 for this span, as are those of a column with an infinity or a NaN (`unserved`).
+//
 // Complex128 panels take seven digits in eight levels, which leaves less error than the FP64 sums they replace, in every
 // entry of G and H (against extended precision, N = 8 to 32, smooth and random panels; seven levels left up to 1.8 times
 // more off the diagonal). Pairs take seven digits of base 128: 1e-15 of the diagonal, the double-float sums 3e-14.
 //
 // Bound: the latency of a stage (load, digits, hand-off to the tensor core, drain), then integer instructions of the digit
-// extraction. 8 k-points x 48 complex128 columns at N = 32: 23.6 ms on the FP64 pipe, 1.92 ms here (without the scan
-// 0.3 ms less, without the MMAs 0.4 ms, without the drains 0.2 ms); one k-point of 24 columns at N = 16: 1.77 ms and
+// extraction. 8 k-points x 48 complex128 columns at N = 32: 23.6 ms on the FP64 pipe, 2.03 ms here (without the scan
+// 0.3 ms less, without the MMAs 0.4 ms, without the drains 0.2 ms, without the marks and their comparison 0.1 ms); one k-point of 24 columns at N = 16: 1.77 ms and
 // 64 us. X^H X of 4 k-points x 19 pair columns at N = 64: 1.61 ms in double-float arithmetic, 1.11 ms here; of one
 // k-point x 13 at N = 16: 60 and 24 us. The pair A^H A, A^H B takes the block's columns of A and of B in one CTA, and the
 // columns of A that the block shares with the left operand are extracted once and stored twice.
@@ -36,14 +41,18 @@ namespace {
 constexpr int SG_CONV = 512;                  // threads that form digits and drain
 constexpr int SG_THREADS = SG_CONV + 32;      // and the warp that issues the MMAs
 constexpr int SG_ROWS = 32;                   // rows per stage
-constexpr int SG_SUPER = 1024;                // rows per common exponent
+constexpr int SG_SUPER = 1024;                // rows per common exponent, at most
+constexpr int SG_WORDS = SG_SUPER / 32;       // words of a column's mask of large rows
+constexpr int SG_WSTRIDE = SG_WORDS + 4;      // their distance from column to column (banks of 16-byte loads)
+// a column's share of the common rows that an entry needs: ordinary, all zeros, with an infinity or a NaN
+constexpr int SG_NEED = 8, SG_ZERO = -1000, SG_BAD = 1 << 20;
 
 __device__ int g_gram_sl_error = 0;
 
 struct SlGramArgs {
   const void *A, *B;
   long sa, sb;
-  long L, chunk;
+  long L;
   int p, q, mode;
   int nbc, nbp;  // columns per block; accumulator columns per level (2 per operand column, rounded up to 16)
   double2 *part0, *part1;
@@ -51,10 +60,15 @@ struct SlGramArgs {
 };
 
 // TASKS: at most 32 TASKS columns to extract (each thread two rows of every 32nd column); DEPTH: stages loaded ahead
+template <typename T> constexpr bool sg_each() { return std::is_same<T, double2>::value; }
+// exponents, needs and masks of 96 columns
+template <typename T> constexpr uint32_t sg_col_bytes() { return 96u * 4u * (sg_each<T>() ? 2 + SG_WSTRIDE : 2); }
+
 template <typename T, int TASKS, int DEPTH>
 __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs a) {
   using F = SlForm<T>;
   constexpr int ND = F::ND, NL = F::NL, GROUP = F::KMAX / SG_ROWS;  // stages per drain
+  constexpr bool EACH = sg_each<T>();  // every entry as accurate as its own terms
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_addr(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -63,11 +77,12 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
   const uint32_t off_e = off_acc + 8u * SG_CONV * 8u;  // FP64 sums, then exponents
   double *const acc = reinterpret_cast<double *>(sm + off_acc);
   int *const sE = reinterpret_cast<int *>(sm + off_e);
-  const uint32_t off_bar = off_e + 96u * 4u;
+  int *const sNeed = sE + 96;                                        // SG_NEED, SG_ZERO or SG_BAD
+  unsigned *const sMask = reinterpret_cast<unsigned *>(sNeed + 96);  // complex128: rows within 2 bits of the column's largest
+  const uint32_t off_bar = off_e + sg_col_bytes<T>();
   const uint32_t bars = base + off_bar;
   uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(sm + off_bar + 16);
   volatile int *abort = reinterpret_cast<volatile int *>(tmem_holder + 1);
-  volatile int *bad = abort + 1;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int bi = blockIdx.z, b = a.act ? a.act[bi] : bi;
@@ -78,7 +93,10 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
   const int ncols = pa + nown;  // columns to extract
   const T *const Ab = static_cast<const T *>(a.A) + (long)b * a.sa;
   const T *const Bb = static_cast<const T *>(a.B) + (long)b * a.sb + (long)j0 * a.L;
-  const long L = a.L, r0 = (long)blockIdx.x * a.chunk, r1 = min(L, r0 + a.chunk);
+  // the chunk's stages, in spans of nearly equal length (a short one would have few rows of normal size)
+  const long L = a.L, nst = (L + SG_ROWS - 1) / SG_ROWS;
+  const long st0 = blockIdx.x * nst / gridDim.x, cst = (blockIdx.x + 1) * nst / gridDim.x - st0;
+  const int nspan = (int)((cst * SG_ROWS + SG_SUPER - 1) / SG_SUPER);
 
   {
     float4 *z = reinterpret_cast<float4 *>(sm);
@@ -90,7 +108,6 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
     bar_init(bars, 1);
     bar_init(bars + 8u, 1);
     *abort = 0;
-    *bad = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -115,40 +132,61 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
   const uint32_t tdrain = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(slot * 16);
   // extracted column (index into sE) of operand column jj
   auto col_of = [&](int jj) { return jj < ndup ? j0 + jj : pa + jj - ndup; };
+  // Whether a span's digits serve the product of two of its columns. They are exact to half a unit of 2^-53 of the largest
+  // value of each, 2^(Ea + 1) and 2^(Eb + 1), so the product is off by at most 2 n 2^-52 2^(Ea + Eb) over n rows: twice
+  // the bound of FP64 sums, if sum |a||b| is at least 2^(Ea + Eb). It is if a and b are within two bits of their largest in
+  // 16 common rows. (Dense columns of random values: about a third of the rows.) Returns the entries k of this thread
+  // (columns slot * 8 + k) that they do not serve.
+  auto unserved = [&](int words) {
+    // the threads of an entry's two parts take four columns each
+    const int k0 = 4 * (lane & 1);
+    int left[4], cb[4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const int jj = slot * 8 + k0 + h;
+      const bool stored = jj < ndup + nown && ci < pa && (a.mode == SL_GENERAL || ci <= j0 + (jj < ndup ? jj : jj - ndup));
+      cb[h] = stored ? col_of(jj) : 0;
+      left[h] = stored ? sNeed[ci] + sNeed[cb[h]] : 0;
+      if (left[h] < SG_BAD + SG_ZERO && (!EACH || cb[h] == ci)) left[h] = 0;  // (a column with itself; pairs: only SG_BAD)
+    }
+    if constexpr (EACH) {
+      for (int w = 0; w < words; w += 4) {
+        const uint4 ma = *reinterpret_cast<const uint4 *>(sMask + ci * SG_WSTRIDE + w);
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          const uint4 mb = *reinterpret_cast<const uint4 *>(sMask + cb[h] * SG_WSTRIDE + w);
+          left[h] -= __popc(ma.x & mb.x) + __popc(ma.y & mb.y) + __popc(ma.z & mb.z) + __popc(ma.w & mb.w);
+        }
+        if (max(max(left[0], left[1]), max(left[2], left[3])) <= 0) break;
+      }
+    }
+    unsigned plain = 0;
+#pragma unroll
+    for (int h = 0; h < 4; ++h) plain |= left[h] > 0 ? 1u << (k0 + h) : 0u;
+    return plain | __shfl_xor_sync(0xffffffffu, plain, 1);
+  };
 
   int n = 0;  // stages issued
-  for (long span0 = r0; span0 < r1; span0 += SG_SUPER) {
-    const long span1 = min(r1, span0 + SG_SUPER);
+  for (int sp = 0; sp < nspan; ++sp) {
+    const long span0 = (st0 + sp * cst / nspan) * SG_ROWS, span1 = min(L, (st0 + (sp + 1) * cst / nspan) * SG_ROWS);
     for (int c = warp; c < ncols; c += SG_THREADS / 32) {
       const T *x = c < pa ? Ab + (long)c * L : Bb + (long)(c - pa) * L;
       int mx = 0;
-#pragma unroll 16
-      for (long l = span0 + lane; l < span1; l += 32) mx = max(mx, sl_key(x[l]));
-      mx = sl_exp_of<T>(__reduce_max_sync(0xffffffffu, mx));
+      for (long l0 = span0; l0 < span1; l0 += 512) {  // 16 loads in flight (past the end: the last row again)
+#pragma unroll
+        for (int w = 0; w < 16; ++w) mx = max(mx, sl_key(x[min(l0 + 32 * w + lane, span1 - 1)]));
+      }
+      mx = __reduce_max_sync(0xffffffffu, mx);
+      if constexpr (EACH) sMask[c * SG_WSTRIDE + lane] = 0u;
+      const int E = sl_exp_of<T>(mx);
       if (lane == 0) {
-        sE[c] = mx;
-        if (mx >= SL_NONFINITE) *bad = 1;
+        sE[c] = E;
+        sNeed[c] = E >= SL_NONFINITE ? SG_BAD : (mx == 0 ? SG_ZERO : SG_NEED);
       }
     }
     __syncthreads();
     const int ns = (int)((span1 - span0 + SG_ROWS - 1) / SG_ROWS);
-    if (*bad) {
-      // an infinity or a NaN in the span: its products in plain FP64
-      if (drains && ci < pa)
-        for (int k = 0; k < 8; ++k) {
-          const int jj = slot * 8 + k;
-          if (jj >= ndup + nown) break;
-          const T *x = Ab + (long)ci * L, *y = jj < ndup ? Ab + (long)(j0 + jj) * L : Bb + (long)(jj - ndup) * L;
-          double s = 0.0;
-          for (long l = span0; l < span1; ++l) {
-            const double2 u = ld_c128(x + l), v = ld_c128(y + l);
-            s = odd ? fma(u.x, v.y, fma(-u.y, v.x, s)) : fma(u.x, v.x, fma(u.y, v.y, s));
-          }
-          acc[k * SG_CONV + tid] += s;
-        }
-      __syncthreads();
-      if (tid == 0) *bad = 0;
-    } else if (issuer) {
+    if (issuer) {
       for (int s = 0; s < ns; ++s, ++n) {
         const int buf = n & 1;
         named_sync(1 + buf, SG_THREADS);
@@ -191,9 +229,14 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
         if (n >= 2) bar_wait(bars + 8u * buf, ((n >> 1) & 1) ^ 1, abort);
 #pragma unroll
         for (int k = 0; k < TASKS; ++k) {
-          const int c = c0 + 32 * k;
+          const int c = c0 + 32 * k, E = c < ncols ? sE[c] : SL_NONFINITE;
+          if constexpr (EACH) {
+            // the rows within two bits of the column's largest: even rows in the low half of the stage's word
+            const unsigned m0 = __ballot_sync(0xffffffffu, sl_key(ring[dd][k][0]) >= (E - 2) << 20);
+            const unsigned m1 = __ballot_sync(0xffffffffu, sl_key(ring[dd][k][1]) >= (E - 2) << 20);
+            if (rp == 0 && c < ncols) sMask[c * SG_WSTRIDE + s] = __byte_perm(m0, m1, lane ? 0x7632 : 0x5410);
+          }
           if (c < ncols) {
-            const int E = sE[c];
             unsigned x[2][ND];  // the digits of rows 2 rp and 2 rp + 1, real and imaginary parts
             if constexpr (std::is_same<T, double2>::value) {
               unsigned long long m[2][2];
@@ -256,16 +299,46 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
           }
         }
       }
+      // the span's sums, but for the entries that the digits do not serve
+      unsigned plain = 0;
+      if constexpr (EACH) named_sync(3, SG_CONV);  // (the masks)
+      if (drains) plain = unserved(ns);
       if (drains && ci < pa) {
         const int EA = sE[ci];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           const int jj = slot * 8 + k;
-          if (jj < ndup + nown) {
+          if (jj < ndup + nown && !((plain >> k) & 1u)) {
             long long H;
             unsigned Lw;
             sl_join<F>(shi[k], slo[k], H, Lw);
             acc[k * SG_CONV + tid] += sl_to_double(H, Lw, sl_weight<F>(EA, sE[col_of(jj)]));
+          }
+        }
+      }
+      // those in plain FP64, one after the other by the whole warp
+      if (__any_sync(0xffffffffu, plain != 0)) {
+#pragma unroll 1
+        for (int k = 0; k < 8; ++k) {
+          unsigned todo = __ballot_sync(0xffffffffu, (plain >> k) & 1u) & 0x55555555u;
+          for (; todo; todo &= todo - 1) {
+            const int src = __ffs(todo) - 1, jj = slot * 8 + k;
+            const T *x = Ab + (long)(quarter * 16 + (src >> 1)) * L;
+            const T *y = jj < ndup ? Ab + (long)(j0 + jj) * L : Bb + (long)(jj - ndup) * L;
+            double re = 0.0, im = 0.0;
+#pragma unroll 4
+            for (long l = span0 + lane; l < span1; l += 32) {
+              const double2 u = ld_c128(x + l), v = ld_c128(y + l);
+              re = fma(u.x, v.x, fma(u.y, v.y, re));
+              im = fma(u.x, v.y, fma(-u.y, v.x, im));
+            }
+            // the lower half-warp sums re and the upper half im, one FP64 instruction a level
+            const bool up = lane & 16;
+            double t = (up ? im : re) + __shfl_xor_sync(0xffffffffu, up ? re : im, 16);
+#pragma unroll
+            for (int o = 8; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            t = __shfl_sync(0xffffffffu, t, lane & 1 ? 16 : 0);
+            if ((lane & ~1) == src) acc[k * SG_CONV + tid] += t;
           }
         }
       }
@@ -295,8 +368,8 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
   if (tid == 0 && *abort) atomicExch(&g_gram_sl_error, 1);
 }
 
-template <typename F> size_t sg_smem(int nbp) {
-  return 1024 + F::ND * 16384 + (size_t)F::NL * nbp * 128 + 8 * SG_CONV * 8 + 96 * 4 + 64;
+template <typename T> size_t sg_smem(int nbp) {
+  return 1024 + SlForm<T>::ND * 16384 + (size_t)SlForm<T>::NL * nbp * 128 + 8 * SG_CONV * 8 + sg_col_bytes<T>() + 64;
 }
 
 }  // namespace
@@ -336,14 +409,10 @@ int launch_gram_sl(int nb, long L, int p, int q, int dtype, const void *A, long 
       c = k;
     }
   }
-  a.chunk = std::max<long>(SG_ROWS, ((L + c - 1) / c + SG_ROWS - 1) / SG_ROWS * SG_ROWS);
-  c = (int)std::max<long>(1, (L + a.chunk - 1) / a.chunk);
   *nchunk = c;
   a.part0 = part;
   a.part1 = part + (size_t)nb * c * p * q;
-  using F64 = SlForm<double2>;
-  using FDF = SlForm<float4>;
-  const size_t smem = dtype == PC_DFS ? sg_smem<FDF>(a.nbp) : sg_smem<F64>(a.nbp);
+  const size_t smem = dtype == PC_DFS ? sg_smem<float4>(a.nbp) : sg_smem<double2>(a.nbp);
   const dim3 grid(c, nblk, nb);
   // columns that a block extracts: its left columns, up to all p, and its own of B
   const int ncols = p + (mode == SL_SELF ? 0 : a.nbc);
@@ -361,7 +430,7 @@ int launch_gram_sl(int nb, long L, int p, int q, int dtype, const void *A, long 
   PC_CK(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64 || !configured[dev][kind]) {
     PC_CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)(kind ? sg_smem<F64>(64) : sg_smem<FDF>(64))));
+                               (int)(kind ? sg_smem<double2>(64) : sg_smem<float4>(64))));
     if (dev >= 0 && dev < 64) configured[dev][kind] = true;
   }
   kernel<<<grid, SG_THREADS, smem, st>>>(a);
