@@ -281,7 +281,9 @@ int pc_gram_pair_noalloc(int nb, long L, int p, int dtype, const void *S, long s
  * (batch stride p*q), Y_b has q columns (batch stride sy). p <= 64, q <= 64. dtype applies to S and Y. PC_C128: on the
  * tensor cores (FP16 digits against one exponent per row of S and column of C, integer sums, one rounding), and in plain
  * FP64 where that would leave an output less accurate than its own terms (all of them far below the row's largest) and
- * where a row has an infinity or a NaN: an output is off by about as much as FP64 sums of its terms. PC_C64: FP32. */
+ * where a row has an infinity or a NaN: an output is off by about as much as FP64 sums of its terms. PC_C64: FP32.
+ * Asynchronous on `stream`: if a wait inside the tensor-core kernel runs out of time (a second; never seen), the rows that
+ * it was to write are NaN. The Gram products and the solves, which synchronise, return PC_ECUDA for that. */
 int pc_block_update(int nb, long L, int p, int q, int dtype, const void *S, long ss, const void *C, void *Y,
                     long sy, void *stream);
 

@@ -252,10 +252,10 @@ size_t gram_scratch_bytes(int nb, long L, int p, int q) {
 }
 
 int launch_gram(int nb, long L, int p, int q, int dtype, const void *A, long sa, const void *B, long sb, void *G,
-                void *scratch, size_t scratch_bytes, cudaStream_t st, const int *act, int nb_alloc, long sg) {
+                void *scratch, size_t scratch_bytes, cudaStream_t st, int *tmo, const int *act, int nb_alloc, long sg) {
   if (nb == 0 || p == 0 || q == 0) return PC_OK;
   if (dtype == PC_C64 && (p > 16 || q > 16)) {
-    const int rc = launch_gram_tc(nb, L, p, q, A, sa, B, sb, G, scratch, scratch_bytes, st, act, nb_alloc, sg);
+    const int rc = launch_gram_tc(nb, L, p, q, A, sa, B, sb, G, scratch, scratch_bytes, st, tmo, act, nb_alloc, sg);
     if (rc != PC_EUNSUPPORTED) return rc;
   }
   if (gram_scratch_bytes(nb, L, p, q) > scratch_bytes) {
@@ -265,7 +265,7 @@ int launch_gram(int nb, long L, int p, int q, int dtype, const void *A, long sa,
   if (dtype == PC_C128) {
     int c = 0;
     const int rc = launch_gram_sl(nb, L, p, q, PC_C128, A, sa, B, sb, SL_GENERAL, static_cast<double2 *>(scratch),
-                                  gram_scratch_chunks(nb, L), &c, st, act);
+                                  gram_scratch_chunks(nb, L), &c, st, tmo, act);
     if (rc) return rc;
     launch_gram_reduce(nb, c, p, q, static_cast<double2 *>(scratch), act, G, st, sg);
     PC_CK_LAUNCH();
@@ -432,7 +432,8 @@ static int launch_gram_pair_t(int nb, long L, int p, const void *S, const void *
 }
 
 int launch_gram_pair(int nb, long L, int p, int dtype, const void *S, const void *AS, long ss, void *G, void *H,
-                     void *scratch, size_t scratch_bytes, cudaStream_t st, const int *act, int nb_alloc, long sg) {
+                     void *scratch, size_t scratch_bytes, cudaStream_t st, int *tmo, const int *act, int nb_alloc,
+                     long sg) {
   if (nb == 0 || p == 0) return PC_OK;
   if (p > 64) {
     set_error("gram_pair: at most 64 columns");
@@ -443,13 +444,14 @@ int launch_gram_pair(int nb, long L, int p, int dtype, const void *S, const void
     return PC_EINVAL;
   }
   if (dtype == PC_C64) {
-    const int rc = launch_gram_pair_tc(nb, L, p, S, AS, ss, G, H, scratch, scratch_bytes, st, act, nb_alloc, sg);
+    const int rc = launch_gram_pair_tc(nb, L, p, S, AS, ss, G, H, scratch, scratch_bytes, st, tmo, act, nb_alloc, sg);
     if (rc != PC_EUNSUPPORTED) return rc;
   }
   double2 *part = static_cast<double2 *>(scratch);
   int nchunk = gram_chunks(nb, L), rc;
   if (dtype == PC_C128) {
     rc = launch_gram_sl(nb, L, p, p, PC_C128, S, ss, AS, ss, SL_PAIR, part, gram_scratch_chunks(nb, L), &nchunk, st,
+                        tmo,
                         act);
   } else {
     long chunk = (L + nchunk - 1) / nchunk;
@@ -469,16 +471,17 @@ size_t gram_pair_coupled_scratch_bytes(int nb, long L, int p, int q2) {
 
 int launch_gram_pair_coupled(int nb, long L, int p, int q2, int dtype, const void *S, const void *AS, long ss,
                              const void *R, long sr, void *G, void *H, void *RQ, void *scratch, size_t scratch_bytes,
-                             cudaStream_t st, const int *act, int nb_alloc, long sg, long srq) {
+                             cudaStream_t st, int *tmo, const int *act, int nb_alloc, long sg, long srq) {
   if (nb == 0 || p == 0) return PC_OK;
   if (dtype == PC_C64) {
     const int rc = launch_gram_pair_coupled_tc(nb, L, p, q2, S, AS, ss, R, sr, G, H, RQ, scratch, scratch_bytes, st,
+                                               tmo,
                                                act, nb_alloc, sg, srq);
     if (rc != PC_EUNSUPPORTED) return rc;
   }
-  int rc = launch_gram_pair(nb, L, p, dtype, S, AS, ss, G, H, scratch, scratch_bytes, st, act, nb_alloc, sg);
+  int rc = launch_gram_pair(nb, L, p, dtype, S, AS, ss, G, H, scratch, scratch_bytes, st, tmo, act, nb_alloc, sg);
   if (rc) return rc;
-  return launch_gram(nb, L, q2, p, dtype, R, sr, S, ss, RQ, scratch, scratch_bytes, st, act, nb_alloc, srq);
+  return launch_gram(nb, L, q2, p, dtype, R, sr, S, ss, RQ, scratch, scratch_bytes, st, tmo, act, nb_alloc, srq);
 }
 
 // ------------------------------------------------------------------------------------------------ block update
@@ -635,7 +638,8 @@ static int update_width(int q, std::initializer_list<int> widths) {
 }
 
 int launch_block_update(int nb, long L, int p, int q, int dtype, const void *S, long ss, const void *C, long sc,
-                        void *Y, long sy, cudaStream_t st, const int *act, const void *Z, long sz, bool each) {
+                        void *Y, long sy, cudaStream_t st, int *tmo, const int *act, const void *Z, long sz,
+                        bool each) {
   if (nb == 0 || q == 0) return PC_OK;
   if (p > UPD_PMAX) {
     set_error("block_update: at most 64 input columns");
@@ -645,7 +649,7 @@ int launch_block_update(int nb, long L, int p, int q, int dtype, const void *S, 
   // rows and up; `each` also where C picks single columns, 1.6 against 4.0 ms for 48 -> 16 of 8 k-points at N = 32); not
   // the addend and the sum of no columns, which no solve asks for
   if (dtype == PC_C128 && p > 0 && !Z)
-    return launch_update_sl(nb, L, p, q, PC_C128, S, ss, C, sc, Y, sy, nullptr, 0, st, act, each);
+    return launch_update_sl(nb, L, p, q, PC_C128, S, ss, C, sc, Y, sy, nullptr, 0, st, tmo, act, each);
   if (dtype == PC_C128) {
     block_update_t<double, 8>(nb, L, p, q, S, ss, C, sc, Y, sy, st, act, Z, sz);
   } else {
@@ -668,8 +672,8 @@ int launch_block_update_sum(int nb, long L, int p, int q, const void *S, const v
   if (nb == 0 || q == 0) return PC_OK;
   const uintptr_t at = (uintptr_t)S | (uintptr_t)S2 | (uintptr_t)Y;
   if (p > UPD_PMAX || q > 16 || ((L | ss | sy) & 1) || (at & 15)) {
-    const int rc = launch_block_update(nb, L, p, q, PC_C64, S, ss, C, sc, Y, sy, st, nullptr);
-    return rc ? rc : launch_block_update(nb, L, p, q, PC_C64, S2, ss, C2, sc, Y, sy, st, nullptr, Y, sy);
+    const int rc = launch_block_update(nb, L, p, q, PC_C64, S, ss, C, sc, Y, sy, st, nullptr, nullptr);
+    return rc ? rc : launch_block_update(nb, L, p, q, PC_C64, S2, ss, C2, sc, Y, sy, st, nullptr, nullptr, Y, sy);
   }
   const dim3 g((unsigned)((L / 2 + 255) / 256), 1, nb);
   auto run = [&](auto kernel) {
@@ -1178,11 +1182,14 @@ extern "C" int pc_gram(int nb, long L, int p, int q, int dtype, const void *A, l
   PC_REQUIRE(nb >= 0 && L >= 0 && p >= 0 && q >= 0 && p <= 64 && q <= 64, "pc_gram: bad sizes");
   PC_REQUIRE(dtype == PC_C128 || dtype == PC_C64, "pc_gram: bad dtype");
   DevBuf tmp;
+  TimeoutWord tmo;
   PC_CK(tmp.reserve(std::max<size_t>(16, gram_scratch_bytes(nb, L, p, q))));
-  int rc = launch_gram(nb, L, p, q, dtype, A, sa, B, sb, G, tmp.p, tmp.bytes, (cudaStream_t)stream, nullptr);
+  int rc = tmo.start();
+  if (rc) return rc;
+  rc = launch_gram(nb, L, p, q, dtype, A, sa, B, sb, G, tmp.p, tmp.bytes, (cudaStream_t)stream, tmo.word, nullptr);
   if (rc) return rc;
   PC_CK(cudaStreamSynchronize((cudaStream_t)stream));  // tmp is released on return
-  return PC_OK;
+  return tmo.check();
 }
 
 extern "C" int pc_gram_pair(int nb, long L, int p, int dtype, const void *S, long ss, const void *AS, void *G,
@@ -1191,11 +1198,14 @@ extern "C" int pc_gram_pair(int nb, long L, int p, int dtype, const void *S, lon
   PC_REQUIRE(nb >= 0 && L >= 0 && p >= 1 && p <= 64, "pc_gram_pair: bad sizes");
   PC_REQUIRE(dtype == PC_C128 || dtype == PC_C64, "pc_gram_pair: bad dtype");
   DevBuf tmp;
+  TimeoutWord tmo;
   PC_CK(tmp.reserve(std::max<size_t>(16, gram_pair_scratch_bytes(nb, L, p))));
-  int rc = launch_gram_pair(nb, L, p, dtype, S, AS, ss, G, H, tmp.p, tmp.bytes, (cudaStream_t)stream, nullptr);
+  int rc = tmo.start();
+  if (rc) return rc;
+  rc = launch_gram_pair(nb, L, p, dtype, S, AS, ss, G, H, tmp.p, tmp.bytes, (cudaStream_t)stream, tmo.word, nullptr);
   if (rc) return rc;
   PC_CK(cudaStreamSynchronize((cudaStream_t)stream));
-  return PC_OK;
+  return tmo.check();
 }
 
 extern "C" int pc_gram_pair_coupled(int nb, long L, int p, int q, const void *S, long ss, const void *AS,
@@ -1203,12 +1213,15 @@ extern "C" int pc_gram_pair_coupled(int nb, long L, int p, int q, const void *S,
   PC_REQUIRE(S && AS && R && G && H && RQ, "pc_gram_pair_coupled: null argument");
   PC_REQUIRE(nb >= 0 && L >= 0 && p >= 1 && p <= 64 && q >= 1 && q <= 64, "pc_gram_pair_coupled: bad sizes");
   DevBuf tmp;
+  TimeoutWord tmo;
   PC_CK(tmp.reserve(std::max<size_t>(16, gram_pair_coupled_scratch_bytes(nb, L, p, q))));
-  int rc = launch_gram_pair_coupled(nb, L, p, q, PC_C64, S, AS, ss, R, sr, G, H, RQ, tmp.p, tmp.bytes,
-                                    (cudaStream_t)stream, nullptr);
+  int rc = tmo.start();
+  if (rc) return rc;
+  rc = launch_gram_pair_coupled(nb, L, p, q, PC_C64, S, AS, ss, R, sr, G, H, RQ, tmp.p, tmp.bytes,
+                                    (cudaStream_t)stream, tmo.word, nullptr);
   if (rc) return rc;
   PC_CK(cudaStreamSynchronize((cudaStream_t)stream));  // tmp is released on return
-  return PC_OK;
+  return tmo.check();
 }
 
 extern "C" int pc_block_update(int nb, long L, int p, int q, int dtype, const void *S, long ss, const void *C, void *Y,
@@ -1216,7 +1229,8 @@ extern "C" int pc_block_update(int nb, long L, int p, int q, int dtype, const vo
   PC_REQUIRE(S && C && Y, "pc_block_update: null argument");
   PC_REQUIRE(nb >= 0 && L >= 0 && p >= 0 && q >= 0 && p <= 64 && q <= 64, "pc_block_update: bad sizes");
   PC_REQUIRE(dtype == PC_C128 || dtype == PC_C64, "pc_block_update: bad dtype");
-  return launch_block_update(nb, L, p, q, dtype, S, ss, C, (long)p * q, Y, sy, (cudaStream_t)stream, nullptr, nullptr, 0,
+  return launch_block_update(nb, L, p, q, dtype, S, ss, C, (long)p * q, Y, sy, (cudaStream_t)stream, nullptr, nullptr,
+                             nullptr, 0,
                              true);
 }
 

@@ -47,8 +47,6 @@ constexpr int SG_WSTRIDE = SG_WORDS + 4;      // their distance from column to c
 // a column's share of the common rows that an entry needs: ordinary, all zeros, with an infinity or a NaN
 constexpr int SG_NEED = 8, SG_ZERO = -1000, SG_BAD = 1 << 20;
 
-__device__ int g_gram_sl_error = 0;
-
 struct SlGramArgs {
   const void *A, *B;
   long sa, sb;
@@ -57,6 +55,7 @@ struct SlGramArgs {
   int nbc, nbp;  // columns per block; accumulator columns per level (2 per operand column, rounded up to 16)
   double2 *part0, *part1;
   const int *act;
+  int *tmo;
 };
 
 // TASKS: at most 32 TASKS columns to extract (each thread two rows of every 32nd column); DEPTH: stages loaded ahead
@@ -365,7 +364,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
   }
-  if (tid == 0 && *abort) atomicExch(&g_gram_sl_error, 1);
+  if (tid == 0 && *abort) report_timeout(a.tmo);
 }
 
 template <typename T> size_t sg_smem(int nbp) {
@@ -381,7 +380,7 @@ int sl_gram_chunks(int nb, long L) {
 }
 
 int launch_gram_sl(int nb, long L, int p, int q, int dtype, const void *A, long sa, const void *B, long sb, int mode,
-                   double2 *part, int maxchunk, int *nchunk, cudaStream_t st, const int *act) {
+                   double2 *part, int maxchunk, int *nchunk, cudaStream_t st, int *tmo, const int *act) {
   SlGramArgs a{};
   a.A = A;
   a.B = B;
@@ -392,6 +391,7 @@ int launch_gram_sl(int nb, long L, int p, int q, int dtype, const void *A, long 
   a.q = q;
   a.mode = mode;
   a.act = act;
+  a.tmo = tmo;
   // blocks of up to 32 operand columns (8 levels of 64 accumulator columns fill TMEM); a pair's block has two per column
   const int most_cols = mode == SL_PAIR ? 16 : 32, nblk = (q + most_cols - 1) / most_cols;
   a.nbc = (q + nblk - 1) / nblk;
@@ -436,18 +436,6 @@ int launch_gram_sl(int nb, long L, int p, int q, int dtype, const void *A, long 
   kernel<<<grid, SG_THREADS, smem, st>>>(a);
   PC_CK_LAUNCH();
   return PC_OK;
-}
-
-int sliced_check() {
-  int v = 0;
-  PC_CK(cudaMemcpyFromSymbol(&v, g_gram_sl_error, sizeof(int)));
-  if (v) {
-    const int zero = 0;
-    PC_CK(cudaMemcpyToSymbol(g_gram_sl_error, &zero, sizeof(int)));
-    set_error("sliced Gram kernel: a pipeline wait ran out of time");
-    return PC_ECUDA;
-  }
-  return update_sl_check();
 }
 
 }  // namespace pc

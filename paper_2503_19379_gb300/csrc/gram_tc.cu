@@ -36,8 +36,11 @@
 #include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdint>
 #include <cstdlib>
+#include <mutex>
+#include <vector>
 
 #include "pc_internal.cuh"
 #include "sliced.cuh"
@@ -56,8 +59,6 @@ constexpr int TC_NTR = 6;     // transform warps (2..7)
 constexpr int TC_NDR = 12;    // drain warps (8..19), three per TMEM lane quarter
 constexpr int TC_NMAX = 160;  // MMA columns: three accumulators of N columns in the 512 TMEM columns
 constexpr int TC_MAXT = 512;  // K tiles per chunk at most: the drain's FP32 running sums span <= 256 groups
-
-__device__ int g_gram_tc_error = 0;
 
 __device__ __forceinline__ void mma_tf32(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                          uint32_t accumulate) {
@@ -103,6 +104,7 @@ struct TcArgs {
   double *partG, *partH;  // pair: [nb][nchunk][p][p] double2 each; general: partH = [nb][nchunk][p][q]
   double *partQ;          // coupling block (RB > 0): R^H A as [nb][nchunk][q2][p] double2
   const int *act;
+  int *tmo;
 };
 
 __global__ void __launch_bounds__(TC_THREADS, 1) gram_tc_kernel(const TcArgs a, const __grid_constant__ CUtensorMap tmA,
@@ -370,7 +372,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) gram_tc_kernel(const TcArgs a, 
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(a.tmem_cols) : "memory");
   }
-  if (threadIdx.x == 0 && *abort) atomicExch(&g_gram_tc_error, 1);
+  if (threadIdx.x == 0 && *abort) report_timeout(a.tmo);
 }
 
 constexpr int TC_SMEM_MAX = 232448;  // opt-in shared memory per block
@@ -430,7 +432,7 @@ bool make_map(CUtensorMap *map, const void *base, long L, long rows, int box_row
 
 // pair mode with R (q2 > 0): B1 = [B; R], the coupling block R^H A written to partQ (after the G and H partials)
 int launch_tc(int nb, int nb_alloc, long L, int p, int q, bool pair, const void *A, long sa, const void *B, long sb,
-              double2 *part, size_t scratch_bytes, cudaStream_t st, const int *act, int *nchunk_out,
+              double2 *part, size_t scratch_bytes, cudaStream_t st, int *tmo, const int *act, int *nchunk_out,
               bool transpose = false, const void *R = nullptr, long sr = 0, int q2 = 0) {
   TcArgs a{};
   a.cppA = sa / L;
@@ -470,6 +472,7 @@ int launch_tc(int nb, int nb_alloc, long L, int p, int q, bool pair, const void 
   a.partH = pair ? reinterpret_cast<double *>(part + (size_t)nb * c * p * p) : reinterpret_cast<double *>(part);
   a.partQ = a.q2 > 0 ? reinterpret_cast<double *>(part + 2 * (size_t)nb * c * p * p) : nullptr;
   a.act = act;
+  a.tmo = tmo;
   static bool configured = false;
   if (!configured) {
     PC_CK(cudaFuncSetAttribute(gram_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_MAX));
@@ -520,11 +523,12 @@ int tc_min_chunks(long L) { return (int)((2 * L / TC_KT + TC_MAXT - 1) / TC_MAXT
 // G = S^H S and H = S^H AS (complex64 panels, p <= 64) on the tensor cores; PC_EUNSUPPORTED when the shape or
 // alignment does not fit (the caller then takes the CUDA-core kernel).
 int launch_gram_pair_tc(int nb, long L, int p, const void *S, const void *AS, long ss, void *G, void *H,
-                        void *scratch, size_t scratch_bytes, cudaStream_t st, const int *act, int nb_alloc, long sg) {
+                        void *scratch, size_t scratch_bytes, cudaStream_t st, int *tmo, const int *act, int nb_alloc,
+                        long sg) {
   if (!tc_shape_ok(L, p, p, S, ss, AS, ss)) return PC_EUNSUPPORTED;
   int c = 0;
   double2 *part = static_cast<double2 *>(scratch);
-  int rc = launch_tc(nb, nb_alloc > 0 ? nb_alloc : nb, L, p, p, true, S, ss, AS, ss, part, scratch_bytes, st, act,
+  int rc = launch_tc(nb, nb_alloc > 0 ? nb_alloc : nb, L, p, p, true, S, ss, AS, ss, part, scratch_bytes, st, tmo, act,
                      &c);
   if (rc) return rc;
   launch_gram_pair_reduce(nb, c, p, part, act, G, H, st, sg);
@@ -536,12 +540,12 @@ int launch_gram_pair_tc(int nb, long L, int p, const void *S, const void *AS, lo
 // rounded up <= 160 MMA columns); PC_EUNSUPPORTED as above.
 int launch_gram_pair_coupled_tc(int nb, long L, int p, int q2, const void *S, const void *AS, long ss, const void *R,
                                 long sr, void *G, void *H, void *RQ, void *scratch, size_t scratch_bytes,
-                                cudaStream_t st, const int *act, int nb_alloc, long sg, long srq) {
+                                cudaStream_t st, int *tmo, const int *act, int nb_alloc, long sg, long srq) {
   if (q2 < 1 || !tc_shape_ok(L, p, p, S, ss, AS, ss) || !tc_shape_ok(L, q2, q2, R, sr, R, sr))
     return PC_EUNSUPPORTED;
   int c = 0;
   double2 *part = static_cast<double2 *>(scratch);
-  int rc = launch_tc(nb, nb_alloc > 0 ? nb_alloc : nb, L, p, p, true, S, ss, AS, ss, part, scratch_bytes, st, act,
+  int rc = launch_tc(nb, nb_alloc > 0 ? nb_alloc : nb, L, p, p, true, S, ss, AS, ss, part, scratch_bytes, st, tmo, act,
                      &c, false, R, sr, q2);
   if (rc) return rc;
   launch_gram_pair_reduce(nb, c, p, part, act, G, H, st, sg);
@@ -553,15 +557,18 @@ int launch_gram_pair_coupled_tc(int nb, long L, int p, int q2, const void *S, co
 
 // G = A^H B (complex64, p <= 64 columns of A, q <= 128 of B) on the tensor cores; PC_EUNSUPPORTED as above.
 int launch_gram_tc(int nb, long L, int p, int q, const void *A, long sa, const void *B, long sb, void *G,
-                   void *scratch, size_t scratch_bytes, cudaStream_t st, const int *act, int nb_alloc, long sg) {
+                   void *scratch, size_t scratch_bytes, cudaStream_t st, int *tmo, const int *act, int nb_alloc,
+                   long sg) {
   if (!tc_shape_ok(L, p, q, A, sa, B, sb)) return PC_EUNSUPPORTED;
   int c = 0;
   double2 *part = static_cast<double2 *>(scratch);
   // the wider panel takes the MMA rows (2 x its columns of the 128): B^H A, written conjugate-transposed
   const bool swap = q > p && q <= 64;
   int rc = swap ? launch_tc(nb, nb_alloc > 0 ? nb_alloc : nb, L, q, p, false, B, sb, A, sa, part, scratch_bytes, st,
+                            tmo,
                             act, &c, true)
                 : launch_tc(nb, nb_alloc > 0 ? nb_alloc : nb, L, p, q, false, A, sa, B, sb, part, scratch_bytes, st,
+                            tmo,
                             act, &c);
   if (rc) return rc;
   launch_gram_reduce(nb, c, p, q, part, act, G, st, sg);
@@ -569,17 +576,56 @@ int launch_gram_tc(int nb, long L, int p, int q, const void *A, long sa, const v
   return PC_OK;
 }
 
-// reads and clears the abort flags of the tensor-core Gram kernels (after a synchronisation)
-int gram_tc_check() {
-  int v = 0;
-  PC_CK(cudaMemcpyFromSymbol(&v, g_gram_tc_error, sizeof(int)));
-  if (v) {
-    const int zero = 0;
-    PC_CK(cudaMemcpyToSymbol(g_gram_tc_error, &zero, sizeof(int)));
-    set_error("tensor-core Gram kernel: a pipeline wait ran out of time");
-    return PC_ECUDA;
+// ---------------------------------------------------------------- time-out words
+namespace {
+
+// Free words; pages of them stay until the process ends (a context may outlive the library's static objects)
+struct WordPool {
+  std::mutex mutex;
+  std::vector<int *> words;
+  std::atomic<int> inject{0};  // the start() that finds a time-out, counted from now; 0: none (pc_inject_tc_timeout)
+};
+WordPool &pool() {
+  static WordPool *p = new WordPool;
+  return *p;
+}
+constexpr int WORDS_PER_PAGE = 256;
+
+}  // namespace
+
+int TimeoutWord::start() {
+  if (!word) {
+    std::lock_guard<std::mutex> lock(pool().mutex);
+    std::vector<int *> &words = pool().words;
+    if (words.empty()) {
+      int *page = nullptr;
+      PC_CK(cudaHostAlloc(reinterpret_cast<void **>(&page), sizeof(int) * WORDS_PER_PAGE, cudaHostAllocPortable));
+      for (int i = WORDS_PER_PAGE; i-- > 0;) words.push_back(page + i);
+    }
+    word = words.back();
+    words.pop_back();
   }
-  return sliced_check();
+  int left = pool().inject.load();
+  while (left > 0 && !pool().inject.compare_exchange_weak(left, left - 1)) {
+  }
+  __atomic_store_n(word, left == 1 ? 1 : 0, __ATOMIC_RELEASE);
+  return PC_OK;
+}
+
+int TimeoutWord::check() {
+  if (!word || !__atomic_exchange_n(word, 0, __ATOMIC_ACQ_REL)) return PC_OK;
+  set_error("a tensor-core kernel's pipeline wait ran out of time");
+  return PC_ECUDA;
+}
+
+TimeoutWord::~TimeoutWord() {
+  if (!word) return;
+  std::lock_guard<std::mutex> lock(pool().mutex);
+  pool().words.push_back(word);
 }
 
 }  // namespace pc
+
+// For tests: the n-th call or solve from now that watches for a time-out finds one, whatever its kernels do (the chunks and
+// the FP64 finish of a solve count as solves).
+extern "C" void pc_inject_tc_timeout(int n) { pc::pool().inject = n; }

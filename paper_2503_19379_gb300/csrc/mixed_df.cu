@@ -622,13 +622,13 @@ int launch_op_df_resid(pc_ctx *ctx, int nb, int m, const void *X, long sx, const
 // ---------------------------------------------------------------- block update Y = X C + Z
 // On the tensor cores (update_sl.cu).
 int launch_update_df(int nb, long L, int p, int q, const void *X, long sx, const void *C, long sc, void *Y, long sy,
-                     const void *Z, long sz, cudaStream_t st, const int *act) {
+                     const void *Z, long sz, cudaStream_t st, int *tmo, const int *act) {
   if (nb == 0 || q == 0) return PC_OK;
   if (p < 1 || p > 32) {
     set_error("update_df: 1 to 32 input columns");
     return PC_EINVAL;
   }
-  return launch_update_sl(nb, L, p, q, PC_DFS, X, sx, C, sc, Y, sy, Z, sz, st, act);
+  return launch_update_sl(nb, L, p, q, PC_DFS, X, sx, C, sc, Y, sy, Z, sz, st, tmo, act);
 }
 
 // ---------------------------------------------------------------- Gram G = X^H X of the FP64 block
@@ -639,7 +639,7 @@ size_t gram_df_scratch_bytes(int nb, long L, int p) {
 }
 
 int launch_gram_df(int nb, long L, int p, const void *X, long sx, void *G, void *scratch, size_t scratch_bytes,
-                   cudaStream_t st, const int *act) {
+                   cudaStream_t st, int *tmo, const int *act) {
   if (nb == 0 || p == 0) return PC_OK;
   if (p > 32 || gram_df_scratch_bytes(nb, L, p) > scratch_bytes) {
     set_error("gram_df: at most 32 columns and enough scratch");
@@ -647,7 +647,8 @@ int launch_gram_df(int nb, long L, int p, const void *X, long sx, void *G, void 
   }
   double2 *part = static_cast<double2 *>(scratch);
   int nchunk = 0;
-  const int rc = launch_gram_sl(nb, L, p, p, PC_DFS, X, sx, X, sx, SL_SELF, part, sl_gram_chunks(nb, L), &nchunk, st, act);
+  const int rc = launch_gram_sl(nb, L, p, p, PC_DFS, X, sx, X, sx, SL_SELF, part, sl_gram_chunks(nb, L), &nchunk, st,
+                                tmo, act);
   if (rc) return rc;
   launch_gram_self_reduce(nb, nchunk, p, part, act, G, st);
   PC_CK_LAUNCH();

@@ -125,6 +125,21 @@ struct DevBuf {
 }  // namespace pc
 
 // ---------------------------------------------------------------- the context
+namespace pc {
+// Where the tensor-core kernels of one call or solve say that a bounded wait ran out (their results are then garbage):
+// a word of pinned host memory from a pool, so that looking at it after a synchronisation costs nothing and no other
+// call, stream or thread sees it. `tmo` of the launch functions below; null where nobody looks (an update writes NaN).
+struct TimeoutWord {
+  int *word = nullptr;
+  int start();  // takes a word from the pool (kept until destruction) and clears it
+  int check();  // after a synchronisation: PC_ECUDA if a wait ran out since start(); clears the word
+  TimeoutWord() = default;
+  TimeoutWord(const TimeoutWord &) = delete;
+  TimeoutWord &operator=(const TimeoutWord &) = delete;
+  ~TimeoutWord();
+};
+}  // namespace pc
+
 struct pc_ctx {
   int N = 0, logN = 0;
   long n = 0;  // N^3
@@ -154,6 +169,7 @@ struct pc_ctx {
   pc::DevBuf kparam;        // KParam [nb]
   pc::DevBuf symd;          // per-k axis symbols d_i(m) complex128 [nb][3][N]; general lattice: [nb][3][3][N]
   pc::DevBuf scratch;       // general scratch (partial sums)
+  pc::TimeoutWord tmo;      // of the solve in progress
   int kcap = 0;             // capacity (k-points) of kparam / symd
   // host tables of the axis symbols (see axis_symbols), and pinned staging of upload_kpoints
   std::vector<double> symS, symZ, symE;
@@ -247,11 +263,11 @@ int launch_precond_c64(pc_ctx *ctx, int nb, int m, const void *R, long sr, void 
 // nb_alloc: k-points in the panel arrays (the act list indexes them); <= 0 means nb.
 // sg: batch stride of the output matrices in elements; <= 0 means packed (p q, or p p for the pair).
 int launch_gram(int nb, long L, int p, int q, int dtype, const void *A, long sa, const void *B, long sb, void *G,
-                void *scratch, size_t scratch_bytes, cudaStream_t st, const int *act, int nb_alloc = -1,
+                void *scratch, size_t scratch_bytes, cudaStream_t st, int *tmo, const int *act, int nb_alloc = -1,
                 long sg = 0);
 size_t gram_scratch_bytes(int nb, long L, int p, int q);
 int launch_gram_pair(int nb, long L, int p, int dtype, const void *S, const void *AS, long ss, void *G, void *H,
-                     void *scratch, size_t scratch_bytes, cudaStream_t st, const int *act, int nb_alloc = -1,
+                     void *scratch, size_t scratch_bytes, cudaStream_t st, int *tmo, const int *act, int nb_alloc = -1,
                      long sg = 0);
 size_t gram_pair_scratch_bytes(int nb, long L, int p);
 // reductions of per-chunk partial sums ([nb][nchunk][p][q] double2; the pair: G block then H block, upper triangles)
@@ -262,25 +278,26 @@ void launch_gram_reduce(int nb, int nchunk, int p, int q, const double2 *part, c
                         cudaStream_t st, long sg = 0);
 // complex64 Gram products on the tensor cores (gram_tc.cu); PC_EUNSUPPORTED when the shape does not fit
 int launch_gram_pair_tc(int nb, long L, int p, const void *S, const void *AS, long ss, void *G, void *H,
-                        void *scratch, size_t scratch_bytes, cudaStream_t st, const int *act, int nb_alloc, long sg);
+                        void *scratch, size_t scratch_bytes, cudaStream_t st, int *tmo, const int *act, int nb_alloc,
+                        long sg);
 int launch_gram_pair_coupled_tc(int nb, long L, int p, int q2, const void *S, const void *AS, long ss, const void *R,
                                 long sr, void *G, void *H, void *RQ, void *scratch, size_t scratch_bytes,
-                                cudaStream_t st, const int *act, int nb_alloc, long sg, long srq);
+                                cudaStream_t st, int *tmo, const int *act, int nb_alloc, long sg, long srq);
 // G = S^H S, H = S^H AS (p columns) and RQ = R^H S (q2 x p) for nb k-points; one tensor-core pass for complex64
 // where the shape allows, else launch_gram_pair and launch_gram
 int launch_gram_pair_coupled(int nb, long L, int p, int q2, int dtype, const void *S, const void *AS, long ss,
                              const void *R, long sr, void *G, void *H, void *RQ, void *scratch, size_t scratch_bytes,
-                             cudaStream_t st, const int *act, int nb_alloc = -1, long sg = 0, long srq = 0);
+                             cudaStream_t st, int *tmo, const int *act, int nb_alloc = -1, long sg = 0, long srq = 0);
 size_t gram_pair_coupled_scratch_bytes(int nb, long L, int p, int q2);
 int launch_gram_tc(int nb, long L, int p, int q, const void *A, long sa, const void *B, long sb, void *G,
-                   void *scratch, size_t scratch_bytes, cudaStream_t st, const int *act, int nb_alloc, long sg);
+                   void *scratch, size_t scratch_bytes, cudaStream_t st, int *tmo, const int *act, int nb_alloc,
+                   long sg);
 // chunks per k-point that the tensor-core Gram takes at least for panels of L rows (its partial sums need that many)
 int tc_min_chunks(long L);
-// reads and clears the time-out flag of the tensor-core Gram kernel (call after a synchronisation)
-int gram_tc_check();
 // Y = S C (+ Z, a complex64 addend, if Z is not null); arithmetic in the precision of dtype
 int launch_block_update(int nb, long L, int p, int q, int dtype, const void *S, long ss, const void *C, long sc,
-                        void *Y, long sy, cudaStream_t st, const int *act, const void *Z = nullptr, long sz = 0,
+                        void *Y, long sy, cudaStream_t st, int *tmo, const int *act, const void *Z = nullptr,
+                        long sz = 0,
                         bool each = false);
 int launch_block_update_sum(int nb, long L, int p, int q, const void *S, const void *C, const void *S2, const void *C2,
                             long ss, long sc, void *Y, long sy, cudaStream_t st);
@@ -333,10 +350,10 @@ size_t op_df_resid_scratch_bytes(pc_ctx *ctx, int nb, int m);
 void launch_residual_reduce(int nb, int nchunk, int m, const double *part, const int *act, double *norms,
                             cudaStream_t st);
 int launch_update_df(int nb, long L, int p, int q, const void *X, long sx, const void *C, long sc, void *Y, long sy,
-                     const void *Z, long sz, cudaStream_t st, const int *act);
+                     const void *Z, long sz, cudaStream_t st, int *tmo, const int *act);
 // G = X^H X of a block of double-float pairs (p <= 32 columns) in double-float arithmetic, G complex128
 int launch_gram_df(int nb, long L, int p, const void *X, long sx, void *G, void *scratch, size_t scratch_bytes,
-                   cudaStream_t st, const int *act);
+                   cudaStream_t st, int *tmo, const int *act);
 size_t gram_df_scratch_bytes(int nb, long L, int p);
 // the mixed-precision LOBPCG driver (solver_mixed.cu); k-points already reduced, gammas per k-point
 // k-points whose phase 2 stalled or reached maxiter are not finished: their indices and the buffer (0 or 1 of

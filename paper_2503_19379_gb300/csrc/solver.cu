@@ -500,15 +500,17 @@ extern "C" int pc_solve(pc_ctx *ctx, int nk, const double *kpts, int nbands, dou
   ctx->fp64_finish.assign(nb, 0);
   int rc = upload_kpoints(ctx, nb, kr.data(), gam.data());
   if (rc) return rc;
+  if ((rc = ctx->tmo.start())) return rc;
   if (ctx->opts.precision == PC_PREC_MIXED) {
     std::vector<std::pair<int, int>> handover;
     rc = solve_mixed(ctx, nb, kr.data(), gam, zero, nbands, m, tol, evals, evecs, iters, resid, &handover);
-    const int tc = gram_tc_check();  // a time-out inside the tensor-core Gram kernel voids the result
+    const int tc = ctx->tmo.check();  // a time-out inside a tensor-core kernel voids the result
     if (tc) return tc;
     if (rc < 0 || handover.empty()) return rc;
     return fp64_finish(ctx, kpts, nbands, m, tol, evals, evecs, iters, resid, handover, rc);
   }
 
+  int *const tmo = ctx->tmo.word;
   const long sS = 3L * m * L;  // panel stride per k-point (elements)
   const size_t panel = sizeof(double2) * (size_t)sS * nb;
   for (int i = 0; i < 2; ++i) {
@@ -577,7 +579,7 @@ extern "C" int pc_solve(pc_ctx *ctx, int nk, const double *kpts, int nbands, dou
   // G = S^H S and H = S^H AS, Hermitian: p (p + 1) / 2 entries each, 8 flops per complex product
   auto GRAM = [&](int nbk, int p, const void *Sx, const void *ASx) {
     return run_stage(ctx, PC_STAGE_GRAM, 2, 2.0 * 8.0 * p * (p + 1) / 2.0 * Ld * nbk, 2.0 * p * Ld * cb * nbk, [&] {
-      return launch_gram_pair(nbk, L, p, PC_C128, Sx, ASx, sS, Gm, Hm, scratch, scr, st, d_act);
+      return launch_gram_pair(nbk, L, p, PC_C128, Sx, ASx, sS, Gm, Hm, scratch, scr, st, tmo, d_act);
     });
   };
   auto RR = [&](int nbk, int nn) {
@@ -586,7 +588,7 @@ extern "C" int pc_solve(pc_ctx *ctx, int nk, const double *kpts, int nbands, dou
   };
   auto UPD = [&](int nbk, int p, const void *Sx, const void *Cx, long sc, void *Y) {
     return run_stage(ctx, PC_STAGE_UPDATE, 1, 8.0 * p * m * Ld * nbk, (double)(p + m) * Ld * cb * nbk,
-                     [&] { return launch_block_update(nbk, L, p, m, PC_C128, Sx, sS, Cx, sc, Y, sS, st, d_act); });
+                     [&] { return launch_block_update(nbk, L, p, m, PC_C128, Sx, sS, Cx, sc, Y, sS, st, tmo, d_act); });
   };
   auto DEFL = [&](int nbk, void *X) {
     return run_stage(ctx, PC_STAGE_OTHER, 1, 4.0 * Ld * m * nbk, 2.0 * Ld * cb * m * nbk,
@@ -621,6 +623,7 @@ extern "C" int pc_solve(pc_ctx *ctx, int nk, const double *kpts, int nbands, dou
     PC_CK(cudaMemcpyAsync(h_theta.data(), theta, sizeof(double) * nb * m, cudaMemcpyDeviceToHost, st));
     PC_CK(cudaMemcpyAsync(h_norms.data(), norms, sizeof(double) * nb * m * 2, cudaMemcpyDeviceToHost, st));
     PC_CK(cudaStreamSynchronize(st));
+    if ((rc = ctx->tmo.check())) return rc;
     if ((rc = harvest_timing(ctx))) return rc;
     if (verbose) {
       for (int b : act) {
@@ -750,6 +753,7 @@ extern "C" int pc_solve(pc_ctx *ctx, int nk, const double *kpts, int nbands, dou
   }
 #undef RUN
   PC_CK(cudaStreamSynchronize(st));
+  if ((rc = ctx->tmo.check())) return rc;
   if (iters)
     for (int b = 0; b < nb; ++b) iters[b] = itcount[b];
   return status;

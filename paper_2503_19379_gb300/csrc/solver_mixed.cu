@@ -178,12 +178,14 @@ class MixedSolve {
     RUN(DEFL(g.act, S.F[0], sF, PC_C64));
     RUN(OP32(na, m, S.F[0], sF, S.AF[0], sF));
     RUN(run_stage(ctx, PC_STAGE_GRAM, 2, 8.0 * m * (m + 1) * S.Ld * na, 2.0 * m * S.Ld * 8.0 * na, [&] {
-      return launch_gram_pair(na, L, m, PC_C64, S.F[0], S.AF[0], sF, S.Gm, S.Hm, g.scratch, S.scr, g.st, g.d_act, nb,
+      return launch_gram_pair(na, L, m, PC_C64, S.F[0], S.AF[0], sF, S.Gm, S.Hm, g.scratch, S.scr, g.st,
+                              ctx->tmo.word, g.d_act, nb,
                               S.sG);
     }));
     RUN(RR(na, m, false));
     RUN(run_stage(ctx, PC_STAGE_UPDATE, 1, 8.0 * m * m * S.Ld * na, 2.0 * m * S.Ld * 8.0 * na, [&] {
-      return launch_block_update(na, L, m, m, PC_C64, S.F[0], sF, S.coef, S.sC, S.F[1], sF, g.st, g.d_act);
+      return launch_block_update(na, L, m, m, PC_C64, S.F[0], sF, S.coef, S.sC, S.F[1], sF, g.st, ctx->tmo.word,
+                                 g.d_act);
     }));
     RUN(OP32(na, m, S.F[1], sF, S.AF[1], sF));
     g.cur = 1;
@@ -399,7 +401,8 @@ class MixedSolve {
     RUN(run_stage(ctx, PC_STAGE_GRAM, 3, 8.0 * (nc * (nc + 1) + m * nc) * S.Ld * na,
                   (2.0 * nc + m) * S.Ld * 8.0 * na, [&] {
                     return launch_gram_pair_coupled(na, L, nc, m, PC_C64, S.F[cur], S.AF[cur], sF, S.R32, sX, S.Gm,
-                                                    S.Hm, S.RQ, g.scratch, S.scr, g.st, g.d_act, nb, S.sG, S.sRS);
+                                                    S.Hm, S.RQ, g.scratch, S.scr, g.st, ctx->tmo.word, g.d_act, nb,
+                                                    S.sG, S.sRS);
                   }));
     act1.clear();
     act2.clear();
@@ -408,7 +411,7 @@ class MixedSolve {
       RUN(set_act(act2));
       const int n2 = (int)act2.size();
       RUN(run_stage(ctx, PC_STAGE_DFLOAT, 2, 4.0 * m * (m + 1) * S.Ld * n2, m * S.Ld * 16.0 * n2, [&] {
-        return launch_gram_df(n2, L, m, S.X64[cur], sX, S.GX, g.scratch, S.scr, g.st, g.d_act);
+        return launch_gram_df(n2, L, m, S.X64[cur], sX, S.GX, g.scratch, S.scr, g.st, ctx->tmo.word, g.d_act);
       }));
       RUN(set_act(g.act));
     }
@@ -416,14 +419,15 @@ class MixedSolve {
     // ---- P' = [W P] coef_{W,P} (complex64), then X' per phase
     RUN(run_stage(ctx, PC_STAGE_UPDATE, 1, 8.0 * nq * m * S.Ld * na, (double)(nq + m) * S.Ld * 8.0 * na, [&] {
       return launch_block_update(na, L, nq, m, PC_C64, S.F[cur] + (long)m * L, sF, S.coef + (long)m * m, S.sC,
-                                 S.F[nxt] + 2L * m * L, sF, g.st, g.d_act);
+                                 S.F[nxt] + 2L * m * L, sF, g.st, ctx->tmo.word, g.d_act);
     }));
     if (!act1.empty()) {
       RUN(set_act(act1));
       const int n1 = (int)act1.size();
       // X' = X C_X + P' (the P' just formed is [W P] C_{W,P}): reads 2m columns instead of the 3m of [X W P]
       RUN(run_stage(ctx, PC_STAGE_UPDATE, 1, 8.0 * m * m * S.Ld * n1, 3.0 * m * S.Ld * 8.0 * n1, [&] {
-        return launch_block_update(n1, L, m, m, PC_C64, S.F[cur], sF, S.coef, S.sC, S.F[nxt], sF, g.st, g.d_act,
+        return launch_block_update(n1, L, m, m, PC_C64, S.F[cur], sF, S.coef, S.sC, S.F[nxt], sF, g.st, ctx->tmo.word,
+                                   g.d_act,
                                    S.F[nxt] + 2L * m * L, sF);
       }));
       RUN(DEFL(act1, S.F[nxt], sF, PC_C64));
@@ -434,7 +438,7 @@ class MixedSolve {
       const int n2 = (int)act2.size();
       RUN(run_stage(ctx, PC_STAGE_DFLOAT, 1, 8.0 * m * m * S.Ld * n2, (2.0 * 16.0 + 8.0) * m * S.Ld * n2, [&] {
         return launch_update_df(n2, L, m, m, S.X64[cur], sX, S.coef, S.sC, S.X64[nxt], sX,
-                                S.F[nxt] + 2L * m * L, sF, g.st, g.d_act);
+                                S.F[nxt] + 2L * m * L, sF, g.st, ctx->tmo.word, g.d_act);
       }));
       RUN(DEFL(act2, S.X64[nxt], sX, PC_DFS));
       RUN(OP64R(n2, S.X64[nxt], nxt));

@@ -57,6 +57,12 @@ __device__ inline bool bar_wait(uint32_t bar, uint32_t parity, volatile int *abo
     }
   }
 }
+// a wait ran out: told to the host through a word of pinned memory (null: the call has none)
+__device__ __forceinline__ void report_timeout(int *word) {
+  if (!word) return;
+  *(volatile int *)word = 1;
+  __threadfence_system();
+}
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(

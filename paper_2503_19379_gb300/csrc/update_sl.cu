@@ -48,8 +48,6 @@ constexpr int SU_COLS = 16;  // columns per stage
 constexpr int SU_BAD = 1 << 20;
 constexpr int SU_SLACK = 5;  // most bits between an output's largest term and its row's (launch_update_sl)
 
-__device__ int g_update_sl_error = 0;
-
 struct SlUpdateArgs {
   const void *S;
   long ss;
@@ -64,6 +62,7 @@ struct SlUpdateArgs {
   int slack;
   uint32_t tmem_cols;
   const int *act;
+  int *tmo;
 };
 
 // four consecutive accumulator columns of this warp's lanes, without waiting
@@ -487,7 +486,20 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(a.tmem_cols) : "memory");
   }
-  if (tid == 0 && *abort) atomicExch(&g_update_sl_error, 1);
+  if (*abort) {
+    // nothing of this CTA can be trusted
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+    for (long tile = blockIdx.x; tile < a.ntile; tile += gridDim.x) {
+      const long l = tile * 128 + r;
+      for (int j = g; j < nbc && l < L; j += 4) {
+        if constexpr (F64)
+          Yb[(long)j * L + l] = make_double2(nan, nan);
+        else
+          Yb[(long)j * L + l] = make_float4((float)nan, (float)nan, (float)nan, (float)nan);
+      }
+    }
+    if (tid == 0) report_timeout(a.tmo);
+  }
 }
 
 template <typename T, int NS, bool EACH = false>
@@ -533,7 +545,7 @@ int launch_su(SlUpdateArgs a, int nb, cudaStream_t st) {
 }  // namespace
 
 int launch_update_sl(int nb, long L, int p, int q, int dtype, const void *S, long ss, const void *C, long sc, void *Y,
-                     long sy, const void *Z, long sz, cudaStream_t st, const int *act, bool each) {
+                     long sy, const void *Z, long sz, cudaStream_t st, int *tmo, const int *act, bool each) {
   SlUpdateArgs a{};
   a.S = S;
   a.ss = ss;
@@ -547,6 +559,7 @@ int launch_update_sl(int nb, long L, int p, int q, int dtype, const void *S, lon
   a.p = p;
   a.q = q;
   a.act = act;
+  a.tmo = tmo;
   if (dtype == PC_DFS) return p <= SU_COLS ? launch_su<float4, 1>(a, nb, st) : launch_su<float4, 2>(a, nb, st);
   // EACH: the error of a digit product is 2^-60.2 sqrt(2 p) (rms) of the largest term that a row of S and a column of C
   // could form. An output with a term within 2^slack of that is off by 2^-54 of its own terms, no more than FP64 sums. The
@@ -559,18 +572,6 @@ int launch_update_sl(int nb, long L, int p, int q, int dtype, const void *S, lon
     case 3: return each ? launch_su<double2, 3, true>(a, nb, st) : launch_su<double2, 3>(a, nb, st);
     default: return each ? launch_su<double2, 4, true>(a, nb, st) : launch_su<double2, 4>(a, nb, st);
   }
-}
-
-int update_sl_check() {
-  int v = 0;
-  PC_CK(cudaMemcpyFromSymbol(&v, g_update_sl_error, sizeof(int)));
-  if (v) {
-    const int zero = 0;
-    PC_CK(cudaMemcpyToSymbol(g_update_sl_error, &zero, sizeof(int)));
-    set_error("sliced update kernel: a pipeline wait ran out of time");
-    return PC_ECUDA;
-  }
-  return PC_OK;
 }
 
 }  // namespace pc

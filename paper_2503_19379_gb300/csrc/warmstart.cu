@@ -744,9 +744,9 @@ extern "C" int pc_ws_backward(int N, int nb, int S, const float *params, const f
   const size_t gbytes = std::max<size_t>(16, gram_scratch_bytes(S, L, nb, nb));
   const long sx = (long)nb * L;
   // subspace loss and its gradient in X
-  rc = launch_gram(S, L, nb, nb, PC_C64, X, sx, X, sx, G, gscr, gbytes, st, nullptr);
+  rc = launch_gram(S, L, nb, nb, PC_C64, X, sx, X, sx, G, gscr, gbytes, st, nullptr, nullptr);
   if (rc) return rc;
-  rc = launch_gram(S, L, nb, nb, PC_C64, X, sx, V, sx, B, gscr, gbytes, st, nullptr);
+  rc = launch_gram(S, L, nb, nb, PC_C64, X, sx, V, sx, B, gscr, gbytes, st, nullptr, nullptr);
   if (rc) return rc;
   loss_kernel<<<S, NBMAX * NBMAX, 0, st>>>(G, B, y, lam, w_val, nb, S, dloss, Cx, Cv, dy);
   PC_CK_LAUNCH();
