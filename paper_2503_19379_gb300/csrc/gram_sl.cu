@@ -18,12 +18,15 @@
 // a column is within two bits of its largest are marked while the digits are formed, and an entry whose columns share too
 // few of them is formed in plain FP64 for this span, as are those of a column with an infinity or a NaN (`unserved`).
 //
+// Every wait is bounded. A warp whose wait runs out, or that finds the abort flag set, leaves its stages; at the end of
+// the span all roles leave together, the MMAs in flight are waited for, and the host is told (TimeoutWord).
+//
 // Complex128 panels take seven digits in eight levels, which leaves less error than the FP64 sums they replace, in every
 // entry of G and H (against extended precision, N = 8 to 32, smooth and random panels; seven levels left up to 1.8 times
 // more off the diagonal). Pairs take seven digits of base 128: 1e-15 of the diagonal, the double-float sums 3e-14.
 //
 // Bound: the latency of a stage (load, digits, hand-off to the tensor core, drain), then integer instructions of the digit
-// extraction. 8 k-points x 48 complex128 columns at N = 32: 23.6 ms on the FP64 pipe, 2.03 ms here (without the scan
+// extraction. 8 k-points x 48 complex128 columns at N = 32: 23.6 ms on the FP64 pipe, 2.06 ms here (without the scan
 // 0.3 ms less, without the MMAs 0.4 ms, without the drains 0.2 ms, without the marks and their comparison 0.1 ms); one k-point of 24 columns at N = 16: 1.77 ms and
 // 64 us. X^H X of 4 k-points x 19 pair columns at N = 64: 1.61 ms in double-float arithmetic, 1.11 ms here; of one
 // k-point x 13 at N = 16: 60 and 24 us. The pair A^H A, A^H B takes the block's columns of A and of B in one CTA, and the
@@ -80,7 +83,8 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
   unsigned *const sMask = reinterpret_cast<unsigned *>(sNeed + 96);  // complex128: rows within 2 bits of the column's largest
   const uint32_t off_bar = off_e + sg_col_bytes<T>();
   const uint32_t bars = base + off_bar;
-  uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(sm + off_bar + 16);
+  const uint32_t ready = bars + 16u;  // by operand buffer: bars, its MMAs are done; ready, its digits are there
+  uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(sm + off_bar + 32);
   volatile int *abort = reinterpret_cast<volatile int *>(tmem_holder + 1);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -106,6 +110,8 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
   if (tid == 0) {
     bar_init(bars, 1);
     bar_init(bars + 8u, 1);
+    bar_init(ready, SG_CONV / 32);
+    bar_init(ready + 8u, SG_CONV / 32);
     *abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -166,6 +172,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
   };
 
   int n = 0;  // stages issued
+  bool live = true;  // no wait of this warp has run out
   for (int sp = 0; sp < nspan; ++sp) {
     const long span0 = (st0 + sp * cst / nspan) * SG_ROWS, span1 = min(L, (st0 + (sp + 1) * cst / nspan) * SG_ROWS);
     for (int c = warp; c < ncols; c += SG_THREADS / 32) {
@@ -188,7 +195,10 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
     if (issuer) {
       for (int s = 0; s < ns; ++s, ++n) {
         const int buf = n & 1;
-        named_sync(1 + buf, SG_THREADS);
+        if (!warp_wait(ready + 8u * buf, (n >> 1) & 1, abort)) {
+          live = false;
+          break;
+        }
         if (elect_one()) {
           tc_fence_after();
 #pragma unroll
@@ -219,13 +229,16 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
       for (int d = 0; d < DEPTH; ++d)
 #pragma unroll
         for (int k = 0; k < TASKS; ++k) load(ring[d][k], k, d);
-      for (int s0 = 0; s0 < ns; s0 += DEPTH)
+      for (int s0 = 0; s0 < ns && live; s0 += DEPTH)
 #pragma unroll
       for (int dd = 0; dd < DEPTH; ++dd) {
         const int s = s0 + dd;
         if (s >= ns) break;
         const int buf = n & 1;
-        if (n >= 2) bar_wait(bars + 8u * buf, ((n >> 1) & 1) ^ 1, abort);
+        if (n >= 2 && !warp_wait(bars + 8u * buf, ((n >> 1) & 1) ^ 1, abort)) {
+          live = false;
+          break;
+        }
 #pragma unroll
         for (int k = 0; k < TASKS; ++k) {
           const int c = c0 + 32 * k, E = c < ncols ? sE[c] : SL_NONFINITE;
@@ -276,10 +289,14 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
         }
         fence_proxy_async();
         tc_fence_before();
-        named_arrive(1 + buf, SG_THREADS);
+        __syncwarp();
+        if (lane == 0) bar_arrive(ready + 8u * buf);
         ++n;
         if ((s & (GROUP - 1)) == GROUP - 1 || s == ns - 1) {
-          bar_wait(bars + 8u * buf, ((n - 1) >> 1) & 1, abort);
+          if (!warp_wait(bars + 8u * buf, ((n - 1) >> 1) & 1, abort)) {
+            live = false;
+            break;
+          }
           tc_fence_after();
           if (drains) {
 #pragma unroll
@@ -300,7 +317,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
       }
       // the span's sums, but for the entries that the digits do not serve
       unsigned plain = 0;
-      if constexpr (EACH) named_sync(3, SG_CONV);  // (the masks)
+      if constexpr (EACH) named_sync(1, SG_CONV);  // (the masks)
       if (drains) plain = unserved(ns);
       if (drains && ci < pa) {
         const int EA = sE[ci];
@@ -342,7 +359,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
         }
       }
     }
-    __syncthreads();
+    if (__syncthreads_or(!live)) break;  // all roles leave together
   }
   if (drains && ci < pa) {
     const long o = ((long)bi * gridDim.x + blockIdx.x) * a.p * a.q;
@@ -357,7 +374,8 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
         reinterpret_cast<double *>(part + o + (long)ci * a.q + j)[odd] = acc[k * SG_CONV + tid];
     }
   }
-  if (issuer && lane == 0 && *abort && n > 0) bar_wait(bars + 8u * ((n - 1) & 1), ((n - 1) >> 1) & 1, abort, false);
+  // on abort: the MMAs in flight (the issuer counts those that it issued)
+  if (issuer && *abort && n > 0) warp_wait(bars + 8u * ((n - 1) & 1), ((n - 1) >> 1) & 1, abort, false);
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {

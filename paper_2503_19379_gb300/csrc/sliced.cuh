@@ -245,9 +245,6 @@ __device__ __forceinline__ void sl_mma_step(uint32_t tmem, uint32_t a, uint32_t 
   }
 }
 
-__device__ __forceinline__ void named_arrive(int id, int count) {
-  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
-}
 __device__ __forceinline__ void named_sync(int id, int count) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }

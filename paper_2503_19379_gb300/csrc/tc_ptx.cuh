@@ -57,6 +57,10 @@ __device__ inline bool bar_wait(uint32_t bar, uint32_t parity, volatile int *abo
     }
   }
 }
+// bar_wait by a whole warp: the same answer in every lane
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int *abort, bool honour_abort = true) {
+  return __all_sync(0xffffffffu, bar_wait(bar, parity, abort, honour_abort));
+}
 // a wait ran out: told to the host through a word of pinned memory (null: the call has none)
 __device__ __forceinline__ void report_timeout(int *word) {
   if (!word) return;

@@ -19,6 +19,8 @@
 // FP64 pipe retires about 2 operations per clock and SM).
 //
 // A tile's first two stages are converted before the epilogue of the tile before it, so that the MMAs run meanwhile.
+// Every wait is bounded. A warp whose wait runs out, or that finds the abort flag set, does nothing more; all leave
+// together at the next tile, wait for the MMAs in flight and write NaN over the CTA's rows.
 //
 // Complex128 takes eight digits (the error against extended precision is 4.7e-17 of the result, that of FP64 sums 1.3e-16
 // to 3.4e-16; seven digits left 1.1e-15). Pairs take eight digits of base 128 (2.5e-15, the double-float sums 2.0e-14;
@@ -100,7 +102,8 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
   uint2 *const sNear = reinterpret_cast<uint2 *>(sM + 1536);
   const uint32_t off_bar = off_e + (uint32_t)(1536 + 128 + su_each_words(EACH)) * 4u;
   const uint32_t bars = base + off_bar;
-  uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(sm + off_bar + 16);
+  const uint32_t ready = bars + 16u;  // bars: the MMAs of an operand buffer are done; ready: digits are there, in turn
+  uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(sm + off_bar + 32);
   volatile int *abort = reinterpret_cast<volatile int *>(tmem_holder + 1);
   volatile int *badC = abort + 1;
 
@@ -119,6 +122,8 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
   if (tid == 0) {
     bar_init(bars, 1);
     bar_init(bars + 8u, 1);
+    bar_init(ready, SU_THREADS / 32);
+    bar_init(ready + 8u, SU_THREADS / 32);
     *abort = 0;
     *badC = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -233,9 +238,12 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
       }
     }
   };
+  bool live = true;  // no wait of this warp has run out; the steps below do nothing after that
+  int nready = 0, issued = -1;  // arrivals on `ready`; the last stage whose MMAs this warp issued
   auto convert = [&](int s, int n, long tile, int ex) {
     const int buf = n & 1;
-    if (n >= 2) bar_wait(bars + 8u * buf, ((n >> 1) & 1) ^ 1, abort);
+    if (live && n >= 2) live = warp_wait(bars + 8u * buf, ((n >> 1) & 1) ^ 1, abort);
+    if (!live) return;
     unsigned char *o = sm + r * 128 + (((buf * 4 + g) ^ (r & 7)) << 4);
     if constexpr (F64) {
       unsigned long long m[8];
@@ -277,9 +285,15 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
   };
   // the MMAs of stages s0 .. s1 - 1 (converted by all threads), the first of them the n-th
   auto issue = [&](int s0, int s1, int n) {
+    if (!live) return;
     tc_fence_before();
+    __syncwarp();
+    const uint32_t bar = ready + 8u * (nready & 1), phase = (nready >> 1) & 1;
+    if (lane == 0) bar_arrive(bar);
+    ++nready;
     if (warp == 0) {
-      named_sync(1 + (n & 1), SU_THREADS);
+      if (!(live = warp_wait(bar, phase, abort))) return;
+      issued = n + s1 - s0 - 1;
       if (elect_one()) {
         tc_fence_after();
         for (int s = s0; s < s1; ++s) {
@@ -291,8 +305,6 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
         }
       }
       __syncwarp();
-    } else {
-      named_arrive(1 + (n & 1), SU_THREADS);
     }
   };
   // This warp's columns of Y: 2 slot + 8 it, and the next
@@ -358,7 +370,8 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
   };
   // the tile whose n-th stage was its last
   auto epilogue = [&](long tile, int n, int par) {
-    bar_wait(bars + 8u * (n & 1), (n >> 1) & 1, abort);
+    if (live) live = warp_wait(bars + 8u * (n & 1), (n >> 1) & 1, abort);
+    if (!live) return;
     tc_fence_after();
     // epilogue: lane = row, four accumulator columns (two columns of Y) at a time
     const int row = quarter * 32 + lane;
@@ -440,7 +453,7 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
       }
     }
     sE[par * 512 + g * 128 + r] = ex;
-    __syncthreads();
+    if (__syncthreads_or(!live)) break;  // all warps leave together
 #pragma unroll
     for (int k = 0; k < 4; ++k) ex = max(ex, sE[par * 512 + k * 128 + r]);
     if constexpr (EACH) {
@@ -473,13 +486,12 @@ __global__ void __launch_bounds__(SU_THREADS, 1) update_sl_kernel(const SlUpdate
     ppar = par;
     par = par == 2 ? 0 : par + 1;
   }
-  if (EACH) __syncthreads();  // (sM of the last tile)
-  if (prev >= 0) {
+  if (!__syncthreads_or(!live) && prev >= 0) {  // (and sM of the last tile)
     load_z(prev);
     epilogue(prev, n - 1, ppar);
   }
   __syncwarp();
-  if (tid == 0 && *abort && n > 0) bar_wait(bars + 8u * ((n - 1) & 1), ((n - 1) >> 1) & 1, abort, false);
+  if (warp == 0 && *abort && issued >= 0) warp_wait(bars + 8u * (issued & 1), (issued >> 1) & 1, abort, false);
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
