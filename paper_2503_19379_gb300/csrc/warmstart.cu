@@ -207,8 +207,9 @@ __global__ void __launch_bounds__(TPB) pool_value_kernel(const float *__restrict
 
 // X[s][b][comp][i] = periodic linear interpolation of the coarse block: along each axis fine point i = 4 j + r takes
 // (1 - r/4) c_j + (r/4) c_{j+1}. A thread forms the four fine points of one coarse x: eight coarse values for four
-// points, two 16-byte stores. Bound: HBM writes (62 us with one point a thread at 16 samples x 8 bands, N = 32).
+// points, two 16-byte stores (WIDE: X is 16-byte aligned; else four of 8 bytes). Bound: HBM writes (62 us with one point a thread at 16 samples x 8 bands, N = 32).
 // grid (ceil(N^3 / 1024), 3 nb, S)
+template <bool WIDE>
 __global__ void __launch_bounds__(TPB) upsample_kernel(const float2 *__restrict__ coarse, float2 *__restrict__ X,
                                                        int logN) {
   const int N = 1 << logN, M = N >> 2, logM = logN - 2;
@@ -237,9 +238,14 @@ __global__ void __launch_bounds__(TPB) upsample_kernel(const float2 *__restrict_
     }
     out[r] = acc;
   }
-  float4 *o = reinterpret_cast<float4 *>(X + col * n + i);
-  o[0] = make_float4(out[0].x, out[0].y, out[1].x, out[1].y);
-  o[1] = make_float4(out[2].x, out[2].y, out[3].x, out[3].y);
+  if constexpr (WIDE) {
+    float4 *o = reinterpret_cast<float4 *>(X + col * n + i);
+    o[0] = make_float4(out[0].x, out[0].y, out[1].x, out[1].y);
+    o[1] = make_float4(out[2].x, out[2].y, out[3].x, out[3].y);
+  } else {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) X[col * n + i + r] = out[r];
+  }
 }
 
 // ------------------------------------------------------------------------------------------------------ loss
@@ -706,8 +712,8 @@ extern "C" int pc_ws_forward(int N, int nb, int S, const float *params, const fl
   PC_CK_LAUNCH();
   pool_value_kernel<<<S, TPB, 0, st>>>(z, params, of, dphi, nb, m3, pool, y);
   PC_CK_LAUNCH();
-  upsample_kernel<<<dim3((unsigned)((n / 4 + TPB - 1) / TPB), 3 * nb, S), TPB, 0, st>>>(coarse, static_cast<float2 *>(X),
-                                                                                   logN);
+  const auto upsample = reinterpret_cast<uintptr_t>(X) & 15 ? upsample_kernel<false> : upsample_kernel<true>;
+  upsample<<<dim3((unsigned)((n / 4 + TPB - 1) / TPB), 3 * nb, S), TPB, 0, st>>>(coarse, static_cast<float2 *>(X), logN);
   PC_CK_LAUNCH();
   PC_CK(cudaStreamSynchronize(st));  // the host copy of phi goes out of scope
   return PC_OK;
