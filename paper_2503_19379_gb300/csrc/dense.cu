@@ -173,53 +173,61 @@ __global__ void __launch_bounds__(RED_X *RED_Y) gram_reduce_kernel(const double2
 }
 
 // Narrow complex64 products (p, q <= 16): 8 x 8 tiles of outputs, a thread holding 8 x 4 of them for its rows (threads
-// 0-127 the first four columns of B, 128-255 the others). The sums of a thread (about 20 rows) are FP32, added over the
-// lanes in FP32 and over the warps and chunks in FP64. Bound: HBM. The tensor-core kernel's hand-offs per K tile cost
+// 0-127 the first four columns of B, 128-255 the others). A thread sums 64 rows in FP32; these are added over the lanes in
+// FP32 and from there on (over the batches of 64 rows, the warps and the chunks) in FP64, whatever the length of a chunk.
+// Bound: HBM. The tensor-core kernel's hand-offs per K tile cost
 // the same for narrow panels as for wide ones: 16 samples x 8 columns at N = 32, 317 us there.
 // grid (nchunk, tiles of p x tiles of q, nb)
-constexpr int GN_T = 8;
+constexpr int GN_T = 8, GN_ROWS = 64 * 128;  // rows of a block between two transfers to FP64
 
 __global__ void __launch_bounds__(256, 2) gram_narrow_kernel(const float2 *__restrict__ A, long sa,
                                                              const float2 *__restrict__ B, long sb, long L, int p, int q,
                                                              long chunk, double2 *__restrict__ part,
                                                              const int *__restrict__ act) {
-  __shared__ float red[8][64];
+  __shared__ double red[8][64];
   const int bi = blockIdx.z, b = act ? act[bi] : bi;
   const int tq = (q + GN_T - 1) / GN_T, i0 = (int)blockIdx.y / tq * GN_T, jt = (int)blockIdx.y % tq * GN_T;
   const int half = threadIdx.x >> 7, j0 = jt + 4 * half, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float2 *Ab = A + (long)b * sa + (long)i0 * L, *Bb = B + (long)b * sb;
   const int np = min(GN_T, p - i0), nq = min(4, q - j0);  // (nq <= 0: nothing of this half is wanted)
-  float acc[64];  // (i, j, part): 8 i + 2 j + part
-#pragma unroll
-  for (int u = 0; u < 64; ++u) acc[u] = 0.f;
   const long beg = (long)blockIdx.x * chunk, end = min(L, beg + chunk);
-  for (long l = beg + (threadIdx.x & 127); l < end; l += 128) {
-    float2 a[GN_T], v[4];
+  double sum0 = 0.0, sum1 = 0.0;  // of the warp: entries 2 lane and 2 lane + 1
+  for (long b0 = beg; b0 < end; b0 += GN_ROWS) {
+    float acc[64];  // (i, j, part): 8 i + 2 j + part
 #pragma unroll
-    for (int i = 0; i < GN_T; ++i) a[i] = i < np ? Ab[(long)i * L + l] : make_float2(0.f, 0.f);
+    for (int u = 0; u < 64; ++u) acc[u] = 0.f;
+    const long stop = min(end, b0 + GN_ROWS);
+#pragma unroll 1
+    for (long l = b0 + (threadIdx.x & 127); l < stop; l += 128) {
+      float2 a[GN_T], v[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) v[j] = j < nq ? Bb[(long)(j0 + j) * L + l] : make_float2(0.f, 0.f);
+      for (int i = 0; i < GN_T; ++i) a[i] = i < np ? Ab[(long)i * L + l] : make_float2(0.f, 0.f);
 #pragma unroll
-    for (int i = 0; i < GN_T; ++i)
+      for (int j = 0; j < 4; ++j) v[j] = j < nq ? Bb[(long)(j0 + j) * L + l] : make_float2(0.f, 0.f);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float &x = acc[8 * i + 2 * j], &y = acc[8 * i + 2 * j + 1];
-        x = fmaf(a[i].x, v[j].x, fmaf(a[i].y, v[j].y, x));
-        y = fmaf(a[i].x, v[j].y, fmaf(-a[i].y, v[j].x, y));
-      }
-  }
-  // lane l of the warp ends with the warp's sums 2 l and 2 l + 1: each step halves the entries a lane holds
+      for (int i = 0; i < GN_T; ++i)
 #pragma unroll
-  for (int w = 16, cnt = 32; w > 0; w >>= 1, cnt >>= 1) {
-    const bool up = lane & w;
-#pragma unroll
-    for (int u = 0; u < cnt; ++u) {
-      const float give = up ? acc[u] : acc[u + cnt], keep = up ? acc[u + cnt] : acc[u];
-      acc[u] = keep + __shfl_xor_sync(0xffffffffu, give, w);
+        for (int j = 0; j < 4; ++j) {
+          float &x = acc[8 * i + 2 * j], &y = acc[8 * i + 2 * j + 1];
+          x = fmaf(a[i].x, v[j].x, fmaf(a[i].y, v[j].y, x));
+          y = fmaf(a[i].x, v[j].y, fmaf(-a[i].y, v[j].x, y));
+        }
     }
+    // lane l of the warp ends with the warp's sums 2 l and 2 l + 1: each step halves the entries a lane holds
+#pragma unroll
+    for (int w = 16, cnt = 32; w > 0; w >>= 1, cnt >>= 1) {
+      const bool up = lane & w;
+#pragma unroll
+      for (int u = 0; u < cnt; ++u) {
+        const float give = up ? acc[u] : acc[u + cnt], keep = up ? acc[u + cnt] : acc[u];
+        acc[u] = keep + __shfl_xor_sync(0xffffffffu, give, w);
+      }
+    }
+    sum0 += (double)acc[0];
+    sum1 += (double)acc[1];
   }
-  red[warp][2 * lane] = acc[0];
-  red[warp][2 * lane + 1] = acc[1];
+  red[warp][2 * lane] = sum0;
+  red[warp][2 * lane + 1] = sum1;
   __syncthreads();
   if ((threadIdx.x & 127) < 32) {
     const int e = threadIdx.x & 31, i = e >> 2, j = e & 3;  // complex output (i, j) of this half
@@ -227,8 +235,8 @@ __global__ void __launch_bounds__(256, 2) gram_narrow_kernel(const float2 *__res
       double x = 0.0, y = 0.0;
 #pragma unroll
       for (int w = 0; w < 4; ++w) {
-        x += (double)red[4 * half + w][2 * e];
-        y += (double)red[4 * half + w][2 * e + 1];
+        x += red[4 * half + w][2 * e];
+        y += red[4 * half + w][2 * e + 1];
       }
       part[((long)bi * gridDim.x + blockIdx.x) * p * q + (i0 + i) * q + j0 + j] = make_double2(x, y);
     }
