@@ -188,8 +188,17 @@ __global__ void __launch_bounds__(TPB) pool_value_kernel(const float *__restrict
   __shared__ float sp[C2];
   const int s = blockIdx.x, lane = threadIdx.x & 31;
   for (int c = threadIdx.x >> 5; c < C2; c += TPB / 32) {  // one warp per channel
-    float acc = 0.0f;
-    for (long q = lane; q < m3; q += 32) acc += z[((long)s * C2 + c) * m3 + q];
+    // eight sums a lane (256 | m3 from N = 32; 64 points at N = 16): short FP32 chains, loads in flight
+    float part[8] = {};
+    for (long q = lane; q < m3; q += 256)
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (q + 32 * k < m3) part[k] += z[((long)s * C2 + c) * m3 + q + 32 * k];
+#pragma unroll
+    for (int h = 4; h; h >>= 1)
+#pragma unroll
+      for (int k = 0; k < h; ++k) part[k] += part[k + h];
+    float acc = part[0];
 #pragma unroll
     for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (lane == 0) sp[c] = acc / (float)m3;
