@@ -10,11 +10,16 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("nb,p,L", [(1300, 2, 98304), (64, 4, 786432), (1, 9, 64), (3, 16, 8193)])
-def test_long_narrow_panels(nb, p, L):
+@pytest.fixture(scope="module")
+def pcmod():
     from paper_2503_19379_gb300 import build as b
     b.build()
-    import paper_2503_19379_gb300 as pcmod
+    import paper_2503_19379_gb300 as p
+    return p
+
+
+@pytest.mark.parametrize("nb,p,L", [(1300, 2, 98304), (64, 4, 786432), (1, 9, 64), (3, 16, 8193)])
+def test_long_narrow_panels(pcmod, nb, p, L):
     v = torch.tensor([1.1 + 0.3j, 1.3 + 0.7j, 0.9 + 1.01j, 3.1], dtype=torch.complex64, device="cuda")[torch.arange(p) % 4]
     A = v[None, :, None].expand(nb, p, L).contiguous()
     w = v.to(torch.complex128)

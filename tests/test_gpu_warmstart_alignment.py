@@ -8,11 +8,16 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("N,nb,S", [(16, 3, 2), (32, 8, 3)])
-def test_x_offset_by_one_element(N, nb, S):
+@pytest.fixture(scope="module")
+def pcmod():
     from paper_2503_19379_gb300 import build as b
     b.build()
-    import paper_2503_19379_gb300 as pcmod
+    import paper_2503_19379_gb300 as p
+    return p
+
+
+@pytest.mark.parametrize("N,nb,S", [(16, 3, 2), (32, 8, 3)])
+def test_x_offset_by_one_element(pcmod, N, nb, S):
     from paper_2503_19379_gb300 import pc
     g = np.random.default_rng(N)
     net = pcmod.WarmStart(N, nb, S)
