@@ -221,7 +221,8 @@ __global__ void __launch_bounds__(256) fft_z_symbol_kernel(const cplx<T> *__rest
       const T rs = (T)1 / sigma, inv = scale * rs;  // one division: 1 / N^3 is a power of two
       if (!laplacian) {
         const C s = cadd(cadd(cmul(d1, r1), cmul(d2, r2)), cmul(d3, r3));  // d^T r
-        const T f = fac * rs;
+        // fac / sigma from the reciprocal: the product, corrected by its remainder (rounded as the quotient)
+        const T f0 = fac * rs, f = fma(fma(-f0, sigma, fac), rs, f0);
         r1 = csub(r1, cscale(cmulc(d1, s), f));  // conj(d1) * s
         r2 = csub(r2, cscale(cmulc(d2, s), f));
         r3 = csub(r3, cscale(cmulc(d3, s), f));
