@@ -493,54 +493,51 @@ int launch_gram_pair_coupled(int nb, long L, int p, int q2, int dtype, const voi
 }
 
 // ------------------------------------------------------------------------------------------------ block update
-// Y_b[:, j] = sum_i S_b[:, i] C_b[i, j] (+ Z_b[:, j] when Z is given); grid (ceil(L/256), ceil(q/QB), nb); one row
-// per thread, QB outputs. Products and sums run in the precision T of S and Y; Z is a complex64 addend (the
-// complex64 correction added to the FP64 block in the mixed-precision update). Each column group re-reads S, so
-// the launcher takes the width that covers q in the fewest groups with the fewest idle columns (complex64: one
-// group of up to 24 columns, 48 accumulator registers).
+// complex64: Y_b[:, j] = sum_i S_b[:, i] C_b[i, j] (+ Z_b[:, j] when Z is given); grid (ceil(L/256), ceil(q/QB), nb); one
+// row per thread, QB outputs, FP32 products and sums. Each column group re-reads S, so the launcher takes the width that
+// covers q in the fewest groups with the fewest idle columns (one group of up to 24 columns, 48 accumulator registers).
 constexpr int UPD_PMAX = 64;
 
-template <typename T, int QB>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
-    block_update_kernel(const cplx<T> *__restrict__ S, long ss, const double2 *__restrict__ Cm, long sc,
-                        cplx<T> *__restrict__ Y, long sy, const float2 *__restrict__ Z, long sz, long L, int p, int q,
+template <int QB>
+__global__ void __launch_bounds__(256, 3)
+    block_update_kernel(const float2 *__restrict__ S, long ss, const double2 *__restrict__ Cm, long sc,
+                        float2 *__restrict__ Y, long sy, const float2 *__restrict__ Z, long sz, long L, int p, int q,
                         const int *__restrict__ act) {
-  using C = cplx<T>;
-  __shared__ C Cs[UPD_PMAX][QB];
+  __shared__ float2 Cs[UPD_PMAX][QB];
   const int b = act ? act[blockIdx.z] : (int)blockIdx.z;
   const int j0 = blockIdx.y * QB;
   const double2 *Cb = Cm + (long)b * sc;
   for (int i = threadIdx.x; i < p * QB; i += blockDim.x) {
     const int r = i / QB, c = i - r * QB;
     const double2 v = (j0 + c < q) ? Cb[r * q + j0 + c] : cmake<double2>(0.0, 0.0);
-    Cs[r][c] = cmake<C>((T)v.x, (T)v.y);
+    Cs[r][c] = make_float2((float)v.x, (float)v.y);
   }
   __syncthreads();
   const long l = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (l >= L) return;
-  const C *Sb = S + (long)b * ss;
-  C acc[QB];
+  const float2 *Sb = S + (long)b * ss;
+  float2 acc[QB];
 #pragma unroll
-  for (int c = 0; c < QB; ++c) acc[c] = cmake<C>((T)0, (T)0);
+  for (int c = 0; c < QB; ++c) acc[c] = make_float2(0.f, 0.f);
   for (int i = 0; i < p; ++i) {
-    const C sv = Sb[(long)i * L + l];
+    const float2 sv = Sb[(long)i * L + l];
 #pragma unroll
     for (int c = 0; c < QB; ++c) {
-      const C cv = Cs[i][c];
-      acc[c].x = fma(sv.x, cv.x, fma(-sv.y, cv.y, acc[c].x));
-      acc[c].y = fma(sv.x, cv.y, fma(sv.y, cv.x, acc[c].y));
+      const float2 cv = Cs[i][c];
+      acc[c].x = fmaf(sv.x, cv.x, fmaf(-sv.y, cv.y, acc[c].x));
+      acc[c].y = fmaf(sv.x, cv.y, fmaf(sv.y, cv.x, acc[c].y));
     }
   }
-  C *Yb = Y + (long)b * sy;
+  float2 *Yb = Y + (long)b * sy;
   const float2 *Zb = Z ? Z + (long)b * sz : nullptr;
 #pragma unroll
   for (int c = 0; c < QB; ++c)
     if (j0 + c < q) {
-      C v = acc[c];
+      float2 v = acc[c];
       if (Zb) {
         const float2 z = Zb[(long)(j0 + c) * L + l];
-        v.x += (T)z.x;
-        v.y += (T)z.y;
+        v.x += z.x;
+        v.y += z.y;
       }
       Yb[(long)(j0 + c) * L + l] = v;
     }
@@ -610,25 +607,22 @@ __global__ void __launch_bounds__(256, 2)
     }
 }
 
-template <typename T, int QB>
-static void block_update_t(int nb, long L, int p, int q, const void *S, long ss, const void *C, long sc, void *Y,
-                           long sy, cudaStream_t st, const int *act, const void *Z, long sz) {
-  if constexpr (std::is_same<T, float>::value) {
-    // two rows a thread once that leaves two blocks per SM (8 k-points x 1536 rows, 39 -> 12: 18 us with one row, 23 with
-    // two)
-    const uintptr_t at = (uintptr_t)S | (uintptr_t)Y | (uintptr_t)Z;
-    const dim3 g((unsigned)((L / 2 + 255) / 256), (unsigned)((q + QB - 1) / QB), nb);
-    if (((L | ss | sy | sz) & 1) == 0 && (at & 15) == 0 && (long)g.x * g.y * g.z >= 2L * sm_count()) {
-      block_update2_kernel<QB><<<g, 256, 0, st>>>(static_cast<const float2 *>(S), ss, static_cast<const double2 *>(C), sc,
-                                                  static_cast<float2 *>(Y), sy, static_cast<const float2 *>(Z), sz, L, p,
-                                                  q, act, nullptr, nullptr);
-      return;
-    }
+template <int QB>
+static void block_update_c64(int nb, long L, int p, int q, const void *S, long ss, const void *C, long sc, void *Y,
+                             long sy, cudaStream_t st, const int *act, const void *Z, long sz) {
+  // two rows a thread once that leaves two blocks per SM (8 k-points x 1536 rows, 39 -> 12: 18 us with one row, 23 with two)
+  const uintptr_t at = (uintptr_t)S | (uintptr_t)Y | (uintptr_t)Z;
+  const dim3 g((unsigned)((L / 2 + 255) / 256), (unsigned)((q + QB - 1) / QB), nb);
+  if (((L | ss | sy | sz) & 1) == 0 && (at & 15) == 0 && (long)g.x * g.y * g.z >= 2L * sm_count()) {
+    block_update2_kernel<QB><<<g, 256, 0, st>>>(static_cast<const float2 *>(S), ss, static_cast<const double2 *>(C), sc,
+                                                static_cast<float2 *>(Y), sy, static_cast<const float2 *>(Z), sz, L, p,
+                                                q, act, nullptr, nullptr);
+    return;
   }
   const dim3 grid((unsigned)((L + 255) / 256), (unsigned)((q + QB - 1) / QB), nb);
-  block_update_kernel<T, QB><<<grid, 256, 0, st>>>(static_cast<const cplx<T> *>(S), ss,
-                                                   static_cast<const double2 *>(C), sc, static_cast<cplx<T> *>(Y), sy,
-                                                   static_cast<const float2 *>(Z), sz, L, p, q, act);
+  block_update_kernel<QB><<<grid, 256, 0, st>>>(static_cast<const float2 *>(S), ss, static_cast<const double2 *>(C), sc,
+                                                static_cast<float2 *>(Y), sy, static_cast<const float2 *>(Z), sz, L, p, q,
+                                                act);
 }
 
 // the column-group width for q outputs among `widths`: fewest idle columns, then fewest groups
@@ -653,22 +647,25 @@ int launch_block_update(int nb, long L, int p, int q, int dtype, const void *S, 
     set_error("block_update: at most 64 input columns");
     return PC_EINVAL;
   }
-  // complex128: on the tensor cores (update_sl.cu: faster than the FP64 pipe at every size measured, 8 -> 4 columns of 1536
-  // rows and up; `each` also where C picks single columns, 1.6 against 4.0 ms for 48 -> 16 of 8 k-points at N = 32); not
-  // the addend and the sum of no columns, which no solve asks for
-  if (dtype == PC_C128 && p > 0 && !Z)
-    return launch_update_sl(nb, L, p, q, PC_C128, S, ss, C, sc, Y, sy, nullptr, 0, st, tmo, act, each);
   if (dtype == PC_C128) {
-    block_update_t<double, 8>(nb, L, p, q, S, ss, C, sc, Y, sy, st, act, Z, sz);
-  } else {
-    switch (update_width(q, {8, 10, 12, 16, 20, 24})) {
-      case 8: block_update_t<float, 8>(nb, L, p, q, S, ss, C, sc, Y, sy, st, act, Z, sz); break;
-      case 10: block_update_t<float, 10>(nb, L, p, q, S, ss, C, sc, Y, sy, st, act, Z, sz); break;
-      case 12: block_update_t<float, 12>(nb, L, p, q, S, ss, C, sc, Y, sy, st, act, Z, sz); break;
-      case 16: block_update_t<float, 16>(nb, L, p, q, S, ss, C, sc, Y, sy, st, act, Z, sz); break;
-      case 20: block_update_t<float, 20>(nb, L, p, q, S, ss, C, sc, Y, sy, st, act, Z, sz); break;
-      default: block_update_t<float, 24>(nb, L, p, q, S, ss, C, sc, Y, sy, st, act, Z, sz); break;
+    // on the tensor cores (update_sl.cu: faster than the FP64 pipe at every size measured, 8 -> 4 columns of 1536 rows
+    // and up; `each` also where C picks single columns, 1.6 against 4.0 ms for 48 -> 16 of 8 k-points at N = 32)
+    if (Z || (p == 0 && act)) {
+      set_error("block_update: complex128 blocks take no addend, and no list of k-points with a sum of no columns");
+      return PC_EINVAL;
     }
+    if (p > 0) return launch_update_sl(nb, L, p, q, PC_C128, S, ss, C, sc, Y, sy, nullptr, 0, st, tmo, act, each);
+    for (int b = 0; b < nb; ++b)
+      PC_CK(cudaMemsetAsync(static_cast<double2 *>(Y) + (long)b * sy, 0, sizeof(double2) * (size_t)q * L, st));
+    return PC_OK;
+  }
+  switch (update_width(q, {8, 10, 12, 16, 20, 24})) {
+    case 8: block_update_c64<8>(nb, L, p, q, S, ss, C, sc, Y, sy, st, act, Z, sz); break;
+    case 10: block_update_c64<10>(nb, L, p, q, S, ss, C, sc, Y, sy, st, act, Z, sz); break;
+    case 12: block_update_c64<12>(nb, L, p, q, S, ss, C, sc, Y, sy, st, act, Z, sz); break;
+    case 16: block_update_c64<16>(nb, L, p, q, S, ss, C, sc, Y, sy, st, act, Z, sz); break;
+    case 20: block_update_c64<20>(nb, L, p, q, S, ss, C, sc, Y, sy, st, act, Z, sz); break;
+    default: block_update_c64<24>(nb, L, p, q, S, ss, C, sc, Y, sy, st, act, Z, sz); break;
   }
   PC_CK_LAUNCH();
   return PC_OK;

@@ -78,8 +78,6 @@ __device__ __forceinline__ df df_mul(df x, df y) {
   e = fmaf(x.lo, y.hi, e);
   return quick_two_sum(p, e);
 }
-// multiplication by a power of two (exact)
-__device__ __forceinline__ df df_scale2(df x, float s) { return df{x.hi * s, x.lo * s}; }
 
 // complex double-float
 struct cdf {
@@ -98,55 +96,6 @@ __device__ __forceinline__ cdf cdf_mulc(cdf a, cdf b) {
 }
 __device__ __forceinline__ cdf cdf_scale(cdf a, df s) { return cdf{df_mul(a.re, s), df_mul(a.im, s)}; }
 
-// s += a b for double-float a, b, s: the product's rounding error is exact via fma, the sum via two_sum, then one
-// renormalisation (15 FP32 operations); about 2^-44 relative per step
-__device__ __forceinline__ void df_mac(df &s, df a, df b) {
-  const float p = a.hi * b.hi;
-  float e = fmaf(a.hi, b.hi, -p);
-  e = fmaf(a.hi, b.lo, e);
-  e = fmaf(a.lo, b.hi, e);
-  const float t = s.hi + p;
-  const float bb = t - s.hi;
-  const float err = (s.hi - (t - bb)) + (p - bb);
-  s = quick_two_sum(t, err + (s.lo + e));
-}
-// s += a b for complex double-float
-__device__ __forceinline__ void cdf_mac(cdf &s, cdf a, cdf b) {
-  df_mac(s.re, a.re, b.re);
-  df_mac(s.re, df_neg(a.im), b.im);
-  df_mac(s.im, a.re, b.im);
-  df_mac(s.im, a.im, b.re);
-}
-__device__ __forceinline__ cdf cdf_scale2(cdf a, float s) { return cdf{df_scale2(a.re, s), df_scale2(a.im, s)}; }
-
-// A double-float sum built term by term without renormalising after every term: s is the FP32 running sum of the
-// leading products, e collects every rounding error exactly captured on the way (two_sum of the running sum, the
-// fma residual of each leading product) plus the small cross terms hi*lo + lo*hi. One term costs 12 FP32 operations
-// (df_mac: 15), and the value is quick_two_sum(s, e) at the end; e stays ~2^-24 |s|, so its own rounding is ~2^-48
-// of the sum, like the renormalised form.
-struct dfsum {
-  float s, e;
-};
-// a += x c
-__device__ __forceinline__ void dfsum_mac(dfsum &a, df x, df c) {
-  const float p = x.hi * c.hi;
-  const float ep = fmaf(x.hi, c.hi, -p);
-  const float t = a.s + p;
-  const float bb = t - a.s;
-  const float es = (a.s - (t - bb)) + (p - bb);
-  a.s = t;
-  a.e += es + ep;
-  a.e = fmaf(x.hi, c.lo, a.e);
-  a.e = fmaf(x.lo, c.hi, a.e);
-}
-// a += f for an FP32 f
-__device__ __forceinline__ void dfsum_addf(dfsum &a, float f) {
-  const float t = a.s + f;
-  const float bb = t - a.s;
-  a.e += (a.s - (t - bb)) + (f - bb);
-  a.s = t;
-}
-__device__ __forceinline__ df dfsum_value(dfsum a) { return quick_two_sum(a.s, a.e); }
 // x + f for a double-float x and an FP32 f
 __device__ __forceinline__ df df_addf(df x, float f) {
   const df s = two_sum(x.hi, f);

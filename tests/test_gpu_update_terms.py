@@ -78,3 +78,15 @@ def test_scales_far_from_one(pcmod):
     S[0, 5], C[0, 6], C[0, :, 4], S[0, :, 77] = 0.0, 0.0, 0.0, 0.0
     C[0, :3, 7] = C[0, 4:, 7] = 0.0  # output 7: only the scaled column
     assert error_of_terms(pcmod, S, C) <= 2.0 ** -51 + 2.0 ** -52.2 * np.sqrt(40)
+
+
+@pytest.mark.parametrize("dtype", [torch.complex128, torch.complex64])
+def test_sum_of_no_columns(pcmod, dtype):
+    """p = 0 through the C ABI: zeros in the outputs, nothing past them."""
+    from paper_2503_19379_gb300 import pc
+    Y = torch.ones(3, 5, 37, dtype=dtype, device="cuda")
+    z = torch.zeros(1, dtype=torch.complex128, device="cuda")
+    rc = pcmod.lib().pc_block_update(3, 37, 0, 4, pc._dtype_code(Y), pc._dev(z), 0, pc._dev(z), pc._dev(Y), 5 * 37,
+                                     pc._stream(None))
+    assert rc == 0
+    assert bool((Y[:, :4] == 0).all()) and bool((Y[:, 4] == 1).all())
