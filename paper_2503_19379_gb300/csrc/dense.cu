@@ -273,7 +273,7 @@ int launch_gram(int nb, long L, int p, int q, int dtype, const void *A, long sa,
   if (dtype == PC_C128) {
     int c = 0;
     const int rc = launch_gram_sl(nb, L, p, q, PC_C128, A, sa, B, sb, SL_GENERAL, static_cast<double2 *>(scratch),
-                                  gram_scratch_chunks(nb, L), &c, st, tmo, act);
+                                  gram_scratch_chunks(nb, L), &c, st, tmo, act, true);
     if (rc) return rc;
     launch_gram_reduce(nb, c, p, q, static_cast<double2 *>(scratch), act, G, st, sg);
     PC_CK_LAUNCH();
@@ -441,7 +441,7 @@ static int launch_gram_pair_t(int nb, long L, int p, const void *S, const void *
 
 int launch_gram_pair(int nb, long L, int p, int dtype, const void *S, const void *AS, long ss, void *G, void *H,
                      void *scratch, size_t scratch_bytes, cudaStream_t st, int *tmo, const int *act, int nb_alloc,
-                     long sg) {
+                     long sg, bool each) {
   if (nb == 0 || p == 0) return PC_OK;
   if (p > 64) {
     set_error("gram_pair: at most 64 columns");
@@ -459,8 +459,7 @@ int launch_gram_pair(int nb, long L, int p, int dtype, const void *S, const void
   int nchunk = gram_chunks(nb, L), rc;
   if (dtype == PC_C128) {
     rc = launch_gram_sl(nb, L, p, p, PC_C128, S, ss, AS, ss, SL_PAIR, part, gram_scratch_chunks(nb, L), &nchunk, st,
-                        tmo,
-                        act);
+                        tmo, act, each);
   } else {
     long chunk = (L + nchunk - 1) / nchunk;
     chunk = (chunk + GRAM_TL - 1) / GRAM_TL * GRAM_TL;
@@ -1207,7 +1206,8 @@ extern "C" int pc_gram_pair(int nb, long L, int p, int dtype, const void *S, lon
   PC_CK(tmp.reserve(std::max<size_t>(16, gram_pair_scratch_bytes(nb, L, p))));
   int rc = tmo.start();
   if (rc) return rc;
-  rc = launch_gram_pair(nb, L, p, dtype, S, AS, ss, G, H, tmp.p, tmp.bytes, (cudaStream_t)stream, tmo.word, nullptr);
+  rc = launch_gram_pair(nb, L, p, dtype, S, AS, ss, G, H, tmp.p, tmp.bytes, (cudaStream_t)stream, tmo.word, nullptr, -1,
+                        0, true);
   if (rc) return rc;
   PC_CK(cudaStreamSynchronize((cudaStream_t)stream));
   return tmo.check();

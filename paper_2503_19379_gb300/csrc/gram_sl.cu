@@ -14,9 +14,10 @@
 // scaled and added to FP64 sums in shared memory.
 //
 // Digits are exact relative to the largest values of the two columns in the span, which need not meet: columns that are
-// large in different rows have a product far below that of their largest values. So the rows of a complex128 span in which
-// a column is within two bits of its largest are marked while the digits are formed, and an entry whose columns share too
-// few of them is formed in plain FP64 for this span, as are those of a column with an infinity or a NaN (`unserved`).
+// large in different rows have a product far below that of their largest values. The solves take that, since an entry's
+// error counts against the norms of its columns there. For other callers (EACH) the rows of a span in which a column is
+// within two bits of its largest are marked while the digits are formed, and an entry whose columns share too few of them
+// is formed in plain FP64 for this span, as are, for all, those of a column with an infinity or a NaN (`unserved`).
 //
 // Every wait is bounded. A warp whose wait runs out, or that finds the abort flag set, leaves its stages; at the end of
 // the span all roles leave together, the MMAs in flight are waited for, and the host is told (TimeoutWord).
@@ -27,7 +28,8 @@
 //
 // Bound: the latency of a stage (load, digits, hand-off to the tensor core, drain), then integer instructions of the digit
 // extraction. 8 k-points x 48 complex128 columns at N = 32: 23.6 ms on the FP64 pipe, 2.06 ms here (without the scan
-// 0.3 ms less, without the MMAs 0.4 ms, without the drains 0.2 ms, without the marks and their comparison 0.1 ms); one k-point of 24 columns at N = 16: 1.77 ms and
+// 0.3 ms less, without the MMAs 0.4 ms, without the drains 0.2 ms, without the marks and their comparison 0.1 ms; with
+// marks in the solves too, whose converged columns are far from dense, the FP64 solve at N = 64 took 16% longer); one k-point of 24 columns at N = 16: 1.77 ms and
 // 64 us. X^H X of 4 k-points x 19 pair columns at N = 64: 1.61 ms in double-float arithmetic, 1.11 ms here; of one
 // k-point x 13 at N = 16: 60 and 24 us. The pair A^H A, A^H B takes the block's columns of A and of B in one CTA, and the
 // columns of A that the block shares with the left operand are extracted once and stored twice.
@@ -61,16 +63,15 @@ struct SlGramArgs {
   int *tmo;
 };
 
-// TASKS: at most 32 TASKS columns to extract (each thread two rows of every 32nd column); DEPTH: stages loaded ahead
-template <typename T> constexpr bool sg_each() { return std::is_same<T, double2>::value; }
 // exponents, needs and masks of 96 columns
-template <typename T> constexpr uint32_t sg_col_bytes() { return 96u * 4u * (sg_each<T>() ? 2 + SG_WSTRIDE : 2); }
+constexpr uint32_t sg_col_bytes(bool each) { return 96u * 4u * (each ? 2 + SG_WSTRIDE : 2); }
 
-template <typename T, int TASKS, int DEPTH>
+// TASKS: at most 32 TASKS columns to extract (each thread two rows of every 32nd column); DEPTH: stages loaded ahead; EACH:
+// every entry to the accuracy of its own terms
+template <typename T, int TASKS, int DEPTH, bool EACH>
 __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs a) {
   using F = SlForm<T>;
   constexpr int ND = F::ND, NL = F::NL, GROUP = F::KMAX / SG_ROWS;  // stages per drain
-  constexpr bool EACH = sg_each<T>();  // every entry as accurate as its own terms
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_addr(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -81,7 +82,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
   int *const sE = reinterpret_cast<int *>(sm + off_e);
   int *const sNeed = sE + 96;                                        // SG_NEED, SG_ZERO or SG_BAD
   unsigned *const sMask = reinterpret_cast<unsigned *>(sNeed + 96);  // complex128: rows within 2 bits of the column's largest
-  const uint32_t off_bar = off_e + sg_col_bytes<T>();
+  const uint32_t off_bar = off_e + sg_col_bytes(EACH);
   const uint32_t bars = base + off_bar;
   const uint32_t ready = bars + 16u;  // by operand buffer: bars, its MMAs are done; ready, its digits are there
   uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(sm + off_bar + 32);
@@ -385,8 +386,8 @@ __global__ void __launch_bounds__(SG_THREADS, 1) gram_sl_kernel(const SlGramArgs
   if (tid == 0 && *abort) report_timeout(a.tmo);
 }
 
-template <typename T> size_t sg_smem(int nbp) {
-  return 1024 + SlForm<T>::ND * 16384 + (size_t)SlForm<T>::NL * nbp * 128 + 8 * SG_CONV * 8 + sg_col_bytes<T>() + 64;
+template <typename T> size_t sg_smem(int nbp, bool each) {
+  return 1024 + SlForm<T>::ND * 16384 + (size_t)SlForm<T>::NL * nbp * 128 + 8 * SG_CONV * 8 + sg_col_bytes(each) + 64;
 }
 
 }  // namespace
@@ -398,7 +399,7 @@ int sl_gram_chunks(int nb, long L) {
 }
 
 int launch_gram_sl(int nb, long L, int p, int q, int dtype, const void *A, long sa, const void *B, long sb, int mode,
-                   double2 *part, int maxchunk, int *nchunk, cudaStream_t st, int *tmo, const int *act) {
+                   double2 *part, int maxchunk, int *nchunk, cudaStream_t st, int *tmo, const int *act, bool each) {
   SlGramArgs a{};
   a.A = A;
   a.B = B;
@@ -430,25 +431,27 @@ int launch_gram_sl(int nb, long L, int p, int q, int dtype, const void *A, long 
   *nchunk = c;
   a.part0 = part;
   a.part1 = part + (size_t)nb * c * p * q;
-  const size_t smem = dtype == PC_DFS ? sg_smem<float4>(a.nbp) : sg_smem<double2>(a.nbp);
+  const size_t smem = dtype == PC_DFS ? sg_smem<float4>(a.nbp, false) : sg_smem<double2>(a.nbp, each);
   const dim3 grid(c, nblk, nb);
   // columns that a block extracts: its left columns, up to all p, and its own of B
   const int ncols = p + (mode == SL_SELF ? 0 : a.nbc);
-  const int kind = dtype == PC_DFS ? 0 : (ncols <= 32 ? 1 : (ncols <= 64 ? 2 : 3));
+  const int kind = dtype == PC_DFS ? 0 : (ncols <= 32 ? 1 : (ncols <= 64 ? 2 : 3)) + (each ? 3 : 0);
   if (kind == 0 && ncols > 32) {
     set_error("gram_sl: at most 32 columns of double-float pairs");
     return PC_EINVAL;
   }
-  const auto kernel = kind == 0   ? gram_sl_kernel<float4, 1, 3>
-                      : kind == 1 ? gram_sl_kernel<double2, 1, 3>
-                      : kind == 2 ? gram_sl_kernel<double2, 2, 1>
-                                  : gram_sl_kernel<double2, 3, 1>;
-  static bool configured[64][4] = {};  // per device
+  using Kernel = void (*)(SlGramArgs);
+  static constexpr Kernel kernels[7] = {gram_sl_kernel<float4, 1, 3, false>,  gram_sl_kernel<double2, 1, 3, false>,
+                                        gram_sl_kernel<double2, 2, 1, false>, gram_sl_kernel<double2, 3, 1, false>,
+                                        gram_sl_kernel<double2, 1, 3, true>,  gram_sl_kernel<double2, 2, 1, true>,
+                                        gram_sl_kernel<double2, 3, 1, true>};
+  const Kernel kernel = kernels[kind];
+  static bool configured[64][7] = {};  // per device
   int dev = 0;
   PC_CK(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64 || !configured[dev][kind]) {
     PC_CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)(kind ? sg_smem<double2>(64) : sg_smem<float4>(64))));
+                               (int)(kind ? sg_smem<double2>(64, each) : sg_smem<float4>(64, false))));
     if (dev >= 0 && dev < 64) configured[dev][kind] = true;
   }
   kernel<<<grid, SG_THREADS, smem, st>>>(a);

@@ -262,13 +262,14 @@ int launch_precond(pc_ctx *ctx, int nb, int m, int dtype, const void *R, long sr
 int launch_precond_c64(pc_ctx *ctx, int nb, int m, const void *R, long sr, void *W, long sw, const int *act);
 // nb_alloc: k-points in the panel arrays (the act list indexes them); <= 0 means nb.
 // sg: batch stride of the output matrices in elements; <= 0 means packed (p q, or p p for the pair).
+// each: see launch_gram_sl (complex128 pairs; launch_gram always takes it)
 int launch_gram(int nb, long L, int p, int q, int dtype, const void *A, long sa, const void *B, long sb, void *G,
                 void *scratch, size_t scratch_bytes, cudaStream_t st, int *tmo, const int *act, int nb_alloc = -1,
                 long sg = 0);
 size_t gram_scratch_bytes(int nb, long L, int p, int q);
 int launch_gram_pair(int nb, long L, int p, int dtype, const void *S, const void *AS, long ss, void *G, void *H,
                      void *scratch, size_t scratch_bytes, cudaStream_t st, int *tmo, const int *act, int nb_alloc = -1,
-                     long sg = 0);
+                     long sg = 0, bool each = false);
 size_t gram_pair_scratch_bytes(int nb, long L, int p);
 // reductions of per-chunk partial sums ([nb][nchunk][p][q] double2; the pair: G block then H block, upper triangles)
 void launch_gram_pair_reduce(int nb, int nchunk, int p, const double2 *part, const int *act, void *G, void *H,

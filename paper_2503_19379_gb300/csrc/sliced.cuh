@@ -251,11 +251,11 @@ __device__ __forceinline__ void named_sync(int id, int count) {
 
 // Gram products of FP64-accurate panels (gram_sl.cu), dtype PC_C128 or PC_DFS, one array part[bi][chunk][p][q] per
 // product: SL_GENERAL A^H B; SL_PAIR A^H A, then A^H B, both upper triangles (q = p); SL_SELF the upper triangle of
-// A^H A
+// A^H A; each (PC_C128): every entry to the accuracy of its own terms, otherwise to that of the columns' norms
 constexpr int SL_GENERAL = 0, SL_PAIR = 1, SL_SELF = 2;
 int sl_gram_chunks(int nb, long L);
 int launch_gram_sl(int nb, long L, int p, int q, int dtype, const void *A, long sa, const void *B, long sb, int mode,
-                   double2 *part, int maxchunk, int *nchunk, cudaStream_t st, int *tmo, const int *act);
+                   double2 *part, int maxchunk, int *nchunk, cudaStream_t st, int *tmo, const int *act, bool each = false);
 
 // Y = S C (+ Z, a complex64 addend, for pairs) for PC_C128 (1 <= p <= 64) or PC_DFS (1 <= p <= 32) blocks (update_sl.cu);
 // each (PC_C128): every output to the accuracy of its own terms, otherwise to that of its row's largest
