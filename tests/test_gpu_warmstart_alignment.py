@@ -25,7 +25,8 @@ def test_x_offset_by_one_element(pcmod, N, nb, S):
     m0 = torch.from_numpy(g.uniform(0.1, 1.0, (2, 3, N, N, N)).astype(np.float32)).cuda()
     sidx = torch.tensor([i % 2 for i in range(S)], dtype=torch.int32, device="cuda")
     k = np.ascontiguousarray(g.uniform(-3, 3, (S, 3)))
-    V = torch.randn(S, nb, 3, N, N, N, dtype=torch.complex64, device="cuda") / np.sqrt(3 * N ** 3)
+    gen = torch.Generator(device="cuda").manual_seed(N)
+    V = torch.randn(S, nb, 3, N, N, N, dtype=torch.complex64, device="cuda", generator=gen) / np.sqrt(3 * N ** 3)
     lam = torch.from_numpy(np.sort(g.uniform(2.0, 60.0, (S, nb)), axis=1)).cuda()
     X, y = net.forward(m0, sidx, k)
     grad, loss = net.backward(m0, sidx, X, y, V, lam)
