@@ -3,8 +3,8 @@
 //   two_sum(a, b):  s = fl(a + b), e = (a - (s - bb)) + (b - bb), bb = s - a   (Knuth), a + b = s + e exactly;
 //   two_prod(a, b): p = fl(a b),   e = fma(a, b, -p),                             a b = p + e exactly;
 // (Dekker 1971; Hida, Li and Bailey, "Library for double-double and quad-double arithmetic", 2001).
-// On GB300 the FP32 pipe is ~62x faster than the FP64 pipe, so the FP64-accurate parts of the mixed-precision solve
-// (the block X, its operator image, the X-X Gram block) run in this format: ~10 FP32 operations per operation, a
+// On GB300 the FP32 pipe is ~62x faster than the FP64 pipe, so the FP64-accurate block X of the mixed-precision solve is
+// kept in this format, and its operator image is formed in it: ~10 FP32 operations per operation, a
 // relative error of ~2^-44 instead of 2^-53, which the eigensolver does not resolve (its FP64 residual floor is
 // ~1e-10 here).
 #pragma once

@@ -1,7 +1,7 @@
 // The FP64-accurate kernels of the mixed-precision solve, in double-float arithmetic (dfloat.cuh) on the FP32 pipe
 // (GB300: 75 TFLOP/s FP32 against 1.2 TFLOP/s FP64). The solver's block X is stored as double-float pairs (PC_DFS,
-// one float4 per complex element), so these kernels do no FP64 arithmetic at all; the public stencil entry point
-// takes complex128 and converts on load and store.
+// one float4 per complex element), so the stencils do no FP64 arithmetic on it; the public entry point takes complex128
+// and converts on load and store.
 //   op_df_kernel / opz_df_kernel  AX = Op X (the stencil of stencil.cu; differences, shifts, M0, gamma in
 //                     double-float), or, in the solver, the residual epilogue: R = AX - X Theta and complex64 copies
 //                     of R, X and AX, plus column norms (AX itself is not stored)
@@ -19,9 +19,11 @@ namespace pc {
 // ---------------------------------------------------------------- packed complex double-float
 // A complex double-float as two packed FP32 pairs, hi = (re.hi, im.hi) and lo = (re.lo, im.lo): every operation runs on
 // both parts with one instruction (add, mul, fma .f32x2). Their rate in results is that of the scalar ones (measured: 124
-// and 119 per clock and SM), in half the issue slots, and the stencils below are bound by issue (71% of the cycles
-// with the FMA pipe 60% busy; complex128 blocks of 15 k-points x 16 fields at N = 32: 1.10 ms with scalar operations,
-// 1.01 ms with these). The operations and their order are those of dfloat.cuh: the same bits.
+// and 119 per clock and SM), in half the issue slots, and the stencils below are bound by issue in the solver's pair
+// storage (71% of the cycles with scalar operations, the FMA pipe 60% busy). On complex128 blocks the FP64 pipe bounds
+// them, 76% busy with the conversions to pairs and back, of halo points too (issue 37%, FMA 22%): 15 k-points x 16
+// fields at N = 32 take 1.10 ms with scalar operations and 1.00 ms with these. The operations and their order are those
+// of dfloat.cuh: the same bits.
 __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, 0xbf800000bf800000ull, a); }  // b (-1, -1) + a
 __device__ __forceinline__ f32x2 swap2(f32x2 v) {
   const float2 t = unpack2(v);

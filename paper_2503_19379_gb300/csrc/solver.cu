@@ -18,6 +18,8 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <vector>
 
 #include "pc_internal.cuh"
@@ -124,6 +126,59 @@ void spurious_mask(const std::vector<int> &redo, int m, int nbands, double tol, 
     }
 }
 
+namespace {
+
+constexpr size_t PINNED_MIN = 16 << 10;   // blocks: powers of two from here
+constexpr size_t PINNED_KEPT = 8 << 20;  // bytes of returned blocks that are kept
+
+struct PinnedPool {
+  std::mutex mutex;
+  std::map<size_t, std::vector<void *>> blocks;  // returned ones by size
+  size_t kept = 0;
+  long allocations = 0;
+};
+PinnedPool &pinned_pool() {
+  static PinnedPool *p = new PinnedPool;  // (a context may outlive the library's static objects)
+  return *p;
+}
+
+}  // namespace
+
+cudaError_t pinned_take(size_t need, void **p, size_t *bytes) {
+  size_t size = PINNED_MIN;
+  while (size < need) size *= 2;
+  PinnedPool &pool = pinned_pool();
+  {
+    std::lock_guard<std::mutex> lock(pool.mutex);
+    std::vector<void *> &v = pool.blocks[size];
+    if (!v.empty()) {
+      *p = v.back();
+      *bytes = size;
+      v.pop_back();
+      pool.kept -= size;
+      return cudaSuccess;
+    }
+    ++pool.allocations;
+  }
+  const cudaError_t e = cudaHostAlloc(p, size, cudaHostAllocPortable);
+  if (e == cudaSuccess) *bytes = size;
+  return e;
+}
+
+void pinned_give(void *p, size_t bytes) {
+  if (!p) return;
+  PinnedPool &pool = pinned_pool();
+  {
+    std::lock_guard<std::mutex> lock(pool.mutex);
+    if (pool.kept + bytes <= PINNED_KEPT) {
+      pool.blocks[bytes].push_back(p);
+      pool.kept += bytes;
+      return;
+    }
+  }
+  cudaFreeHost(p);
+}
+
 int upload_kpoints(pc_ctx *ctx, int nb, const double *kpts, const double *gammas, bool wait) {
   if (nb <= 0) return PC_OK;
   const int tabs = ctx->lat ? 9 : 3;  // symbol tables per k-point: d_i by axis, or the parts (i, j) of d_i
@@ -204,6 +259,12 @@ int harvest_timing(pc_ctx *ctx) {
 }  // namespace pc
 
 using namespace pc;
+
+// For tests: pinned blocks allocated so far.
+extern "C" long pc_pinned_allocations(void) {
+  std::lock_guard<std::mutex> lock(pc::pinned_pool().mutex);
+  return pc::pinned_pool().allocations;
+}
 
 extern "C" const char *pc_last_error(void) { return g_err; }
 

@@ -22,8 +22,8 @@
 // Every wait is bounded. A warp whose wait runs out, or that finds the abort flag set, does nothing more; all leave
 // together at the next tile, wait for the MMAs in flight and write NaN over the CTA's rows.
 //
-// Complex128 takes eight digits (the error against extended precision is 4.7e-17 of the result, that of FP64 sums 1.3e-16
-// to 3.4e-16; seven digits left 1.1e-15). Pairs take eight digits of base 128 (2.5e-15, the double-float sums 2.0e-14;
+// Complex128 takes eight digits (smooth fields, 24 to 64 columns, against extended precision: off by 4.7e-17 of the
+// result's norm, FP64 sums by 2.9e-16 to 4.7e-16; seven digits left 1.1e-15). Pairs take eight digits of base 128 (2.5e-15, the double-float sums 2.0e-14;
 // seven left 5.4e-14 where C is near the identity).
 //
 // Bound: instructions of the digit extraction and the epilogue. Complex128, 8 k-points, 48 -> 16 columns at N = 32:
