@@ -497,36 +497,42 @@ int launch_gram_pair_coupled(int nb, long L, int p, int q2, int dtype, const voi
 // covers q in the fewest groups with the fewest idle columns (one group of up to 24 columns, 48 accumulator registers).
 constexpr int UPD_PMAX = 64;
 
-template <int QB>
+// SUM: a second product S2 C2 of the same widths follows in the same sums.
+template <int QB, bool SUM>
 __global__ void __launch_bounds__(256, 3)
     block_update_kernel(const float2 *__restrict__ S, long ss, const double2 *__restrict__ Cm, long sc,
                         float2 *__restrict__ Y, long sy, const float2 *__restrict__ Z, long sz, long L, int p, int q,
-                        const int *__restrict__ act) {
+                        const int *__restrict__ act, const float2 *__restrict__ S2, const double2 *__restrict__ Cm2) {
   __shared__ float2 Cs[UPD_PMAX][QB];
   const int b = act ? act[blockIdx.z] : (int)blockIdx.z;
   const int j0 = blockIdx.y * QB;
-  const double2 *Cb = Cm + (long)b * sc;
-  for (int i = threadIdx.x; i < p * QB; i += blockDim.x) {
-    const int r = i / QB, c = i - r * QB;
-    const double2 v = (j0 + c < q) ? Cb[r * q + j0 + c] : cmake<double2>(0.0, 0.0);
-    Cs[r][c] = make_float2((float)v.x, (float)v.y);
-  }
-  __syncthreads();
   const long l = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (l >= L) return;
-  const float2 *Sb = S + (long)b * ss;
   float2 acc[QB];
 #pragma unroll
   for (int c = 0; c < QB; ++c) acc[c] = make_float2(0.f, 0.f);
-  for (int i = 0; i < p; ++i) {
-    const float2 sv = Sb[(long)i * L + l];
 #pragma unroll
-    for (int c = 0; c < QB; ++c) {
-      const float2 cv = Cs[i][c];
-      acc[c].x = fmaf(sv.x, cv.x, fmaf(-sv.y, cv.y, acc[c].x));
-      acc[c].y = fmaf(sv.x, cv.y, fmaf(sv.y, cv.x, acc[c].y));
+  for (int pass = 0; pass < (SUM ? 2 : 1); ++pass) {
+    const double2 *Cb = (pass ? Cm2 : Cm) + (long)b * sc;
+    if (pass) __syncthreads();
+    for (int i = threadIdx.x; i < p * QB; i += blockDim.x) {
+      const int r = i / QB, c = i - r * QB;
+      const double2 v = (j0 + c < q) ? Cb[r * q + j0 + c] : cmake<double2>(0.0, 0.0);
+      Cs[r][c] = make_float2((float)v.x, (float)v.y);
+    }
+    __syncthreads();
+    if (l >= L) continue;
+    const float2 *Sb = (pass ? S2 : S) + (long)b * ss;
+    for (int i = 0; i < p; ++i) {
+      const float2 sv = Sb[(long)i * L + l];
+#pragma unroll
+      for (int c = 0; c < QB; ++c) {
+        const float2 cv = Cs[i][c];
+        acc[c].x = fmaf(sv.x, cv.x, fmaf(-sv.y, cv.y, acc[c].x));
+        acc[c].y = fmaf(sv.x, cv.y, fmaf(sv.y, cv.x, acc[c].y));
+      }
     }
   }
+  if (l >= L) return;
   float2 *Yb = Y + (long)b * sy;
   const float2 *Zb = Z ? Z + (long)b * sz : nullptr;
 #pragma unroll
@@ -609,19 +615,24 @@ __global__ void __launch_bounds__(256, 2)
 template <int QB>
 static void block_update_c64(int nb, long L, int p, int q, const void *S, long ss, const void *C, long sc, void *Y,
                              long sy, cudaStream_t st, const int *act, const void *Z, long sz) {
-  // two rows a thread once that leaves two blocks per SM (8 k-points x 1536 rows, 39 -> 12: 18 us with one row, 23 with two)
-  const uintptr_t at = (uintptr_t)S | (uintptr_t)Y | (uintptr_t)Z;
-  const dim3 g((unsigned)((L / 2 + 255) / 256), (unsigned)((q + QB - 1) / QB), nb);
-  if (((L | ss | sy | sz) & 1) == 0 && (at & 15) == 0 && (long)g.x * g.y * g.z >= 2L * sm_count()) {
-    block_update2_kernel<QB><<<g, 256, 0, st>>>(static_cast<const float2 *>(S), ss, static_cast<const double2 *>(C), sc,
-                                                static_cast<float2 *>(Y), sy, static_cast<const float2 *>(Z), sz, L, p,
-                                                q, act, nullptr, nullptr);
-    return;
+  // Two rows a thread from 16 outputs and two blocks per SM on. 2 k-points at N = 64, with one row and two: 57 -> 16, 20
+  // and 24 columns 469 and 384, 515 and 416, 531 and 428 us, but 57 -> 8 and 12 columns 203 and 349, 241 and 365 us: the
+  // loads of few outputs are what takes the time there, and one row a thread has more of them in flight. 8 k-points x 1536
+  // rows, 39 -> 12: 18 us with one row, 23 with two.
+  if constexpr (QB >= 16) {
+    const uintptr_t at = (uintptr_t)S | (uintptr_t)Y | (uintptr_t)Z;
+    const dim3 g((unsigned)((L / 2 + 255) / 256), (unsigned)((q + QB - 1) / QB), nb);
+    if (((L | ss | sy | sz) & 1) == 0 && (at & 15) == 0 && (long)g.x * g.y * g.z >= 2L * sm_count()) {
+      block_update2_kernel<QB><<<g, 256, 0, st>>>(static_cast<const float2 *>(S), ss, static_cast<const double2 *>(C), sc,
+                                                  static_cast<float2 *>(Y), sy, static_cast<const float2 *>(Z), sz, L, p,
+                                                  q, act, nullptr, nullptr);
+      return;
+    }
   }
   const dim3 grid((unsigned)((L + 255) / 256), (unsigned)((q + QB - 1) / QB), nb);
-  block_update_kernel<QB><<<grid, 256, 0, st>>>(static_cast<const float2 *>(S), ss, static_cast<const double2 *>(C), sc,
-                                                static_cast<float2 *>(Y), sy, static_cast<const float2 *>(Z), sz, L, p, q,
-                                                act);
+  block_update_kernel<QB, false><<<grid, 256, 0, st>>>(static_cast<const float2 *>(S), ss,
+                                                       static_cast<const double2 *>(C), sc, static_cast<float2 *>(Y), sy,
+                                                       static_cast<const float2 *>(Z), sz, L, p, q, act, nullptr, nullptr);
 }
 
 // the column-group width for q outputs among `widths`: fewest idle columns, then fewest groups
@@ -670,27 +681,23 @@ int launch_block_update(int nb, long L, int p, int q, int dtype, const void *S, 
   return PC_OK;
 }
 
-// Y = S C + S2 C2, complex64, p <= 64 columns each (q <= 16: one pass over S and S2; the general shapes in two)
+// Y = S C + S2 C2, complex64, p <= 64 columns each: in one pass over S and S2 up to 16 outputs (with the rows a thread that
+// block_update_c64 takes for them), otherwise in two
 int launch_block_update_sum(int nb, long L, int p, int q, const void *S, const void *C, const void *S2, const void *C2,
                             long ss, long sc, void *Y, long sy, cudaStream_t st) {
   if (nb == 0 || q == 0) return PC_OK;
   const uintptr_t at = (uintptr_t)S | (uintptr_t)S2 | (uintptr_t)Y;
-  if (p > UPD_PMAX || q > 16 || ((L | ss | sy) & 1) || (at & 15)) {
+  const bool two_rows = q > 12;
+  if (p > UPD_PMAX || q > 16 || (two_rows && (((L | ss | sy) & 1) || (at & 15)))) {
     const int rc = launch_block_update(nb, L, p, q, PC_C64, S, ss, C, sc, Y, sy, st, nullptr, nullptr);
     return rc ? rc : launch_block_update(nb, L, p, q, PC_C64, S2, ss, C2, sc, Y, sy, st, nullptr, nullptr, Y, sy);
   }
-  const dim3 g((unsigned)((L / 2 + 255) / 256), 1, nb);
-  auto run = [&](auto kernel) {
-    kernel<<<g, 256, 0, st>>>(static_cast<const float2 *>(S), ss, static_cast<const double2 *>(C), sc,
-                              static_cast<float2 *>(Y), sy, nullptr, 0, L, p, q, nullptr,
-                              static_cast<const float2 *>(S2), static_cast<const double2 *>(C2));
-  };
-  if (q <= 8)
-    run(block_update2_kernel<8>);
-  else if (q <= 12)
-    run(block_update2_kernel<12>);
-  else
-    run(block_update2_kernel<16>);
+  const dim3 g((unsigned)(((two_rows ? L / 2 : L) + 255) / 256), 1, nb);
+  const auto kernel = q <= 8 ? block_update_kernel<8, true>
+                             : (two_rows ? block_update2_kernel<16> : block_update_kernel<12, true>);
+  kernel<<<g, 256, 0, st>>>(static_cast<const float2 *>(S), ss, static_cast<const double2 *>(C), sc,
+                            static_cast<float2 *>(Y), sy, nullptr, 0, L, p, q, nullptr, static_cast<const float2 *>(S2),
+                            static_cast<const double2 *>(C2));
   PC_CK_LAUNCH();
   return PC_OK;
 }

@@ -16,7 +16,7 @@ def pcmod():
     return p
 
 
-@pytest.mark.parametrize("N,nb,S", [(16, 3, 2), (32, 8, 3)])
+@pytest.mark.parametrize("N,nb,S", [(16, 3, 2), (32, 8, 3), (16, 10, 2), (16, 16, 2)])
 def test_x_offset_by_one_element(pcmod, N, nb, S):
     from paper_2503_19379_gb300 import pc
     g = np.random.default_rng(N)
