@@ -27,7 +27,7 @@
 // seven left 5.4e-14 where C is near the identity).
 //
 // Bound: instructions of the digit extraction and the epilogue. Complex128, 8 k-points, 48 -> 16 columns at N = 32:
-// 4.00 ms on the FP64 pipe (1.21 TFLOP/s, all of it), 0.48 ms here (EACH: 0.51 ms for smooth fields and dense C; 2.1 ms
+// 4.00 ms on the FP64 pipe (1.21 TFLOP/s, all of it), 0.48 ms here (EACH: 0.52 ms for smooth fields and dense C; 2.1 ms
 // for C near the identity, where a fifth of the outputs takes FP64); 4 k-points, 57 -> 19 at N = 64: 27.5 and 2.7 ms; one
 // k-point, 24 -> 8 at N = 16: 54.8 and 17.0 us; the smallest size tried (8 -> 4 columns of 1536 rows): 21.9 and 17.9 us.
 // Pairs, 4 k-points, 19 -> 19 columns at N = 64: 2.03 ms in double-float arithmetic, 1.16 ms here (without the MMAs
